@@ -158,7 +158,8 @@ __global__ void compact_kernel(int64_t k_total, const uint32_t* __restrict__ fla
   out_val[o] = static_cast<uint32_t>(slot);
 }
 
-constexpr int kRB = 64;  // list entries staged per round
+constexpr int kRB = kTilePixels;  // list entries staged per step: one per thread
+constexpr int kGroup = 64;        // staged entries screened at once per pixel (two mask words)
 constexpr int kDeepTest = 256;  // re-checked Gaussians a deep tile tests per pixel at most
 
 // Float-pair constants of the compositing rule (Sec. 3.1 Eq. 1 conventions).
@@ -166,91 +167,150 @@ constexpr double kAlphaMinD = 1.0 / 255.0, kAlphaMaxD = 0.99, kTMinD = 1e-4;
 constexpr double kLn2D = 0.69314718055994530942;
 #define FS_F2C(d) f2{static_cast<float>(d), static_cast<float>((d) - static_cast<double>(static_cast<float>(d)))}
 
-// 2^-q for q >= 0 as a float pair (about 1e-11 relative): q = k + j/64 + s,
+// One row of w = W l + b at the pixel offset l (exact small half-integers) as
+// a float pair: the products' and sums' rounding errors are gathered in one
+// float and put back once (a compensated dot product, Ogita, Rump and Oishi
+// 2005), about 25 operations where a chain of float-pair products and sums
+// takes 34.
+__device__ __forceinline__ f2 f2_row(float wh0, float wl0, float wh1, float wl1, float bh,
+                                     float bl, float lx, float ly) {
+  const f2 p0 = two_prod(wh0, lx), p1 = two_prod(wh1, ly);
+  const f2 s = two_sum(p0.hi, p1.hi);
+  const f2 u = two_sum(s.hi, bh);
+  float err = __fadd_rn(p0.lo, p1.lo);
+  err = __fmaf_rn(wl0, lx, err);
+  err = __fmaf_rn(wl1, ly, err);
+  err = __fadd_rn(err, s.lo);
+  err = __fadd_rn(err, u.lo);
+  err = __fadd_rn(err, bl);
+  return fast_two_sum(u.hi, err);
+}
+
+// a^2 + b^2 of float pairs, likewise with one gathered error.
+__device__ __forceinline__ f2 f2_norm2(f2 a, f2 b) {
+  const f2 p0 = two_prod(a.hi, a.hi), p1 = two_prod(b.hi, b.hi);
+  const f2 s = two_sum(p0.hi, p1.hi);
+  float err = __fadd_rn(p0.lo, p1.lo);
+  err = __fmaf_rn(a.hi + a.hi, a.lo, err);
+  err = __fmaf_rn(b.hi + b.hi, b.lo, err);
+  err = __fadd_rn(err, s.lo);
+  return fast_two_sum(s.hi, err);
+}
+
+// o 2^-q for q >= 0 as a float pair (about 1e-11 relative): q = k + j/64 + s,
 // 2^-q = 2^-k * 2^(-j/64) * e^(-s ln 2) with a degree-4 Taylor polynomial of
-// e^-x for x = s ln 2 in [0, ln2/64) (truncation below 1.3e-12).
-__device__ __forceinline__ f2 f2_exp2_neg(f2 q, const float2* __restrict__ tab) {
+// e^-x for x = s ln 2 in [0, ln2/64) (truncation below 1.3e-12).  x and the
+// product with the table stay unnormalised (hi, lo) pairs; the polynomial
+// takes x's low part to first order.
+__device__ __forceinline__ f2 f2_exp2_neg(f2 q, float o, const float2* __restrict__ tab) {
   const float k = floorf(q.hi);
   const float r = q.hi - k;                        // exact
   const float jf = floorf(r * 64.f);
   const float s = r - jf * (1.f / 64.f);           // exact (Sterbenz)
-  const f2 t = two_sum(s, q.lo);
-  const f2 x = f2_mul(t, FS_F2C(kLn2D));
-  const float xh = x.hi;
-  const float p = xh * xh * fmaf(xh, fmaf(xh, 1.f / 24.f, -1.f / 6.f), 0.5f);
-  f2 e = f2_add(f2_from(1.f), f2_neg(x));
-  e = f2_add(e, f2_from(p));
+  const f2 t = fast_two_sum(s, q.lo);              // s is 0 or a multiple of ulp(q.hi)
+  const f2 ln2 = FS_F2C(kLn2D);
+  const float xh = __fmul_rn(t.hi, ln2.hi);
+  float xl = __fmaf_rn(t.hi, ln2.hi, -xh);
+  xl = __fmaf_rn(t.hi, ln2.lo, xl);
+  xl = __fmaf_rn(t.lo, ln2.hi, xl);
+  float p = xh * xh * fmaf(xh, fmaf(xh, 1.f / 24.f, -1.f / 6.f), 0.5f);
+  p = __fmaf_rn(xh, xl, p);
+  const f2 e0 = fast_two_sum(1.f, -xh);
+  const f2 e1 = fast_two_sum(e0.hi, p);
+  const float el = __fadd_rn(e1.lo, __fsub_rn(e0.lo, xl));
   const float2 tj = tab[static_cast<int>(jf)];
-  e = f2_mul(e, f2{tj.x, tj.y});
-  const float sc = __int_as_float((127 - static_cast<int>(k)) << 23);  // 2^-k, k <= 126
-  return {e.hi * sc, e.lo * sc};
+  const float mh = __fmul_rn(e1.hi, tj.x);
+  float ml = __fmaf_rn(e1.hi, tj.x, -mh);
+  ml = __fmaf_rn(e1.hi, tj.y, ml);
+  ml = __fmaf_rn(el, tj.x, ml);
+  const float os = o * __int_as_float((127 - static_cast<int>(k)) << 23);  // o 2^-k, k <= 126
+  f2 a = two_prod(mh, os);
+  a.lo = __fmaf_rn(ml, os, a.lo);
+  return fast_two_sum(a.hi, a.lo);
 }
 
-// Staged list entry: W (float pairs), b = W (ctr - m) relative to the tile
-// centre (float pairs), opacity, q_cut + slack, re-check row (-1: none).
-struct Staged {
-  f2 w[4];
-  f2 b[2];
-  float o, qc;
-  int j;
+// Staged list entries, one array per 16-byte part so that lanes that read
+// different entries spread over the banks: W (hi and lo parts), b = W (ctr - m)
+// relative to the tile centre, the cut with slack, the opacity and the
+// re-check row (-1: none).
+struct Stage {
+  float4 w_hi[kRB];
+  float4 w_lo[kRB];
+  float4 bq[kRB];  // (b0 hi, b1 hi, q_cut + slack, opacity)
+  float2 b_lo[kRB];
+  int j[kRB];
 };
 
-__device__ __forceinline__ Staged stage_entry(const ProjRecord& r, float cx, float cy, int j) {
-  Staged st;
-  st.w[0] = {r.w_hi.x, r.w_lo.x};
-  st.w[1] = {r.w_hi.y, r.w_lo.y};
-  st.w[2] = {r.w_hi.z, r.w_lo.z};
-  st.w[3] = {r.w_hi.w, r.w_lo.w};
+__device__ __forceinline__ void stage_entry(Stage& S, int e, const ProjRecord& r, float cx,
+                                            float cy, int j) {
+  const f2 w0 = {r.w_hi.x, r.w_lo.x}, w1 = {r.w_hi.y, r.w_lo.y};
+  const f2 w2 = {r.w_hi.z, r.w_lo.z}, w3 = {r.w_hi.w, r.w_lo.w};
   // b = W (ctr - m) with the difference of the centre and the float-pair mean
   const f2 dx = f2_sub(f2_from(cx), f2{r.m.x, r.m.z});
   const f2 dy = f2_sub(f2_from(cy), f2{r.m.y, r.m.w});
-  st.b[0] = f2_add(f2_mul(st.w[0], dx), f2_mul(st.w[1], dy));
-  st.b[1] = f2_add(f2_mul(st.w[2], dx), f2_mul(st.w[3], dy));
-  st.o = r.misc.x;
+  const f2 b0 = f2_add(f2_mul(w0, dx), f2_mul(w1, dy));
+  const f2 b1 = f2_add(f2_mul(w2, dx), f2_mul(w3, dy));
+  S.w_hi[e] = r.w_hi;
+  S.w_lo[e] = r.w_lo;
   // near the cut the FP32 screen |W_hi l + b_hi|^2 is off by far less than 0.05
-  st.qc = r.misc.y + 0.05f;
-  st.j = j;
-  return st;
+  S.bq[e] = make_float4(b0.hi, b1.hi, r.misc.y + 0.05f, r.misc.x);
+  S.b_lo[e] = make_float2(b0.lo, b1.lo);
+  S.j[e] = j;
 }
 
 // Reduced-precision record: W16 and the FP32 mean are exact float values, so
 // b = W (ctr - m) is formed from the exact difference in float pairs.
-__device__ __forceinline__ Staged stage_compact(const CompactRecord& r, float o, float cx,
-                                                float cy, int j) {
-  Staged st;
+__device__ __forceinline__ void stage_compact(Stage& S, int e, const CompactRecord& r, float o,
+                                              float cx, float cy, int j) {
   const float2 wa = __half22float2(*reinterpret_cast<const __half2*>(&r.w01));
   const float2 wb = __half22float2(*reinterpret_cast<const __half2*>(&r.w23));
-  st.w[0] = f2_from(wa.x);
-  st.w[1] = f2_from(wa.y);
-  st.w[2] = f2_from(wb.x);
-  st.w[3] = f2_from(wb.y);
   const f2 dx = two_sum(cx, -r.mx), dy = two_sum(cy, -r.my);
-  st.b[0] = f2_add(f2_mul(st.w[0], dx), f2_mul(st.w[1], dy));
-  st.b[1] = f2_add(f2_mul(st.w[2], dx), f2_mul(st.w[3], dy));
-  st.o = o;
-  st.qc = fmaxf(log2f(255.f * o), 0.f) * 1.001f + 1e-3f + 0.05f;
-  st.j = j;
-  return st;
+  const f2 b0 = f2_add(f2_mul_f(dx, wa.x), f2_mul_f(dy, wa.y));
+  const f2 b1 = f2_add(f2_mul_f(dx, wb.x), f2_mul_f(dy, wb.y));
+  S.w_hi[e] = make_float4(wa.x, wa.y, wb.x, wb.y);
+  S.w_lo[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  S.bq[e] = make_float4(b0.hi, b1.hi, fmaxf(log2f(255.f * o), 0.f) * 1.001f + 1e-3f + 0.05f, o);
+  S.b_lo[e] = make_float2(b0.lo, b1.lo);
+  S.j[e] = j;
 }
 
 // FP32 screen: can the entry's alpha >= 1/255 region reach this pixel?
-__device__ __forceinline__ bool reaches(const Staged& e, float lx, float ly) {
-  const float q0 = fmaf(e.w[0].hi, lx, fmaf(e.w[1].hi, ly, e.b[0].hi));
-  const float q1 = fmaf(e.w[2].hi, lx, fmaf(e.w[3].hi, ly, e.b[1].hi));
-  return fmaf(q0, q0, q1 * q1) <= e.qc;
+__device__ __forceinline__ bool reaches(const Stage& S, int e, float lx, float ly) {
+  const float4 w = S.w_hi[e], b = S.bq[e];
+  const float q0 = fmaf(w.x, lx, fmaf(w.y, ly, b.x));
+  const float q1 = fmaf(w.z, lx, fmaf(w.w, ly, b.y));
+  return fmaf(q0, q0, q1 * q1) <= b.z;
 }
 
-// One CTA per 16x16 tile of a view, one thread per pixel.  Pass 1 finds, per
-// pixel, the last list position holding a re-checked Gaussian that can reach
-// the pixel; pass 2 composites the pixel in float pairs up to that position
-// (deep tiles: up to its stop).
+// Bit k: staged entry e0 + k (k < 32, e0 + k < count) reaches the pixel.  The
+// staging array is read past `count` (its old entries, masked off here).
+__device__ __forceinline__ uint32_t reach_mask(const Stage& S, int e0, int count, float lx,
+                                               float ly) {
+  if (e0 >= count) return 0u;
+  uint32_t m = 0u;
+#pragma unroll 8
+  for (int k = 0; k < 32; ++k) m |= reaches(S, e0 + k, lx, ly) ? 1u << k : 0u;
+  return count - e0 >= 32 ? m : m & ((1u << (count - e0)) - 1u);
+}
+
+// One CTA per 16x16 tile of a view, one thread per pixel (warps of 8x4
+// pixels).  Pass 1 finds, per pixel, the last list position holding a
+// re-checked Gaussian that can reach the pixel; pass 2 composites the pixel
+// in float pairs up to that position (deep tiles: up to its stop).
+//
+// The work is the ~130 FP32 operations of a (pixel, entry) pair, and an entry
+// covers only some of a warp's pixels.  So a pixel first collects the staged
+// entries that reach it, 64 at a time, in a bit mask (about ten operations an
+// entry), and then walks its own bits: lanes work on different entries at the
+// same time and a warp takes as many steps as its busiest pixel has entries,
+// not as many as its pixels have between them.
 template <typename LabelT>
-__global__ void __launch_bounds__(kTilePixels, 6) recheck_blend_kernel(
+__global__ void __launch_bounds__(kTilePixels, 4) recheck_blend_kernel(
     const ViewParams* __restrict__ views, RecheckLists L, const uint64_t* __restrict__ skip,
     const ProjRecord* __restrict__ rec, const CompactRecord* __restrict__ rec16,
     const float4* __restrict__ pos_op, int64_t n, int E, const int32_t* __restrict__ map,
     double* __restrict__ R, unsigned long long* __restrict__ counters) {
-  __shared__ Staged s_e[kRB];
+  __shared__ Stage S;
   __shared__ float2 s_tab[64];
   const ViewParams& vp = views[blockIdx.y];
   const int tile = blockIdx.x;
@@ -266,9 +326,10 @@ __global__ void __launch_bounds__(kTilePixels, 6) recheck_blend_kernel(
     const float hi = static_cast<float>(d);
     s_tab[threadIdx.x] = make_float2(hi, static_cast<float>(d - static_cast<double>(hi)));
   }
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int x0 = (tile % vp.tiles_x) * kTile, y0 = (tile / vp.tiles_x) * kTile;
-  const int x = x0 + (threadIdx.x & (kTile - 1));
-  const int y = y0 + (threadIdx.x / kTile);
+  const int x = x0 + 8 * (warp & 1) + (lane & 7);
+  const int y = y0 + 4 * (warp >> 1) + (lane >> 3);
   int label = -1;
   if (x < vp.width && y < vp.height) {
     const int l = static_cast<int>(
@@ -280,28 +341,35 @@ __global__ void __launch_bounds__(kTilePixels, 6) recheck_blend_kernel(
   // pixel centre (x + 0.5, y + 0.5) relative to the tile centre: exact
   const float lx = static_cast<float>(x - x0) + 0.5f - 0.5f * kTile;
   const float ly = static_cast<float>(y - y0) + 0.5f - 0.5f * kTile;
+  // the slots of a view are view * n + index
+  const uint32_t slot0 = static_cast<uint32_t>(static_cast<int64_t>(blockIdx.y) * n);
+  auto stage = [&](uint32_t slot, int j) {
+    if (rec16)
+      stage_compact(S, tid, rec16[slot], pos_op[slot - slot0].w, cx, cy, j);
+    else
+      stage_entry(S, tid, rec[slot], cx, cy, j);
+  };
 
-  // pass 1: last re-checked entry (chunk << 32 | index) that may reach the pixel
+  // pass 1: last re-checked entry (chunk << 32 | index) that may reach the
+  // pixel.  Re-checked entries are rare: a step without one costs its loads
+  // and one barrier.
   int64_t last = -1;
   for (int c = 0; c < n_chunks; ++c) {
     const uint2 rg = L.ranges[c][gtile];
     for (uint32_t b0 = rg.x; b0 < rg.y; b0 += kRB) {
-      const int cnt = static_cast<int>(min(static_cast<uint32_t>(kRB), rg.y - b0));
+      const uint32_t at = b0 + tid;
+      const uint32_t slot = at < rg.y ? L.val[c][at] : slot0;
+      const int j = at < rg.y ? map[slot - slot0] : -1;
+      if (__syncthreads_or(j >= 0) == 0) continue;
+      S.j[tid] = j;
+      if (j >= 0) stage(slot, j);
       __syncthreads();
-      if (threadIdx.x < cnt) {
-        const uint32_t slot = L.val[c][b0 + threadIdx.x];
-        const uint32_t gi = static_cast<uint32_t>(slot % static_cast<uint64_t>(n));
-        const int j = map[gi];
-        s_e[threadIdx.x].j = j;
-        if (j >= 0)
-          s_e[threadIdx.x] = rec16 ? stage_compact(rec16[slot], pos_op[gi].w, cx, cy, j)
-                                   : stage_entry(rec[slot], cx, cy, j);
+      if (label >= 0) {
+        const int cnt = static_cast<int>(min(static_cast<uint32_t>(kRB), rg.y - b0));
+        for (int e = 0; e < cnt; ++e)
+          if (S.j[e] >= 0 && reaches(S, e, lx, ly)) last = (static_cast<int64_t>(c) << 32) | (b0 + e);
       }
       __syncthreads();
-      if (label >= 0)
-        for (int e = 0; e < cnt; ++e)
-          if (s_e[e].j >= 0 && reaches(s_e[e], lx, ly))
-            last = (static_cast<int64_t>(c) << 32) | (b0 + e);
     }
   }
 
@@ -314,17 +382,14 @@ __global__ void __launch_bounds__(kTilePixels, 6) recheck_blend_kernel(
     for (int k0 = 0; k0 < L.n_flagged; k0 += kRB) {
       const int cnt = min(kRB, L.n_flagged - k0);
       __syncthreads();
-      if (threadIdx.x < cnt) {
-        const uint32_t gi = L.flagged[k0 + threadIdx.x];
-        const int64_t slot = static_cast<int64_t>(blockIdx.y) * n + gi;
-        s_e[threadIdx.x].j = -1;
-        if (L.cnt[slot])
-          s_e[threadIdx.x] = rec16 ? stage_compact(rec16[slot], pos_op[gi].w, cx, cy, 0)
-                                   : stage_entry(rec[slot], cx, cy, 0);
+      if (tid < cnt) {
+        const uint32_t slot = slot0 + L.flagged[k0 + tid];
+        S.j[tid] = -1;
+        if (L.cnt[slot]) stage(slot, 0);
       }
       __syncthreads();
       for (int e = 0; e < cnt; ++e)
-        if (s_e[e].j >= 0 && reaches(s_e[e], lx, ly)) reached = true;
+        if (S.j[e] >= 0 && reaches(S, e, lx, ly)) reached = true;
     }
     deep_px = reached;
   }
@@ -339,46 +404,64 @@ __global__ void __launch_bounds__(kTilePixels, 6) recheck_blend_kernel(
   for (int c = 0; c < n_chunks && !done_all; ++c) {
     const uint2 rg = L.ranges[c][gtile];
     for (uint32_t b0 = rg.x; b0 < rg.y; b0 += kRB) {
-      if (__syncthreads_count(live) == 0) {
+      if (__syncthreads_or(live) == 0) {
         done_all = true;
         break;
       }
       const int cnt = static_cast<int>(min(static_cast<uint32_t>(kRB), rg.y - b0));
-      if (threadIdx.x < cnt) {
-        const uint32_t slot = L.val[c][b0 + threadIdx.x];
-        const uint32_t gi = static_cast<uint32_t>(slot % static_cast<uint64_t>(n));
-        s_e[threadIdx.x] = rec16 ? stage_compact(rec16[slot], pos_op[gi].w, cx, cy, map[gi])
-                                 : stage_entry(rec[slot], cx, cy, map[gi]);
+      if (tid < cnt) {
+        const uint32_t slot = L.val[c][b0 + tid];
+        stage(slot, map[slot - slot0]);
       }
       __syncthreads();
-      if (live) {
-        const int64_t pos0 = (static_cast<int64_t>(c) << 32) | b0;
-        int e_end = cnt;
-        if (!to_stop) e_end = static_cast<int>(min(static_cast<int64_t>(cnt), last - pos0 + 1));
-        for (int e = 0; e < e_end; ++e) {
-          const Staged& en = s_e[e];
-          if (!reaches(en, lx, ly)) continue;  // alpha < 1/255 in any precision
-          ++evals;
-          const f2 w0 = f2_add(f2_add(f2_mul_f(en.w[0], lx), f2_mul_f(en.w[1], ly)), en.b[0]);
-          const f2 w1 = f2_add(f2_add(f2_mul_f(en.w[2], lx), f2_mul_f(en.w[3], ly)), en.b[1]);
-          const f2 q = f2_add(f2_mul(w0, w0), f2_mul(w1, w1));
-          f2 a = f2_mul_f(f2_exp2_neg(q, s_tab), en.o);
+      // the pixel's entries of this step: all of them, or up to its last one
+      const int64_t pos0 = (static_cast<int64_t>(c) << 32) | b0;
+      const int e_end =
+          to_stop ? cnt : static_cast<int>(min(static_cast<int64_t>(cnt), last - pos0 + 1));
+      for (int g0 = 0; g0 < cnt; g0 += kGroup) {
+        if (!__any_sync(0xffffffffu, live && g0 < e_end)) break;
+        uint32_t m0 = 0u, m1 = 0u;
+        if (live) {
+          m0 = reach_mask(S, g0, e_end, lx, ly);
+          m1 = reach_mask(S, g0 + 32, e_end, lx, ly);
+        }
+        evals += __popc(m0) + __popc(m1);
+        while (m0 | m1) {
+          int e = g0;
+          if (m0) {
+            e += __ffs(m0) - 1;
+            m0 &= m0 - 1u;
+          } else {
+            e += 31 + __ffs(m1);
+            m1 &= m1 - 1u;
+          }
+          const float4 wh = S.w_hi[e], wl = S.w_lo[e], bq = S.bq[e];
+          const float2 bl = S.b_lo[e];
+          const f2 w0 = f2_row(wh.x, wl.x, wh.y, wl.y, bq.x, bl.x, lx, ly);
+          const f2 w1 = f2_row(wh.z, wl.z, wh.w, wl.w, bq.y, bl.y, lx, ly);
+          f2 a = f2_exp2_neg(f2_norm2(w0, w1), bq.w, s_tab);
           if (f2_lt(a_max, a)) a = a_max;
           if (f2_lt(a, a_min)) continue;
-          const f2 t = f2_mul(T, f2_sub(f2_from(1.f), a));
+          // T (1 - a): 1 - a needs no normalisation for the product
+          const f2 om = fast_two_sum(1.f, -a.hi);
+          f2 t = two_prod(T.hi, om.hi);
+          t.lo = __fmaf_rn(T.hi, __fsub_rn(om.lo, a.lo), __fmaf_rn(T.lo, om.hi, t.lo));
+          t = fast_two_sum(t.hi, t.lo);
           if (f2_lt(t, t_min)) {
             live = false;
+            evals -= __popc(m0) + __popc(m1);  // not reached
             break;
           }
-          if (en.j >= 0) {
+          const int j = S.j[e];
+          if (j >= 0) {
             const f2 ct = f2_mul(a, T);
-            atomicAdd(&R[static_cast<int64_t>(en.j) * E + label],
+            atomicAdd(&R[static_cast<int64_t>(j) * E + label],
                       static_cast<double>(ct.hi) + static_cast<double>(ct.lo));
           }
           T = t;
         }
-        if (live && !to_stop && pos0 + cnt > last) live = false;
       }
+      if (live && !to_stop && pos0 + cnt > last) live = false;
     }
   }
   // still compositing where a saturated tile's kept lists end: the exact
