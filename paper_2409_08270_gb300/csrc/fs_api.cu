@@ -198,7 +198,7 @@ struct fs_ctx {
   bool compact = false;  // reduced-precision records (FP16 whitening matrix, FP32 mean)
   bool census = false;   // blend counts its pairs (slower variant)
   bool sigma3 = false;   // 3-sigma tile coverage (per-slot tile columns in `cols`)
-  DevBuf dkey, rk_flag, rk_offs, rk_F, rk_map, rk_R, rk_Rb, cols;
+  DevBuf dkey, rk_flag, rk_offs, rk_F, rk_map, rk_R, rk_Rb, rk_tiles, cols;
   DevBuf rd_flag, rd_offs, rd_val, render_out;  // novel-view mask rendering
   DevBuf chunk_bnd;                             // captured solves: chunk boundaries
   HostBuf render_out_host;
@@ -237,7 +237,7 @@ DevBuf* const* workspace_bufs(fs_ctx* c, size_t* count) {
                     &c->lv_a, &c->lk_b, &c->lv_b, &c->ranges, &c->sort_tmp, &c->scan_tmp,
                     &c->mask_stage, &c->table_tmp, &c->table32_tmp, &c->bits_tmp,
                     &c->label_tmp, &c->margin_tmp, &c->dkey, &c->rk_flag, &c->rk_offs,
-                    &c->rk_F, &c->rk_map, &c->rk_R, &c->rk_Rb, &c->kl_ranges, &c->kl_satc,
+                    &c->rk_F, &c->rk_map, &c->rk_R, &c->rk_Rb, &c->rk_tiles, &c->kl_ranges, &c->kl_satc,
                     &c->kl_bound, &c->key_range, &c->lb_tmp, &c->key_a2, &c->val_a2,
                     &c->key_b2, &c->val_b2, &c->cols, &c->rd_flag, &c->rd_offs, &c->rd_val,
                     &c->render_out, &c->chunk_bnd, &c->free_tab};
@@ -344,7 +344,8 @@ fs_status fs_destroy(fs_ctx* c) {
                     &c->sort_tmp, &c->scan_tmp, &c->total, &c->counters, &c->mask_stage,
                     &c->table_tmp, &c->table32_tmp, &c->bits_tmp, &c->label_tmp, &c->margin_tmp,
                     &c->dkey, &c->rk_flag, &c->rk_offs, &c->rk_F, &c->rk_map, &c->rk_R,
-                    &c->rk_Rb, &c->kl_ranges, &c->kl_satc, &c->kl_bound, &c->key_range, &c->lb_tmp,
+                    &c->rk_Rb, &c->rk_tiles, &c->kl_ranges, &c->kl_satc, &c->kl_bound, &c->key_range,
+                    &c->lb_tmp,
                     &c->key_a2, &c->val_a2, &c->key_b2, &c->val_b2, &c->cols,
                     &c->rd_flag, &c->rd_offs, &c->rd_val, &c->render_out, &c->chunk_bnd,
                     &c->free_tab};
@@ -1038,7 +1039,8 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
 fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, int64_t kcap,
                               const BatchLayout& L, const fs::ViewParams* vd, const ProjPtrs& P,
                               const uint32_t* key_src, uint64_t* skip, int32_t mask_dtype,
-                              int32_t E, const int32_t* map, double* R, cudaStream_t stream) {
+                              int32_t E, const uint32_t* F, int64_t nF, const int32_t* map,
+                              double* R, cudaStream_t stream) {
   const int total_tiles = L.total_tiles;
   const int tile_bits = std::max(1, ceil_log2(total_tiles));
   const int64_t k_total = static_cast<int64_t>(nb) * n;
@@ -1073,8 +1075,12 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
   Ls.val[0] = c->lv_a.as<uint32_t>();
   Ls.ranges[0] = c->ranges.as<uint2>();
   Ls.chunks = 1;
-  c->stats.kernel_launches += 1;
-  FS_CUDA(fs::launch_recheck_blend(vd, nb, L.max_tiles, Ls, skip, P.rec, P.rec16,
+  Ls.flagged = F;
+  Ls.n_flagged = static_cast<int>(std::min<int64_t>(nF, 0x7FFFFFFF));
+  Ls.cnt = P.cnt;
+  Ls.foot = P.foot;
+  c->stats.kernel_launches += 2;
+  FS_CUDA(fs::launch_recheck_blend(vd, nb, L.max_tiles, Ls, skip, c->rk_tiles.p, c->n_sm, P.rec, P.rec16,
                                    s->pos_op.as<float4>(), n, E, mask_dtype, map, R, ctr, stream),
           "re-check blend");
   return FS_OK;
@@ -1144,6 +1150,7 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
     FS_TRY(c->sat.ensure(sat_bytes, "tile flags"));
     FS_TRY(c->subsat.ensure(sat_bytes, "deep tile flags"));
     FS_TRY(c->ranges.ensure(static_cast<size_t>(total_tiles) * 8, "tile ranges"));
+    FS_TRY(c->rk_tiles.ensure(fs::recheck_tiles_bytes(total_tiles), "re-check tiles"));
     fs::ViewParams* vd = c->views.as<fs::ViewParams>();
     uint64_t* skip = c->sat.as<uint64_t>();
     uint64_t* deep = c->subsat.as<uint64_t>();
@@ -1186,11 +1193,12 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
       Ls.flagged = F;
       Ls.n_flagged = static_cast<int>(std::min<int64_t>(nF, 0x7FFFFFFF));
       Ls.cnt = P.cnt;
+      Ls.foot = P.foot;
       FS_CUDA(cudaMemsetAsync(Rb, 0, rbytes, stream), "batch rows clear");
       FS_CUDA(cudaMemsetAsync(ctr + fs::kRecheckIncomplete, 0, 8, stream), "incomplete clear");
-      c->stats.kernel_launches += 1;
-      FS_CUDA(fs::launch_recheck_blend(vd, nb, L.max_tiles, Ls, skip, P.rec, P.rec16,
-                                       s->pos_op.as<float4>(), n, E, mask_dtype, map, Rb, ctr,
+      c->stats.kernel_launches += 2;
+      FS_CUDA(fs::launch_recheck_blend(vd, nb, L.max_tiles, Ls, skip, c->rk_tiles.p, c->n_sm,
+                                       P.rec, P.rec16, s->pos_op.as<float4>(), n, E, mask_dtype, map, Rb, ctr,
                                        stream),
               "re-check blend");
       FS_CUDA(cudaMemcpyAsync(ctr_h + fs::kRecheckIncomplete, ctr + fs::kRecheckIncomplete, 8,
@@ -1204,8 +1212,8 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
       }
       c->stats.recheck_rebinned += 1;  // kept lists end too early: bin these tiles anew
     }
-    FS_TRY(recheck_batch_rebin(c, s, n, nb, kcap, L, vd, P, key_src, skip, mask_dtype, E, map, R,
-                               stream));
+    FS_TRY(recheck_batch_rebin(c, s, n, nb, kcap, L, vd, P, key_src, skip, mask_dtype, E, F, nF,
+                               map, R, stream));
   }
   c->stats.kernel_launches += 1;
   FS_CUDA(fs::launch_assign_rows(R, F, nF, E, gamma, table, table_dtype, bits, label, margin,

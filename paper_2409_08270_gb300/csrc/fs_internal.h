@@ -202,17 +202,19 @@ struct RecheckLists {
   const uint8_t* sat_chunk;
   const uint64_t* deep;
   // the re-checked Gaussians (n_flagged of them) and the batch's per-slot
-  // visibility: a deep tile walks only the pixels one of them can reach
-  // (NULL: every labelled pixel of a deep tile)
+  // visibility and footprints: which of them contribute at a pixel
   const uint32_t* flagged;
   int n_flagged;
   const uint32_t* cnt;
+  const Footprint* foot;
 };
+// Scratch of launch_recheck_blend for a batch of total_tiles tiles (bytes).
+size_t recheck_tiles_bytes(int64_t total_tiles);
 // Float-pair compositing of the tiles whose skip bit is clear; adds alpha*T of
 // Gaussian i (map[i] >= 0) at a pixel of label e into R[map[i] * E + e].
 cudaError_t launch_recheck_blend(const ViewParams* views, int n_views, int max_tiles_per_view,
-                                 const RecheckLists& lists, const uint64_t* skip,
-                                 const ProjRecord* rec, const CompactRecord* rec16,
+                                 const RecheckLists& lists, const uint64_t* skip, void* tiles_tmp,
+                                 int n_sm, const ProjRecord* rec, const CompactRecord* rec16,
                                  const float4* pos_op, int64_t n, int E, int mask_dtype,
                                  const int32_t* map, double* R, unsigned long long* counters,
                                  cudaStream_t stream);

@@ -15,10 +15,10 @@
 // chunks, kept in memory) or from a dedicated binning of just the tiles the
 // re-checked Gaussians reach.  A tile that saturated in the main pass has no
 // list entries in later chunks; when a re-checked Gaussian sits in such a
-// chunk ("deep" tile), every pixel of the tile is walked to its stop, and a
-// pixel still compositing at the end of the kept lists (the FP32 and the
-// exact stop decisions differ there) is reported so the caller redoes the
-// batch with the dedicated binning.
+// chunk ("deep" tile), a pixel it reaches is walked to its stop, and a pixel
+// still compositing at the end of the kept lists (the FP32 and the exact stop
+// decisions differ there) is reported so the caller redoes the batch with the
+// dedicated binning.
 //
 // alpha = o 2^-|W (p - m)|^2 from the float-pair whitening record of the
 // projection; 2^-q follows Tang's table-driven method (ACM TOMS 15(2), 1989):
@@ -26,6 +26,8 @@
 // polynomial of e^-x on the remaining [0, ln2/64).
 #include <cuda_fp16.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "fs_binning.cuh"
 #include "fs_common.cuh"
@@ -158,9 +160,11 @@ __global__ void compact_kernel(int64_t k_total, const uint32_t* __restrict__ fla
   out_val[o] = static_cast<uint32_t>(slot);
 }
 
-constexpr int kRB = kTilePixels;  // list entries staged per step: one per thread
-constexpr int kGroup = 64;        // staged entries screened at once per pixel (two mask words)
-constexpr int kDeepTest = 256;  // re-checked Gaussians a deep tile tests per pixel at most
+constexpr int kRound = 32;       // list entries a warp stages and composites at once
+constexpr int kRing = 64;        // a warp's ring of kept entries: a partial round and a step
+constexpr int kFlagTest = 256;   // re-checked Gaussians counted per pixel at most (see below)
+constexpr int kRWarps = 4;       // warps of a block
+constexpr int kSubs = 8;         // 8x4-pixel pieces of a tile, one warp's work each
 
 // Float-pair constants of the compositing rule (Sec. 3.1 Eq. 1 conventions).
 constexpr double kAlphaMinD = 1.0 / 255.0, kAlphaMaxD = 0.99, kTMinD = 1e-4;
@@ -229,16 +233,16 @@ __device__ __forceinline__ f2 f2_exp2_neg(f2 q, float o, const float2* __restric
   return fast_two_sum(a.hi, a.lo);
 }
 
-// Staged list entries, one array per 16-byte part so that lanes that read
-// different entries spread over the banks: W (hi and lo parts), b = W (ctr - m)
+// Staged list entries of one warp, one array per 16-byte part so that lanes that
+// read different entries spread over the banks: W (hi and lo parts), b = W (ctr - m)
 // relative to the tile centre, the cut with slack, the opacity and the
 // re-check row (-1: none).
 struct Stage {
-  float4 w_hi[kRB];
-  float4 w_lo[kRB];
-  float4 bq[kRB];  // (b0 hi, b1 hi, q_cut + slack, opacity)
-  float2 b_lo[kRB];
-  int j[kRB];
+  float4 w_hi[kRound];
+  float4 w_lo[kRound];
+  float4 bq[kRound];  // (b0 hi, b1 hi, q_cut + slack, opacity)
+  float2 b_lo[kRound];
+  int j[kRound];
 };
 
 __device__ __forceinline__ void stage_entry(Stage& S, int e, const ProjRecord& r, float cx,
@@ -282,196 +286,250 @@ __device__ __forceinline__ bool reaches(const Stage& S, int e, float lx, float l
   return fmaf(q0, q0, q1 * q1) <= b.z;
 }
 
-// Bit k: staged entry e0 + k (k < 32, e0 + k < count) reaches the pixel.  The
-// staging array is read past `count` (its old entries, masked off here).
-__device__ __forceinline__ uint32_t reach_mask(const Stage& S, int e0, int count, float lx,
-                                               float ly) {
-  if (e0 >= count) return 0u;
-  uint32_t m = 0u;
-#pragma unroll 8
-  for (int k = 0; k < 32; ++k) m |= reaches(S, e0 + k, lx, ly) ? 1u << k : 0u;
-  return count - e0 >= 32 ? m : m & ((1u << (count - e0)) - 1u);
+// alpha of one (pixel, staged entry) pair, clamped: a float pair.
+__device__ __forceinline__ f2 pair_alpha(const Stage& S, int e, float lx, float ly,
+                                         const float2* __restrict__ tab) {
+  const float4 wh = S.w_hi[e], wl = S.w_lo[e], bq = S.bq[e];
+  const float2 bl = S.b_lo[e];
+  const f2 w0 = f2_row(wh.x, wl.x, wh.y, wl.y, bq.x, bl.x, lx, ly);
+  const f2 w1 = f2_row(wh.z, wl.z, wh.w, wl.w, bq.y, bl.y, lx, ly);
+  const f2 a_max = FS_F2C(kAlphaMaxD);
+  const f2 a = f2_exp2_neg(f2_norm2(w0, w1), bq.w, tab);
+  return f2_lt(a_max, a) ? a_max : a;
 }
 
-// One CTA per 16x16 tile of a view, one thread per pixel (warps of 8x4
-// pixels).  Pass 1 finds, per pixel, the last list position holding a
-// re-checked Gaussian that can reach the pixel; pass 2 composites the pixel
-// in float pairs up to that position (deep tiles: up to its stop).
+// list[1 + k] (k < list[0]): view << 24 | tile of every tile whose skip bit
+// is clear, in no particular order.
+__global__ void __launch_bounds__(256) collect_tiles_kernel(const ViewParams* __restrict__ views,
+                                                            const uint64_t* __restrict__ skip,
+                                                            uint32_t* __restrict__ count,
+                                                            uint32_t* __restrict__ list) {
+  const ViewParams& vp = views[blockIdx.y];
+  const int tile = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+  if (tile >= vp.tiles_x * vp.tiles_y) return;
+  const int g = vp.tile_base + tile;
+  if ((skip[g >> 6] >> (g & 63)) & 1ull) return;
+  list[atomicAdd(count, 1u)] = (blockIdx.y << 24) | static_cast<uint32_t>(tile);
+}
+
+// Composites again the pixels that a re-checked Gaussian contributes to, in
+// float pairs, front to back, until the last one's contribution or the stop.
+// A work item is an 8x4-pixel piece of a listed tile; every warp of the grid
+// takes items from a counter until none is left, and no warp waits for
+// another.
 //
-// The work is the ~130 FP32 operations of a (pixel, entry) pair, and an entry
-// covers only some of a warp's pixels.  So a pixel first collects the staged
-// entries that reach it, 64 at a time, in a bit mask (about ten operations an
-// entry), and then walks its own bits: lanes work on different entries at the
-// same time and a warp takes as many steps as its busiest pixel has entries,
-// not as many as its pixels have between them.
+// Bound by the ~130 FP32 operations of a (pixel, entry) pair and by the
+// latency of the list and record gathers ahead of them.  An entry covers only
+// some of a warp's pixels, and few pieces of a tile hold a pixel to re-check,
+// so
+//  * a piece first counts, per pixel, the re-checked Gaussians that
+//    contribute (the exact alpha test); without one it is done;
+//  * the tile's list is read 32 entries at a time, one per lane, and the
+//    slots that can reach the piece's rectangle go to the warp's ring (a
+//    plain FP32 test); 32 of them at a time are staged as float pairs, so that
+//    every lane has one to stage;
+//  * a pixel then screens the 32 into a bit mask and walks its own bits: lanes
+//    work on different entries at the same time, and a round takes as many
+//    steps as its busiest pixel has entries, not as many as its pixels have
+//    between them.
+// With more than kFlagTest re-checked Gaussians every labelled pixel of the
+// listed tiles is walked to its stop instead of counting.
 template <typename LabelT>
-__global__ void __launch_bounds__(kTilePixels, 4) recheck_blend_kernel(
-    const ViewParams* __restrict__ views, RecheckLists L, const uint64_t* __restrict__ skip,
+__global__ void __launch_bounds__(32 * kRWarps, 8) recheck_blend_kernel(
+    const ViewParams* __restrict__ views, RecheckLists L, const uint32_t* __restrict__ n_tiles,
+    const uint32_t* __restrict__ tiles, uint32_t* __restrict__ ticket,
     const ProjRecord* __restrict__ rec, const CompactRecord* __restrict__ rec16,
     const float4* __restrict__ pos_op, int64_t n, int E, const int32_t* __restrict__ map,
     double* __restrict__ R, unsigned long long* __restrict__ counters) {
-  __shared__ Stage S;
+  __shared__ Stage s_stage[kRWarps];
+  __shared__ uint32_t s_ring[kRWarps][kRing];
   __shared__ float2 s_tab[64];
-  const ViewParams& vp = views[blockIdx.y];
-  const int tile = blockIdx.x;
-  if (tile >= vp.tiles_x * vp.tiles_y) return;
-  const int gtile = vp.tile_base + tile;
-  if ((skip[gtile >> 6] >> (gtile & 63)) & 1ull) return;
-  const int n_chunks = L.sat_chunk ? min(L.chunks, static_cast<int>(L.sat_chunk[gtile]) + 1)
-                                   : L.chunks;
-  const bool truncated = n_chunks < L.chunks;
-  const bool deep = L.deep && ((L.deep[gtile >> 6] >> (gtile & 63)) & 1ull);
+  const int lane = threadIdx.x & 31;
+  Stage& S = s_stage[threadIdx.x >> 5];
+  uint32_t* const ring = s_ring[threadIdx.x >> 5];
   if (threadIdx.x < 64) {
     const double d = exp2(-static_cast<double>(threadIdx.x) / 64.0);
     const float hi = static_cast<float>(d);
     s_tab[threadIdx.x] = make_float2(hi, static_cast<float>(d - static_cast<double>(hi)));
   }
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int x0 = (tile % vp.tiles_x) * kTile, y0 = (tile / vp.tiles_x) * kTile;
-  const int x = x0 + 8 * (warp & 1) + (lane & 7);
-  const int y = y0 + 4 * (warp >> 1) + (lane >> 3);
-  int label = -1;
-  if (x < vp.width && y < vp.height) {
-    const int l = static_cast<int>(
-        static_cast<const LabelT*>(vp.mask)[static_cast<int64_t>(y) * vp.width + x]);
-    if (l >= 0 && l < E) label = l;
-  }
-  const float cx = static_cast<float>(x0) + 0.5f * kTile;
-  const float cy = static_cast<float>(y0) + 0.5f * kTile;
-  // pixel centre (x + 0.5, y + 0.5) relative to the tile centre: exact
-  const float lx = static_cast<float>(x - x0) + 0.5f - 0.5f * kTile;
-  const float ly = static_cast<float>(y - y0) + 0.5f - 0.5f * kTile;
-  // the slots of a view are view * n + index
-  const uint32_t slot0 = static_cast<uint32_t>(static_cast<int64_t>(blockIdx.y) * n);
-  auto stage = [&](uint32_t slot, int j) {
-    if (rec16)
-      stage_compact(S, tid, rec16[slot], pos_op[slot - slot0].w, cx, cy, j);
-    else
-      stage_entry(S, tid, rec[slot], cx, cy, j);
-  };
-
-  // pass 1: last re-checked entry (chunk << 32 | index) that may reach the
-  // pixel.  Re-checked entries are rare: a step without one costs its loads
-  // and one barrier.
-  int64_t last = -1;
-  for (int c = 0; c < n_chunks; ++c) {
-    const uint2 rg = L.ranges[c][gtile];
-    for (uint32_t b0 = rg.x; b0 < rg.y; b0 += kRB) {
-      const uint32_t at = b0 + tid;
-      const uint32_t slot = at < rg.y ? L.val[c][at] : slot0;
-      const int j = at < rg.y ? map[slot - slot0] : -1;
-      if (__syncthreads_or(j >= 0) == 0) continue;
-      S.j[tid] = j;
-      if (j >= 0) stage(slot, j);
-      __syncthreads();
-      if (label >= 0) {
-        const int cnt = static_cast<int>(min(static_cast<uint32_t>(kRB), rg.y - b0));
-        for (int e = 0; e < cnt; ++e)
-          if (S.j[e] >= 0 && reaches(S, e, lx, ly)) last = (static_cast<int64_t>(c) << 32) | (b0 + e);
-      }
-      __syncthreads();
-    }
-  }
-
-  // deep tiles: a pixel is walked to its stop only where a re-checked
-  // Gaussian visible in this view can reach it (the others hold nothing to
-  // re-check); with many re-checked Gaussians every labelled pixel is
-  bool deep_px = deep;
-  if (deep && L.flagged && L.n_flagged <= kDeepTest) {
-    bool reached = false;
-    for (int k0 = 0; k0 < L.n_flagged; k0 += kRB) {
-      const int cnt = min(kRB, L.n_flagged - k0);
-      __syncthreads();
-      if (tid < cnt) {
-        const uint32_t slot = slot0 + L.flagged[k0 + tid];
-        S.j[tid] = -1;
-        if (L.cnt[slot]) stage(slot, 0);
-      }
-      __syncthreads();
-      for (int e = 0; e < cnt; ++e)
-        if (S.j[e] >= 0 && reaches(S, e, lx, ly)) reached = true;
-    }
-    deep_px = reached;
-  }
-
-  // pass 2: float-pair compositing
-  const f2 a_min = FS_F2C(kAlphaMinD), a_max = FS_F2C(kAlphaMaxD), t_min = FS_F2C(kTMinD);
-  f2 T = f2_from(1.f);
-  bool live = label >= 0 && (deep_px || last >= 0);
-  const bool to_stop = deep_px;
+  __syncthreads();
+  const uint32_t n_items = kSubs * *n_tiles;
+  const uint32_t lt = (1u << lane) - 1u;
+  const f2 a_min = FS_F2C(kAlphaMinD), t_min = FS_F2C(kTMinD);
   unsigned long long evals = 0;
-  bool done_all = false;
-  for (int c = 0; c < n_chunks && !done_all; ++c) {
-    const uint2 rg = L.ranges[c][gtile];
-    for (uint32_t b0 = rg.x; b0 < rg.y; b0 += kRB) {
-      if (__syncthreads_or(live) == 0) {
-        done_all = true;
-        break;
+  for (;;) {
+    uint32_t item = 0u;
+    if (lane == 0) item = atomicAdd(ticket, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= n_items) break;
+    const uint32_t vt = tiles[item / kSubs];
+    const int view = static_cast<int>(vt >> 24), tile = static_cast<int>(vt & 0xFFFFFFu);
+    const int sub = static_cast<int>(item % kSubs);
+    const ViewParams& vp = views[view];
+    const int gtile = vp.tile_base + tile;
+    const int tx = tile % vp.tiles_x, ty = tile / vp.tiles_x;
+    const int x = tx * kTile + 8 * (sub & 1) + (lane & 7);
+    const int y = ty * kTile + 4 * (sub >> 1) + (lane >> 3);
+    int label = -1;
+    if (x < vp.width && y < vp.height) {
+      const int l = static_cast<int>(
+          static_cast<const LabelT*>(vp.mask)[static_cast<int64_t>(y) * vp.width + x]);
+      if (l >= 0 && l < E) label = l;
+    }
+    if (!__any_sync(0xffffffffu, label >= 0)) continue;
+    const float cx = static_cast<float>(tx * kTile) + 0.5f * kTile;
+    const float cy = static_cast<float>(ty * kTile) + 0.5f * kTile;
+    // pixel centre (x + 0.5, y + 0.5) and the piece's centre relative to the
+    // tile centre: exact
+    const float lx = static_cast<float>(x) + 0.5f - cx, ly = static_cast<float>(y) + 0.5f - cy;
+    const float rx = 8.f * static_cast<float>(sub & 1) - 4.f;
+    const float ry = 4.f * static_cast<float>(sub >> 1) - 6.f;
+    const uint32_t slot0 = static_cast<uint32_t>(static_cast<int64_t>(view) * n);
+
+    // can the slot reach one of the piece's pixel centres? (FP32, with the
+    // slack of the per-pixel screen)
+    auto meets = [&](uint32_t slot) -> bool {
+      float4 w;
+      float bx, by, qc;
+      if (rec16) {
+        const CompactRecord r = rec16[slot];
+        const float2 wa = __half22float2(*reinterpret_cast<const __half2*>(&r.w01));
+        const float2 wb = __half22float2(*reinterpret_cast<const __half2*>(&r.w23));
+        w = make_float4(wa.x, wa.y, wb.x, wb.y);
+        bx = (cx + rx) - r.mx;
+        by = (cy + ry) - r.my;
+        qc = r.q_cut;
+      } else {
+        const ProjRecord& r = rec[slot];
+        const float4 m = r.m;
+        w = r.w_hi;
+        bx = ((cx + rx) - m.x) - m.z;
+        by = ((cy + ry) - m.y) - m.w;
+        qc = r.misc.y;
       }
-      const int cnt = static_cast<int>(min(static_cast<uint32_t>(kRB), rg.y - b0));
-      if (tid < cnt) {
-        const uint32_t slot = L.val[c][b0 + tid];
-        stage(slot, map[slot - slot0]);
+      const float d0 = fmaxf(0.f, fabsf(fmaf(w.x, bx, w.y * by)) -
+                                      fmaf(fabsf(w.x), 3.5f, fabsf(w.y) * 1.5f));
+      const float d1 = fmaxf(0.f, fabsf(fmaf(w.z, bx, w.w * by)) -
+                                      fmaf(fabsf(w.z), 3.5f, fabsf(w.w) * 1.5f));
+      return fmaf(d0, d0, d1 * d1) <= qc + 0.05f;
+    };
+    // ring entries first .. first + count - 1 into the stage, one per lane
+    auto stage = [&](int first, int count) {
+      if (lane < count) {
+        const uint32_t slot = ring[(first + lane) & (kRing - 1)];
+        const int j = map[slot - slot0];
+        if (rec16)
+          stage_compact(S, lane, rec16[slot], pos_op[slot - slot0].w, cx, cy, j);
+        else
+          stage_entry(S, lane, rec[slot], cx, cy, j);
       }
-      __syncthreads();
-      // the pixel's entries of this step: all of them, or up to its last one
-      const int64_t pos0 = (static_cast<int64_t>(c) << 32) | b0;
-      const int e_end =
-          to_stop ? cnt : static_cast<int>(min(static_cast<int64_t>(cnt), last - pos0 + 1));
-      for (int g0 = 0; g0 < cnt; g0 += kGroup) {
-        if (!__any_sync(0xffffffffu, live && g0 < e_end)) break;
-        uint32_t m0 = 0u, m1 = 0u;
-        if (live) {
-          m0 = reach_mask(S, g0, e_end, lx, ly);
-          m1 = reach_mask(S, g0 + 32, e_end, lx, ly);
+      __syncwarp();
+    };
+    // appends the lanes' slots that are kept at ring position `at`
+    auto append = [&](bool keep, uint32_t slot, int at) -> int {
+      const uint32_t bal = __ballot_sync(0xffffffffu, keep);
+      if (keep) ring[(at + __popc(bal & lt)) & (kRing - 1)] = slot;
+      __syncwarp();
+      return __popc(bal);
+    };
+
+    // the re-checked Gaussians that contribute at each pixel: of those whose
+    // footprint lists this tile, the ones with alpha >= 1/255
+    int left = 0;
+    if (L.n_flagged <= kFlagTest) {
+      for (int k0 = 0; k0 < L.n_flagged; k0 += 32) {
+        bool on = k0 + lane < L.n_flagged;
+        const uint32_t slot = slot0 + (on ? L.flagged[k0 + lane] : 0u);
+        on = on && L.cnt[slot] != 0u;
+        if (on) {
+          const Footprint f = L.foot[slot];
+          int r0, r1, c0, c1;
+          footprint_rows(f, &r0, &r1);
+          on = ty >= r0 && ty <= r1 && row_span(f, ty, vp.width, &c0, &c1) &&
+               clip_cols(vp, slot, &c0, &c1) && tx >= c0 && tx <= c1;
         }
-        evals += __popc(m0) + __popc(m1);
-        while (m0 | m1) {
-          int e = g0;
-          if (m0) {
-            e += __ffs(m0) - 1;
-            m0 &= m0 - 1u;
-          } else {
-            e += 31 + __ffs(m1);
-            m1 &= m1 - 1u;
-          }
-          const float4 wh = S.w_hi[e], wl = S.w_lo[e], bq = S.bq[e];
-          const float2 bl = S.b_lo[e];
-          const f2 w0 = f2_row(wh.x, wl.x, wh.y, wl.y, bq.x, bl.x, lx, ly);
-          const f2 w1 = f2_row(wh.z, wl.z, wh.w, wl.w, bq.y, bl.y, lx, ly);
-          f2 a = f2_exp2_neg(f2_norm2(w0, w1), bq.w, s_tab);
-          if (f2_lt(a_max, a)) a = a_max;
-          if (f2_lt(a, a_min)) continue;
-          // T (1 - a): 1 - a needs no normalisation for the product
-          const f2 om = fast_two_sum(1.f, -a.hi);
-          f2 t = two_prod(T.hi, om.hi);
-          t.lo = __fmaf_rn(T.hi, __fsub_rn(om.lo, a.lo), __fmaf_rn(T.lo, om.hi, t.lo));
-          t = fast_two_sum(t.hi, t.lo);
-          if (f2_lt(t, t_min)) {
-            live = false;
-            evals -= __popc(m0) + __popc(m1);  // not reached
-            break;
-          }
+        const int m = append(on && meets(slot), slot, 0);
+        stage(0, m);
+        if (label >= 0)
+          for (int e = 0; e < m; ++e)
+            if (reaches(S, e, lx, ly) && !f2_lt(pair_alpha(S, e, lx, ly, s_tab), a_min)) ++left;
+        __syncwarp();
+      }
+    } else if (label >= 0) {
+      left = 0x7FFFFFFF;
+    }
+
+    f2 T = f2_from(1.f);
+    // one round: `count` kept entries from ring position `first` on
+    auto composite = [&](int first, int count) {
+      stage(first, count);
+      uint32_t m = 0u;
+      if (left > 0) {
+#pragma unroll 8
+        for (int k = 0; k < kRound; ++k) m |= reaches(S, k, lx, ly) ? 1u << k : 0u;
+        if (count < kRound) m &= (1u << count) - 1u;
+      }
+      evals += __popc(m);
+      while (m) {
+        const int e = __ffs(m) - 1;
+        m &= m - 1u;
+        const f2 a = pair_alpha(S, e, lx, ly, s_tab);
+        if (f2_lt(a, a_min)) continue;
+        // T (1 - a): 1 - a needs no normalisation for the product
+        const f2 om = fast_two_sum(1.f, -a.hi);
+        f2 t = two_prod(T.hi, om.hi);
+        t.lo = __fmaf_rn(T.hi, __fsub_rn(om.lo, a.lo), __fmaf_rn(T.lo, om.hi, t.lo));
+        t = fast_two_sum(t.hi, t.lo);
+        if (f2_lt(t, t_min)) {
+          left = 0;  // the pixel's stop
+        } else {
           const int j = S.j[e];
           if (j >= 0) {
             const f2 ct = f2_mul(a, T);
             atomicAdd(&R[static_cast<int64_t>(j) * E + label],
                       static_cast<double>(ct.hi) + static_cast<double>(ct.lo));
+            --left;
           }
           T = t;
         }
+        if (left == 0) {
+          evals -= __popc(m);  // not evaluated
+          break;
+        }
       }
-      if (live && !to_stop && pos0 + cnt > last) live = false;
+      __syncwarp();
+    };
+    if (!__any_sync(0xffffffffu, left > 0)) continue;
+    const int n_chunks =
+        L.sat_chunk ? min(L.chunks, static_cast<int>(L.sat_chunk[gtile]) + 1) : L.chunks;
+    int head = 0, queued = 0;
+    bool some = true;
+    for (int c = 0; c < n_chunks && some; ++c) {
+      const uint2 rg = L.ranges[c][gtile];
+      const uint32_t* __restrict__ val = L.val[c];
+      uint32_t next = rg.x + lane < rg.y ? val[rg.x + lane] : 0u;
+      for (uint32_t b0 = rg.x; b0 < rg.y && some; b0 += 32) {
+        const uint32_t slot = next;
+        if (b0 + 32 + lane < rg.y) next = val[b0 + 32 + lane];
+        queued += append(b0 + lane < rg.y && meets(slot), slot, head + queued);
+        if (queued >= kRound) {
+          composite(head, kRound);
+          head += kRound;
+          queued -= kRound;
+          some = __any_sync(0xffffffffu, left > 0);
+        }
+      }
     }
+    if (some && queued > 0) composite(head, queued);
+    // still compositing where a deep tile's kept lists end: the exact walk
+    // needs entries the main pass never listed
+    const bool deep = L.deep && ((L.deep[gtile >> 6] >> (gtile & 63)) & 1ull);
+    if (n_chunks < L.chunks && deep && __any_sync(0xffffffffu, left > 0) && lane == 0)
+      atomicAdd(&counters[kRecheckIncomplete], 1ull);
   }
-  // still compositing where a saturated tile's kept lists end: the exact
-  // walk needs entries the main pass never listed
-  const bool incomplete = live && truncated && to_stop;
-  const int n_inc = __syncthreads_count(incomplete);
-  if (threadIdx.x == 0 && n_inc) atomicAdd(&counters[kRecheckIncomplete], 1ull);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) evals += __shfl_xor_sync(0xffffffffu, evals, o);
-  if ((threadIdx.x & 31) == 0 && evals) atomicAdd(&counters[kRecheckPairs], evals);
+  if (lane == 0 && evals) atomicAdd(&counters[kRecheckPairs], evals);
 }
 
 __global__ void add_rows_kernel(int64_t count, const double* __restrict__ src,
@@ -537,21 +595,34 @@ cudaError_t launch_compact(int64_t k_total, const uint32_t* flag, const uint32_t
   return cudaGetLastError();
 }
 
+size_t recheck_tiles_bytes(int64_t total_tiles) {
+  return 256 + static_cast<size_t>(total_tiles) * sizeof(uint32_t);
+}
+
 cudaError_t launch_recheck_blend(const ViewParams* views, int n_views, int max_tiles_per_view,
-                                 const RecheckLists& lists, const uint64_t* skip,
-                                 const ProjRecord* rec, const CompactRecord* rec16,
+                                 const RecheckLists& lists, const uint64_t* skip, void* tiles_tmp,
+                                 int n_sm, const ProjRecord* rec, const CompactRecord* rec16,
                                  const float4* pos_op, int64_t n, int E, int mask_dtype,
                                  const int32_t* map, double* R, unsigned long long* counters,
                                  cudaStream_t stream) {
   if (n_views == 0 || max_tiles_per_view == 0) return cudaSuccess;
   if (lists.chunks < 1 || lists.chunks > kMaxChunks) return cudaErrorInvalidValue;
-  const dim3 grid(static_cast<unsigned>(max_tiles_per_view), static_cast<unsigned>(n_views));
+  uint32_t* words = static_cast<uint32_t*>(tiles_tmp);  // [0] tiles listed, [1] items taken
+  uint32_t* tiles = words + 64;
+  cudaError_t e = cudaMemsetAsync(words, 0, 2 * sizeof(uint32_t), stream);
+  if (e != cudaSuccess) return e;
+  const dim3 grid(blocks_for(max_tiles_per_view, 256), static_cast<unsigned>(n_views));
+  collect_tiles_kernel<<<grid, 256, 0, stream>>>(views, skip, words, tiles);
+  // one full set of resident blocks, fewer when the batch has fewer pieces
+  const int64_t items = static_cast<int64_t>(n_views) * max_tiles_per_view * kSubs;
+  const unsigned blocks = static_cast<unsigned>(
+      std::min<int64_t>(8 * static_cast<int64_t>(n_sm), (items + kRWarps - 1) / kRWarps));
   if (mask_dtype == 4)
-    recheck_blend_kernel<uint8_t><<<grid, kTilePixels, 0, stream>>>(
-        views, lists, skip, rec, rec16, pos_op, n, E, map, R, counters);
+    recheck_blend_kernel<uint8_t><<<blocks, 32 * kRWarps, 0, stream>>>(
+        views, lists, words, tiles, words + 1, rec, rec16, pos_op, n, E, map, R, counters);
   else
-    recheck_blend_kernel<int32_t><<<grid, kTilePixels, 0, stream>>>(
-        views, lists, skip, rec, rec16, pos_op, n, E, map, R, counters);
+    recheck_blend_kernel<int32_t><<<blocks, 32 * kRWarps, 0, stream>>>(
+        views, lists, words, tiles, words + 1, rec, rec16, pos_op, n, E, map, R, counters);
   return cudaGetLastError();
 }
 
