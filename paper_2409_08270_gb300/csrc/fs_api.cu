@@ -147,9 +147,7 @@ int ceil_log2(int64_t x) {
 // kernels launched by exclusive_scan / radix_sort_pairs for n elements
 int64_t scan_launches(int64_t n) { return n > 0 ? 3 : 0; }
 int64_t radix_launches(int64_t n, int bits) {
-  if (n <= 1 || bits <= 0) return 0;
-  const int64_t nb = (n + 4095) / 4096;
-  return static_cast<int64_t>(fs::radix_passes(bits)) * (2 + scan_launches(nb * 512));
+  return n > 1 && bits > 0 ? 1 + fs::radix_passes(bits) : 0;
 }
 
 }  // namespace
@@ -675,7 +673,8 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
     bool alt2 = false;
     FS_CUDA(fs::radix_sort_pairs(c->lk_a.as<uint32_t>(), val_dst->as<uint32_t>(),
                                  c->lk_b.as<uint32_t>(), c->lv_b.as<uint32_t>(), plan_cap,
-                                 tile_bits, c->sort_tmp.p, &alt2, stream, 0u, 0xFFFFFFFFu, total),
+                                 tile_bits, c->sort_tmp.p, &alt2, stream, ctr, false, 0u, 0xFFFFFFFFu,
+                                 total),
             "tile sort");
     const uint32_t* lkey = alt2 ? c->lk_b.as<uint32_t>() : c->lk_a.as<uint32_t>();
     if (alt2)
@@ -719,7 +718,7 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
   FS_TRY(stage_begin(c, FS_STAGE_TILE_SORT, stream, false, &tt));
   FS_CUDA(fs::radix_sort_pairs(c->lk_a.as<uint32_t>(), val_dst->as<uint32_t>(),
                                c->lk_b.as<uint32_t>(), c->lv_b.as<uint32_t>(), I, tile_bits,
-                               c->sort_tmp.p, &alt2, stream),
+                               c->sort_tmp.p, &alt2, stream, ctr),
           "tile sort");
   const uint32_t* lkey = alt2 ? c->lk_b.as<uint32_t>() : c->lk_a.as<uint32_t>();
   if (alt2)
@@ -881,7 +880,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
     int tp = -1;
     FS_TRY(stage_begin(c, FS_STAGE_PROJECT, strm, plan != nullptr, &tp));
     FS_CUDA(fs::launch_project(n, nbb, pr.vd, s->pos_op.as<float4>(), s->cov.as<float4>(),
-                               PP.rec, PP.rec16, PP.foot, PP.cnt, pr.key, pr.val, PP.dlo, krq,
+                               PP.rec, PP.rec16, PP.foot, PP.cnt, pr.key, PP.dlo, krq,
                                strm),
             "project");
     FS_TRY(stage_end(c, tp, strm));
@@ -947,7 +946,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
     int td = -1;
     FS_TRY(stage_begin(c, FS_STAGE_DEPTH_SORT, stream, plan != nullptr, &td));
     FS_CUDA(fs::radix_sort_pairs(pr.key, pr.val, pr.key_alt, pr.val_alt, k_total, key_bits,
-                                 c->sort_tmp.p, &alt, stream, kmin, span, nullptr,
+                                 c->sort_tmp.p, &alt, stream, ctr, true, kmin, span, nullptr,
                                  plan ? krd : nullptr),
             "depth sort");
     uint32_t* sorted_key = alt ? pr.key_alt : pr.key;
@@ -1062,7 +1061,7 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
   bool alt = false;
   FS_CUDA(fs::radix_sort_pairs(c->key_b.as<uint32_t>(), c->val_b.as<uint32_t>(),
                                c->key_a.as<uint32_t>(), c->val_a.as<uint32_t>(), C, 32,
-                               c->sort_tmp.p, &alt, stream),
+                               c->sort_tmp.p, &alt, stream, ctr),
           "candidate sort");
   uint32_t* sorted_key = alt ? c->key_a.as<uint32_t>() : c->key_b.as<uint32_t>();
   uint32_t* sorted_val = alt ? c->val_a.as<uint32_t>() : c->val_b.as<uint32_t>();
@@ -1160,8 +1159,8 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
     if (!keep) {
       c->stats.kernel_launches += 1;
       FS_CUDA(fs::launch_project(n, nb, vd, s->pos_op.as<float4>(), s->cov.as<float4>(), P.rec,
-                                 P.rec16, P.foot, P.cnt, c->key_a.as<uint32_t>(),
-                                 c->val_a.as<uint32_t>(), P.dlo, nullptr, stream),
+                                 P.rec16, P.foot, P.cnt, c->key_a.as<uint32_t>(), P.dlo, nullptr,
+                                 stream),
               "project");
       key_src = c->key_a.as<uint32_t>();
     }
@@ -1303,8 +1302,7 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
     FS_CUDA(cudaMemsetAsync(krq, 0xFF, 4, stream), "key range");
     FS_CUDA(cudaMemsetAsync(krq + 1, 0, 8, stream), "key range");
     FS_CUDA(fs::launch_project(n, nb, vd, s->pos_op.as<float4>(), s->cov.as<float4>(), P.rec,
-                               P.rec16, P.foot, P.cnt, c->key_a.as<uint32_t>(),
-                               c->val_a.as<uint32_t>(), P.dlo, krq, stream),
+                               P.rec16, P.foot, P.cnt, c->key_a.as<uint32_t>(), P.dlo, krq, stream),
             "project");
     FS_CUDA(cudaMemcpyAsync(krh, krq, 12, cudaMemcpyDeviceToHost, stream), "key range readback");
     FS_CUDA(cudaStreamSynchronize(stream), "key range readback");
@@ -1320,7 +1318,8 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
     bool alt = false;
     FS_CUDA(fs::radix_sort_pairs(c->key_a.as<uint32_t>(), c->val_a.as<uint32_t>(),
                                  c->key_b.as<uint32_t>(), c->val_b.as<uint32_t>(), k_total,
-                                 key_bits, c->sort_tmp.p, &alt, stream, kmin, span),
+                                 key_bits, c->sort_tmp.p, &alt, stream, c->counters.as<unsigned long long>(),
+                                 true, kmin, span),
             "depth sort");
     uint32_t* sorted_key = alt ? c->key_b.as<uint32_t>() : c->key_a.as<uint32_t>();
     uint32_t* sorted_val = alt ? c->val_b.as<uint32_t>() : c->val_a.as<uint32_t>();
@@ -1820,22 +1819,28 @@ fs_status fs_test_sort_pairs(int32_t device, uint32_t* keys, uint32_t* vals, int
     return fail(FS_INVALID_ARGUMENT, "fs_test_sort_pairs: bad arrays, n or bits");
   if (n == 0) return FS_OK;
   DeviceGuard g(device);
-  DevBuf ak, av, tmp;
+  DevBuf ak, av, tmp, ctr;
   FS_TRY(ak.ensure(static_cast<size_t>(n) * 4, "sort keys"));
   FS_TRY(av.ensure(static_cast<size_t>(n) * 4, "sort vals"));
   FS_TRY(tmp.ensure(fs::radix_temp_bytes(n), "sort temp"));
+  FS_TRY(ctr.ensure(8 * fs::kNumCounters, "sort counters"));
   bool alt = false;
-  cudaError_t e = fs::radix_sort_pairs(keys, vals, ak.as<uint32_t>(), av.as<uint32_t>(), n, bits,
-                                       tmp.p, &alt, nullptr);
+  cudaError_t e = cudaMemset(ctr.p, 0, 8 * fs::kNumCounters);
+  if (e == cudaSuccess)
+    e = fs::radix_sort_pairs(keys, vals, ak.as<uint32_t>(), av.as<uint32_t>(), n, bits, tmp.p,
+                             &alt, nullptr, ctr.as<unsigned long long>());
   if (e == cudaSuccess && alt) {
     e = cudaMemcpy(keys, ak.p, static_cast<size_t>(n) * 4, cudaMemcpyDeviceToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(vals, av.p, static_cast<size_t>(n) * 4, cudaMemcpyDeviceToDevice);
   }
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  unsigned long long h[fs::kNumCounters] = {};
+  if (e == cudaSuccess) e = cudaMemcpy(h, ctr.p, sizeof(h), cudaMemcpyDeviceToHost);
   ak.release();
   av.release();
   tmp.release();
+  ctr.release();
   if (e != cudaSuccess) return cuda_fail(e, "fs_test_sort_pairs");
+  if (h[fs::kLookbackTimeout]) return fail(FS_TIMEOUT, "fs_test_sort_pairs: a bounded wait gave up");
   return FS_OK;
 }
 

@@ -18,6 +18,9 @@ struct ProjRecord;
 struct CompactRecord;
 struct Footprint;
 
+// Polls of a predecessor's look-back word before the wait gives up (about 2 s).
+constexpr int kLookbackSpinLimit = 1 << 26;
+
 // scan / sort (fs_sort.cu) --------------------------------------------------
 // Temporary storage needed by exclusive_scan for n elements (bytes).
 size_t scan_temp_bytes(int64_t n);
@@ -31,14 +34,16 @@ size_t radix_temp_bytes(int64_t n);
 // Stable LSD radix sort of (key, val) pairs on the low `bits` bits of
 // min(key - kmin, span) (the keys themselves are moved unchanged).
 // Ping-pongs between (keys, vals) and (keys_alt, vals_alt); *in_alt tells the
-// caller which pair holds the result.  n_dev (may be NULL): the count to sort
-// is min(n, *n_dev), read on the device (the grid is sized for n); range_dev
-// (may be NULL): kmin and span from a device key range {min, max}.
+// caller which pair holds the result.  counters (may be NULL): a look-back
+// wait that gives up is counted there (kLookbackTimeout).  iota: the values
+// are 0 .. n - 1, whatever `vals` holds.  n_dev (may be NULL): the count to
+// sort is min(n, *n_dev), read on the device (the grid is sized for n);
+// range_dev (may be NULL): kmin and span from a device key range {min, max}.
 cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
                              uint32_t* vals_alt, int64_t n, int bits, void* temp, bool* in_alt,
-                             cudaStream_t stream, uint32_t kmin = 0u,
-                             uint32_t span = 0xFFFFFFFFu, const uint32_t* n_dev = nullptr,
-                             const uint32_t* range_dev = nullptr);
+                             cudaStream_t stream, unsigned long long* counters, bool iota = false,
+                             uint32_t kmin = 0u, uint32_t span = 0xFFFFFFFFu,
+                             const uint32_t* n_dev = nullptr, const uint32_t* range_dev = nullptr);
 
 // projection / binning (fs_project.cu) --------------------------------------
 // pos_op[n] = (m, o); cov[3n] = Sigma3D as float pairs (FP64 once per scene)
@@ -49,14 +54,14 @@ cudaError_t launch_scene_prep(int64_t n, const float* mean, const void* quat, in
 // rec16 != NULL: reduced-precision records (FP16 whitening matrix, FP32 mean)
 // are written to rec16 instead of the float-pair records to rec.  Records are
 // written for visible slots only (nothing reads the others'); footprints,
-// counts, keys, values and low depth words for every slot.
+// counts, keys and low depth words for every slot.
 // key_range (3 uint32, may be NULL): atomic min / max of the visible slots'
 // depth keys and their number (the caller initialises it to {0xFFFFFFFF, 0,
 // 0}).  After the depth sort the visible slots are the first ones.
 cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, const float4* pos_op,
                            const float4* cov, ProjRecord* rec, CompactRecord* rec16,
-                           Footprint* foot, uint32_t* cnt, uint32_t* key, uint32_t* val,
-                           uint32_t* depth_lo, uint32_t* key_range, cudaStream_t stream);
+                           Footprint* foot, uint32_t* cnt, uint32_t* key, uint32_t* depth_lo,
+                           uint32_t* key_range, cudaStream_t stream);
 // re-orders runs of equal 32-bit depth keys by the depth's low word, then slot
 // (n_total elements; slot / n is the view of a slot)
 cudaError_t launch_depth_tie_fix(int64_t n_total, int64_t n, const uint32_t* key, uint32_t* val,
@@ -84,8 +89,6 @@ cudaError_t launch_bin_fused(int64_t p0, int64_t n_pos, int64_t n, const ViewPar
                              unsigned long long* counters, cudaStream_t stream,
                              const int64_t* range_dev = nullptr);
 size_t bin_fused_temp_bytes(int64_t n_pos);
-// Polls of a predecessor's look-back word before the wait gives up (about 2 s).
-constexpr int kLookbackSpinLimit = 1 << 26;
 // Diagnostic: the fused binning on one block whose predecessor never
 // publishes, with a wait bound of spin_limit polls (lookback: 512 B, total:
 // one word, counters: kNumCounters; the other arrays need one element each).

@@ -35,7 +35,7 @@ constexpr int64_t kNA_N = FS_NOALLOC_MAX_GAUSSIANS;
 constexpr int kNA_Side = FS_NOALLOC_MAX_SIDE;
 constexpr int64_t kNA_Entries = FS_NOALLOC_MAX_LIST_ENTRIES;
 constexpr int kNA_Tiles = (kNA_Side / kTile) * (kNA_Side / kTile);
-constexpr size_t kNA_SortTmp = 512 * 1024;  // >= radix_temp_bytes(kNA_Entries), checked at run time
+constexpr size_t kNA_SortTmp = 544 * 1024;  // >= radix_temp_bytes(kNA_Entries), checked at run time
 constexpr size_t kNA_ScanTmp = 4 * 1024;    // >= scan_temp_bytes(kNA_N), checked at run time
 
 constexpr size_t al(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
@@ -229,11 +229,12 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
     const int tiles = vp.tiles_x * vp.tiles_y;
     // pageable source: the copy has taken the bytes when the call returns
     NA_CUDA(cudaMemcpyAsync(vd, &vp, sizeof(vp), cudaMemcpyHostToDevice, strm), "view upload");
-    NA_CUDA(launch_project(n, 1, vd, pos, cov, rec, nullptr, foot, cnt, key_a, val_a, dlo, nullptr,
+    NA_CUDA(launch_project(n, 1, vd, pos, cov, rec, nullptr, foot, cnt, key_a, dlo, nullptr,
                            strm),
             "project");
     bool alt = false;
-    NA_CUDA(radix_sort_pairs(key_a, val_a, key_b, val_b, n, 32, sort_tmp, &alt, strm), "sort");
+    NA_CUDA(radix_sort_pairs(key_a, val_a, key_b, val_b, n, 32, sort_tmp, &alt, strm, ctr, true),
+            "sort");
     uint32_t* skey = alt ? key_b : key_a;
     uint32_t* sval = alt ? val_b : val_a;
     NA_CUDA(launch_depth_tie_fix(n, n, skey, sval, dlo, strm), "ties");
@@ -261,7 +262,8 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
                             strm),
                 "emit");
         bool alt2 = false;
-        NA_CUDA(radix_sort_pairs(lk_a, lv_a, lk_b, lv_b, I, bits_for(tiles), sort_tmp, &alt2, strm),
+        NA_CUDA(radix_sort_pairs(lk_a, lv_a, lk_b, lv_b, I, bits_for(tiles), sort_tmp, &alt2, strm,
+                                 ctr),
                 "tile sort");
         const uint32_t* lkey = alt2 ? lk_b : lk_a;
         const uint32_t* lval = alt2 ? lv_b : lv_a;
@@ -279,6 +281,8 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
   unsigned long long h_ctr[kNumCounters];
   NA_CUDA(cudaMemcpyAsync(h_ctr, ctr, sizeof(h_ctr), cudaMemcpyDeviceToHost, strm), "readback");
   NA_CUDA(cudaStreamSynchronize(strm), "readback");
+  if (h_ctr[kLookbackTimeout])
+    return na_fail(FS_TIMEOUT, "fs_solve_noalloc: a sort's bounded wait gave up");
   if (h_ctr[kBinningMismatch])
     return na_fail(FS_CUDA_ERROR, "fs_solve_noalloc: internal binning mismatch");
   return FS_OK;

@@ -142,8 +142,8 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
     int64_t n, int n_views, const ViewParams* __restrict__ views_g,
     const float4* __restrict__ pos_op, const float4* __restrict__ cov3,
     ProjRecord* __restrict__ rec, CompactRecord* __restrict__ rec16, Footprint* __restrict__ foot,
-    uint32_t* __restrict__ cnt, uint32_t* __restrict__ key, uint32_t* __restrict__ val,
-    uint32_t* __restrict__ depth_lo, uint32_t* __restrict__ key_range) {
+    uint32_t* __restrict__ cnt, uint32_t* __restrict__ key, uint32_t* __restrict__ depth_lo,
+    uint32_t* __restrict__ key_range) {
   __shared__ ViewParams views[kMaxViewsPerBatch];
   for (int k = threadIdx.x; k < n_views * (int)(sizeof(ViewParams) / 4); k += blockDim.x)
     reinterpret_cast<uint32_t*>(views)[k] = reinterpret_cast<const uint32_t*>(views_g)[k];
@@ -421,7 +421,6 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
       ++n_vis;
     }
     key[slot] = k;
-    val[slot] = static_cast<uint32_t>(slot);
     depth_lo[slot] = float_order_key(depth_l);
   }
   }
@@ -949,18 +948,18 @@ cudaError_t launch_scene_prep(int64_t n, const float* mean, const void* quat, in
 
 cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, const float4* pos_op,
                            const float4* cov, ProjRecord* rec, CompactRecord* rec16,
-                           Footprint* foot, uint32_t* cnt, uint32_t* key, uint32_t* val,
-                           uint32_t* depth_lo, uint32_t* key_range, cudaStream_t stream) {
+                           Footprint* foot, uint32_t* cnt, uint32_t* key, uint32_t* depth_lo,
+                           uint32_t* key_range, cudaStream_t stream) {
   if (n == 0 || n_views == 0) return cudaSuccess;
   const int threads = 256;
   const int64_t blocks = (n + threads - 1) / threads;
   // the reduced-precision form takes the FP32 projection
   if (rec16)
     project_kernel<true><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-        n, n_views, views, pos_op, cov, rec, rec16, foot, cnt, key, val, depth_lo, key_range);
+        n, n_views, views, pos_op, cov, rec, rec16, foot, cnt, key, depth_lo, key_range);
   else
     project_kernel<false><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-        n, n_views, views, pos_op, cov, rec, rec16, foot, cnt, key, val, depth_lo, key_range);
+        n, n_views, views, pos_op, cov, rec, rec16, foot, cnt, key, depth_lo, key_range);
   return cudaGetLastError();
 }
 

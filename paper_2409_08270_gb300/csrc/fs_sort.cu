@@ -1,11 +1,16 @@
 // Device exclusive scan and stable LSD radix sort of (uint32 key, uint32 value)
 // pairs, used for the depth order and the tile binning of Sec. 3.1.
 //
-// Both work on tiles of 4096 elements per 256-thread block.  The radix sort
-// is the classic three-step pass (per-block digit histogram, scan of the
-// histogram in digit-major order, stable scatter).  No step waits on another
-// block.
+// The radix sort reads the keys once for the digit histograms of all passes;
+// each pass is then one launch that reads and writes every pair once: a block
+// ranks a tile of pairs, learns where its digits' runs start from its
+// predecessors' published counts (decoupled look-back, Merrill and Garland
+// 2016; one launch per pass, Adinets and Merrill 2022) and writes the runs.
+// Blocks take tiles in launch order (a ticket), so a block only ever waits for
+// blocks that have started, and every wait is bounded.
+#include <algorithm>
 #include <atomic>
+#include <utility>
 
 #include "fs_internal.h"
 
@@ -13,6 +18,7 @@ namespace fs {
 
 namespace {
 
+// the scan: tiles of 4096 elements per 256-thread block
 constexpr int kThreads = 256;
 constexpr int kRounds = 16;
 constexpr int kTileElems = kThreads * kRounds;
@@ -121,13 +127,16 @@ __global__ void __launch_bounds__(kThreads) scan_down_kernel(const uint32_t* __r
   }
 }
 
+// ---------------------------------------------------------------------------
+// radix sort
+// ---------------------------------------------------------------------------
+
 // Digits are taken from min(key - kmin, span): a key range [kmin, kmin + span)
 // (and everything above it mapped to span) needs only the bits of span.
-// A pass takes DB bits (8 or 9: a 17-bit tile key sorts in two passes).
-template <int DB>
-__device__ __forceinline__ uint32_t digit_of(uint32_t key, uint32_t kmin, uint32_t span,
-                                             int shift) {
-  return (min(key - kmin, span) >> shift) & ((1u << DB) - 1u);
+// A pass takes 8 or 9 bits (a 17-bit tile key sorts in two passes).
+__device__ __forceinline__ uint32_t digit_of(uint32_t key, uint32_t kmin, uint32_t span, int shift,
+                                             int bits) {
+  return (min(key - kmin, span) >> shift) & ((1u << bits) - 1u);
 }
 
 // Sizes read on the device (a launch captured once and replayed): the element
@@ -144,158 +153,295 @@ __device__ __forceinline__ void device_sizes(const uint32_t* n_dev, const uint32
   }
 }
 
-template <int DB>
-__global__ void __launch_bounds__(kThreads) radix_hist_kernel(const uint32_t* __restrict__ keys,
-                                                              int64_t n, int shift, int64_t nb,
-                                                              uint32_t kmin, uint32_t span,
-                                                              uint32_t* __restrict__ hist,
-                                                              const uint32_t* __restrict__ n_dev,
-                                                              const uint32_t* __restrict__ range_dev) {
-  constexpr int kRad = 1 << DB;
-  device_sizes(n_dev, range_dev, &n, &kmin, &span);
-  __shared__ uint32_t s_h[kRad];
-  for (int d = threadIdx.x; d < kRad; d += kThreads) s_h[d] = 0;
-  __syncthreads();
-  const int64_t base = static_cast<int64_t>(blockIdx.x) * kTileElems;
-  // all of the thread's loads in flight before the first count
-  uint32_t key[kRounds];
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const int64_t j = base + r * kThreads + threadIdx.x;
-    key[r] = j < n ? keys[j] : 0u;
-  }
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const int64_t j = base + r * kThreads + threadIdx.x;
-    if (j < n) atomicAdd(&s_h[digit_of<DB>(key[r], kmin, span, shift)], 1u);
-  }
-  __syncthreads();
-  for (int d = threadIdx.x; d < kRad; d += kThreads)
-    hist[static_cast<int64_t>(d) * nb + blockIdx.x] = s_h[d];
-}
+constexpr int kMaxPasses = 4;
+constexpr int kMaxRadix = 512;
+constexpr int kHistThreads = 512;
 
-// Shared memory of one scatter block (dynamic: the 9-bit form needs 52 KB).
-template <int DB>
-struct ScatterSmem {
-  uint32_t key[kTileElems];
-  uint32_t val[kTileElems];
-  uint32_t wcnt[kWarps][1 << DB];  // per-warp digit counts, then warp prefixes
-  uint32_t loc[1 << DB];           // local start of each digit's run
-  uint32_t glob[1 << DB];          // global start of this block's run per digit
-  uint32_t warp_sums[kWarps];
+// Head of the sort's scratch, cleared before the first launch; the status
+// words of the passes follow.
+struct SortHead {
+  uint32_t ticket[kMaxPasses];
+  uint32_t hist_blocks;  // histogram blocks that are done
+  uint32_t pad[59];
+  uint32_t hist[kMaxPasses][kMaxRadix];  // digit counts, then digit starts
 };
 
-// Stable scatter of one radix pass.  Each warp ranks its 512 elements (16
-// coalesced columns of 32) by digit with a warp match per column and per-warp
-// digit counters, so equal digits keep their input order; the block then
-// turns (digit, warp) counts into local offsets, places its 4096 elements
-// digit-sorted in shared memory and writes each digit's run to its global
-// offset with consecutive threads on consecutive addresses.
-template <int DB>
-__global__ void __launch_bounds__(kThreads) radix_scatter_kernel(
-    const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals, int64_t n, int shift,
-    int64_t nb, uint32_t kmin, uint32_t span, const uint32_t* __restrict__ hist_pre,
-    uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out,
-    const uint32_t* __restrict__ n_dev, const uint32_t* __restrict__ range_dev) {
-  constexpr int kRad = 1 << DB;
+struct PassShape {
+  int passes;
+  int shift[kMaxPasses], bits[kMaxPasses];
+};
+
+// Digit counts of every pass from one read of the keys (shared-memory counts
+// per block, added up in global memory); the last block to finish turns them
+// into the digits' starts.  Bound by HBM: 4 B a key.
+__global__ void __launch_bounds__(kHistThreads) radix_hist_kernel(
+    const uint32_t* __restrict__ keys, int64_t n, PassShape shape, uint32_t kmin, uint32_t span,
+    SortHead* __restrict__ head, const uint32_t* __restrict__ n_dev,
+    const uint32_t* __restrict__ range_dev) {
+  __shared__ uint32_t s_h[kMaxPasses][kMaxRadix];
+  __shared__ uint32_t s_warp[kHistThreads / 32];
+  __shared__ bool s_last;
   device_sizes(n_dev, range_dev, &n, &kmin, &span);
-  constexpr int kPer = kRad / kThreads;  // digits per thread in the block-wide steps
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  ScatterSmem<DB>& S = *reinterpret_cast<ScatterSmem<DB>*>(smem_raw);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t base = static_cast<int64_t>(blockIdx.x) * kTileElems;
-  const int n_here =
-      static_cast<int>(max(static_cast<int64_t>(0), min(static_cast<int64_t>(kTileElems), n - base)));
-  const int wbase = warp * (kTileElems / kWarps);  // 512 elements per warp
+  for (int k = threadIdx.x; k < kMaxPasses * kMaxRadix; k += kHistThreads) (&s_h[0][0])[k] = 0u;
+  __syncthreads();
+  const int64_t step = static_cast<int64_t>(gridDim.x) * kHistThreads;
+  constexpr int kAhead = 8;  // loads in flight per thread
+  for (int64_t j0 = static_cast<int64_t>(blockIdx.x) * kHistThreads + threadIdx.x; j0 < n;
+       j0 += kAhead * step) {
+    uint32_t key[kAhead];
 #pragma unroll
-  for (int k = 0; k < kRad / 32; ++k) S.wcnt[warp][lane + 32 * k] = 0;
-  __syncwarp();
+    for (int i = 0; i < kAhead; ++i) key[i] = j0 + i * step < n ? keys[j0 + i * step] : 0u;
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      if (j0 + i * step >= n) break;
+      for (int p = 0; p < shape.passes; ++p)
+        atomicAdd(&s_h[p][digit_of(key[i], kmin, span, shape.shift[p], shape.bits[p])], 1u);
+    }
+  }
+  __syncthreads();
+  for (int p = 0; p < shape.passes; ++p)
+    for (int d = threadIdx.x; d < (1 << shape.bits[p]); d += kHistThreads)
+      if (s_h[p][d]) atomicAdd(&head->hist[p][d], s_h[p][d]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&head->hist_blocks, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int p = 0; p < shape.passes; ++p) {
+    const int d = threadIdx.x;
+    const uint32_t c = d < (1 << shape.bits[p]) ? __ldcg(&head->hist[p][d]) : 0u;
+    uint32_t inc = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    uint32_t pre = 0;
+    for (int w = 0; w < warp; ++w) pre += s_warp[w];
+    if (d < (1 << shape.bits[p])) head->hist[p][d] = pre + inc - c;
+    __syncthreads();
+  }
+}
+
+// A published word of (tile, digit): the tile's own count or the inclusive
+// prefix over all tiles up to it, in the low bits; 0: not published yet.
+template <typename Word>
+struct LookWord {
+  static constexpr int kShift = 8 * sizeof(Word) - 2;
+  static constexpr Word kCount = static_cast<Word>(1) << kShift;
+  static constexpr Word kPrefix = static_cast<Word>(2) << kShift;
+  static constexpr Word kMask = kCount - 1;
+};
+
+// Shared memory of one pass block of T threads with K pairs each.
+template <int DB, int T, int K>
+struct PassSmem {
+  uint32_t key[T * K];
+  uint32_t val[T * K];
+  uint16_t wcnt[T / 32][1 << DB];  // per-warp digit counts, then warp prefixes
+  uint32_t loc[1 << DB];           // local start of each digit's run
+  uint32_t off[1 << DB];           // global start of the block's run minus its local start
+  uint32_t warp_sums[T / 32];
+  uint32_t tile;
+};
+
+// One stable pass.  A block takes T * K consecutive pairs.  Each warp ranks
+// its 32 * K keys (coalesced columns of 32) by digit with one ballot per digit
+// bit and per-warp digit counters, so equal digits keep their input order.
+// The block publishes its digit counts, places its pairs digit-sorted in
+// shared memory while its predecessors' counts arrive, adds those up (one
+// digit or two per thread, four predecessors at a time) and writes each
+// digit's run with consecutive threads on consecutive addresses.
+//
+// Bound by issue and latency (about 145 warp instructions per 32 pairs, most
+// of them the ballots; 45 % of issue slots busy, DRAM at a quarter of its
+// rate), so resident warps count; 16-bit digit counters leave shared memory
+// for them.  Against the histogram, scan (of a digit-by-tile matrix) and
+// scatter launches of a pass that this replaces, five a pass, small sorts lose
+// most of their launches (16,000 pairs: 81 -> 48 us) and large ones gain
+// little (4.8 10^7 pairs of 24 bits with their ties: 1.36 -> 1.32 ms).
+template <int DB, int T, int K, int kBlocks, typename Word>
+__global__ void __launch_bounds__(T, kBlocks) radix_pass_kernel(
+    const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals, int64_t n, int pass,
+    int shift, uint32_t kmin, uint32_t span, SortHead* __restrict__ head,
+    Word* __restrict__ status, Word* __restrict__ next_status, int next_radix, int next_pairs,
+    uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out,
+    const uint32_t* __restrict__ n_dev, const uint32_t* __restrict__ range_dev,
+    unsigned long long* __restrict__ counters) {
+  constexpr int kRad = 1 << DB;
+  constexpr int kTileN = T * K;
+  constexpr int kWarps = T / 32;
+  constexpr int kPer = kRad > T ? kRad / T : 1;  // digits per thread, next to each other
+  static_assert(kRad <= T || kRad % T == 0, "every digit has a thread");
+  using W = LookWord<Word>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  PassSmem<DB, T, K>& S = *reinterpret_cast<PassSmem<DB, T, K>*>(smem_raw);
+  device_sizes(n_dev, range_dev, &n, &kmin, &span);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) S.tile = atomicAdd(&head->ticket[pass], 1u);
+  uint32_t* const cnt2 = reinterpret_cast<uint32_t*>(S.wcnt[warp]);
+#pragma unroll
+  for (int k = 0; k < kRad / 64; ++k) cnt2[lane + 32 * k] = 0;
+  __syncthreads();
+  const uint32_t tile = S.tile;
+  const int64_t base = static_cast<int64_t>(tile) * kTileN;
+  if (base >= n) return;  // the grid was sized for more (device-side count)
+  const int n_here = static_cast<int>(min(static_cast<int64_t>(kTileN), n - base));
+  const int wbase = warp * 32 * K;
+  // the block's share of the next pass's status words, cleared
+  if (next_radix) {
+    const int64_t words = (n + next_pairs - 1) / next_pairs * next_radix;
+    const int64_t share = (words + (n - 1) / kTileN) / ((n + kTileN - 1) / kTileN);
+    const int64_t end = min(words, (tile + 1) * share);
+    for (int64_t k = tile * share + threadIdx.x; k < end; k += T) next_status[k] = 0;
+  }
 
   const uint32_t lt = lanemask_lt();
-  uint32_t key[kRounds], rank[kRounds];
+  uint32_t key[K];
+  uint32_t at[K];  // digit << 16 | rank among the warp's equal digits
   // all of the warp's key loads in flight at once (the ranking below has
   // warp barriers, which no load is moved across)
 #pragma unroll
-  for (int i = 0; i < kRounds; ++i) {
+  for (int i = 0; i < K; ++i) {
     const int j = wbase + i * 32 + lane;
     key[i] = j < n_here ? keys[base + j] : 0u;
   }
 #pragma unroll
-  for (int i = 0; i < kRounds; ++i) {
-    const int j = wbase + i * 32 + lane;
-    const bool ok = j < n_here;
-    const uint32_t d = ok ? digit_of<DB>(key[i], kmin, span, shift) : static_cast<uint32_t>(kRad);
+  for (int i = 0; i < K; ++i) {
+    // places past the end take the last digit: they come last, and their
+    // count is taken off below
+    const uint32_t d = wbase + i * 32 + lane < n_here ? digit_of(key[i], kmin, span, shift, DB)
+                                                      : static_cast<uint32_t>(kRad - 1);
     // lanes holding the same digit: one ballot per digit bit
-    uint32_t peers = __ballot_sync(0xffffffffu, ok);
-    if (!ok) peers = ~peers;
+    uint32_t peers = 0xffffffffu;
 #pragma unroll
     for (int b = 0; b < DB; ++b) {
       const bool bit = (d >> b) & 1u;
       const uint32_t bb = __ballot_sync(0xffffffffu, bit);
       peers &= bit ? bb : ~bb;
     }
-    const uint32_t before = ok ? S.wcnt[warp][d] : 0u;
-    rank[i] = before + __popc(peers & lt);
+    const uint32_t before = S.wcnt[warp][d];
+    at[i] = (d << 16) | (before + __popc(peers & lt));
     __syncwarp();
-    if (ok && (peers & lt) == 0) S.wcnt[warp][d] = before + __popc(peers);
+    if ((peers & lt) == 0) S.wcnt[warp][d] = static_cast<uint16_t>(before + __popc(peers));
     __syncwarp();
   }
   __syncthreads();
-  // per digit (thread t holds digits t * kPer .. t * kPer + kPer - 1): warp
-  // prefixes, then the block-wide digit offsets
-  uint32_t running[kPer], own = 0;
+  // the thread's digits: their counts over the warps (left as warp prefixes),
+  // published
+  const int d0 = threadIdx.x * kPer;
+  const bool has = d0 < kRad;
+  uint32_t own[kPer], sum = 0;
+  Word* const row = status + static_cast<int64_t>(tile) * kRad;
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
-    const int d = threadIdx.x * kPer + q;
-    running[q] = 0;
+    own[q] = 0;
+    if (has) {
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      const uint32_t c = S.wcnt[w][d];
-      S.wcnt[w][d] = running[q];
-      running[q] += c;
+      for (int w = 0; w < kWarps; ++w) {
+        const uint32_t c = S.wcnt[w][d0 + q];
+        S.wcnt[w][d0 + q] = static_cast<uint16_t>(own[q]);
+        own[q] += c;
+      }
+      sum += own[q];
+      if (d0 + q == kRad - 1) own[q] -= static_cast<uint32_t>(kTileN - n_here);
+      *reinterpret_cast<volatile Word*>(row + d0 + q) =
+          (tile == 0 ? W::kPrefix : W::kCount) | own[q];
     }
-    own += running[q];
   }
-  uint32_t tot;
-  uint32_t ex = block_exclusive_scan(own, S.warp_sums, &tot);
+  // local digit starts
+  uint32_t inc = sum;
 #pragma unroll
-  for (int q = 0; q < kPer; ++q) {
-    const int d = threadIdx.x * kPer + q;
-    S.loc[d] = ex;
-    ex += running[q];
-    S.glob[d] = hist_pre[static_cast<int64_t>(d) * nb + blockIdx.x];
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) S.warp_sums[warp] = inc;
+  __syncthreads();
+  uint32_t loc = inc - sum;
+  for (int w = 0; w < warp; ++w) loc += S.warp_sums[w];
+  if (has) {
+#pragma unroll
+    for (int q = 0, l = loc; q < kPer; ++q) {
+      S.loc[d0 + q] = l;
+      l += own[q];
+    }
   }
   __syncthreads();
+  // the tile's pairs, digit-sorted in shared memory
 #pragma unroll
-  for (int i = 0; i < kRounds; ++i) {
+  for (int i = 0; i < K; ++i) {
+    const uint32_t dg = at[i] >> 16;
+    at[i] = S.loc[dg] + S.wcnt[warp][dg] + (at[i] & 0xFFFFu);
+    S.key[at[i]] = key[i];
+  }
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
     const int j = wbase + i * 32 + lane;
-    if (j < n_here) {
-      const uint32_t d = digit_of<DB>(key[i], kmin, span, shift);
-      const uint32_t pos = S.loc[d] + S.wcnt[warp][d] + rank[i];
-      S.key[pos] = key[i];
-      S.val[pos] = vals[base + j];
+    const uint32_t v = j >= n_here ? 0u : vals ? vals[base + j] : static_cast<uint32_t>(base + j);
+    S.val[at[i]] = v;
+  }
+  if (has) {
+    // look-back: predecessors' counts down to the nearest prefix
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int d = d0 + q;
+      uint32_t excl = 0;
+      bool found = tile == 0;
+      for (int64_t t = static_cast<int64_t>(tile) - 1; !found; t -= 4) {
+        Word w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          w[k] = t - k >= 0 ? *reinterpret_cast<const volatile Word*>(status + (t - k) * kRad + d)
+                            : W::kPrefix;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (found) break;
+          for (int spins = 0; (w[k] & ~W::kMask) == 0; ++spins) {
+            if (spins == kLookbackSpinLimit) {  // gave up: report, count it as an empty prefix
+              if (counters) atomicAdd(&counters[kLookbackTimeout], 1ull);
+              w[k] = W::kPrefix;
+              break;
+            }
+            __nanosleep(32);
+            w[k] = *reinterpret_cast<const volatile Word*>(status + (t - k) * kRad + d);
+          }
+          excl += static_cast<uint32_t>(w[k] & W::kMask);
+          found = (w[k] & W::kPrefix) != 0;
+        }
+      }
+      if (tile > 0) *reinterpret_cast<volatile Word*>(row + d) = W::kPrefix | (excl + own[q]);
+      S.off[d] = head->hist[pass][d] + excl - S.loc[d];
     }
   }
   __syncthreads();
   // coalesced write-out of the digit runs
 #pragma unroll
-  for (int i = 0; i < kRounds; ++i) {
-    const int j = i * kThreads + threadIdx.x;
+  for (int i = 0; i < K; ++i) {
+    const int j = i * T + threadIdx.x;
     if (j < n_here) {
       const uint32_t k = S.key[j];
-      const uint32_t d = digit_of<DB>(k, kmin, span, shift);
-      const uint32_t dst = S.glob[d] + (static_cast<uint32_t>(j) - S.loc[d]);
+      const uint32_t dst = S.off[digit_of(k, kmin, span, shift, DB)] + static_cast<uint32_t>(j);
       keys_out[dst] = k;
       vals_out[dst] = S.val[j];
     }
   }
 }
 
-template <int DB>
-cudaError_t radix_pass(const uint32_t* src_k, const uint32_t* src_v, uint32_t* dst_k,
-                       uint32_t* dst_v, int64_t n, int shift, int64_t nb, uint32_t kmin,
-                       uint32_t span, uint32_t* hist, void* scan_tmp, cudaStream_t stream,
-                       const uint32_t* n_dev, const uint32_t* range_dev);
+__global__ void __launch_bounds__(256) iota_kernel(uint32_t* __restrict__ out, int64_t n) {
+  const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (k < n) out[k] = static_cast<uint32_t>(k);
+}
+
+cudaError_t launch_iota(uint32_t* out, int64_t n, cudaStream_t stream) {
+  if (n <= 0) return cudaSuccess;
+  iota_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(out, n);
+  return cudaGetLastError();
+}
 
 inline int64_t tiles_of(int64_t n) { return (n + kTileElems - 1) / kTileElems; }
 
@@ -319,21 +465,39 @@ cudaError_t exclusive_scan(const uint32_t* in, const uint32_t* gather, uint32_t*
   return cudaGetLastError();
 }
 
-size_t radix_temp_bytes(int64_t n) {
-  const int64_t nb = tiles_of(n);
-  const int64_t hist = nb * 512;  // the widest digit
-  return static_cast<size_t>(hist) * sizeof(uint32_t) + scan_temp_bytes(hist) + 256;
-}
-
 namespace {
 
-template <int DB>
+constexpr int64_t kWideSort = static_cast<int64_t>(1) << 30;  // counts need 64-bit words
+
+// Pairs of a pass block: 512 threads with 8 pairs (three blocks per SM) or 16
+// (two blocks per SM).  9-bit passes take 8: with 512 digits more resident
+// warps are worth more than longer runs (tile sorts of the 100-view,
+// 10^6-Gaussian workload 2.95 ms against 3.33).  8-bit passes take 16 (its
+// depth sorts 2.74 ms against 2.88) unless that would leave fewer than two
+// blocks per SM of 152.
+constexpr int kPassThreads = 512;
+constexpr int64_t kSmallSort = 2 * 152 * 16 * kPassThreads;
+int pass_items(int64_t n, int bits) { return bits == 9 || n < kSmallSort ? 8 : 16; }
+int64_t pass_tiles(int64_t n, int bits) {
+  const int64_t pairs = kPassThreads * pass_items(n, bits);
+  return (n + pairs - 1) / pairs;
+}
+
+// Status words of one pass: a word per (tile, digit), two passes' worth in
+// turn (a pass clears the next one's).
+size_t status_bytes(int64_t n) {
+  const int64_t tiles = (n + 8 * kPassThreads - 1) / (8 * kPassThreads);  // the smallest tile
+  return static_cast<size_t>(tiles) * kMaxRadix * (n < kWideSort ? 4 : 8);
+}
+
+template <int DB, int K, typename Word>
 cudaError_t radix_pass(const uint32_t* src_k, const uint32_t* src_v, uint32_t* dst_k,
-                       uint32_t* dst_v, int64_t n, int shift, int64_t nb, uint32_t kmin,
-                       uint32_t span, uint32_t* hist, void* scan_tmp, cudaStream_t stream,
-                       const uint32_t* n_dev, const uint32_t* range_dev) {
-  constexpr int kRad = 1 << DB;
-  const size_t smem = sizeof(ScatterSmem<DB>);
+                       uint32_t* dst_v, int64_t n, int pass, int shift, uint32_t kmin,
+                       uint32_t span, SortHead* head, void* status, void* next_status,
+                       int next_radix, int next_pairs, cudaStream_t stream, const uint32_t* n_dev,
+                       const uint32_t* range_dev, unsigned long long* counters) {
+  constexpr int T = kPassThreads, kBlocks = K > 8 ? 2 : 3;
+  const size_t smem = sizeof(PassSmem<DB, T, K>);
   // dynamic shared memory above 48 KB needs the opt-in, once per device
   static std::atomic<uint64_t> attr_set{0};
   int dev = 0;
@@ -341,22 +505,25 @@ cudaError_t radix_pass(const uint32_t* src_k, const uint32_t* src_v, uint32_t* d
   if (e0 != cudaSuccess) return e0;
   const uint64_t bit = 1ull << (dev & 63);
   if (!(attr_set.load() & bit)) {
-    cudaError_t e = cudaFuncSetAttribute(radix_scatter_kernel<DB>,
+    cudaError_t e = cudaFuncSetAttribute(radix_pass_kernel<DB, T, K, kBlocks, Word>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     attr_set.fetch_or(bit);
   }
-  radix_hist_kernel<DB><<<static_cast<unsigned>(nb), kThreads, 0, stream>>>(
-      src_k, n, shift, nb, kmin, span, hist, n_dev, range_dev);
-  cudaError_t e = exclusive_scan(hist, nullptr, hist, nb * kRad, nullptr, scan_tmp, stream);
-  if (e != cudaSuccess) return e;
-  radix_scatter_kernel<DB><<<static_cast<unsigned>(nb), kThreads, smem, stream>>>(
-      src_k, src_v, n, shift, nb, kmin, span, hist, dst_k, dst_v, n_dev, range_dev);
+  const int64_t tiles = (n + T * K - 1) / (T * K);
+  radix_pass_kernel<DB, T, K, kBlocks, Word><<<static_cast<unsigned>(tiles), T, smem, stream>>>(
+      src_k, src_v, n, pass, shift, kmin, span, head, static_cast<Word*>(status),
+      static_cast<Word*>(next_status), next_radix, next_pairs, dst_k, dst_v, n_dev, range_dev,
+      counters);
   return cudaGetLastError();
 }
 
 }  // namespace
+
+size_t radix_temp_bytes(int64_t n) {
+  return sizeof(SortHead) + 2 * status_bytes(n) + 256;
+}
 
 int radix_passes(int bits) {
   if (bits <= 0) return 0;
@@ -365,37 +532,57 @@ int radix_passes(int bits) {
 
 cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
                              uint32_t* vals_alt, int64_t n, int bits, void* temp, bool* in_alt,
-                             cudaStream_t stream, uint32_t kmin, uint32_t span,
-                             const uint32_t* n_dev, const uint32_t* range_dev) {
+                             cudaStream_t stream, unsigned long long* counters, bool iota,
+                             uint32_t kmin, uint32_t span, const uint32_t* n_dev,
+                             const uint32_t* range_dev) {
   *in_alt = false;
-  if (n <= 1 || bits <= 0) return cudaSuccess;
-  const int64_t nb = tiles_of(n);
-  uint32_t* hist = static_cast<uint32_t*>(temp);
-  void* scan_tmp = reinterpret_cast<char*>(temp) +
-                   ((static_cast<size_t>(nb) * 512 * sizeof(uint32_t) + 255) / 256) * 256;
   // digit widths: 8 bits, or 9 where that saves a whole pass (17 -> 9 + 8)
-  const int passes = radix_passes(bits);
-  int wide = bits - 8 * passes;  // passes that take 9 bits
-  if (wide < 0) wide = 0;
+  PassShape shape{};
+  shape.passes = n > 1 ? radix_passes(bits) : 0;
+  if (shape.passes > kMaxPasses) return cudaErrorInvalidValue;
+  if (shape.passes == 0) return iota ? launch_iota(vals, n, stream) : cudaSuccess;
+  const int wide = std::max(0, bits - 8 * shape.passes);  // passes that take 9 bits
+  for (int p = 0, shift = 0; p < shape.passes; ++p) {
+    shape.bits[p] = p < wide ? 9 : 8;
+    shape.shift[p] = shift;
+    shift += shape.bits[p];
+  }
+  SortHead* head = static_cast<SortHead*>(temp);
+  char* status[2];
+  status[0] = static_cast<char*>(temp) + sizeof(SortHead);
+  status[1] = status[0] + status_bytes(n);
+  const int64_t nt = pass_tiles(n, shape.bits[0]);
+  const size_t word = n < kWideSort ? 4 : 8;
+  cudaError_t e = cudaMemsetAsync(
+      temp, 0, sizeof(SortHead) + static_cast<size_t>(nt << shape.bits[0]) * word, stream);
+  if (e != cudaSuccess) return e;
+  const int64_t hist_blocks = std::min<int64_t>((n + 4 * kHistThreads - 1) / (4 * kHistThreads), 608);
+  radix_hist_kernel<<<static_cast<unsigned>(hist_blocks), kHistThreads, 0, stream>>>(
+      keys, n, shape, kmin, span, head, n_dev, range_dev);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   uint32_t *src_k = keys, *src_v = vals, *dst_k = keys_alt, *dst_v = vals_alt;
-  int shift = 0;
-  for (int p = 0; p < passes; ++p) {
-    const bool nine = p < wide;
-    cudaError_t e = nine ? radix_pass<9>(src_k, src_v, dst_k, dst_v, n, shift, nb, kmin, span,
-                                         hist, scan_tmp, stream, n_dev, range_dev)
-                         : radix_pass<8>(src_k, src_v, dst_k, dst_v, n, shift, nb, kmin, span,
-                                         hist, scan_tmp, stream, n_dev, range_dev);
+  for (int p = 0; p < shape.passes; ++p) {
+    const bool more = p + 1 < shape.passes;
+    const int next_radix = more ? 1 << shape.bits[p + 1] : 0;
+    const int next_pairs = more ? kPassThreads * pass_items(n, shape.bits[p + 1]) : 1;
+    const uint32_t* v = iota && p == 0 ? nullptr : src_v;
+    auto run = [&](auto pass) {
+      return pass(src_k, v, dst_k, dst_v, n, p, shape.shift[p], kmin, span, head, status[p & 1],
+                  status[(p + 1) & 1], next_radix, next_pairs, stream, n_dev, range_dev, counters);
+    };
+    const bool wide_counts = n >= kWideSort;
+    if (shape.bits[p] == 9)
+      e = wide_counts ? run(radix_pass<9, 8, uint64_t>) : run(radix_pass<9, 8, uint32_t>);
+    else if (pass_items(n, 8) == 8)
+      e = run(radix_pass<8, 8, uint32_t>);
+    else
+      e = wide_counts ? run(radix_pass<8, 16, uint64_t>) : run(radix_pass<8, 16, uint32_t>);
     if (e != cudaSuccess) return e;
-    shift += nine ? 9 : 8;
-    uint32_t* tk = src_k;
-    uint32_t* tv = src_v;
-    src_k = dst_k;
-    src_v = dst_v;
-    dst_k = tk;
-    dst_v = tv;
+    std::swap(src_k, dst_k);
+    std::swap(src_v, dst_v);
     *in_alt = !*in_alt;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace fs
