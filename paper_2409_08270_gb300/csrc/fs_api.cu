@@ -619,10 +619,7 @@ fs_status ensure_window(fs_ctx* c, int64_t n, int vb, int32_t V, bool keep) {
   FS_TRY(c->val_a.ensure(static_cast<size_t>(kcap) * 4, "vals"));
   FS_TRY(c->key_b.ensure(static_cast<size_t>(kcap) * 4, "keys"));
   FS_TRY(c->val_b.ensure(static_cast<size_t>(kcap) * 4, "vals"));
-  FS_TRY(c->offs.ensure(static_cast<size_t>(kcap) * 4, "offsets"));
-  FS_TRY(c->scan_tmp.ensure(fs::scan_temp_bytes(kcap), "scan temp"));
   FS_TRY(c->sort_tmp.ensure(fs::radix_temp_bytes(kcap), "sort temp"));
-  FS_TRY(c->ccnt.ensure(static_cast<size_t>(kcap) * 4, "chunk counts"));
   return FS_OK;
 }
 
@@ -662,7 +659,7 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
   if (range_dev) {
     uint32_t* total = c->total.as<uint32_t>();
     const uint32_t capacity = static_cast<uint32_t>(plan_cap);
-    FS_CUDA(fs::launch_bin_fused(0, n_pos, n, vd, sorted_val, P.foot, sat, c->lk_a.as<uint32_t>(),
+    FS_CUDA(fs::launch_bin_fused(0, n_pos, n, vd, nb, sorted_val, P.foot, sat, c->lk_a.as<uint32_t>(),
                                  val_dst->as<uint32_t>(), capacity, c->lb_tmp.p, total, ctr,
                                  stream, range_dev),
             "binning");
@@ -693,7 +690,7 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
     c->stats.kernel_launches += 1;
     int tb = -1;
     FS_TRY(stage_begin(c, FS_STAGE_BINNING, stream, false, &tb));
-    FS_CUDA(fs::launch_bin_fused(p0, n_pos, n, vd, sorted_val, P.foot, sat,
+    FS_CUDA(fs::launch_bin_fused(p0, n_pos, n, vd, nb, sorted_val, P.foot, sat,
                                  c->lk_a.as<uint32_t>(), val_dst->as<uint32_t>(), capacity,
                                  c->lb_tmp.p, c->total.as<uint32_t>(), ctr, stream),
             "binning");
@@ -1044,6 +1041,9 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
   const int tile_bits = std::max(1, ceil_log2(total_tiles));
   const int64_t k_total = static_cast<int64_t>(nb) * n;
   unsigned long long* ctr = c->counters.as<unsigned long long>();
+  FS_TRY(c->ccnt.ensure(static_cast<size_t>(kcap) * 4, "candidate flags"));
+  FS_TRY(c->offs.ensure(static_cast<size_t>(kcap) * 4, "candidate offsets"));
+  FS_TRY(c->scan_tmp.ensure(fs::scan_temp_bytes(kcap), "scan temp"));
   c->stats.kernel_launches += 1 + scan_launches(k_total);
   FS_CUDA(fs::launch_candidates(k_total, n, vd, P.cnt, P.foot, skip, c->ccnt.as<uint32_t>(),
                                 stream),

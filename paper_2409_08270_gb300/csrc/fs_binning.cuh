@@ -7,9 +7,9 @@
 namespace fs {
 
 // Inflated r2 used for binning (conservative against FP32 rounding).  The
-// binning arithmetic uses explicit round-to-nearest intrinsics so that the
-// count (projection kernel) and the emission (emit kernel) evaluate it
-// bit-identically whatever the compiler contracts elsewhere.
+// binning arithmetic uses explicit round-to-nearest intrinsics so that every
+// kernel that bins evaluates it bit-identically whatever the compiler contracts
+// elsewhere.
 __device__ __forceinline__ float binning_r2(float r2) {
   return __fadd_rn(__fmul_rn(r2, 1.001f), 1e-3f);
 }
@@ -45,12 +45,11 @@ __device__ __forceinline__ bool any_free(const uint64_t* __restrict__ sat, int a
   return false;
 }
 
-// Unsaturated tiles of rows [r0, r1] x columns [c0, c1] of a view, from its
-// prefix table (four reads).
-__device__ __forceinline__ uint32_t free_in_box(const ViewParams& vp, int r0, int r1, int c0,
-                                                int c1) {
-  const int w1 = vp.tiles_x + 1;
-  const uint32_t* t = vp.free_tab;
+// Unsaturated tiles of rows [r0, r1] x columns [c0, c1] of a view of tiles_x
+// columns, from its prefix table t (four reads).
+__device__ __forceinline__ uint32_t free_in_box(const uint32_t* __restrict__ t, int tiles_x,
+                                                int r0, int r1, int c0, int c1) {
+  const int w1 = tiles_x + 1;
   return t[(r1 + 1) * w1 + c1 + 1] - t[r0 * w1 + c1 + 1] - t[(r1 + 1) * w1 + c0] +
          t[r0 * w1 + c0];
 }
@@ -92,10 +91,10 @@ __device__ __forceinline__ bool row_span(const Footprint& f, int ty, int width, 
 
 // Under 3-sigma coverage, [tx0, tx1] narrowed to the slot's tile columns
 // (false if nothing is left); unchanged under exact coverage.
-__device__ __forceinline__ bool clip_cols(const ViewParams& vp, int64_t slot, int* tx0,
-                                          int* tx1) {
-  if (!vp.cols) return true;
-  const uint32_t c = vp.cols[slot];
+__device__ __forceinline__ bool clip_cols(const uint32_t* __restrict__ cols, int64_t slot,
+                                          int* tx0, int* tx1) {
+  if (!cols) return true;
+  const uint32_t c = cols[slot];
   *tx0 = max(*tx0, static_cast<int>(c & 0xFFFFu));
   *tx1 = min(*tx1, static_cast<int>(c >> 16));
   return *tx0 <= *tx1;

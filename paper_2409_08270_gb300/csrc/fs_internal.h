@@ -67,23 +67,14 @@ cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, cons
 cudaError_t launch_depth_tie_fix(int64_t n_total, int64_t n, const uint32_t* key, uint32_t* val,
                                  const uint32_t* depth_lo, cudaStream_t stream,
                                  const uint32_t* n_dev = nullptr);
-// Binning of sorted positions [p0, p0 + n_pos): one list entry (key = tile
-// id, value = slot) per (tile, Gaussian) whose footprint reaches the tile,
-// unless the tile's `sat` bit is set.
-cudaError_t launch_chunk_count(int64_t p0, int64_t n_pos, int64_t n, const ViewParams* views,
-                               const uint32_t* sorted_val, const Footprint* foot,
-                               const uint64_t* sat, uint32_t* out_cnt, cudaStream_t stream);
-cudaError_t launch_emit(int64_t p0, int64_t n_pos, int64_t n, const ViewParams* views,
-                        const uint32_t* sorted_val, const uint32_t* offsets,
-                        const uint32_t* chunk_cnt, const Footprint* foot,
-                        const uint64_t* sat, uint32_t* out_key, uint32_t* out_val,
-                        unsigned long long* counters, cudaStream_t stream);
-// Count, scan and emit of sorted positions [p0, p0 + n_pos) in one launch
-// (decoupled look-back).  Entries at positions >= capacity are not written;
+// Binning of sorted positions [p0, p0 + n_pos): one list entry (key = tile id,
+// value = slot) per (tile, Gaussian) whose footprint reaches the tile, unless
+// the tile's `sat` bit is set, in one launch (count, decoupled look-back,
+// emit).  Entries at positions >= capacity are not written;
 // *total (device) receives the entry count.  lookback: bin_fused_temp_bytes
 // of scratch (cleared by the launcher).
 cudaError_t launch_bin_fused(int64_t p0, int64_t n_pos, int64_t n, const ViewParams* views,
-                             const uint32_t* sorted_val, const Footprint* foot,
+                             int n_views, const uint32_t* sorted_val, const Footprint* foot,
                              const uint64_t* sat, uint32_t* out_key, uint32_t* out_val,
                              uint32_t capacity, void* lookback, uint32_t* total,
                              unsigned long long* counters, cudaStream_t stream,

@@ -36,7 +36,7 @@ constexpr int kNA_Side = FS_NOALLOC_MAX_SIDE;
 constexpr int64_t kNA_Entries = FS_NOALLOC_MAX_LIST_ENTRIES;
 constexpr int kNA_Tiles = (kNA_Side / kTile) * (kNA_Side / kTile);
 constexpr size_t kNA_SortTmp = 544 * 1024;  // >= radix_temp_bytes(kNA_Entries), checked at run time
-constexpr size_t kNA_ScanTmp = 4 * 1024;    // >= scan_temp_bytes(kNA_N), checked at run time
+constexpr size_t kNA_BinTmp = 2 * 1024;     // >= bin_fused_temp_bytes(kNA_N), checked at run time
 
 constexpr size_t al(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
@@ -51,9 +51,7 @@ constexpr size_t oKeyA = oCnt + al(kNA_N * 4);
 constexpr size_t oValA = oKeyA + al(kNA_N * 4);
 constexpr size_t oKeyB = oValA + al(kNA_N * 4);
 constexpr size_t oValB = oKeyB + al(kNA_N * 4);
-constexpr size_t oOffs = oValB + al(kNA_N * 4);
-constexpr size_t oCcnt = oOffs + al(kNA_N * 4);
-constexpr size_t oDlo = oCcnt + al(kNA_N * 4);
+constexpr size_t oDlo = oValB + al(kNA_N * 4);
 constexpr size_t oLkA = oDlo + al(kNA_N * 4);
 constexpr size_t oLvA = oLkA + al(kNA_Entries * 4);
 constexpr size_t oLkB = oLvA + al(kNA_Entries * 4);
@@ -63,8 +61,8 @@ constexpr size_t oState = oRanges + al(kNA_Tiles * 8);
 constexpr size_t oSat = oState + al(static_cast<size_t>(kNA_Side) * kNA_Side * 4);
 constexpr size_t oSubsat = oSat + al(kNA_Tiles);
 constexpr size_t oSortTmp = oSubsat + al(4 * kNA_Tiles);
-constexpr size_t oScanTmp = oSortTmp + al(kNA_SortTmp);
-constexpr size_t oWords = oScanTmp + al(kNA_ScanTmp);  // total (u32), error word (u32)
+constexpr size_t oBinTmp = oSortTmp + al(kNA_SortTmp);
+constexpr size_t oWords = oBinTmp + al(kNA_BinTmp);  // total (u32), error word (u32)
 constexpr size_t oCounters = oWords + 256;
 constexpr size_t kNA_Bytes = oCounters + al(kNumCounters * 8);
 
@@ -161,7 +159,7 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
           return na_fail(FS_INVALID_ARGUMENT, "fs_solve_noalloc: camera R is not a rotation");
       }
   }
-  if (radix_temp_bytes(kNA_Entries) > kNA_SortTmp || scan_temp_bytes(kNA_N) > kNA_ScanTmp)
+  if (radix_temp_bytes(kNA_Entries) > kNA_SortTmp || bin_fused_temp_bytes(kNA_N) > kNA_BinTmp)
     return na_fail(FS_UNSUPPORTED, "fs_solve_noalloc: internal scratch layout too small");
 
   int prev = -1;
@@ -188,8 +186,6 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
   uint32_t* val_a = reinterpret_cast<uint32_t*>(S + oValA);
   uint32_t* key_b = reinterpret_cast<uint32_t*>(S + oKeyB);
   uint32_t* val_b = reinterpret_cast<uint32_t*>(S + oValB);
-  uint32_t* offs = reinterpret_cast<uint32_t*>(S + oOffs);
-  uint32_t* ccnt = reinterpret_cast<uint32_t*>(S + oCcnt);
   uint32_t* dlo = reinterpret_cast<uint32_t*>(S + oDlo);
   uint32_t* lk_a = reinterpret_cast<uint32_t*>(S + oLkA);
   uint32_t* lv_a = reinterpret_cast<uint32_t*>(S + oLvA);
@@ -200,7 +196,7 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
   uint64_t* sat = reinterpret_cast<uint64_t*>(S + oSat);
   uint64_t* subsat = reinterpret_cast<uint64_t*>(S + oSubsat);
   void* sort_tmp = S + oSortTmp;
-  void* scan_tmp = S + oScanTmp;
+  void* lookback = S + oBinTmp;
   uint32_t* total_d = reinterpret_cast<uint32_t*>(S + oWords);
   unsigned int* err_d = reinterpret_cast<unsigned int*>(S + oWords + 4);
   unsigned long long* ctr = reinterpret_cast<unsigned long long*>(S + oCounters);
@@ -248,8 +244,10 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
       const int64_t p1 = (ci == chunks - 1) ? n : (n >> (chunks - 1 - ci));
       const int64_t n_pos = p1 - p0;
       if (n_pos <= 0) continue;
-      NA_CUDA(launch_chunk_count(p0, n_pos, n, vd, sval, foot, sat, ccnt, strm), "count");
-      NA_CUDA(exclusive_scan(ccnt, nullptr, offs, n_pos, total_d, scan_tmp, strm), "scan");
+      NA_CUDA(launch_bin_fused(p0, n_pos, n, vd, 1, sval, foot, sat, lk_a, lv_a,
+                               static_cast<uint32_t>(kNA_Entries), lookback, total_d, ctr, strm,
+                               nullptr),
+              "binning");
       uint32_t I = 0;
       NA_CUDA(cudaMemcpyAsync(&I, total_d, 4, cudaMemcpyDeviceToHost, strm), "readback");
       NA_CUDA(cudaStreamSynchronize(strm), "readback");
@@ -258,9 +256,6 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
                        "fs_solve_noalloc: a view needs more than FS_NOALLOC_MAX_LIST_ENTRIES "
                        "(tile, Gaussian) pairs in one depth chunk; the table is incomplete");
       if (I > 0) {
-        NA_CUDA(launch_emit(p0, n_pos, n, vd, sval, offs, ccnt, foot, sat, lk_a, lv_a, ctr,
-                            strm),
-                "emit");
         bool alt2 = false;
         NA_CUDA(radix_sort_pairs(lk_a, lv_a, lk_b, lv_b, I, bits_for(tiles), sort_tmp, &alt2, strm,
                                  ctr),
@@ -282,7 +277,7 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
   NA_CUDA(cudaMemcpyAsync(h_ctr, ctr, sizeof(h_ctr), cudaMemcpyDeviceToHost, strm), "readback");
   NA_CUDA(cudaStreamSynchronize(strm), "readback");
   if (h_ctr[kLookbackTimeout])
-    return na_fail(FS_TIMEOUT, "fs_solve_noalloc: a sort's bounded wait gave up");
+    return na_fail(FS_TIMEOUT, "fs_solve_noalloc: a bounded wait of the binning or a sort gave up");
   if (h_ctr[kBinningMismatch])
     return na_fail(FS_CUDA_ERROR, "fs_solve_noalloc: internal binning mismatch");
   return FS_OK;

@@ -522,23 +522,26 @@ __global__ void depth_tie_fix_kernel(int64_t n_total, int64_t n, const uint32_t*
 
 // ---------------------------------------------------------------------------
 // Per depth chunk: count and emit the (tile, Gaussian) entries of sorted
-// positions [p0, p0 + n_pos) on tiles not yet saturated.  A warp takes 32
-// consecutive positions and spreads all of their tile rows over its lanes,
-// one (Gaussian, row) per lane per round, so large footprints do not hold up
-// small ones.  The owner of row r is found by a binary search over the
-// lanes' inclusive row counts.
+// positions [p0, p0 + n_pos) on tiles not yet saturated.
 // ---------------------------------------------------------------------------
 
+// What the binning reads of a view, kept in shared memory: consecutive sorted
+// positions belong to any of the batch's views, and 32 different views'
+// parameters read through L1 take a line each.
+struct BinView {
+  int tile_base, tiles_x, width, cell;  // cell: the view's first prefix-table entry
+};
+
 struct RowJob {
-  uint32_t g;      // slot of the owning Gaussian (view * n + index)
   int row;         // tile row
   int owner;       // lane that holds the owning Gaussian
   bool ok;         // r < R
 };
 
-// Every lane of the warp must call this (it shuffles).
-__device__ __forceinline__ RowJob row_job(int r, int R, uint32_t incl_rows, uint32_t g_lane,
-                                          int ty0_lane) {
+// Row r of the warp's 32 Gaussians' tile rows, in order: the owner is found by
+// a binary search over the lanes' inclusive row counts.  Every lane of the
+// warp must call this (it shuffles).
+__device__ __forceinline__ RowJob row_job(int r, int R, uint32_t incl_rows, int ty0_lane) {
   // owner = number of lanes whose inclusive row count is <= r
   int lo = 0;
 #pragma unroll
@@ -548,81 +551,59 @@ __device__ __forceinline__ RowJob row_job(int r, int R, uint32_t incl_rows, uint
   }
   const int owner = min(lo, 31);
   const uint32_t pi = __shfl_sync(0xffffffffu, incl_rows, max(owner - 1, 0));
-  const uint32_t g = __shfl_sync(0xffffffffu, g_lane, owner);
   const int ty0 = __shfl_sync(0xffffffffu, ty0_lane, owner);
   RowJob j;
   j.ok = r < R;
-  j.g = g;
   j.owner = owner;
   j.row = ty0 + (r - static_cast<int>(owner > 0 ? pi : 0u));
   return j;
 }
 
-// Unsaturated tiles of one job's row: [a, b] (global ids) and their number.
-__device__ __forceinline__ uint32_t job_free(const RowJob& jb, SlotView sv,
-                                             const ViewParams* __restrict__ views,
-                                             const Footprint* __restrict__ foot,
-                                             const uint64_t* __restrict__ sat, int* a, int* b) {
-  *a = 0;
-  *b = -1;
-  if (!jb.ok) return 0;
-  const int v = static_cast<int>(sv(jb.g));
-  const Footprint f = foot[jb.g];
-  int tx0, tx1;
-  if (!row_span(f, jb.row, views[v].width, &tx0, &tx1)) return 0;
-  if (!clip_cols(views[v], jb.g, &tx0, &tx1)) return 0;
-  const int base = views[v].tile_base + jb.row * views[v].tiles_x;
-  *a = base + tx0;
-  *b = base + tx1;
-  return count_free(sat, *a, *b);
-}
-
-// The lane's sorted position j (if < n_pos): its slot g, first tile row ty0
-// and number of tile rows -- none when every tile of its footprint's
-// bounding box is already saturated, as is the case for most slots of later
-// depth chunks.  Over the footprint x(dy) - mx stays within +-hx, hx^2 =
-// syr (a^2 + b2); the box takes one more pixel on each side than the rows'
-// spans, so it holds every span whatever their rounding.
-__device__ __forceinline__ void lane_rows(int64_t j, int64_t n_pos, int64_t p0, SlotView sv,
-                                          const ViewParams* __restrict__ views,
-                                          const uint32_t* __restrict__ sorted_val,
-                                          const Footprint* __restrict__ foot,
-                                          const uint64_t* __restrict__ sat, uint32_t* g,
-                                          int* ty0, uint32_t* nrows) {
-  *g = 0;
-  *ty0 = 0;
-  *nrows = 0;
-  if (j >= n_pos) return;
-  const uint32_t gg = sorted_val[p0 + j];
-  *g = gg;
-  const Footprint f = foot[gg];
+// Number of tile rows of a slot's footprint (first row *ty0) -- none when every
+// tile of the footprint's bounding box is already saturated, as is the case
+// for most slots of later depth chunks.  Over the footprint x(dy) - mx stays
+// within +-hx, hx^2 = syr (a^2 + b2); the box takes one more pixel on each
+// side than the rows' spans, so it holds every span whatever their rounding.
+__device__ __forceinline__ uint32_t live_rows(const Footprint& f, uint32_t slot, const BinView& vp,
+                                              const uint32_t* __restrict__ cols,
+                                              const uint32_t* __restrict__ free_tab,
+                                              const uint64_t* __restrict__ sat, int* ty0) {
   int t0, t1;
   footprint_rows(f, &t0, &t1);
   *ty0 = t0;
-  if (t1 < t0) return;
-  const ViewParams& vp = views[sv(gg)];
+  if (t1 < t0) return 0u;
   const float hx = sqrtf(f.syr * fmaf(f.a, f.a, f.b2));
   const float x0 = fmaxf(ceilf(f.mx - hx - 2.5f), 0.f);
   const float x1 = fminf(floorf(f.mx + hx + 1.5f), static_cast<float>(vp.width - 1));
-  if (!(x0 <= x1)) return;
+  if (!(x0 <= x1)) return 0u;
   int c0 = static_cast<int>(x0) / kTile, c1 = static_cast<int>(x1) / kTile;
-  if (vp.cols) {  // 3-sigma coverage
-    const uint32_t c = vp.cols[gg];
+  if (cols) {  // 3-sigma coverage
+    const uint32_t c = cols[slot];
     c0 = max(c0, static_cast<int>(c & 0xFFFFu));
     c1 = min(c1, static_cast<int>(c >> 16));
-    if (c0 > c1) return;
+    if (c0 > c1) return 0u;
   }
-  if (vp.free_tab) {
-    if (free_in_box(vp, t0, t1, c0, c1)) *nrows = static_cast<uint32_t>(t1 - t0 + 1);
-    return;
-  }
+  const uint32_t rows = static_cast<uint32_t>(t1 - t0 + 1);
+  if (free_tab) return free_in_box(free_tab + vp.cell, vp.tiles_x, t0, t1, c0, c1) ? rows : 0u;
   for (int ty = t0; ty <= t1; ++ty) {
     const int base = vp.tile_base + ty * vp.tiles_x;
-    if (any_free(sat, base + c0, base + c1)) {
-      *nrows = static_cast<uint32_t>(t1 - t0 + 1);
-      return;
-    }
+    if (any_free(sat, base + c0, base + c1)) return rows;
   }
+  return 0u;
+}
+
+// Unsaturated tiles of one tile row of a footprint: [*a, *b] (global ids) and
+// their number.
+__device__ __forceinline__ uint32_t row_free(const Footprint& f, uint32_t slot, int row,
+                                             const BinView& vp, const uint32_t* __restrict__ cols,
+                                             const uint64_t* __restrict__ sat, int* a, int* b) {
+  int tx0, tx1;
+  if (!row_span(f, row, vp.width, &tx0, &tx1)) return 0;
+  if (!clip_cols(cols, slot, &tx0, &tx1)) return 0;
+  const int base = vp.tile_base + row * vp.tiles_x;
+  *a = base + tx0;
+  *b = base + tx1;
+  return count_free(sat, *a, *b);
 }
 
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x, int lane) {
@@ -634,138 +615,82 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x, int lane) {
   return x;
 }
 
-__global__ void __launch_bounds__(256) chunk_count_kernel(
-    int64_t p0, int64_t n_pos, SlotView sv, const ViewParams* __restrict__ views,
-    const uint32_t* __restrict__ sorted_val,
-    const Footprint* __restrict__ foot, const uint64_t* __restrict__ sat,
-    uint32_t* __restrict__ out_cnt) {
-
-  __shared__ uint32_t s_cnt[8][32];
-  const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t g, nrows;
-  int ty0;
-  lane_rows(j, n_pos, p0, sv, views, sorted_val, foot, sat, &g, &ty0, &nrows);
-  const uint32_t incl = warp_incl_scan(nrows, lane);
-  const int R = static_cast<int>(__shfl_sync(0xffffffffu, incl, 31));
-  s_cnt[warp][lane] = 0;
-  __syncwarp();
-  for (int r0 = 0; r0 < R; r0 += 32) {
-    const RowJob jb = row_job(r0 + lane, R, incl, g, ty0);
-    int a, b;
-    const uint32_t fr = job_free(jb, sv, views, foot, sat, &a, &b);
-    if (jb.ok && fr) atomicAdd(&s_cnt[warp][jb.owner], fr);
+// The k-th (from 0) unsaturated tile id from `a` on; there must be one.
+__device__ __forceinline__ uint32_t nth_free(const uint64_t* __restrict__ sat, int a, int k) {
+  int w = a >> 6;
+  uint64_t bits = ~sat[w] & (~0ull << (a & 63));
+  for (int c = __popcll(bits); k >= c; c = __popcll(bits)) {
+    k -= c;
+    bits = ~sat[++w];
   }
-  __syncwarp();
-  if (j < n_pos) out_cnt[j] = s_cnt[warp][lane];
-}
-
-// Writes (tile, g) for every unsaturated tile id in [a, b], from position o,
-// never at or past `end`; returns the next position.
-__device__ __forceinline__ uint32_t emit_free(const uint64_t* __restrict__ sat, int a, int b,
-                                              uint32_t g, uint32_t* __restrict__ out_key,
-                                              uint32_t* __restrict__ out_val, uint32_t o,
-                                              uint32_t end) {
-  const int wa = a >> 6, wb = b >> 6;
-  for (int w = wa; w <= wb; ++w) {
-    uint64_t m = ~0ull;
-    if (w == wa) m &= ~0ull << (a & 63);
-    if (w == wb) m &= ~0ull >> (63 - (b & 63));
-    uint64_t bits = ~sat[w] & m;
-    while (bits && o < end) {
-      const int bit = __ffsll(static_cast<long long>(bits)) - 1;
-      bits &= bits - 1;
-      out_key[o] = static_cast<uint32_t>(w * 64 + bit);
-      out_val[o] = g;
-      ++o;
-    }
-  }
-  return o;
-}
-
-// Writes the list entries of sorted positions [p0, p0 + n_pos) in depth
-// order: the warp's 32 Gaussians own the contiguous output range starting at
-// offsets[first] (the exclusive scan of chunk_cnt); row r's entries start at
-// that base plus the free tiles of all earlier rows of the warp.
-__global__ void __launch_bounds__(256) emit_kernel(
-    int64_t p0, int64_t n_pos, SlotView sv, const ViewParams* __restrict__ views,
-    const uint32_t* __restrict__ sorted_val, const uint32_t* __restrict__ offsets,
-    const uint32_t* __restrict__ chunk_cnt,
-    const Footprint* __restrict__ foot, const uint64_t* __restrict__ sat,
-    uint32_t* __restrict__ out_key, uint32_t* __restrict__ out_val,
-    unsigned long long* __restrict__ counters) {
-
-  const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  uint32_t g, nrows;
-  int ty0;
-  lane_rows(j, n_pos, p0, sv, views, sorted_val, foot, sat, &g, &ty0, &nrows);
-  const uint32_t incl = warp_incl_scan(nrows, lane);
-  const int R = static_cast<int>(__shfl_sync(0xffffffffu, incl, 31));
-  // the warp's output range [wbeg, wend)
-  const int64_t jw = j - lane;  // first position of the warp
-  const int64_t jl = min(jw + 31, n_pos - 1);
-  uint32_t wbeg = 0, wend = 0;
-  if (lane == 0 && jw < n_pos) {
-    wbeg = offsets[jw];
-    wend = offsets[jl] + chunk_cnt[jl];
-  }
-  wbeg = __shfl_sync(0xffffffffu, wbeg, 0);
-  wend = __shfl_sync(0xffffffffu, wend, 0);
-  uint32_t carry = 0;
-  for (int r0 = 0; r0 < R; r0 += 32) {
-    const RowJob jb = row_job(r0 + lane, R, incl, g, ty0);
-    int a, b;
-    const uint32_t fr = job_free(jb, sv, views, foot, sat, &a, &b);
-    const uint32_t sc = warp_incl_scan(fr, lane);
-    const uint32_t o = wbeg + carry + sc - fr;
-    if (fr) emit_free(sat, a, b, jb.g, out_key, out_val, o, min(o + fr, wend));
-    carry += __shfl_sync(0xffffffffu, sc, 31);
-  }
-  if (lane == 0 && jw < n_pos && wbeg + carry != wend) atomicAdd(&counters[kBinningMismatch], 1ull);
+  for (; k > 0; --k) bits &= bits - 1;
+  return static_cast<uint32_t>(w * 64 + __ffsll(static_cast<long long>(bits)) - 1);
 }
 
 // Count, offset and emit in one pass.  Blocks take virtual ids in launch
 // order (a ticket), so every block's predecessors are running or done.  A
 // block (4 warps: a short wait at its barriers) counts its 128 positions'
-// entries, publishes the count, then adds
-// up its predecessors' published words (decoupled look-back: a word is
-// either a block's own count or the inclusive prefix up to it; the walk
-// stops at the first prefix), publishes its own prefix and emits from its
-// offset.  No block waits on a later one.  Entries at or past `capacity`
-// are not written; *total receives the entry count either way, so the
-// caller can grow the buffer and run the chunk again.  A look-back that
-// polls a predecessor's word more than spin_limit times gives up, counts a
-// time-out (kLookbackTimeout) and uses 0.
+// entries, publishes the count, then adds up its predecessors' published words
+// (decoupled look-back: a word is either a block's own count or the inclusive
+// prefix up to it; the walk stops at the first prefix), publishes its own
+// prefix and emits from its offset.  No block waits on a later one.  Entries
+// at or past `capacity` are not written; *total receives the entry count
+// either way, so the caller can grow the buffer and run the chunk again.  A
+// look-back that polls a predecessor's word more than spin_limit times gives
+// up, counts a time-out (kLookbackTimeout) and uses 0.
+//
+// A warp spreads its 32 positions' tile rows over its lanes, one (slot, row)
+// job per lane per round, so large footprints do not hold up small ones; the
+// entries of a round are then spread over the lanes again, so that 32
+// consecutive list places are written at a time.
 constexpr unsigned long long kLbCount = 1ull << 32;   // word holds the block's own count
 constexpr unsigned long long kLbPrefix = 2ull << 32;  // word holds the inclusive prefix
+constexpr int kBinThreads = 128, kBinWarps = kBinThreads / 32;
 
 template <bool kDeviceRange>
-__global__ void __launch_bounds__(128, 12) bin_fused_kernel(
-    int64_t p0, int64_t n_pos, SlotView sv, const ViewParams* __restrict__ views,
+__global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
+    int64_t p0, int64_t n_pos, SlotView sv, const ViewParams* __restrict__ views, int n_views,
     const uint32_t* __restrict__ sorted_val,
     const Footprint* __restrict__ foot, const uint64_t* __restrict__ sat,
     uint32_t* __restrict__ out_key, uint32_t* __restrict__ out_val, uint32_t capacity,
     unsigned long long* __restrict__ status, uint32_t* __restrict__ ticket,
     uint32_t* __restrict__ total, unsigned long long* __restrict__ counters, int spin_limit,
     const int64_t* __restrict__ range_dev) {
-
-  __shared__ uint32_t s_vb, s_boff;
+  __shared__ uint32_t s_vb, s_boff, s_wtot[kBinWarps];
+  __shared__ BinView s_view[kMaxViewsPerBatch];
   if constexpr (kDeviceRange) {  // the chunk's positions [range_dev[0], range_dev[1])
     p0 = range_dev[0];
     n_pos = range_dev[1] - range_dev[0];
   }
-  __shared__ uint32_t s_wtot[4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_vb = atomicAdd(ticket, 1u);
+  const uint32_t* const cols = views[0].cols;
+  const uint32_t* const free_tab = views[0].free_tab;
+  for (int v = threadIdx.x; v < n_views; v += kBinThreads) {
+    const ViewParams& vp = views[v];
+    s_view[v] = {vp.tile_base, vp.tiles_x, vp.width,
+                 free_tab ? static_cast<int>(vp.free_tab - free_tab) : 0};
+  }
   __syncthreads();
   const uint32_t vb = s_vb;
-  const int64_t j = static_cast<int64_t>(vb) * blockDim.x + threadIdx.x;
-  uint32_t g, nrows;
-  int ty0;
-  lane_rows(j, n_pos, p0, sv, views, sorted_val, foot, sat, &g, &ty0, &nrows);
+  const int64_t j = static_cast<int64_t>(vb) * kBinThreads + threadIdx.x;
+  uint32_t g = 0u, nrows = 0u;
+  int ty0 = 0;
+  if (j < n_pos) {
+    g = sorted_val[p0 + j];
+    nrows = live_rows(foot[g], g, s_view[sv(g)], cols, free_tab, sat, &ty0);
+  }
   const uint32_t incl = warp_incl_scan(nrows, lane);
-  const int R = static_cast<int>(__shfl_sync(0xffffffffu, incl, 31));
+  const int R = static_cast<int>(__shfl_sync(0xffffffffu, incl, 31));  // same for the whole warp
+  // one round's job: the lane's tile range and its free tiles
+  auto job = [&](int r, int* a, int* b, uint32_t* slot) -> uint32_t {
+    const RowJob jb = row_job(r, R, incl, ty0);
+    *slot = __shfl_sync(0xffffffffu, g, jb.owner);
+    *a = 0;
+    *b = -1;
+    if (!jb.ok) return 0u;
+    return row_free(foot[*slot], *slot, jb.row, s_view[sv(*slot)], cols, sat, a, b);
+  };
   // count; the first kStash rounds' jobs are kept in registers for the emission
   constexpr int kStash = 3;
   int st_a[kStash], st_b[kStash];
@@ -777,24 +702,15 @@ __global__ void __launch_bounds__(128, 12) bin_fused_kernel(
     st_b[k] = -1;
     st_fr[k] = 0;
     st_g[k] = 0;
-    if (32 * k < R) {  // R is the same for the whole warp
-      const RowJob jb = row_job(32 * k + lane, R, incl, g, ty0);
-      const uint32_t fr = job_free(jb, sv, views, foot, sat, &st_a[k], &st_b[k]);
-      st_fr[k] = fr;
-      st_g[k] = jb.g;
-      uint32_t sum = fr;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      wtot += sum;
+    if (32 * k < R) {
+      st_fr[k] = job(32 * k + lane, &st_a[k], &st_b[k], &st_g[k]);
+      wtot += __reduce_add_sync(0xffffffffu, st_fr[k]);
     }
   }
   for (int r0 = 32 * kStash; r0 < R; r0 += 32) {
-    const RowJob jb = row_job(r0 + lane, R, incl, g, ty0);
     int a, b;
-    uint32_t fr = job_free(jb, sv, views, foot, sat, &a, &b);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) fr += __shfl_xor_sync(0xffffffffu, fr, o);
-    wtot += fr;
+    uint32_t slot;
+    wtot += __reduce_add_sync(0xffffffffu, job(r0 + lane, &a, &b, &slot));
   }
   if (lane == 0) s_wtot[warp] = wtot;
   __syncthreads();
@@ -802,7 +718,7 @@ __global__ void __launch_bounds__(128, 12) bin_fused_kernel(
   // time (lane l reads predecessor vb - 1 - l)
   if (warp == 0) {
     uint32_t btot = 0;
-    for (int w = 0; w < 4; ++w) btot += s_wtot[w];
+    for (int w = 0; w < kBinWarps; ++w) btot += s_wtot[w];
     if (lane == 0) atomicExch(&status[vb], (vb == 0 ? kLbPrefix : kLbCount) | btot);
     volatile unsigned long long* vs = status;
     uint32_t excl = 0;
@@ -824,10 +740,8 @@ __global__ void __launch_bounds__(128, 12) bin_fused_kernel(
       }
       const uint32_t pre = __ballot_sync(0xffffffffu, (word & ~0xFFFFFFFFull) == kLbPrefix);
       const int first = pre ? __ffs(pre) - 1 : 31;  // nearest predecessor holding a prefix
-      uint32_t v = lane <= first ? static_cast<uint32_t>(word & 0xFFFFFFFFull) : 0u;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      excl += v;
+      excl += __reduce_add_sync(
+          0xffffffffu, lane <= first ? static_cast<uint32_t>(word & 0xFFFFFFFFull) : 0u);
       if (pre) break;
     }
     if (lane == 0) {
@@ -837,34 +751,48 @@ __global__ void __launch_bounds__(128, 12) bin_fused_kernel(
     }
   }
   __syncthreads();
-  uint32_t wbeg = s_boff;
-  for (int w = 0; w < warp; ++w) wbeg += s_wtot[w];
-  const uint32_t wend = wbeg + wtot;
-  // emit, in the same (Gaussian, row) order as the count
-  uint32_t carry = 0;
-#pragma unroll
-  for (int k = 0; k < kStash; ++k) {
-    if (32 * k < R) {
-      const uint32_t fr = st_fr[k];
-      const uint32_t sc = warp_incl_scan(fr, lane);
-      const uint32_t o = wbeg + carry + sc - fr;
-      if (fr && o < capacity)
-        emit_free(sat, st_a[k], st_b[k], st_g[k], out_key, out_val, o,
-                  min(min(o + fr, wend), capacity));
-      carry += __shfl_sync(0xffffffffu, sc, 31);
-    }
-  }
-  for (int r0 = 32 * kStash; r0 < R; r0 += 32) {
-    const RowJob jb = row_job(r0 + lane, R, incl, g, ty0);
-    int a, b;
-    const uint32_t fr = job_free(jb, sv, views, foot, sat, &a, &b);
+  uint32_t o0 = s_boff;
+  for (int w = 0; w < warp; ++w) o0 += s_wtot[w];
+  const uint32_t wend = o0 + wtot;
+  // one round's entries, from list place o0 on
+  auto emit = [&](uint32_t fr, int a, int b, uint32_t slot) {
     const uint32_t sc = warp_incl_scan(fr, lane);
-    const uint32_t o = wbeg + carry + sc - fr;
-    if (fr && o < capacity)
-      emit_free(sat, a, b, jb.g, out_key, out_val, o, min(min(o + fr, wend), capacity));
-    carry += __shfl_sync(0xffffffffu, sc, 31);
+    const uint32_t T = __shfl_sync(0xffffffffu, sc, 31);
+    const int n_tiles = b - a + 1;
+    for (uint32_t e0 = 0; e0 < T; e0 += 32) {
+      const uint32_t e = min(e0 + lane, T - 1);
+      // owner of entry e: the number of lanes whose inclusive count is <= e
+      int lo = 0;
+#pragma unroll
+      for (int s = 16; s >= 1; s >>= 1) {
+        const uint32_t v = __shfl_sync(0xffffffffu, sc, lo + s - 1);
+        if (v <= e) lo += s;
+      }
+      const int ow = min(lo, 31);
+      const uint32_t fr_o = __shfl_sync(0xffffffffu, fr, ow);
+      const uint32_t k = e - (__shfl_sync(0xffffffffu, sc, ow) - fr_o);
+      const int a_o = __shfl_sync(0xffffffffu, a, ow), n_o = __shfl_sync(0xffffffffu, n_tiles, ow);
+      const uint32_t slot_o = __shfl_sync(0xffffffffu, slot, ow);
+      if (e0 + lane < T && o0 + e < capacity) {
+        out_key[o0 + e] = fr_o == static_cast<uint32_t>(n_o)
+                              ? static_cast<uint32_t>(a_o) + k  // no saturated tile among them
+                              : nth_free(sat, a_o, static_cast<int>(k));
+        out_val[o0 + e] = slot_o;
+      }
+    }
+    o0 += T;
+  };
+  // emit, in the same (slot, row) order as the count
+#pragma unroll
+  for (int k = 0; k < kStash; ++k)
+    if (32 * k < R) emit(st_fr[k], st_a[k], st_b[k], st_g[k]);
+  for (int r0 = 32 * kStash; r0 < R; r0 += 32) {
+    int a, b;
+    uint32_t slot;
+    const uint32_t fr = job(r0 + lane, &a, &b, &slot);
+    emit(fr, a, b, slot);
   }
-  if (lane == 0 && wbeg + carry != wend) atomicAdd(&counters[kBinningMismatch], 1ull);
+  if (lane == 0 && o0 != wend) atomicAdd(&counters[kBinningMismatch], 1ull);
 }
 
 // Per view of the batch (one block each), the 2-D prefix sums of its
@@ -974,55 +902,26 @@ cudaError_t launch_depth_tie_fix(int64_t n_total, int64_t n, const uint32_t* key
   return cudaGetLastError();
 }
 
-cudaError_t launch_chunk_count(int64_t p0, int64_t n_pos, int64_t n, const ViewParams* views,
-                               const uint32_t* sorted_val,
-                               const Footprint* foot, const uint64_t* sat, uint32_t* out_cnt,
-                               cudaStream_t stream) {
-  if (n_pos == 0) return cudaSuccess;
-  const int threads = 256;
-  const int64_t blocks = (n_pos + threads - 1) / threads;
-  chunk_count_kernel<<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-      p0, n_pos, SlotView(n > 0 ? n : 1), views, sorted_val, foot, sat, out_cnt);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_emit(int64_t p0, int64_t n_pos, int64_t n, const ViewParams* views,
-                        const uint32_t* sorted_val, const uint32_t* offsets,
-                        const uint32_t* chunk_cnt, const Footprint* foot,
-                        const uint64_t* sat, uint32_t* out_key, uint32_t* out_val,
-                        unsigned long long* counters, cudaStream_t stream) {
-  if (n_pos == 0) return cudaSuccess;
-  const int threads = 256;
-  const int64_t blocks = (n_pos + threads - 1) / threads;
-  emit_kernel<<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-      p0, n_pos, SlotView(n > 0 ? n : 1), views, sorted_val, offsets, chunk_cnt, foot, sat, out_key, out_val,
-      counters);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_bin_fused(int64_t p0, int64_t n_pos, int64_t n, const ViewParams* views,
-                             const uint32_t* sorted_val,
+                             int n_views, const uint32_t* sorted_val,
                              const Footprint* foot, const uint64_t* sat, uint32_t* out_key,
                              uint32_t* out_val, uint32_t capacity, void* lookback,
                              uint32_t* total, unsigned long long* counters, cudaStream_t stream,
                              const int64_t* range_dev) {
   if (n_pos <= 0) return cudaMemsetAsync(total, 0, sizeof(uint32_t), stream);
-  const int threads = 128;
-  const int64_t blocks = (n_pos + threads - 1) / threads;
+  const int64_t blocks = (n_pos + kBinThreads - 1) / kBinThreads;
   uint32_t* ticket = static_cast<uint32_t*>(lookback);
   unsigned long long* status = reinterpret_cast<unsigned long long*>(
       static_cast<char*>(lookback) + 256);
   cudaError_t e = cudaMemsetAsync(lookback, 0, 256 + static_cast<size_t>(blocks) * 8, stream);
   if (e != cudaSuccess) return e;
-  if (range_dev)
-    bin_fused_kernel<true><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-        p0, n_pos, SlotView(n > 0 ? n : 1), views, sorted_val, foot, sat, out_key, out_val, capacity, status, ticket,
-        total, counters, kLookbackSpinLimit, range_dev);
-  else
-    bin_fused_kernel<false><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-        p0, n_pos, SlotView(n > 0 ? n : 1), views, sorted_val, foot, sat, out_key, out_val, capacity, status, ticket,
-        total, counters, kLookbackSpinLimit, nullptr);
-  return cudaGetLastError();
+  auto launch = [&](auto kernel) {
+    kernel<<<static_cast<unsigned>(blocks), kBinThreads, 0, stream>>>(
+        p0, n_pos, SlotView(n > 0 ? n : 1), views, n_views, sorted_val, foot, sat, out_key,
+        out_val, capacity, status, ticket, total, counters, kLookbackSpinLimit, range_dev);
+    return cudaGetLastError();
+  };
+  return range_dev ? launch(bin_fused_kernel<true>) : launch(bin_fused_kernel<false>);
 }
 
 cudaError_t launch_lookback_probe(void* lookback, uint32_t* total, unsigned long long* counters,
@@ -1039,14 +938,14 @@ cudaError_t launch_lookback_probe(void* lookback, uint32_t* total, unsigned long
   const uint32_t one = 1u;
   e = cudaMemcpyAsync(ticket, &one, sizeof(one), cudaMemcpyHostToDevice, stream);
   if (e != cudaSuccess) return e;
-  bin_fused_kernel<false><<<1, 128, 0, stream>>>(0, 1, SlotView(1), views, sorted_val, foot, sat, out_key,
-                                                 out_val, 0u, status, ticket, total, counters,
-                                                 spin_limit, nullptr);
+  bin_fused_kernel<false><<<1, kBinThreads, 0, stream>>>(
+      0, 1, SlotView(1), views, 1, sorted_val, foot, sat, out_key, out_val, 0u, status, ticket,
+      total, counters, spin_limit, nullptr);
   return cudaGetLastError();
 }
 
 size_t bin_fused_temp_bytes(int64_t n_pos) {
-  return 256 + static_cast<size_t>((n_pos + 127) / 128) * 8;
+  return 256 + static_cast<size_t>((n_pos + kBinThreads - 1) / kBinThreads) * 8;
 }
 
 cudaError_t launch_free_tables(const ViewParams* views, int n_views, const uint64_t* sat,

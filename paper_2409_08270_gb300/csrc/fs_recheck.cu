@@ -109,7 +109,7 @@ __global__ void mark_tiles_kernel(int64_t n_flagged, int n_views, int64_t n,
   footprint_rows(f, &ty0, &ty1);
   for (int ty = ty0; ty <= ty1; ++ty) {
     int tx0, tx1;
-    if (!row_span(f, ty, vp.width, &tx0, &tx1) || !clip_cols(vp, slot, &tx0, &tx1)) continue;
+    if (!row_span(f, ty, vp.width, &tx0, &tx1) || !clip_cols(vp.cols, slot, &tx0, &tx1)) continue;
     const int a = vp.tile_base + ty * vp.tiles_x + tx0;
     const int b = vp.tile_base + ty * vp.tiles_x + tx1;
     for (int w = a >> 6; w <= (b >> 6); ++w) {
@@ -141,7 +141,7 @@ __global__ void candidates_kernel(int64_t k_total, int64_t n, const ViewParams* 
     footprint_rows(f, &ty0, &ty1);
     for (int ty = ty0; ty <= ty1 && !hit; ++ty) {
       int tx0, tx1;
-      if (!row_span(f, ty, vp.width, &tx0, &tx1) || !clip_cols(vp, slot, &tx0, &tx1)) continue;
+      if (!row_span(f, ty, vp.width, &tx0, &tx1) || !clip_cols(vp.cols, slot, &tx0, &tx1)) continue;
       const int base = vp.tile_base + ty * vp.tiles_x;
       if (count_free(skip, base + tx0, base + tx1)) hit = 1;
     }
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(32 * kRWarps, 8) recheck_blend_kernel(
           int r0, r1, c0, c1;
           footprint_rows(f, &r0, &r1);
           on = ty >= r0 && ty <= r1 && row_span(f, ty, vp.width, &c0, &c1) &&
-               clip_cols(vp, slot, &c0, &c1) && tx >= c0 && tx <= c1;
+               clip_cols(vp.cols, slot, &c0, &c1) && tx >= c0 && tx <= c1;
         }
         const int m = append(on && meets(slot), slot, 0);
         stage(0, m);
