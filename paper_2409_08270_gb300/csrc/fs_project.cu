@@ -446,10 +446,7 @@ __device__ __forceinline__ void fix_tie_run(int64_t k, int64_t n_total, const Sl
                                             uint32_t kk, const uint32_t* __restrict__ key,
                                             uint32_t* __restrict__ val,
                                             const uint32_t* __restrict__ depth_lo) {
-  const uint32_t v0 = val[k];
-  const uint32_t view = view_of(v0);
-  if (view_of(val[k + 1]) != view) return;                       // no same-view tie here
-  if (k > 0 && key[k - 1] == kk && view_of(val[k - 1]) == view) return;  // not the run's start
+  const uint32_t view = view_of(val[k]);
   int64_t e = k + 2;
   while (e < n_total && key[e] == kk && view_of(val[e]) == view) ++e;
   for (int64_t a = k + 1; a < e; ++a) {
@@ -467,11 +464,15 @@ __device__ __forceinline__ void fix_tie_run(int64_t k, int64_t n_total, const Sl
   }
 }
 
-// Each thread screens four consecutive positions for the start of a run of
-// equal keys within one view.  Equal keys of different views are common (a
-// batch holds many views of the same depths), so the screen compares the
-// views of neighbours from one 16-byte key load and one 16-byte value load
-// (when both arrays are 16-byte aligned) before a run is walked.
+// Each thread takes four consecutive positions, k0 .. k0 + 3.  Equal keys of
+// different views are common (a batch holds many views of the same depths), so
+// it compares keys and views of its positions' neighbours, k0 - 1 .. k0 + 5,
+// from one 16-byte load each (when both arrays are 16-byte aligned) and the
+// words around them.  Nearly every same-view run is a pair: the pairs' low
+// words are gathered together, where walking each run as it is met costs a
+// chain of gathers per run.  Longer runs are walked.  Bound by the gathers:
+// every sixth slot of a 10^6-Gaussian view shares its key (4.8 10^7 slots of
+// 48 views: 328 us, 375 us with every run walked).
 __global__ void depth_tie_fix_kernel(int64_t n_total, int64_t n, const uint32_t* __restrict__ key,
                                      uint32_t* __restrict__ val,
                                      const uint32_t* __restrict__ depth_lo,
@@ -479,44 +480,57 @@ __global__ void depth_tie_fix_kernel(int64_t n_total, int64_t n, const uint32_t*
   if (n_dev) n_total = min(n_total, static_cast<int64_t>(*n_dev));
   const int64_t k0 = 4 * (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
   if (k0 + 1 >= n_total) return;
-  uint32_t t[5];  // keys k0 .. k0 + 4 (0xFFFFFFFF past the end: never a run)
-  uint32_t w[5];  // their values (slots), where a key is present
+  // t[1 + i], w[1 + i]: key and slot of position k0 + i (key 0xFFFFFFFF where
+  // there is none: never a run)
+  uint32_t t[7], w[7];
   const bool full = k0 + 4 <= n_total &&
                     ((reinterpret_cast<uintptr_t>(key) | reinterpret_cast<uintptr_t>(val)) & 15u) == 0;
-  if (full) {
-    const uint4 q = *reinterpret_cast<const uint4*>(key + k0);
-    t[0] = q.x;
-    t[1] = q.y;
-    t[2] = q.z;
-    t[3] = q.w;
-  } else {
+  auto load = [&](const uint32_t* src, uint32_t none, uint32_t* dst) {
+    if (full) {
+      const uint4 q = *reinterpret_cast<const uint4*>(src + k0);
+      dst[1] = q.x;
+      dst[2] = q.y;
+      dst[3] = q.z;
+      dst[4] = q.w;
+    } else {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) t[i] = k0 + i < n_total ? key[k0 + i] : 0xFFFFFFFFu;
-  }
-  t[4] = k0 + 4 < n_total ? key[k0 + 4] : 0xFFFFFFFFu;
+      for (int i = 0; i < 4; ++i) dst[1 + i] = k0 + i < n_total ? src[k0 + i] : none;
+    }
+    dst[0] = k0 > 0 ? src[k0 - 1] : none;
+    dst[5] = k0 + 4 < n_total ? src[k0 + 4] : none;
+    dst[6] = k0 + 5 < n_total ? src[k0 + 5] : none;
+  };
+  load(key, 0xFFFFFFFFu, t);
   bool any = false;  // an equal neighbour somewhere among the four
 #pragma unroll
-  for (int i = 0; i < 4; ++i) any = any || (t[i] != 0xFFFFFFFFu && t[i + 1] == t[i]);
+  for (int i = 1; i <= 4; ++i) any = any || (t[i] != 0xFFFFFFFFu && t[i + 1] == t[i]);
   if (!any) return;
-  if (full) {
-    const uint4 q = *reinterpret_cast<const uint4*>(val + k0);
-    w[0] = q.x;
-    w[1] = q.y;
-    w[2] = q.z;
-    w[3] = q.w;
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = k0 + i < n_total ? val[k0 + i] : 0u;
-  }
-  w[4] = k0 + 4 < n_total ? val[k0 + 4] : 0u;
+  load(val, 0u, w);
   const SlotView view_of(n);
-  uint32_t vw[5];
+  bool tie[6];  // positions k0 + i - 1 and k0 + i: equal keys, one view
 #pragma unroll
-  for (int i = 0; i < 5; ++i) vw[i] = view_of(w[i]);
+  for (int i = 0; i < 6; ++i)
+    tie[i] = t[i] != 0xFFFFFFFFu && t[i + 1] == t[i] && view_of(w[i]) == view_of(w[i + 1]);
+  uint32_t lo[4][2];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    if (t[i] != 0xFFFFFFFFu && t[i + 1] == t[i] && vw[i + 1] == vw[i] && k0 + i + 1 < n_total)
-      fix_tie_run(k0 + i, n_total, view_of, t[i], key, val, depth_lo);
+    if (tie[1 + i] && !tie[i] && !tie[2 + i]) {
+      lo[i][0] = depth_lo[w[1 + i]];
+      lo[i][1] = depth_lo[w[2 + i]];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (!tie[1 + i] || tie[i]) continue;  // no run starts here
+    if (!tie[2 + i]) {
+      // slots of a pair ascend already: equal low words stay
+      if (lo[i][0] > lo[i][1]) {
+        val[k0 + i] = w[2 + i];
+        val[k0 + i + 1] = w[1 + i];
+      }
+    } else {
+      fix_tie_run(k0 + i, n_total, view_of, t[1 + i], key, val, depth_lo);
+    }
   }
 }
 
@@ -797,24 +811,33 @@ __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
 
 // Per view of the batch (one block each), the 2-D prefix sums of its
 // unsaturated tiles: free_tab[r * (tiles_x + 1) + c] = unsaturated tiles in
-// rows < r and columns < c (row 0 and column 0 are zero).  Running sums
-// along each row, then down each column.
+// rows < r and columns < c (row 0 and column 0 are zero).  A warp runs along a
+// row 32 tiles at a time, a thread then down a column.  Views of up to
+// kTableCells cells keep the table in shared memory until it is whole (a
+// 1008x756 view: 17 us through global memory, 8 us so).
+constexpr int kTableCells = 10240;
 __global__ void __launch_bounds__(256) free_table_kernel(const ViewParams* __restrict__ views,
                                                          const uint64_t* __restrict__ sat) {
+  __shared__ uint32_t s_tab[kTableCells];
   const ViewParams& vp = views[blockIdx.x];
-  uint32_t* tab = vp.free_tab;
-  if (!tab) return;
-  const int tx = vp.tiles_x, ty = vp.tiles_y, w1 = tx + 1;
+  uint32_t* const out = vp.free_tab;
+  if (!out) return;
+  const int tx = vp.tiles_x, ty = vp.tiles_y, w1 = tx + 1, base = vp.tile_base;
+  const int64_t cells = static_cast<int64_t>(w1) * (ty + 1);
+  const bool shared = cells <= kTableCells;
+  uint32_t* const tab = shared ? s_tab : out;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int c = threadIdx.x; c < w1; c += blockDim.x) tab[c] = 0u;
-  for (int r = threadIdx.x; r < ty; r += blockDim.x) {
-    const int g0 = vp.tile_base + r * tx;
+  for (int r = warp; r < ty; r += 8) {
     uint32_t* row = tab + static_cast<int64_t>(r + 1) * w1;
+    if (lane == 0) row[0] = 0u;
     uint32_t run = 0;
-    row[0] = 0u;
-    for (int c = 0; c < tx; ++c) {
-      const int g = g0 + c;
-      run += static_cast<uint32_t>(((sat[g >> 6] >> (g & 63)) & 1ull) == 0ull);
-      row[c + 1] = run;
+    for (int c0 = 0; c0 < tx; c0 += 32) {
+      const int g = base + r * tx + c0 + lane;
+      const bool free = c0 + lane < tx && ((sat[g >> 6] >> (g & 63)) & 1ull) == 0ull;
+      const uint32_t bits = __ballot_sync(0xffffffffu, free);
+      if (c0 + lane < tx) row[c0 + lane + 1] = run + __popc(bits & (0xffffffffu >> (31 - lane)));
+      run += __popc(bits);
     }
   }
   __syncthreads();
@@ -826,6 +849,9 @@ __global__ void __launch_bounds__(256) free_table_kernel(const ViewParams* __res
       *e = acc;
     }
   }
+  if (!shared) return;
+  __syncthreads();
+  for (int k = threadIdx.x; k < static_cast<int>(cells); k += blockDim.x) out[k] = s_tab[k];
 }
 
 // [start, end) of every tile's run in the tile-sorted list.  Each thread

@@ -171,19 +171,33 @@ struct PassShape {
   int shift[kMaxPasses], bits[kMaxPasses];
 };
 
-// Digit counts of every pass from one read of the keys (shared-memory counts
-// per block, added up in global memory); the last block to finish turns them
-// into the digits' starts.  Bound by HBM: 4 B a key.
+// Digit counts of every pass from one read of the keys: per block in shared
+// memory, added up in global memory; the last block to finish turns them into
+// the digits' starts.  Bound by the shared-memory atomics, so a block keeps
+// kHistCopies counters per digit side by side, one per lane group: lanes that
+// meet in a bank are then mostly those of one group (4.8 10^7 keys of three
+// digits: 118 us with one counter per digit, 78 us so).
+constexpr int kHistCopies = 8;
+size_t hist_smem(const PassShape& shape) {
+  size_t words = 0;
+  for (int p = 0; p < shape.passes; ++p) words += static_cast<size_t>(kHistCopies) << shape.bits[p];
+  return words * sizeof(uint32_t);
+}
+
 __global__ void __launch_bounds__(kHistThreads) radix_hist_kernel(
     const uint32_t* __restrict__ keys, int64_t n, PassShape shape, uint32_t kmin, uint32_t span,
     SortHead* __restrict__ head, const uint32_t* __restrict__ n_dev,
     const uint32_t* __restrict__ range_dev) {
-  __shared__ uint32_t s_h[kMaxPasses][kMaxRadix];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* const s_h = reinterpret_cast<uint32_t*>(smem_raw);  // [pass][digit][copy]
   __shared__ uint32_t s_warp[kHistThreads / 32];
   __shared__ bool s_last;
   device_sizes(n_dev, range_dev, &n, &kmin, &span);
-  for (int k = threadIdx.x; k < kMaxPasses * kMaxRadix; k += kHistThreads) (&s_h[0][0])[k] = 0u;
+  int words = 0;
+  for (int p = 0; p < shape.passes; ++p) words += kHistCopies << shape.bits[p];
+  for (int k = threadIdx.x; k < words; k += kHistThreads) s_h[k] = 0u;
   __syncthreads();
+  uint32_t* const mine = s_h + threadIdx.x % kHistCopies;
   const int64_t step = static_cast<int64_t>(gridDim.x) * kHistThreads;
   constexpr int kAhead = 8;  // loads in flight per thread
   for (int64_t j0 = static_cast<int64_t>(blockIdx.x) * kHistThreads + threadIdx.x; j0 < n;
@@ -194,14 +208,24 @@ __global__ void __launch_bounds__(kHistThreads) radix_hist_kernel(
 #pragma unroll
     for (int i = 0; i < kAhead; ++i) {
       if (j0 + i * step >= n) break;
-      for (int p = 0; p < shape.passes; ++p)
-        atomicAdd(&s_h[p][digit_of(key[i], kmin, span, shape.shift[p], shape.bits[p])], 1u);
+      uint32_t* h = mine;
+#pragma unroll
+      for (int p = 0; p < kMaxPasses; ++p) {
+        if (p >= shape.passes) break;
+        atomicAdd(&h[kHistCopies * digit_of(key[i], kmin, span, shape.shift[p], shape.bits[p])], 1u);
+        h += kHistCopies << shape.bits[p];
+      }
     }
   }
   __syncthreads();
-  for (int p = 0; p < shape.passes; ++p)
-    for (int d = threadIdx.x; d < (1 << shape.bits[p]); d += kHistThreads)
-      if (s_h[p][d]) atomicAdd(&head->hist[p][d], s_h[p][d]);
+  for (int p = 0, at = 0; p < shape.passes; at += kHistCopies << shape.bits[p], ++p)
+    for (int d = threadIdx.x; d < (1 << shape.bits[p]); d += kHistThreads) {
+      uint32_t sum = 0;
+#pragma unroll
+      for (int c = 0; c < kHistCopies; ++c)  // rotated: threads start at different banks
+        sum += s_h[at + d * kHistCopies + (c + d) % kHistCopies];
+      if (sum) atomicAdd(&head->hist[p][d], sum);
+    }
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_last = atomicAdd(&head->hist_blocks, 1u) == gridDim.x - 1;
@@ -556,8 +580,12 @@ cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
   cudaError_t e = cudaMemsetAsync(
       temp, 0, sizeof(SortHead) + static_cast<size_t>(nt << shape.bits[0]) * word, stream);
   if (e != cudaSuccess) return e;
-  const int64_t hist_blocks = std::min<int64_t>((n + 4 * kHistThreads - 1) / (4 * kHistThreads), 608);
-  radix_hist_kernel<<<static_cast<unsigned>(hist_blocks), kHistThreads, 0, stream>>>(
+  const int64_t hist_blocks = std::min<int64_t>((n + 8 * kHistThreads - 1) / (8 * kHistThreads), 304);
+  const size_t hist_bytes = hist_smem(shape);
+  e = cudaFuncSetAttribute(radix_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(kMaxPasses * kMaxRadix * kHistCopies * 4));
+  if (e != cudaSuccess) return e;
+  radix_hist_kernel<<<static_cast<unsigned>(hist_blocks), kHistThreads, hist_bytes, stream>>>(
       keys, n, shape, kmin, span, head, n_dev, range_dev);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   uint32_t *src_k = keys, *src_v = vals, *dst_k = keys_alt, *dst_v = vals_alt;
