@@ -186,7 +186,8 @@ struct fs_ctx {
   size_t events_used = 0;
   bool stage_outer = false;         // a stage holding others (the re-check) is open
   // workspace
-  DevBuf views, rec, foot, cnt, key_a, val_a, key_b, val_b, offs, ccnt, dlo, state, sat, subsat;
+  DevBuf views, rec, foot, box, key_a, val_a, key_b, val_b, offs, ccnt, dlo, state, sat, subsat;
+  DevBuf live, live_val, live_range;  // slot bits, a chunk's live slots and their number
   DevBuf free_tab;  // the batch's per-view prefix tables of unsaturated tiles
   DevBuf lk_a, lv_a, lk_b, lv_b, ranges, sort_tmp, scan_tmp, total, counters;
   DevBuf mask_stage, table_tmp, table32_tmp, bits_tmp, label_tmp, margin_tmp;
@@ -196,7 +197,7 @@ struct fs_ctx {
   bool compact = false;  // reduced-precision records (FP16 whitening matrix, FP32 mean)
   bool census = false;   // blend counts its pairs (slower variant)
   bool sigma3 = false;   // 3-sigma tile coverage (per-slot tile columns in `cols`)
-  DevBuf dkey, rk_flag, rk_offs, rk_F, rk_map, rk_R, rk_Rb, rk_tiles, cols;
+  DevBuf rk_flag, rk_offs, rk_F, rk_map, rk_R, rk_Rb, rk_tiles, cols;
   DevBuf rd_flag, rd_offs, rd_val, render_out;  // novel-view mask rendering
   DevBuf chunk_bnd;                             // captured solves: chunk boundaries
   HostBuf render_out_host;
@@ -230,15 +231,16 @@ namespace {
 DevBuf* const* workspace_bufs(fs_ctx* c, size_t* count) {
   static thread_local DevBuf* bufs[64];
   size_t k = 0;
-  DevBuf* list[] = {&c->rec, &c->foot, &c->cnt, &c->key_a, &c->val_a, &c->key_b, &c->val_b,
+  DevBuf* list[] = {&c->rec, &c->foot, &c->box, &c->key_a, &c->val_a, &c->key_b, &c->val_b,
                     &c->offs, &c->ccnt, &c->dlo, &c->state, &c->sat, &c->subsat, &c->lk_a,
                     &c->lv_a, &c->lk_b, &c->lv_b, &c->ranges, &c->sort_tmp, &c->scan_tmp,
                     &c->mask_stage, &c->table_tmp, &c->table32_tmp, &c->bits_tmp,
-                    &c->label_tmp, &c->margin_tmp, &c->dkey, &c->rk_flag, &c->rk_offs,
+                    &c->label_tmp, &c->margin_tmp, &c->rk_flag, &c->rk_offs,
                     &c->rk_F, &c->rk_map, &c->rk_R, &c->rk_Rb, &c->rk_tiles, &c->kl_ranges, &c->kl_satc,
                     &c->kl_bound, &c->key_range, &c->lb_tmp, &c->key_a2, &c->val_a2,
                     &c->key_b2, &c->val_b2, &c->cols, &c->rd_flag, &c->rd_offs, &c->rd_val,
-                    &c->render_out, &c->chunk_bnd, &c->free_tab};
+                    &c->render_out, &c->chunk_bnd, &c->free_tab, &c->live, &c->live_val,
+                    &c->live_range};
   for (DevBuf* b : list) bufs[k++] = b;
   *count = k;
   return bufs;
@@ -337,16 +339,16 @@ fs_status fs_destroy(fs_ctx* c) {
     return fail(FS_INVALID_ARGUMENT, "fs_destroy: %d scene(s) still alive", c->scenes);
   DeviceGuard g(c->device);
   cudaDeviceSynchronize();
-  DevBuf* bufs[] = {&c->subsat, &c->ccnt, &c->dlo, &c->state, &c->sat, &c->views, &c->rec, &c->foot, &c->cnt, &c->key_a, &c->val_a, &c->key_b,
+  DevBuf* bufs[] = {&c->subsat, &c->ccnt, &c->dlo, &c->state, &c->sat, &c->views, &c->rec, &c->foot, &c->box, &c->key_a, &c->val_a, &c->key_b,
                     &c->val_b, &c->offs, &c->lk_a, &c->lv_a, &c->lk_b, &c->lv_b, &c->ranges,
                     &c->sort_tmp, &c->scan_tmp, &c->total, &c->counters, &c->mask_stage,
                     &c->table_tmp, &c->table32_tmp, &c->bits_tmp, &c->label_tmp, &c->margin_tmp,
-                    &c->dkey, &c->rk_flag, &c->rk_offs, &c->rk_F, &c->rk_map, &c->rk_R,
+                    &c->rk_flag, &c->rk_offs, &c->rk_F, &c->rk_map, &c->rk_R,
                     &c->rk_Rb, &c->rk_tiles, &c->kl_ranges, &c->kl_satc, &c->kl_bound, &c->key_range,
                     &c->lb_tmp,
                     &c->key_a2, &c->val_a2, &c->key_b2, &c->val_b2, &c->cols,
                     &c->rd_flag, &c->rd_offs, &c->rd_val, &c->render_out, &c->chunk_bnd,
-                    &c->free_tab};
+                    &c->free_tab, &c->live, &c->live_val, &c->live_range};
   for (DevBuf& b : c->kl_val) b.release();
   for (DevBuf* b : bufs) b->release();
   c->views_host.release();
@@ -589,9 +591,8 @@ struct ProjPtrs {
   fs::ProjRecord* rec;       // float-pair records, or NULL
   fs::CompactRecord* rec16;  // reduced-precision records, or NULL
   fs::Footprint* foot;
-  uint32_t* cnt;
+  fs::TileBox* box;
   uint32_t* dlo;
-  uint32_t* dkey;  // resident depth keys (keep only)
   uint32_t* cols;  // 3-sigma tile columns, or NULL (exact coverage)
 };
 
@@ -600,8 +601,7 @@ ProjPtrs proj_ptrs(const fs_ctx* c, bool keep, int32_t v0, int64_t n) {
   return {c->compact ? nullptr : c->rec.as<fs::ProjRecord>() + off,
           c->compact ? c->rec.as<fs::CompactRecord>() + off : nullptr,
           c->foot.as<fs::Footprint>() + off,
-          c->cnt.as<uint32_t>() + off, c->dlo.as<uint32_t>() + off,
-          keep ? c->dkey.as<uint32_t>() + off : nullptr,
+          c->box.as<fs::TileBox>() + off, c->dlo.as<uint32_t>() + off,
           c->sigma3 ? c->cols.as<uint32_t>() + off : nullptr};
 }
 
@@ -611,9 +611,8 @@ fs_status ensure_window(fs_ctx* c, int64_t n, int vb, int32_t V, bool keep) {
   const size_t rec_bytes = c->compact ? sizeof(fs::CompactRecord) : sizeof(fs::ProjRecord);
   FS_TRY(c->rec.ensure(static_cast<size_t>(pcap) * rec_bytes, "records"));
   FS_TRY(c->foot.ensure(static_cast<size_t>(pcap) * sizeof(fs::Footprint), "footprints"));
-  FS_TRY(c->cnt.ensure(static_cast<size_t>(pcap) * 4, "counts"));
+  FS_TRY(c->box.ensure(static_cast<size_t>(pcap) * sizeof(fs::TileBox), "tile boxes"));
   FS_TRY(c->dlo.ensure(static_cast<size_t>(pcap) * 4, "depth low words"));
-  if (keep) FS_TRY(c->dkey.ensure(static_cast<size_t>(pcap) * 4, "depth keys"));
   if (c->sigma3) FS_TRY(c->cols.ensure(static_cast<size_t>(pcap) * 4, "tile columns"));
   FS_TRY(c->key_a.ensure(static_cast<size_t>(kcap) * 4, "keys"));
   FS_TRY(c->val_a.ensure(static_cast<size_t>(kcap) * 4, "vals"));
@@ -638,6 +637,9 @@ fs_status read_total(fs_ctx* c, cudaStream_t stream, int64_t* out) {
 // sorted list values go to *val_dst (grown as needed) and the per-tile ranges
 // to ranges_dst.  Returns the entry count in *I_out.
 //
+// live: the positions are first reduced to the slots with an unsaturated tile
+// in their box (for large chunks behind saturated tiles).
+//
 // Captured form (range_dev != NULL): the chunk's positions are read on the
 // device from range_dev[0 .. 1] (at most n_pos of them: the grid), nothing is
 // read back, and the lists are sized for plan_cap entries (the capture's
@@ -647,21 +649,37 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
                         const ProjPtrs& P,
                         const uint64_t* sat, int total_tiles, int tile_bits, int64_t kcap,
                         bool count_entries, DevBuf* val_dst, uint2* ranges_dst,
-                        cudaStream_t stream, int64_t* I_out, const int64_t* range_dev = nullptr,
-                        int64_t plan_cap = 0) {
+                        cudaStream_t stream, int64_t* I_out, bool live = false,
+                        const int64_t* range_dev = nullptr, int64_t plan_cap = 0) {
   unsigned long long* ctr = c->counters.as<unsigned long long>();
   *I_out = 0;
   FS_CUDA(cudaMemsetAsync(ranges_dst, 0, static_cast<size_t>(total_tiles) * 8, stream),
           "ranges clear");
   FS_TRY(c->lb_tmp.ensure(fs::bin_fused_temp_bytes(n_pos), "binning look-back"));
   // the views' prefix tables of the tiles still unsaturated
+  int tl = -1;
+  FS_TRY(stage_begin(c, FS_STAGE_BINNING, stream, range_dev != nullptr, &tl));
   FS_CUDA(fs::launch_free_tables(vd, nb, sat, stream), "tile prefix tables");
+  const int64_t* range = range_dev;  // what the binning reads its positions from
+  if (live) {
+    int64_t* const rng = c->live_range.as<int64_t>();
+    uint32_t* const slots = c->live_val.as<uint32_t>();
+    FS_CUDA(fs::launch_slot_live(n, vd, nb, P.box, c->live.as<uint32_t>(), stream), "slot bits");
+    FS_CUDA(fs::launch_compact_live(p0, n_pos, n, sorted_val, c->live.as<uint32_t>(), slots, rng,
+                                    c->lb_tmp.p, ctr, stream, range_dev),
+            "live slots");
+    if (!range_dev) c->stats.kernel_launches += 2;
+    sorted_val = slots;
+    range = rng;
+    p0 = 0;
+  }
+  FS_TRY(stage_end(c, tl, stream));
   if (range_dev) {
     uint32_t* total = c->total.as<uint32_t>();
     const uint32_t capacity = static_cast<uint32_t>(plan_cap);
     FS_CUDA(fs::launch_bin_fused(0, n_pos, n, vd, nb, sorted_val, P.foot, sat, c->lk_a.as<uint32_t>(),
                                  val_dst->as<uint32_t>(), capacity, c->lb_tmp.p, total, ctr,
-                                 stream, range_dev),
+                                 stream, range),
             "binning");
     FS_CUDA(fs::launch_graph_check(total, capacity, nullptr, 0, range_dev, n_pos, ctr, stream),
             "plan check");
@@ -692,7 +710,7 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
     FS_TRY(stage_begin(c, FS_STAGE_BINNING, stream, false, &tb));
     FS_CUDA(fs::launch_bin_fused(p0, n_pos, n, vd, nb, sorted_val, P.foot, sat,
                                  c->lk_a.as<uint32_t>(), val_dst->as<uint32_t>(), capacity,
-                                 c->lb_tmp.p, c->total.as<uint32_t>(), ctr, stream),
+                                 c->lb_tmp.p, c->total.as<uint32_t>(), ctr, stream, range),
             "binning");
     FS_TRY(stage_end(c, tb, stream));
     FS_TRY(read_total(c, stream, &I));
@@ -726,6 +744,13 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
   FS_TRY(stage_end(c, tt, stream));
   return FS_OK;
 }
+
+// Chunks of at least this many positions, and a fifth of the batch's slots, are
+// reduced to their live slots before the binning.  The bits cost a pass over
+// every slot of the batch (180 us for 4.8 10^7) and pay where most of the
+// chunk's slots lie behind saturated tiles: its last two chunks 600 and 1041
+// us without, 545 and 645 us with the bits; earlier and smaller chunks lose.
+constexpr int64_t kLiveMin = 1 << 22;
 
 // Front-to-back depth chunk boundaries of a batch of k_total sorted slots:
 // chunk ci covers positions [chunk_begin(ci), chunk_begin(ci + 1)).
@@ -835,6 +860,12 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
     cudaGetLastError();
   }
   FS_TRY(c->key_range.ensure(32, "depth key range"));
+  if (kcap >= kLiveMin) {
+    FS_TRY(c->live.ensure(static_cast<size_t>(fs::live_words(n)) * vb * 4, "slot bits"));
+    // chunks but the first hold at most half the slots (and one)
+    FS_TRY(c->live_val.ensure(static_cast<size_t>(kcap / 2 + 1) * 4, "live slots"));
+    FS_TRY(c->live_range.ensure(16, "live slot range"));
+  }
   struct Prologue {
     BatchLayout L;
     fs::ViewParams* vd = nullptr;  // the batch's views on the device
@@ -877,14 +908,10 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
     int tp = -1;
     FS_TRY(stage_begin(c, FS_STAGE_PROJECT, strm, plan != nullptr, &tp));
     FS_CUDA(fs::launch_project(n, nbb, pr.vd, s->pos_op.as<float4>(), s->cov.as<float4>(),
-                               PP.rec, PP.rec16, PP.foot, PP.cnt, pr.key, PP.dlo, krq,
+                               PP.rec, PP.rec16, PP.foot, PP.box, pr.key, PP.dlo, krq,
                                strm),
             "project");
     FS_TRY(stage_end(c, tp, strm));
-    if (PP.dkey)
-      FS_CUDA(cudaMemcpyAsync(PP.dkey, pr.key, static_cast<size_t>(nbb) * n * 4,
-                              cudaMemcpyDeviceToDevice, strm),
-              "depth key copy");
     if (plan) return FS_OK;  // captured: the key range stays on the device
     FS_CUDA(cudaMemcpyAsync(krhq, krq, 12, cudaMemcpyDeviceToHost, strm), "key range readback");
     FS_CUDA(cudaEventRecord(c->prologue_done[q], strm), "prologue event");
@@ -1010,8 +1037,9 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
         continue;
       }
       int64_t I = 0;
+      const bool live = ci > 0 && n_pos >= kLiveMin && 5 * n_pos >= k_total;
       FS_TRY(bin_positions(c, p0, n_pos, n, vd, nb, sorted_val, P, sat, total_tiles, tile_bits, kcap,
-                           !plan, val_dst, ranges_dst, stream, &I,
+                           !plan, val_dst, ranges_dst, stream, &I, live,
                            plan ? c->chunk_bnd.as<int64_t>() + ci : nullptr,
                            plan ? plan->entries[pi] : 0));
       if (record) record->entries[pi] = I;
@@ -1034,7 +1062,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
 // list per tile) and the re-check compositing of them into R.
 fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, int64_t kcap,
                               const BatchLayout& L, const fs::ViewParams* vd, const ProjPtrs& P,
-                              const uint32_t* key_src, uint64_t* skip, int32_t mask_dtype,
+                              uint64_t* skip, int32_t mask_dtype,
                               int32_t E, const uint32_t* F, int64_t nF, const int32_t* map,
                               double* R, cudaStream_t stream) {
   const int total_tiles = L.total_tiles;
@@ -1045,7 +1073,7 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
   FS_TRY(c->offs.ensure(static_cast<size_t>(kcap) * 4, "candidate offsets"));
   FS_TRY(c->scan_tmp.ensure(fs::scan_temp_bytes(kcap), "scan temp"));
   c->stats.kernel_launches += 1 + scan_launches(k_total);
-  FS_CUDA(fs::launch_candidates(k_total, n, vd, P.cnt, P.foot, skip, c->ccnt.as<uint32_t>(),
+  FS_CUDA(fs::launch_candidates(k_total, n, vd, P.box, P.foot, skip, c->ccnt.as<uint32_t>(),
                                 stream),
           "candidates");
   FS_CUDA(fs::exclusive_scan(c->ccnt.as<uint32_t>(), nullptr, c->offs.as<uint32_t>(), k_total,
@@ -1055,7 +1083,7 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
   FS_TRY(read_total(c, stream, &C));
   if (C == 0) return FS_OK;
   c->stats.kernel_launches += 2 + radix_launches(C, 32);
-  FS_CUDA(fs::launch_compact(k_total, c->ccnt.as<uint32_t>(), c->offs.as<uint32_t>(), key_src,
+  FS_CUDA(fs::launch_compact(k_total, c->ccnt.as<uint32_t>(), c->offs.as<uint32_t>(), P.rec, P.rec16,
                              c->key_b.as<uint32_t>(), c->val_b.as<uint32_t>(), stream),
           "compact");
   bool alt = false;
@@ -1076,7 +1104,7 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
   Ls.chunks = 1;
   Ls.flagged = F;
   Ls.n_flagged = static_cast<int>(std::min<int64_t>(nF, 0x7FFFFFFF));
-  Ls.cnt = P.cnt;
+  Ls.box = P.box;
   Ls.foot = P.foot;
   c->stats.kernel_launches += 2;
   FS_CUDA(fs::launch_recheck_blend(vd, nb, L.max_tiles, Ls, skip, c->rk_tiles.p, c->n_sm, P.rec, P.rec16,
@@ -1155,14 +1183,12 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
     uint64_t* deep = c->subsat.as<uint64_t>();
     FS_CUDA(cudaMemcpyAsync(vd, vh, sizeof(fs::ViewParams) * nb, cudaMemcpyHostToDevice, stream),
             "view upload");
-    const uint32_t* key_src = P.dkey;
     if (!keep) {
       c->stats.kernel_launches += 1;
       FS_CUDA(fs::launch_project(n, nb, vd, s->pos_op.as<float4>(), s->cov.as<float4>(), P.rec,
-                                 P.rec16, P.foot, P.cnt, c->key_a.as<uint32_t>(), P.dlo, nullptr,
+                                 P.rec16, P.foot, P.box, c->key_a.as<uint32_t>(), P.dlo, nullptr,
                                  stream),
               "project");
-      key_src = c->key_a.as<uint32_t>();
     }
     // tiles to re-render: those the flagged Gaussians reach
     FS_CUDA(cudaMemsetAsync(skip, 0xFF, sat_bytes, stream), "skip bits");
@@ -1172,8 +1198,8 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
     const uint32_t* bound = kept ? K->kl_bound.as<uint32_t>() + static_cast<int64_t>(b) * chunks
                                  : nullptr;
     c->stats.kernel_launches += 1;
-    FS_CUDA(fs::launch_mark_tiles(nF, nb, n, F, vd, P.cnt, P.foot, skip, c->total.as<uint32_t>(),
-                                  bound, chunks, P.dkey, P.dlo, satc, deep, stream),
+    FS_CUDA(fs::launch_mark_tiles(nF, nb, n, F, vd, P.box, P.foot, skip, c->total.as<uint32_t>(),
+                                  bound, chunks, P.rec, P.rec16, P.dlo, satc, deep, stream),
             "mark tiles");
     int64_t visible = 0;
     FS_TRY(read_total(c, stream, &visible));
@@ -1191,7 +1217,7 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
       Ls.deep = deep;
       Ls.flagged = F;
       Ls.n_flagged = static_cast<int>(std::min<int64_t>(nF, 0x7FFFFFFF));
-      Ls.cnt = P.cnt;
+      Ls.box = P.box;
       Ls.foot = P.foot;
       FS_CUDA(cudaMemsetAsync(Rb, 0, rbytes, stream), "batch rows clear");
       FS_CUDA(cudaMemsetAsync(ctr + fs::kRecheckIncomplete, 0, 8, stream), "incomplete clear");
@@ -1211,7 +1237,7 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
       }
       c->stats.recheck_rebinned += 1;  // kept lists end too early: bin these tiles anew
     }
-    FS_TRY(recheck_batch_rebin(c, s, n, nb, kcap, L, vd, P, key_src, skip, mask_dtype, E, F, nF,
+    FS_TRY(recheck_batch_rebin(c, s, n, nb, kcap, L, vd, P, skip, mask_dtype, E, F, nF,
                                map, R, stream));
   }
   c->stats.kernel_launches += 1;
@@ -1302,7 +1328,7 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
     FS_CUDA(cudaMemsetAsync(krq, 0xFF, 4, stream), "key range");
     FS_CUDA(cudaMemsetAsync(krq + 1, 0, 8, stream), "key range");
     FS_CUDA(fs::launch_project(n, nb, vd, s->pos_op.as<float4>(), s->cov.as<float4>(), P.rec,
-                               P.rec16, P.foot, P.cnt, c->key_a.as<uint32_t>(), P.dlo, krq, stream),
+                               P.rec16, P.foot, P.box, c->key_a.as<uint32_t>(), P.dlo, krq, stream),
             "project");
     FS_CUDA(cudaMemcpyAsync(krh, krq, 12, cudaMemcpyDeviceToHost, stream), "key range readback");
     FS_CUDA(cudaStreamSynchronize(stream), "key range readback");
@@ -1333,7 +1359,7 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
     FS_CUDA(cudaMemsetAsync(c->sat.p, 0, sat_bytes, stream), "tile flags clear");
     for (int e = 1; e < E; ++e) {
       uint32_t* flag = c->rd_flag.as<uint32_t>();
-      FS_CUDA(fs::launch_member_select(k_vis, n, sorted_val, P.cnt, member_bits, 1ull << e, flag,
+      FS_CUDA(fs::launch_member_select(k_vis, n, sorted_val, P.box, member_bits, 1ull << e, flag,
                                        stream),
               "object slots");
       FS_CUDA(fs::exclusive_scan(flag, nullptr, c->rd_offs.as<uint32_t>(), k_vis,
@@ -1412,8 +1438,8 @@ bool keep_fits(const fs_ctx* c, int64_t n, int32_t V) {
     return false;
   }
   const double need = (c->compact ? 76.0 : 108.0) * static_cast<double>(n) * V;
-  const double have = static_cast<double>(c->rec.bytes + c->foot.bytes + c->cnt.bytes +
-                                          c->dlo.bytes + c->dkey.bytes);
+  const double have = static_cast<double>(c->rec.bytes + c->foot.bytes + c->box.bytes +
+                                          c->dlo.bytes);
   return need <= have + 0.5 * static_cast<double>(free_b);
 }
 

@@ -17,6 +17,7 @@ struct ViewParams;
 struct ProjRecord;
 struct CompactRecord;
 struct Footprint;
+typedef uint2 TileBox;
 
 // Polls of a predecessor's look-back word before the wait gives up (about 2 s).
 constexpr int kLookbackSpinLimit = 1 << 26;
@@ -54,13 +55,13 @@ cudaError_t launch_scene_prep(int64_t n, const float* mean, const void* quat, in
 // rec16 != NULL: reduced-precision records (FP16 whitening matrix, FP32 mean)
 // are written to rec16 instead of the float-pair records to rec.  Records are
 // written for visible slots only (nothing reads the others'); footprints,
-// counts, keys and low depth words for every slot.
+// tile boxes, keys and low depth words for every slot.
 // key_range (3 uint32, may be NULL): atomic min / max of the visible slots'
 // depth keys and their number (the caller initialises it to {0xFFFFFFFF, 0,
 // 0}).  After the depth sort the visible slots are the first ones.
 cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, const float4* pos_op,
                            const float4* cov, ProjRecord* rec, CompactRecord* rec16,
-                           Footprint* foot, uint32_t* cnt, uint32_t* key, uint32_t* depth_lo,
+                           Footprint* foot, TileBox* box, uint32_t* key, uint32_t* depth_lo,
                            uint32_t* key_range, cudaStream_t stream);
 // re-orders runs of equal 32-bit depth keys by the depth's low word, then slot
 // (n_total elements; slot / n is the view of a slot)
@@ -80,6 +81,19 @@ cudaError_t launch_bin_fused(int64_t p0, int64_t n_pos, int64_t n, const ViewPar
                              unsigned long long* counters, cudaStream_t stream,
                              const int64_t* range_dev = nullptr);
 size_t bin_fused_temp_bytes(int64_t n_pos);
+// Words of one view's bits of launch_slot_live (n Gaussians).
+int64_t live_words(int64_t n);
+// One bit per (view, Gaussian) slot of the batch: a tile of its box is
+// unsaturated by the views' prefix tables, which must be current.
+cudaError_t launch_slot_live(int64_t n, const ViewParams* views, int n_views, const TileBox* box,
+                             uint32_t* live, cudaStream_t stream);
+// The live slots among sorted positions [p0, p0 + n_pos) (or range_in[0 .. 1),
+// at most n_pos of them), in order, to out, and {0, their number} to range_out
+// (device).  lookback: bin_fused_temp_bytes(n_pos) of scratch.
+cudaError_t launch_compact_live(int64_t p0, int64_t n_pos, int64_t n, const uint32_t* sorted_val,
+                                const uint32_t* live, uint32_t* out, int64_t* range_out,
+                                void* lookback, unsigned long long* counters, cudaStream_t stream,
+                                const int64_t* range_in);
 // Diagnostic: the fused binning on one block whose predecessor never
 // publishes, with a wait bound of spin_limit polls (lookback: 512 B, total:
 // one word, counters: kNumCounters; the other arrays need one element each).
@@ -166,25 +180,26 @@ cudaError_t launch_scatter_flagged(int64_t n, const uint32_t* flag, const uint32
                                    uint32_t* F, int32_t* map, cudaStream_t stream);
 // clears the skip bits of every tile a flagged Gaussian reaches in the batch;
 // *visible += the number of visible (view, flagged Gaussian) pairs.  With
-// kept chunk lists (bound: the last slot of each depth chunk; dkey / dlo: the
-// batch's depth keys and low words; sat_chunk: the chunk in which each tile
+// kept chunk lists (bound: the last slot of each depth chunk; rec / rec16 and
+// dlo: the batch's records and low depth words, which order its slots; sat_chunk: the chunk in which each tile
 // saturated, 0xFF = never), sets the `deep` bit of every tile that saturated
 // before the flagged Gaussian's own chunk.  bound == NULL: no kept lists.
 cudaError_t launch_mark_tiles(int64_t n_flagged, int n_views, int64_t n, const uint32_t* F,
-                              const ViewParams* views, const uint32_t* cnt, const Footprint* foot,
+                              const ViewParams* views, const TileBox* box, const Footprint* foot,
                               uint64_t* skip, uint32_t* visible, const uint32_t* bound,
-                              int chunks, const uint32_t* dkey, const uint32_t* dlo,
+                              int chunks, const ProjRecord* rec, const CompactRecord* rec16,
+                              const uint32_t* dlo,
                               const uint8_t* sat_chunk, uint64_t* deep, cudaStream_t stream);
 // dst[i] += src[i], i < count
 cudaError_t launch_add_rows(int64_t count, const double* src, double* dst, cudaStream_t stream);
 // flag[slot] = the slot's footprint reaches an unskipped tile
 cudaError_t launch_candidates(int64_t k_total, int64_t n, const ViewParams* views,
-                              const uint32_t* cnt, const Footprint* foot, const uint64_t* skip,
+                              const TileBox* box, const Footprint* foot, const uint64_t* skip,
                               uint32_t* flag, cudaStream_t stream);
-// (out_key, out_val)[offs[slot]] = (key_src[slot], slot) for flagged slots
+// (out_key, out_val)[offs[slot]] = (the slot's depth key, slot) for flagged slots
 cudaError_t launch_compact(int64_t k_total, const uint32_t* flag, const uint32_t* offs,
-                           const uint32_t* key_src, uint32_t* out_key, uint32_t* out_val,
-                           cudaStream_t stream);
+                           const ProjRecord* rec, const CompactRecord* rec16, uint32_t* out_key,
+                           uint32_t* out_val, cudaStream_t stream);
 // Depth-ordered tile lists for the re-check: `chunks` consecutive depth
 // chunks, each with its list values and per-batch-tile ranges; sat_chunk and
 // deep as in launch_mark_tiles (NULL when the lists are complete).
@@ -199,7 +214,7 @@ struct RecheckLists {
   // visibility and footprints: which of them contribute at a pixel
   const uint32_t* flagged;
   int n_flagged;
-  const uint32_t* cnt;
+  const TileBox* box;
   const Footprint* foot;
 };
 // Scratch of launch_recheck_blend for a batch of total_tiles tiles (bytes).
@@ -221,9 +236,9 @@ struct RenderOut {
   float* rho;
   float* depth;
 };
-// flag[k] = 1 iff sorted slot k is visible (cnt != 0) and member[slot % n] & bit
+// flag[k] = 1 iff sorted slot k is visible and member[slot % n] & bit
 cudaError_t launch_member_select(int64_t k_total, int64_t n, const uint32_t* sorted_val,
-                                 const uint32_t* cnt, const uint64_t* member, uint64_t bit,
+                                 const TileBox* box, const uint64_t* member, uint64_t bit,
                                  uint32_t* flag, cudaStream_t stream);
 // out[offs[k]] = sorted_val[k] for flagged k (order kept)
 cudaError_t launch_member_scatter(int64_t k_total, const uint32_t* flag, const uint32_t* offs,

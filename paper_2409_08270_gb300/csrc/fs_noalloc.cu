@@ -46,8 +46,8 @@ constexpr size_t oCov = oPos + al(kNA_N * 16);
 constexpr size_t oViews = oCov + al(kNA_N * 48);
 constexpr size_t oRec = oViews + al(sizeof(ViewParams));
 constexpr size_t oFoot = oRec + al(kNA_N * sizeof(ProjRecord));
-constexpr size_t oCnt = oFoot + al(kNA_N * sizeof(Footprint));
-constexpr size_t oKeyA = oCnt + al(kNA_N * 4);
+constexpr size_t oBox = oFoot + al(kNA_N * sizeof(Footprint));
+constexpr size_t oKeyA = oBox + al(kNA_N * sizeof(TileBox));
 constexpr size_t oValA = oKeyA + al(kNA_N * 4);
 constexpr size_t oKeyB = oValA + al(kNA_N * 4);
 constexpr size_t oValB = oKeyB + al(kNA_N * 4);
@@ -181,7 +181,7 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
   ViewParams* vd = reinterpret_cast<ViewParams*>(S + oViews);
   ProjRecord* rec = reinterpret_cast<ProjRecord*>(S + oRec);
   Footprint* foot = reinterpret_cast<Footprint*>(S + oFoot);
-  uint32_t* cnt = reinterpret_cast<uint32_t*>(S + oCnt);
+  TileBox* box = reinterpret_cast<TileBox*>(S + oBox);
   uint32_t* key_a = reinterpret_cast<uint32_t*>(S + oKeyA);
   uint32_t* val_a = reinterpret_cast<uint32_t*>(S + oValA);
   uint32_t* key_b = reinterpret_cast<uint32_t*>(S + oKeyB);
@@ -225,7 +225,7 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
     const int tiles = vp.tiles_x * vp.tiles_y;
     // pageable source: the copy has taken the bytes when the call returns
     NA_CUDA(cudaMemcpyAsync(vd, &vp, sizeof(vp), cudaMemcpyHostToDevice, strm), "view upload");
-    NA_CUDA(launch_project(n, 1, vd, pos, cov, rec, nullptr, foot, cnt, key_a, dlo, nullptr,
+    NA_CUDA(launch_project(n, 1, vd, pos, cov, rec, nullptr, foot, box, key_a, dlo, nullptr,
                            strm),
             "project");
     bool alt = false;

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
     int64_t n, int n_views, const ViewParams* __restrict__ views_g,
     const float4* __restrict__ pos_op, const float4* __restrict__ cov3,
     ProjRecord* __restrict__ rec, CompactRecord* __restrict__ rec16, Footprint* __restrict__ foot,
-    uint32_t* __restrict__ cnt, uint32_t* __restrict__ key, uint32_t* __restrict__ depth_lo,
+    TileBox* __restrict__ box, uint32_t* __restrict__ key, uint32_t* __restrict__ depth_lo,
     uint32_t* __restrict__ key_range) {
   __shared__ ViewParams views[kMaxViewsPerBatch];
   for (int k = threadIdx.x; k < n_views * (int)(sizeof(ViewParams) / 4); k += blockDim.x)
@@ -171,7 +171,6 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
     const f2 tx = f2x2_first(txy), ty = f2x2_second(txy);
     const f2 tz = f2_dot3_add(vp.R_hi + 6, vp.R_lo + 6, po.x, po.y, po.z, vp.t_hi[2], vp.t_lo[2]);
     bool visible = opaque_enough && f2_greater(tz, vp.near_hi, vp.near_lo);
-    uint32_t count = 0;
     float depth = 0.f, depth_l = 0.f;
     ProjRecord R;
     R.w_hi = R.w_lo = R.m = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -186,7 +185,8 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
     Footprint F;
     F.mx = F.my = F.hy = F.syr = F.dys = F.a = F.b2 = 0.f;
     F.rows = 0x0000FFFFu;  // no tile row (first row 65535 > last row 0)
-    uint32_t col_clip = 0x0000FFFFu;  // 3-sigma coverage: no tile column
+    uint32_t col_clip = kNoBox;       // 3-sigma coverage: no tile column
+    TileBox bx = make_uint2(kNoBox, kNoBox);
     if (visible) {
       float sxx, sxy, syy, det32, mx32, my32;  // 2D covariance and mean for the footprint
       if constexpr (kFast) {
@@ -399,7 +399,18 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
         }
         if (ty0 <= ty1) {
           F.rows = static_cast<uint32_t>(ty0) | (static_cast<uint32_t>(ty1) << 16);
-          count = 1;
+          // the spans of the rows stay within +-hx of the mean; one more pixel
+          // on each side, and a little of hx, cover their rounding
+          const float bxw = 1.00001f * hx;
+          int c0 = static_cast<int>(fmaxf(ceilf(F.mx - bxw - 2.5f), 0.f)) / kTile;
+          int c1 = static_cast<int>(fminf(floorf(F.mx + bxw + 1.5f),
+                                          static_cast<float>(vp.width - 1))) / kTile;
+          if (vp.cols) {
+            c0 = max(c0, static_cast<int>(col_clip & 0xFFFFu));
+            c1 = min(c1, static_cast<int>(col_clip >> 16));
+          }
+          if (c0 <= c1)
+            bx = make_uint2(static_cast<uint32_t>(c0) | (static_cast<uint32_t>(c1) << 16), F.rows);
         } else {
           visible = false;
         }
@@ -413,7 +424,7 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
         rec[slot] = R;
     }
     foot[slot] = F;
-    cnt[slot] = visible ? count : 0u;
+    box[slot] = bx;
     const uint32_t k = visible ? depth_key(depth) : 0xFFFFFFFFu;
     if (visible) {
       kmin = min(kmin, k);
@@ -653,13 +664,49 @@ __device__ __forceinline__ uint32_t nth_free(const uint64_t* __restrict__ sat, i
 // look-back that polls a predecessor's word more than spin_limit times gives
 // up, counts a time-out (kLookbackTimeout) and uses 0.
 //
-// A warp spreads its 32 positions' tile rows over its lanes, one (slot, row)
+// With the positions' number read on the device (kDeviceRange) the blocks past
+// it leave at once.  (One set of resident blocks that loops over the tickets
+// measured slower, 7.06 ms against 5.25 for the 100-view, 10^6-Gaussian
+// workload: its blocks advance in step and look back over each other.)  A warp
+// spreads its 32 positions' tile rows over its lanes, one (slot, row)
 // job per lane per round, so large footprints do not hold up small ones; the
 // entries of a round are then spread over the lanes again, so that 32
 // consecutive list places are written at a time.
 constexpr unsigned long long kLbCount = 1ull << 32;   // word holds the block's own count
 constexpr unsigned long long kLbPrefix = 2ull << 32;  // word holds the inclusive prefix
 constexpr int kBinThreads = 128, kBinWarps = kBinThreads / 32;
+
+// Decoupled look-back by one warp: the sum of the counts of blocks 0 .. vb - 1,
+// 32 predecessors at a time (lane l reads block vb - 1 - l).
+__device__ __forceinline__ uint32_t look_back(const unsigned long long* status, uint32_t vb,
+                                              unsigned long long* counters, int spin_limit,
+                                              int lane) {
+  const volatile unsigned long long* vs = status;
+  uint32_t excl = 0;
+  for (int64_t base = static_cast<int64_t>(vb) - 1; base >= 0; base -= 32) {
+    const int64_t q = base - lane;
+    unsigned long long word = kLbPrefix;  // before block 0: an empty prefix
+    if (q >= 0) {
+      word = vs[q];
+      int spins = 0;
+      while ((word >> 32) == 0ull && spins < spin_limit) {
+        __nanosleep(32);
+        word = vs[q];
+        ++spins;
+      }
+      if ((word >> 32) == 0ull) {  // gave up: report, count it as an empty prefix
+        atomicAdd(&counters[kLookbackTimeout], 1ull);
+        word = kLbPrefix;
+      }
+    }
+    const uint32_t pre = __ballot_sync(0xffffffffu, (word & ~0xFFFFFFFFull) == kLbPrefix);
+    const int first = pre ? __ffs(pre) - 1 : 31;  // nearest predecessor holding a prefix
+    excl += __reduce_add_sync(0xffffffffu,
+                              lane <= first ? static_cast<uint32_t>(word & 0xFFFFFFFFull) : 0u);
+    if (pre) break;
+  }
+  return excl;
+}
 
 template <bool kDeviceRange>
 __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
@@ -674,7 +721,7 @@ __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
   __shared__ BinView s_view[kMaxViewsPerBatch];
   if constexpr (kDeviceRange) {  // the chunk's positions [range_dev[0], range_dev[1])
     p0 = range_dev[0];
-    n_pos = range_dev[1] - range_dev[0];
+    n_pos = min(n_pos, range_dev[1] - range_dev[0]);  // the launch's scratch is sized for n_pos
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_vb = atomicAdd(ticket, 1u);
@@ -688,6 +735,7 @@ __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
   __syncthreads();
   const uint32_t vb = s_vb;
   const int64_t j = static_cast<int64_t>(vb) * kBinThreads + threadIdx.x;
+  if (j - threadIdx.x >= n_pos) return;  // whole block: the grid was sized for more
   uint32_t g = 0u, nrows = 0u;
   int ty0 = 0;
   if (j < n_pos) {
@@ -728,40 +776,16 @@ __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
   }
   if (lane == 0) s_wtot[warp] = wtot;
   __syncthreads();
-  // offset of the block: decoupled look-back over the predecessors, 32 at a
-  // time (lane l reads predecessor vb - 1 - l)
+  // offset of the block
   if (warp == 0) {
     uint32_t btot = 0;
     for (int w = 0; w < kBinWarps; ++w) btot += s_wtot[w];
     if (lane == 0) atomicExch(&status[vb], (vb == 0 ? kLbPrefix : kLbCount) | btot);
-    volatile unsigned long long* vs = status;
-    uint32_t excl = 0;
-    for (int64_t base = static_cast<int64_t>(vb) - 1; base >= 0; base -= 32) {
-      const int64_t q = base - lane;
-      unsigned long long word = kLbPrefix;  // before block 0: an empty prefix
-      if (q >= 0) {
-        word = vs[q];
-        int spins = 0;
-        while ((word >> 32) == 0ull && spins < spin_limit) {
-          __nanosleep(32);
-          word = vs[q];
-          ++spins;
-        }
-        if ((word >> 32) == 0ull) {  // gave up: report, count it as an empty prefix
-          atomicAdd(&counters[kLookbackTimeout], 1ull);
-          word = kLbPrefix;
-        }
-      }
-      const uint32_t pre = __ballot_sync(0xffffffffu, (word & ~0xFFFFFFFFull) == kLbPrefix);
-      const int first = pre ? __ffs(pre) - 1 : 31;  // nearest predecessor holding a prefix
-      excl += __reduce_add_sync(
-          0xffffffffu, lane <= first ? static_cast<uint32_t>(word & 0xFFFFFFFFull) : 0u);
-      if (pre) break;
-    }
+    const uint32_t excl = look_back(status, vb, counters, spin_limit, lane);
     if (lane == 0) {
       if (vb > 0) atomicExch(&status[vb], kLbPrefix | (excl + btot));
       s_boff = excl;
-      if (vb == gridDim.x - 1) *total = excl + btot;
+      if (static_cast<int64_t>(vb + 1) * kBinThreads >= n_pos) *total = excl + btot;
     }
   }
   __syncthreads();
@@ -809,13 +833,118 @@ __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
   if (lane == 0 && o0 != wend) atomicAdd(&counters[kBinningMismatch], 1ull);
 }
 
+// Bit i % 32 of word view * words_per_view + i / 32: an unsaturated tile lies
+// in the tile box of Gaussian i in that view.  A block takes kLiveSlots
+// consecutive slots of one view, whose prefix table it reads from shared
+// memory (views of up to kTableCells cells): in depth order a slot's four
+// table reads each fetch a sector of some other view's table.  Bound by the
+// 8 B a slot.
+constexpr int kTableCells = 10240;
+constexpr int kLiveSlots = 16384;
+__global__ void __launch_bounds__(256) slot_live_kernel(
+    int64_t n, const ViewParams* __restrict__ views, const TileBox* __restrict__ box,
+    int64_t words_per_view, uint32_t* __restrict__ live) {
+  __shared__ uint16_t s_tab[kTableCells];
+  const ViewParams& vp = views[blockIdx.y];
+  const int tx = vp.tiles_x, w1 = tx + 1;
+  const int64_t cells = static_cast<int64_t>(w1) * (vp.tiles_y + 1);
+  const uint32_t* __restrict__ tab = vp.free_tab;
+  const bool shared = cells <= kTableCells;
+  if (shared)
+    for (int k = threadIdx.x; k < static_cast<int>(cells); k += 256)
+      s_tab[k] = static_cast<uint16_t>(tab[k]);
+  __syncthreads();
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kLiveSlots + threadIdx.x;
+  const TileBox* __restrict__ vbox = box + static_cast<int64_t>(blockIdx.y) * n;
+  uint32_t* const out = live + static_cast<int64_t>(blockIdx.y) * words_per_view;
+#pragma unroll 4
+  for (int k = 0; k < kLiveSlots / 256; ++k) {
+    const int64_t i = i0 + 256 * k;
+    bool any = false;
+    if (i < n) {
+      const TileBox b = vbox[i];
+      if (box_visible(b)) {
+        const int c0 = b.x & 0xFFFFu, c1 = (b.x >> 16) + 1;
+        const int r0 = static_cast<int>(b.y & 0xFFFFu) * w1;
+        const int r1 = static_cast<int>((b.y >> 16) + 1) * w1;
+        any = shared ? s_tab[r1 + c1] + s_tab[r0 + c0] != s_tab[r0 + c1] + s_tab[r1 + c0]
+                     : tab[r1 + c1] + tab[r0 + c0] != tab[r0 + c1] + tab[r1 + c0];
+      }
+    }
+    const uint32_t bits = __ballot_sync(0xffffffffu, any);
+    if ((threadIdx.x & 31) == 0 && i < n) out[i >> 5] = bits;
+  }
+}
+
+// Sorted positions [p0, p0 + n_pos) (read from range_in, if given) whose slots
+// are live, in order, and their number as a range for the binning
+// (range_out[0 .. 1] = 0, count).  A warp takes 512 consecutive positions,
+// the slots of 32 per load; the block's place comes from a decoupled look-back
+// as in the binning.
+constexpr int kCompactItems = 16, kCompactWarps = 8;
+constexpr int kCompactTile = 32 * kCompactItems * kCompactWarps;
+__global__ void __launch_bounds__(32 * kCompactWarps) compact_live_kernel(
+    int64_t p0, int64_t n_pos, SlotView sv, const uint32_t* __restrict__ sorted_val,
+    int64_t words_per_view, const uint32_t* __restrict__ live, uint32_t* __restrict__ out,
+    unsigned long long* __restrict__ status, uint32_t* __restrict__ ticket,
+    int64_t* __restrict__ range_out, unsigned long long* __restrict__ counters, int spin_limit,
+    const int64_t* __restrict__ range_in) {
+  __shared__ uint32_t s_vb, s_boff, s_cnt[kCompactWarps];
+  if (range_in) {
+    p0 = range_in[0];
+    n_pos = min(n_pos, range_in[1] - range_in[0]);
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) s_vb = atomicAdd(ticket, 1u);
+  __syncthreads();
+  const uint32_t vb = s_vb;
+  const int64_t j0 = static_cast<int64_t>(vb) * kCompactTile + warp * 32 * kCompactItems + lane;
+  uint32_t g[kCompactItems], bal[kCompactItems], cnt = 0;
+#pragma unroll
+  for (int i = 0; i < kCompactItems; ++i)
+    g[i] = j0 + 32 * i < n_pos ? sorted_val[p0 + j0 + 32 * i] : 0xFFFFFFFFu;
+#pragma unroll
+  for (int i = 0; i < kCompactItems; ++i) {
+    bool on = false;
+    if (g[i] != 0xFFFFFFFFu) {
+      const uint32_t v = sv(g[i]), k = g[i] - v * sv.n;
+      on = (live[v * words_per_view + (k >> 5)] >> (k & 31)) & 1u;
+    }
+    bal[i] = __ballot_sync(0xffffffffu, on);
+    cnt += __popc(bal[i]);
+  }
+  if (lane == 0) s_cnt[warp] = cnt;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t btot = 0;
+    for (int w = 0; w < kCompactWarps; ++w) btot += s_cnt[w];
+    if (lane == 0) atomicExch(&status[vb], (vb == 0 ? kLbPrefix : kLbCount) | btot);
+    const uint32_t excl = look_back(status, vb, counters, spin_limit, lane);
+    if (lane == 0) {
+      if (vb > 0) atomicExch(&status[vb], kLbPrefix | (excl + btot));
+      s_boff = excl;
+      if (vb == gridDim.x - 1) {
+        range_out[0] = 0;
+        range_out[1] = excl + btot;
+      }
+    }
+  }
+  __syncthreads();
+  uint32_t o = s_boff;
+  for (int w = 0; w < warp; ++w) o += s_cnt[w];
+#pragma unroll
+  for (int i = 0; i < kCompactItems; ++i) {
+    if ((bal[i] >> lane) & 1u) out[o + __popc(bal[i] & ((1u << lane) - 1u))] = g[i];
+    o += __popc(bal[i]);
+  }
+}
+
 // Per view of the batch (one block each), the 2-D prefix sums of its
 // unsaturated tiles: free_tab[r * (tiles_x + 1) + c] = unsaturated tiles in
 // rows < r and columns < c (row 0 and column 0 are zero).  A warp runs along a
 // row 32 tiles at a time, a thread then down a column.  Views of up to
 // kTableCells cells keep the table in shared memory until it is whole (a
 // 1008x756 view: 17 us through global memory, 8 us so).
-constexpr int kTableCells = 10240;
 __global__ void __launch_bounds__(256) free_table_kernel(const ViewParams* __restrict__ views,
                                                          const uint64_t* __restrict__ sat) {
   __shared__ uint32_t s_tab[kTableCells];
@@ -902,7 +1031,7 @@ cudaError_t launch_scene_prep(int64_t n, const float* mean, const void* quat, in
 
 cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, const float4* pos_op,
                            const float4* cov, ProjRecord* rec, CompactRecord* rec16,
-                           Footprint* foot, uint32_t* cnt, uint32_t* key, uint32_t* depth_lo,
+                           Footprint* foot, TileBox* box, uint32_t* key, uint32_t* depth_lo,
                            uint32_t* key_range, cudaStream_t stream) {
   if (n == 0 || n_views == 0) return cudaSuccess;
   const int threads = 256;
@@ -910,10 +1039,10 @@ cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, cons
   // the reduced-precision form takes the FP32 projection
   if (rec16)
     project_kernel<true><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-        n, n_views, views, pos_op, cov, rec, rec16, foot, cnt, key, depth_lo, key_range);
+        n, n_views, views, pos_op, cov, rec, rec16, foot, box, key, depth_lo, key_range);
   else
     project_kernel<false><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-        n, n_views, views, pos_op, cov, rec, rec16, foot, cnt, key, depth_lo, key_range);
+        n, n_views, views, pos_op, cov, rec, rec16, foot, box, key, depth_lo, key_range);
   return cudaGetLastError();
 }
 
@@ -940,6 +1069,8 @@ cudaError_t launch_bin_fused(int64_t p0, int64_t n_pos, int64_t n, const ViewPar
   unsigned long long* status = reinterpret_cast<unsigned long long*>(
       static_cast<char*>(lookback) + 256);
   cudaError_t e = cudaMemsetAsync(lookback, 0, 256 + static_cast<size_t>(blocks) * 8, stream);
+  if (e == cudaSuccess && range_dev)  // a chunk may turn out empty
+    e = cudaMemsetAsync(total, 0, sizeof(uint32_t), stream);
   if (e != cudaSuccess) return e;
   auto launch = [&](auto kernel) {
     kernel<<<static_cast<unsigned>(blocks), kBinThreads, 0, stream>>>(
@@ -964,14 +1095,43 @@ cudaError_t launch_lookback_probe(void* lookback, uint32_t* total, unsigned long
   const uint32_t one = 1u;
   e = cudaMemcpyAsync(ticket, &one, sizeof(one), cudaMemcpyHostToDevice, stream);
   if (e != cudaSuccess) return e;
+  // position 128 is the ticket's first and only one, sorted_val[0]
   bin_fused_kernel<false><<<1, kBinThreads, 0, stream>>>(
-      0, 1, SlotView(1), views, 1, sorted_val, foot, sat, out_key, out_val, 0u, status, ticket,
-      total, counters, spin_limit, nullptr);
+      -kBinThreads, kBinThreads + 1, SlotView(1), views, 1, sorted_val, foot, sat, out_key,
+      out_val, 0u, status, ticket, total, counters, spin_limit, nullptr);
   return cudaGetLastError();
 }
 
 size_t bin_fused_temp_bytes(int64_t n_pos) {
   return 256 + static_cast<size_t>((n_pos + kBinThreads - 1) / kBinThreads) * 8;
+}
+
+int64_t live_words(int64_t n) { return (n + 31) / 32; }
+
+cudaError_t launch_slot_live(int64_t n, const ViewParams* views, int n_views, const TileBox* box,
+                             uint32_t* live, cudaStream_t stream) {
+  if (n <= 0 || n_views <= 0) return cudaSuccess;
+  const dim3 grid(static_cast<unsigned>((n + kLiveSlots - 1) / kLiveSlots),
+                  static_cast<unsigned>(n_views));
+  slot_live_kernel<<<grid, 256, 0, stream>>>(n, views, box, live_words(n), live);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_compact_live(int64_t p0, int64_t n_pos, int64_t n, const uint32_t* sorted_val,
+                                const uint32_t* live, uint32_t* out, int64_t* range_out,
+                                void* lookback, unsigned long long* counters, cudaStream_t stream,
+                                const int64_t* range_in) {
+  if (n_pos <= 0) return cudaMemsetAsync(range_out, 0, 2 * sizeof(int64_t), stream);
+  const int64_t blocks = (n_pos + kCompactTile - 1) / kCompactTile;
+  uint32_t* ticket = static_cast<uint32_t*>(lookback);
+  unsigned long long* status = reinterpret_cast<unsigned long long*>(
+      static_cast<char*>(lookback) + 256);
+  cudaError_t e = cudaMemsetAsync(lookback, 0, 256 + static_cast<size_t>(blocks) * 8, stream);
+  if (e != cudaSuccess) return e;
+  compact_live_kernel<<<static_cast<unsigned>(blocks), 32 * kCompactWarps, 0, stream>>>(
+      p0, n_pos, SlotView(n), sorted_val, live_words(n), live, out, status, ticket, range_out,
+      counters, kLookbackSpinLimit, range_in);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_free_tables(const ViewParams* views, int n_views, const uint64_t* sat,

@@ -58,12 +58,21 @@ __global__ void scatter_flagged_kernel(int64_t n, const uint32_t* __restrict__ f
   }
 }
 
+// The slot's depth key: its record holds the FP32 depth.
+__device__ __forceinline__ uint32_t slot_key(const ProjRecord* __restrict__ rec,
+                                             const CompactRecord* __restrict__ rec16,
+                                             uint32_t slot) {
+  return depth_key(rec16 ? rec16[slot].depth : rec[slot].misc.w);
+}
+
 // Position of slot a before-or-equal slot b in the batch's depth order:
 // (depth key, view, low word of the depth, slot).
 __device__ __forceinline__ bool order_le(uint32_t a, uint32_t b, int64_t n,
-                                         const uint32_t* __restrict__ dkey,
+                                         const ProjRecord* __restrict__ rec,
+                                         const CompactRecord* __restrict__ rec16,
                                          const uint32_t* __restrict__ dlo) {
-  if (dkey[a] != dkey[b]) return dkey[a] < dkey[b];
+  const uint32_t ka = slot_key(rec, rec16, a), kb = slot_key(rec, rec16, b);
+  if (ka != kb) return ka < kb;
   const uint32_t va = a / static_cast<uint32_t>(n), vb = b / static_cast<uint32_t>(n);
   if (va != vb) return va < vb;
   if (dlo[a] != dlo[b]) return dlo[a] < dlo[b];
@@ -78,12 +87,13 @@ __device__ __forceinline__ bool order_le(uint32_t a, uint32_t b, int64_t n,
 __global__ void mark_tiles_kernel(int64_t n_flagged, int n_views, int64_t n,
                                   const uint32_t* __restrict__ F,
                                   const ViewParams* __restrict__ views,
-                                  const uint32_t* __restrict__ cnt,
+                                  const TileBox* __restrict__ box,
                                   const Footprint* __restrict__ foot,
                                   unsigned long long* __restrict__ skip,
                                   uint32_t* __restrict__ visible,
                                   const uint32_t* __restrict__ bound, int chunks,
-                                  const uint32_t* __restrict__ dkey,
+                                  const ProjRecord* __restrict__ rec,
+                                  const CompactRecord* __restrict__ rec16,
                                   const uint32_t* __restrict__ dlo,
                                   const uint8_t* __restrict__ sat_chunk,
                                   unsigned long long* __restrict__ deep) {
@@ -91,14 +101,14 @@ __global__ void mark_tiles_kernel(int64_t n_flagged, int n_views, int64_t n,
   if (idx >= n_flagged * n_views) return;
   const int v = static_cast<int>(idx / n_flagged);
   const int64_t slot = static_cast<int64_t>(v) * n + F[idx % n_flagged];
-  if (!cnt[slot]) return;
+  if (!box_visible(box[slot])) return;
   atomicAdd(visible, 1u);
   int my_chunk = 0;
   if (bound) {
     my_chunk = chunks - 1;
     for (int ci = 0; ci < chunks - 1; ++ci)
       if (bound[ci] != 0xFFFFFFFFu &&  // an empty chunk holds nothing
-          order_le(static_cast<uint32_t>(slot), bound[ci], n, dkey, dlo)) {
+          order_le(static_cast<uint32_t>(slot), bound[ci], n, rec, rec16, dlo)) {
         my_chunk = ci;
         break;
       }
@@ -127,13 +137,13 @@ __global__ void mark_tiles_kernel(int64_t n_flagged, int n_views, int64_t n,
 
 // flag[slot] = 1 iff the slot's footprint reaches a tile left unskipped.
 __global__ void candidates_kernel(int64_t k_total, int64_t n, const ViewParams* __restrict__ views,
-                                  const uint32_t* __restrict__ cnt,
+                                  const TileBox* __restrict__ box,
                                   const Footprint* __restrict__ foot,
                                   const uint64_t* __restrict__ skip, uint32_t* __restrict__ flag) {
   const int64_t slot = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (slot >= k_total) return;
   uint32_t hit = 0;
-  if (cnt[slot]) {
+  if (box_visible(box[slot])) {
     const int v = static_cast<int>(slot / n);
     const ViewParams& vp = views[v];
     const Footprint f = foot[slot];
@@ -151,12 +161,12 @@ __global__ void candidates_kernel(int64_t k_total, int64_t n, const ViewParams* 
 
 __global__ void compact_kernel(int64_t k_total, const uint32_t* __restrict__ flag,
                                const uint32_t* __restrict__ offs,
-                               const uint32_t* __restrict__ key_src,
-                               uint32_t* __restrict__ out_key, uint32_t* __restrict__ out_val) {
+                               const ProjRecord* __restrict__ rec,
+                               const CompactRecord* __restrict__ rec16, uint32_t* __restrict__ out_key, uint32_t* __restrict__ out_val) {
   const int64_t slot = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (slot >= k_total || !flag[slot]) return;
   const uint32_t o = offs[slot];
-  out_key[o] = key_src[slot];
+  out_key[o] = slot_key(rec, rec16, static_cast<uint32_t>(slot));
   out_val[o] = static_cast<uint32_t>(slot);
 }
 
@@ -440,7 +450,7 @@ __global__ void __launch_bounds__(32 * kRWarps, 8) recheck_blend_kernel(
       for (int k0 = 0; k0 < L.n_flagged; k0 += 32) {
         bool on = k0 + lane < L.n_flagged;
         const uint32_t slot = slot0 + (on ? L.flagged[k0 + lane] : 0u);
-        on = on && L.cnt[slot] != 0u;
+        on = on && box_visible(L.box[slot]);
         if (on) {
           const Footprint f = L.foot[slot];
           int r0, r1, c0, c1;
@@ -559,15 +569,16 @@ cudaError_t launch_scatter_flagged(int64_t n, const uint32_t* flag, const uint32
 }
 
 cudaError_t launch_mark_tiles(int64_t n_flagged, int n_views, int64_t n, const uint32_t* F,
-                              const ViewParams* views, const uint32_t* cnt, const Footprint* foot,
+                              const ViewParams* views, const TileBox* box, const Footprint* foot,
                               uint64_t* skip, uint32_t* visible, const uint32_t* bound,
-                              int chunks, const uint32_t* dkey, const uint32_t* dlo,
+                              int chunks, const ProjRecord* rec, const CompactRecord* rec16,
+                              const uint32_t* dlo,
                               const uint8_t* sat_chunk, uint64_t* deep, cudaStream_t stream) {
   const int64_t total = n_flagged * n_views;
   if (total == 0) return cudaSuccess;
   mark_tiles_kernel<<<blocks_for(total, 256), 256, 0, stream>>>(
-      n_flagged, n_views, n, F, views, cnt, foot, reinterpret_cast<unsigned long long*>(skip),
-      visible, bound, chunks, dkey, dlo, sat_chunk, reinterpret_cast<unsigned long long*>(deep));
+      n_flagged, n_views, n, F, views, box, foot, reinterpret_cast<unsigned long long*>(skip),
+      visible, bound, chunks, rec, rec16, dlo, sat_chunk, reinterpret_cast<unsigned long long*>(deep));
   return cudaGetLastError();
 }
 
@@ -578,19 +589,19 @@ cudaError_t launch_add_rows(int64_t count, const double* src, double* dst, cudaS
 }
 
 cudaError_t launch_candidates(int64_t k_total, int64_t n, const ViewParams* views,
-                              const uint32_t* cnt, const Footprint* foot, const uint64_t* skip,
+                              const TileBox* box, const Footprint* foot, const uint64_t* skip,
                               uint32_t* flag, cudaStream_t stream) {
   if (k_total == 0) return cudaSuccess;
-  candidates_kernel<<<blocks_for(k_total, 256), 256, 0, stream>>>(k_total, n, views, cnt, foot,
+  candidates_kernel<<<blocks_for(k_total, 256), 256, 0, stream>>>(k_total, n, views, box, foot,
                                                                   skip, flag);
   return cudaGetLastError();
 }
 
 cudaError_t launch_compact(int64_t k_total, const uint32_t* flag, const uint32_t* offs,
-                           const uint32_t* key_src, uint32_t* out_key, uint32_t* out_val,
-                           cudaStream_t stream) {
+                           const ProjRecord* rec, const CompactRecord* rec16, uint32_t* out_key,
+                           uint32_t* out_val, cudaStream_t stream) {
   if (k_total == 0) return cudaSuccess;
-  compact_kernel<<<blocks_for(k_total, 256), 256, 0, stream>>>(k_total, flag, offs, key_src,
+  compact_kernel<<<blocks_for(k_total, 256), 256, 0, stream>>>(k_total, flag, offs, rec, rec16,
                                                                out_key, out_val);
   return cudaGetLastError();
 }

@@ -20,13 +20,13 @@ namespace {
 // flag[k] = 1 iff sorted slot k is visible and its Gaussian has bit `bit`.
 __global__ void __launch_bounds__(256) member_flag_kernel(
     int64_t k_total, int64_t n, const uint32_t* __restrict__ sorted_val,
-    const uint32_t* __restrict__ cnt, const uint64_t* __restrict__ member, uint64_t bit,
+    const TileBox* __restrict__ box, const uint64_t* __restrict__ member, uint64_t bit,
     uint32_t* __restrict__ flag) {
   const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k >= k_total) return;
   const uint32_t slot = sorted_val[k];
   const int64_t i = static_cast<int64_t>(slot) % n;
-  flag[k] = (cnt[slot] != 0u && (member[i] & bit) != 0ull) ? 1u : 0u;
+  flag[k] = (box_visible(box[slot]) && (member[i] & bit) != 0ull) ? 1u : 0u;
 }
 
 // out[offs[k]] = sorted_val[k] where flag[k]: the flagged slots, in order.
@@ -129,11 +129,11 @@ __global__ void __launch_bounds__(kRenderThreads) render_kernel(
 }  // namespace
 
 cudaError_t launch_member_select(int64_t k_total, int64_t n, const uint32_t* sorted_val,
-                                 const uint32_t* cnt, const uint64_t* member, uint64_t bit,
+                                 const TileBox* box, const uint64_t* member, uint64_t bit,
                                  uint32_t* flag, cudaStream_t stream) {
   if (k_total == 0) return cudaSuccess;
   member_flag_kernel<<<static_cast<unsigned>((k_total + 255) / 256), 256, 0, stream>>>(
-      k_total, n, sorted_val, cnt, member, bit, flag);
+      k_total, n, sorted_val, box, member, bit, flag);
   return cudaGetLastError();
 }
 
