@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 def _workload():
     rng = np.random.default_rng(7)
-    n = 200_003
+    n = 260_003
     sizes = [(2600, 1030)] + [(int(rng.integers(17, 200)), int(rng.integers(17, 160)))
                               for _ in range(46)]
     gauss = {"mean": rng.uniform(-1, 1, (n, 3)).astype(np.float32),
