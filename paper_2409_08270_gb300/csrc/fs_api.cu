@@ -178,7 +178,7 @@ void fs::set_last_error(const char* msg) {
 struct fs_ctx {
   int device = 0;
   int views_per_batch = 50;
-  int depth_chunks = 6;  // front-to-back chunks per batch (sizes 1/32, 1/32, 1/16, ..., 1/2)
+  int depth_chunks = 0;  // front-to-back chunks per batch (0: by the batch's size)
   int n_sm = 0;
   bool time_stages = false;
   std::vector<cudaEvent_t> events;  // (start, stop) pairs around timed stages
@@ -270,7 +270,25 @@ void fs::ctx_release_workspace(fs_ctx* c) {
 // Per-solve batching (views per batch, depth chunks), as fs_options sets them.
 void fs::ctx_set_batching(fs_ctx* c, int views_per_batch, int depth_chunks) {
   if (views_per_batch > 0) c->views_per_batch = std::min(views_per_batch, fs::kMaxViewsPerBatch);
-  if (depth_chunks > 0) c->depth_chunks = std::min(depth_chunks, 16);
+  if (depth_chunks >= 0) c->depth_chunks = std::min(depth_chunks, 16);
+}
+
+// Front-to-back depth chunks of a solve of n Gaussians (sizes 1/32, 1/32, 1/16,
+// ..., 1/2 of a batch's visible slots with six): the context's setting, or by n.
+// A chunk costs its launches, a readback and the blend's start on every tile,
+// and spares later chunks the entries of the tiles it saturates, of which there
+// are more the deeper a view's lists are.  Solve times in ms with
+// 1 | 2 | 3 | 4 | 5 | 6 | 7 | 8 chunks:
+//   50k Gaussians, 60 views 300x200      2.0   2.3   2.6   2.8   3.0   3.2   3.4   3.5
+//   300k, 24 views 512x512               3.0   3.1   3.3   3.4   3.6   3.7   3.8   3.9
+//   333k, 37 views 799x601               6.6   6.3   6.3   6.5   6.7   6.9   7.0   7.2
+//   500k, 50 views 1008x756             15.7  13.9  13.6  13.6  13.7  13.9  14.2  14.5
+//   1M, 100 views 1008x756              51.3  37.6  30.2  27.5  26.6  26.7  27.1  27.6
+//   3M, 100 views 1256x828               158   118    97  86.1  79.8  77.2  76.5  76.6
+int fs::ctx_depth_chunks(const fs_ctx* c, int64_t n) {
+  if (c->depth_chunks > 0) return std::min(c->depth_chunks, fs::kMaxChunks);
+  const double by_size = 1.0 + 2.0 * log2(static_cast<double>(std::max<int64_t>(n, 1)) / 262144.0);
+  return std::max(1, std::min(8, static_cast<int>(lround(by_size))));
 }
 
 extern "C" {
@@ -638,7 +656,8 @@ fs_status read_total(fs_ctx* c, cudaStream_t stream, int64_t* out) {
 // to ranges_dst.  Returns the entry count in *I_out.
 //
 // live: the positions are first reduced to the slots with an unsaturated tile
-// in their box (for large chunks behind saturated tiles).
+// in their box (for large chunks behind saturated tiles).  limit > 0: more
+// entries than that are left unsorted and unlisted, and *I_out is -1.
 //
 // Captured form (range_dev != NULL): the chunk's positions are read on the
 // device from range_dev[0 .. 1] (at most n_pos of them: the grid), nothing is
@@ -650,7 +669,8 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
                         const uint64_t* sat, int total_tiles, int tile_bits, int64_t kcap,
                         bool count_entries, DevBuf* val_dst, uint2* ranges_dst,
                         cudaStream_t stream, int64_t* I_out, bool live = false,
-                        const int64_t* range_dev = nullptr, int64_t plan_cap = 0) {
+                        int64_t limit = 0, const int64_t* range_dev = nullptr,
+                        int64_t plan_cap = 0) {
   unsigned long long* ctr = c->counters.as<unsigned long long>();
   *I_out = 0;
   FS_CUDA(cudaMemsetAsync(ranges_dst, 0, static_cast<size_t>(total_tiles) * 8, stream),
@@ -714,6 +734,10 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
             "binning");
     FS_TRY(stage_end(c, tb, stream));
     FS_TRY(read_total(c, stream, &I));
+    if (limit > 0 && I > limit) {
+      *I_out = -1;
+      return FS_OK;
+    }
     if (I >= (static_cast<int64_t>(1) << 31))
       return fail(FS_UNSUPPORTED, "%lld list entries in one chunk; use fewer views per batch",
                   (long long)I);
@@ -751,6 +775,9 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
 // chunk's slots lie behind saturated tiles: its last two chunks 600 and 1041
 // us without, 545 and 645 us with the bits; earlier and smaller chunks lose.
 constexpr int64_t kLiveMin = 1 << 22;
+// A chunk with more list entries than this (8 GB of lists) is halved when the
+// context chose the number of chunks.
+constexpr int64_t kSplitEntries = static_cast<int64_t>(1) << 29;
 
 // Front-to-back depth chunk boundaries of a batch of k_total sorted slots:
 // chunk ci covers positions [chunk_begin(ci), chunk_begin(ci + 1)).
@@ -827,7 +854,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   if (vb < 1) return fail(FS_UNSUPPORTED, "fs_accumulate: scene too large");
   const int64_t kcap = static_cast<int64_t>(vb) * n;
-  const int chunks = std::max(1, std::min(c->depth_chunks, fs::kMaxChunks));
+  const int chunks = fs::ctx_depth_chunks(c, n);
   FS_TRY(ensure_window(c, n, vb, V, keep));
   FS_TRY(stage_masks(c, cams, V, masks, mask_dtype, mask_memory, stream));
   if (keep) FS_TRY(kept_layout(c, cams, V, vb, chunks));
@@ -918,6 +945,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
     return FS_OK;
   };
   FS_TRY(ensure_prologue_events(c));
+  bool split = false;
   if (overlap) FS_TRY(launch_prologue(0, stream));
   for (int32_t v0 = 0, b = 0; v0 < V; v0 += vb, ++b) {
     const int nb = std::min(vb, V - v0);
@@ -1036,25 +1064,39 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
                   "plan check");
         continue;
       }
-      int64_t I = 0;
-      const bool live = ci > 0 && n_pos >= kLiveMin && 5 * n_pos >= k_total;
-      FS_TRY(bin_positions(c, p0, n_pos, n, vd, nb, sorted_val, P, sat, total_tiles, tile_bits, kcap,
-                           !plan, val_dst, ranges_dst, stream, &I, live,
-                           plan ? c->chunk_bnd.as<int64_t>() + ci : nullptr,
-                           plan ? plan->entries[pi] : 0));
-      if (record) record->entries[pi] = I;
+      // a chunk of the context's own choosing is halved while it has too many
+      // entries (its parts are not kept for the re-check, which then bins anew)
+      for (int64_t a0 = p0, a1 = p0 + n_pos; a0 < p0 + n_pos;) {
+        const int64_t n_part = a1 - a0;
+        const int64_t limit =
+            c->depth_chunks == 0 && !plan && !record && n_part > 1 ? kSplitEntries : 0;
+        const bool live = ci > 0 && n_part >= kLiveMin && 5 * n_part >= k_total;
+        int64_t I = 0;
+        FS_TRY(bin_positions(c, a0, n_part, n, vd, nb, sorted_val, P, sat, total_tiles, tile_bits,
+                             kcap, !plan, val_dst, ranges_dst, stream, &I, live, limit,
+                             plan ? c->chunk_bnd.as<int64_t>() + ci : nullptr,
+                             plan ? plan->entries[pi] : 0));
+        if (I < 0) {
+          a1 = a0 + n_part / 2;
+          split = true;
+          continue;
+        }
+        if (record) record->entries[pi] = I;
+        a0 = a1;
+        a1 = p0 + n_pos;
+        if (I == 0) continue;
+        int tb = -1;
+        FS_TRY(stage_begin(c, FS_STAGE_BLEND, stream, plan != nullptr, &tb));
+        FS_CUDA(fs::launch_blend(vd, nb, max_tiles, ranges_dst, val_dst->as<uint32_t>(), P.rec,
+                                 P.rec16, n, E, mask_dtype, table, table_dtype, state, sat, subsat,
+                                 satc, ci, ctr, c->census, stream),
+                "blend");
+        FS_TRY(stage_end(c, tb, stream));
+      }
       p0 = p1;
-      if (I == 0) continue;
-      int tb = -1;
-      FS_TRY(stage_begin(c, FS_STAGE_BLEND, stream, plan != nullptr, &tb));
-      FS_CUDA(fs::launch_blend(vd, nb, max_tiles, ranges_dst, val_dst->as<uint32_t>(), P.rec,
-                               P.rec16, n, E, mask_dtype, table, table_dtype, state, sat, subsat,
-                               satc, ci, ctr, c->census, stream),
-              "blend");
-      FS_TRY(stage_end(c, tb, stream));
     }
   }
-  c->kl_valid = keep;
+  c->kl_valid = keep && !split;
   return FS_OK;
 }
 
@@ -1705,11 +1747,19 @@ fs_status fs_graph_create(fs_ctx* tmpl, const fs_scene* s, const fs_camera* cams
   // 1. a solve that records the shapes and sizes every buffer
   c->stats = fs_stats{};
   ce = cudaMemsetAsync(c->counters.p, 0, c->counters.bytes, g->stream);
-  if (ce == cudaSuccess) ce = cudaMemsetAsync(g->table, 0, nn * E * 8, g->stream);
   if (ce != cudaSuccess) return bail(cuda_fail(ce, "fs_graph_create"));
-  if ((st = accumulate_impl(c, s, cams, V, masks, mask_dtype, FS_MEM_DEVICE, E, g->table, FS_F64,
-                            g->keep, g->stream, &g->plan, nullptr)) != FS_OK)
-    return bail(st);
+  auto record = [&]() -> fs_status {
+    FS_CUDA(cudaMemsetAsync(g->table, 0, nn * E * 8, g->stream), "table clear");
+    return accumulate_impl(c, s, cams, V, masks, mask_dtype, FS_MEM_DEVICE, E, g->table, FS_F64,
+                           g->keep, g->stream, &g->plan, nullptr);
+  };
+  st = record();
+  if (st == FS_UNSUPPORTED && c->depth_chunks == 0) {
+    // too many entries for the chunks its size suggests: the most there are
+    c->depth_chunks = fs::kMaxChunks;
+    st = record();
+  }
+  if (st != FS_OK) return bail(st);
   if ((ce = cudaStreamSynchronize(g->stream)) != cudaSuccess)
     return bail(cuda_fail(ce, "fs_graph_create"));
   const int vb = batch_views(c, n);

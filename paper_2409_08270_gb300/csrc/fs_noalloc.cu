@@ -238,23 +238,32 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
     NA_CUDA(cudaMemsetAsync(subsat, 0, static_cast<size_t>((4 * tiles + 63) / 64) * 8, strm),
             "clear");
     NA_CUDA(launch_state_init(vd, 1, tiles, E, mask_dtype, state, sat, subsat, ctr, strm), "state");
+    // One list per view where its entries fit; where they do not, the next of
+    // six front-to-back depth chunks, whose saturated tiles the rest passes
+    // over.  (12,000 Gaussians, four 384x384 views: 2.57 ms in six chunks a view,
+    // 1.00 ms in one.)
     const int chunks = 6;
     int64_t p0 = 0;
-    for (int ci = 0; ci < chunks; ++ci) {
-      const int64_t p1 = (ci == chunks - 1) ? n : (n >> (chunks - 1 - ci));
-      const int64_t n_pos = p1 - p0;
-      if (n_pos <= 0) continue;
-      NA_CUDA(launch_bin_fused(p0, n_pos, n, vd, 1, sval, foot, sat, lk_a, lv_a,
-                               static_cast<uint32_t>(kNA_Entries), lookback, total_d, ctr, strm,
-                               nullptr),
-              "binning");
+    while (p0 < n) {
+      int64_t p1 = n;
       uint32_t I = 0;
-      NA_CUDA(cudaMemcpyAsync(&I, total_d, 4, cudaMemcpyDeviceToHost, strm), "readback");
-      NA_CUDA(cudaStreamSynchronize(strm), "readback");
-      if (I > static_cast<uint32_t>(kNA_Entries))
-        return na_fail(FS_UNSUPPORTED,
-                       "fs_solve_noalloc: a view needs more than FS_NOALLOC_MAX_LIST_ENTRIES "
-                       "(tile, Gaussian) pairs in one depth chunk; the table is incomplete");
+      for (;;) {
+        NA_CUDA(launch_bin_fused(p0, p1 - p0, n, vd, 1, sval, foot, sat, lk_a, lv_a,
+                                 static_cast<uint32_t>(kNA_Entries), lookback, total_d, ctr, strm,
+                                 nullptr),
+                "binning");
+        NA_CUDA(cudaMemcpyAsync(&I, total_d, 4, cudaMemcpyDeviceToHost, strm), "readback");
+        NA_CUDA(cudaStreamSynchronize(strm), "readback");
+        if (I <= static_cast<uint32_t>(kNA_Entries)) break;
+        int ci = 0;  // the chunk p0 lies in ends at n >> (chunks - 1 - ci)
+        while (ci < chunks - 1 && (n >> (chunks - 1 - ci)) <= p0) ++ci;
+        const int64_t end = ci == chunks - 1 ? n : n >> (chunks - 1 - ci);
+        if (p1 == end)
+          return na_fail(FS_UNSUPPORTED,
+                         "fs_solve_noalloc: a view needs more than FS_NOALLOC_MAX_LIST_ENTRIES "
+                         "(tile, Gaussian) pairs in one depth chunk; the table is incomplete");
+        p1 = end;
+      }
       if (I > 0) {
         bool alt2 = false;
         NA_CUDA(radix_sort_pairs(lk_a, lv_a, lk_b, lv_b, I, bits_for(tiles), sort_tmp, &alt2, strm,

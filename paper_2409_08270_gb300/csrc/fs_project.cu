@@ -677,7 +677,8 @@ constexpr unsigned long long kLbPrefix = 2ull << 32;  // word holds the inclusiv
 constexpr int kBinThreads = 128, kBinWarps = kBinThreads / 32;
 
 // Decoupled look-back by one warp: the sum of the counts of blocks 0 .. vb - 1,
-// 32 predecessors at a time (lane l reads block vb - 1 - l).
+// 32 predecessors at a time (lane l reads block vb - 1 - l).  Sums stop at
+// 2^32 - 1, so a list that is too long is seen as such.
 __device__ __forceinline__ uint32_t look_back(const unsigned long long* status, uint32_t vb,
                                               unsigned long long* counters, int spin_limit,
                                               int lane) {
@@ -701,11 +702,18 @@ __device__ __forceinline__ uint32_t look_back(const unsigned long long* status, 
     }
     const uint32_t pre = __ballot_sync(0xffffffffu, (word & ~0xFFFFFFFFull) == kLbPrefix);
     const int first = pre ? __ffs(pre) - 1 : 31;  // nearest predecessor holding a prefix
-    excl += __reduce_add_sync(0xffffffffu,
-                              lane <= first ? static_cast<uint32_t>(word & 0xFFFFFFFFull) : 0u);
+    const uint32_t v = lane <= first ? static_cast<uint32_t>(word & 0xFFFFFFFFull) : 0u;
+    const uint64_t sum =
+        excl + __reduce_add_sync(0xffffffffu, v & 0xFFFFu) +
+        (static_cast<uint64_t>(__reduce_add_sync(0xffffffffu, v >> 16)) << 16);
+    excl = static_cast<uint32_t>(min(sum, static_cast<uint64_t>(0xFFFFFFFFu)));
     if (pre) break;
   }
   return excl;
+}
+
+__device__ __forceinline__ uint32_t add_sat(uint32_t a, uint32_t b) {
+  return a + b < a ? 0xFFFFFFFFu : a + b;
 }
 
 template <bool kDeviceRange>
@@ -783,9 +791,9 @@ __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
     if (lane == 0) atomicExch(&status[vb], (vb == 0 ? kLbPrefix : kLbCount) | btot);
     const uint32_t excl = look_back(status, vb, counters, spin_limit, lane);
     if (lane == 0) {
-      if (vb > 0) atomicExch(&status[vb], kLbPrefix | (excl + btot));
+      if (vb > 0) atomicExch(&status[vb], kLbPrefix | add_sat(excl, btot));
       s_boff = excl;
-      if (static_cast<int64_t>(vb + 1) * kBinThreads >= n_pos) *total = excl + btot;
+      if (static_cast<int64_t>(vb + 1) * kBinThreads >= n_pos) *total = add_sat(excl, btot);
     }
   }
   __syncthreads();

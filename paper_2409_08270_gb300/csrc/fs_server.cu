@@ -50,7 +50,7 @@ struct SceneEntry {
   fs_scene* scene = nullptr;
   int64_t n = 0;
   bool tuned = false;
-  int views_per_batch = 50, depth_chunks = 6;
+  int views_per_batch = 50, depth_chunks = 0;  // 0 chunks: by the size
   std::mutex tune_mu;
   // graphs on: a captured solve of the scene's last (cameras, E, gamma, mask
   // dtype), its device mask buffers and outputs; one replay at a time
@@ -300,7 +300,7 @@ void worker(fs_server* s, int slot) {
     }
     fs::ctx_set_batching(s->ctx[slot], se->views_per_batch, se->depth_chunks);
     r->info.views_per_batch = se->views_per_batch;
-    r->info.depth_chunks = se->depth_chunks;
+    r->info.depth_chunks = fs::ctx_depth_chunks(s->ctx[slot], se->n);
     const fs_status st =
         s->max_graphs > 0
             ? solve_with_graph(s, slot, *se, r, &r->info.stats)
