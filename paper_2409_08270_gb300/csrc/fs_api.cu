@@ -198,7 +198,7 @@ struct fs_ctx {
   bool census = false;   // blend counts its pairs (slower variant)
   bool sigma3 = false;   // 3-sigma tile coverage (per-slot tile columns in `cols`)
   DevBuf rk_flag, rk_offs, rk_F, rk_map, rk_R, rk_Rb, rk_tiles, cols;
-  DevBuf rd_flag, rd_offs, rd_val, render_out;  // novel-view mask rendering
+  DevBuf rd_val, render_out;  // novel-view mask rendering
   DevBuf chunk_bnd;                             // captured solves: chunk boundaries
   HostBuf render_out_host;
   DevBuf key_range;  // min / max visible depth key of the batch (two slots, by batch parity)
@@ -238,7 +238,7 @@ DevBuf* const* workspace_bufs(fs_ctx* c, size_t* count) {
                     &c->label_tmp, &c->margin_tmp, &c->rk_flag, &c->rk_offs,
                     &c->rk_F, &c->rk_map, &c->rk_R, &c->rk_Rb, &c->rk_tiles, &c->kl_ranges, &c->kl_satc,
                     &c->kl_bound, &c->key_range, &c->lb_tmp, &c->key_a2, &c->val_a2,
-                    &c->key_b2, &c->val_b2, &c->cols, &c->rd_flag, &c->rd_offs, &c->rd_val,
+                    &c->key_b2, &c->val_b2, &c->cols, &c->rd_val,
                     &c->render_out, &c->chunk_bnd, &c->free_tab, &c->live, &c->live_val,
                     &c->live_range};
   for (DevBuf* b : list) bufs[k++] = b;
@@ -365,7 +365,7 @@ fs_status fs_destroy(fs_ctx* c) {
                     &c->rk_Rb, &c->rk_tiles, &c->kl_ranges, &c->kl_satc, &c->kl_bound, &c->key_range,
                     &c->lb_tmp,
                     &c->key_a2, &c->val_a2, &c->key_b2, &c->val_b2, &c->cols,
-                    &c->rd_flag, &c->rd_offs, &c->rd_val, &c->render_out, &c->chunk_bnd,
+                    &c->rd_val, &c->render_out, &c->chunk_bnd,
                     &c->free_tab, &c->live, &c->live_val, &c->live_range};
   for (DevBuf& b : c->kl_val) b.release();
   for (DevBuf* b : bufs) b->release();
@@ -655,6 +655,7 @@ fs_status read_total(fs_ctx* c, cudaStream_t stream, int64_t* out) {
 // sorted list values go to *val_dst (grown as needed) and the per-tile ranges
 // to ranges_dst.  Returns the entry count in *I_out.
 //
+// range (may be NULL): the positions' bounds in device memory (at most n_pos).
 // live: the positions are first reduced to the slots with an unsaturated tile
 // in their box (for large chunks behind saturated tiles).  limit > 0: more
 // entries than that are left unsorted and unlisted, and *I_out is -1.
@@ -668,8 +669,8 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
                         const ProjPtrs& P,
                         const uint64_t* sat, int total_tiles, int tile_bits, int64_t kcap,
                         bool count_entries, DevBuf* val_dst, uint2* ranges_dst,
-                        cudaStream_t stream, int64_t* I_out, bool live = false,
-                        int64_t limit = 0, const int64_t* range_dev = nullptr,
+                        cudaStream_t stream, int64_t* I_out,
+                        const int64_t* range = nullptr, bool live = false, int64_t limit = 0, const int64_t* range_dev = nullptr,
                         int64_t plan_cap = 0) {
   unsigned long long* ctr = c->counters.as<unsigned long long>();
   *I_out = 0;
@@ -680,7 +681,7 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
   int tl = -1;
   FS_TRY(stage_begin(c, FS_STAGE_BINNING, stream, range_dev != nullptr, &tl));
   FS_CUDA(fs::launch_free_tables(vd, nb, sat, stream), "tile prefix tables");
-  const int64_t* range = range_dev;  // what the binning reads its positions from
+  if (range_dev) range = range_dev;
   if (live) {
     int64_t* const rng = c->live_range.as<int64_t>();
     uint32_t* const slots = c->live_val.as<uint32_t>();
@@ -891,7 +892,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
     FS_TRY(c->live.ensure(static_cast<size_t>(fs::live_words(n)) * vb * 4, "slot bits"));
     // chunks but the first hold at most half the slots (and one)
     FS_TRY(c->live_val.ensure(static_cast<size_t>(kcap / 2 + 1) * 4, "live slots"));
-    FS_TRY(c->live_range.ensure(16, "live slot range"));
+    FS_TRY(c->live_range.ensure(256, "live slot range"));
   }
   struct Prologue {
     BatchLayout L;
@@ -1073,7 +1074,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
         const bool live = ci > 0 && n_part >= kLiveMin && 5 * n_part >= k_total;
         int64_t I = 0;
         FS_TRY(bin_positions(c, a0, n_part, n, vd, nb, sorted_val, P, sat, total_tiles, tile_bits,
-                             kcap, !plan, val_dst, ranges_dst, stream, &I, live, limit,
+                             kcap, !plan, val_dst, ranges_dst, stream, &I, nullptr, live, limit,
                              plan ? c->chunk_bnd.as<int64_t>() + ci : nullptr,
                              plan ? plan->entries[pi] : 0));
         if (I < 0) {
@@ -1337,10 +1338,9 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
   const int64_t kcap = static_cast<int64_t>(vb) * n;
   FS_TRY(ensure_window(c, n, vb, V, false));
   FS_TRY(c->key_range.ensure(32, "depth key range"));
-  FS_TRY(c->rd_flag.ensure(static_cast<size_t>(kcap) * 4, "render flags"));
-  FS_TRY(c->rd_offs.ensure(static_cast<size_t>(kcap) * 4, "render offsets"));
   FS_TRY(c->rd_val.ensure(static_cast<size_t>(kcap) * 4, "render slots"));
-  FS_TRY(c->scan_tmp.ensure(fs::scan_temp_bytes(kcap), "scan temp"));
+  FS_TRY(c->lb_tmp.ensure(fs::bin_fused_temp_bytes(kcap), "look-back"));
+  FS_TRY(c->live_range.ensure(256, "slot range"));
   const size_t ro_bytes = sizeof(fs::RenderOut) * fs::kMaxViewsPerBatch;
   FS_TRY(c->render_out.ensure(ro_bytes, "render outputs"));
   FS_TRY(c->render_out_host.ensure(ro_bytes));
@@ -1400,22 +1400,15 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
     FS_TRY(c->state.ensure(static_cast<size_t>(L.pixels) * 4, "pixel state"));
     FS_CUDA(cudaMemsetAsync(c->sat.p, 0, sat_bytes, stream), "tile flags clear");
     for (int e = 1; e < E; ++e) {
-      uint32_t* flag = c->rd_flag.as<uint32_t>();
-      FS_CUDA(fs::launch_member_select(k_vis, n, sorted_val, P.box, member_bits, 1ull << e, flag,
-                                       stream),
+      int64_t* const rng = c->live_range.as<int64_t>();
+      FS_CUDA(fs::launch_member_slots(k_vis, n, sorted_val, member_bits, 1ull << e,
+                                      c->rd_val.as<uint32_t>(), rng, c->lb_tmp.p,
+                                      c->counters.as<unsigned long long>(), stream),
               "object slots");
-      FS_CUDA(fs::exclusive_scan(flag, nullptr, c->rd_offs.as<uint32_t>(), k_vis,
-                                 c->total.as<uint32_t>(), c->scan_tmp.p, stream),
-              "object scan");
-      FS_CUDA(fs::launch_member_scatter(k_vis, flag, c->rd_offs.as<uint32_t>(), sorted_val,
-                                        c->rd_val.as<uint32_t>(), stream),
-              "object scatter");
-      int64_t count = 0;
-      FS_TRY(read_total(c, stream, &count));
       int64_t I = 0;
-      FS_TRY(bin_positions(c, 0, count, n, vd, nb, c->rd_val.as<uint32_t>(), P,
+      FS_TRY(bin_positions(c, 0, k_vis, n, vd, nb, c->rd_val.as<uint32_t>(), P,
                            c->sat.as<uint64_t>(), total_tiles, tile_bits, kcap, false, &c->lv_a,
-                           c->ranges.as<uint2>(), stream, &I));
+                           c->ranges.as<uint2>(), stream, &I, rng));
       FS_CUDA(fs::launch_render(vd, rod, nb, max_tiles, c->ranges.as<uint2>(),
                                 c->lv_a.as<uint32_t>(), P.rec, P.rec16, e, e == 1, tau,
                                 c->state.as<float>(), out_dtype, stream),
@@ -1597,21 +1590,22 @@ fs_status fs_keep_after_removal(fs_ctx* c, const uint64_t* member_bits, int64_t 
   if (n == 0) return FS_OK;
   DeviceGuard g(c->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const size_t nn = static_cast<size_t>(n);
-  FS_TRY(c->rk_flag.ensure(nn * 4, "removal flags"));
-  FS_TRY(c->rk_offs.ensure(nn * 4, "removal offsets"));
-  FS_TRY(c->scan_tmp.ensure(fs::scan_temp_bytes(n), "scan temp"));
-  FS_CUDA(fs::launch_keep_flags(n, member_bits, remove, c->rk_flag.as<uint32_t>(), st),
-          "removal flags");
-  FS_CUDA(fs::exclusive_scan(c->rk_flag.as<uint32_t>(), nullptr, c->rk_offs.as<uint32_t>(), n,
-                             c->total.as<uint32_t>(), c->scan_tmp.p, st),
-          "removal scan");
-  FS_CUDA(fs::launch_keep_scatter(n, c->rk_flag.as<uint32_t>(), c->rk_offs.as<uint32_t>(),
-                                  keep_index, st),
-          "removal scatter");
-  c->stats.kernel_launches += 2 + scan_launches(n);
-  int64_t kept = 0;
-  FS_TRY(read_total(c, st, &kept));
+  FS_TRY(c->lb_tmp.ensure(fs::bin_fused_temp_bytes(n), "look-back"));
+  FS_TRY(c->live_range.ensure(256, "removal count"));
+  // the count's range and counters of this call's own, read back together
+  int64_t* const rng = c->live_range.as<int64_t>();
+  unsigned long long* const ctr = reinterpret_cast<unsigned long long*>(rng + 2);
+  const size_t back = 16 + sizeof(unsigned long long) * fs::kNumCounters;
+  FS_CUDA(cudaMemsetAsync(ctr, 0, back - 16, st), "counters clear");
+  FS_CUDA(fs::launch_keep(n, member_bits, remove, keep_index, rng, c->lb_tmp.p, ctr, st),
+          "removal");
+  c->stats.kernel_launches += 1;
+  int64_t* const h = reinterpret_cast<int64_t*>(c->total_host.as<char>() + 64);
+  FS_CUDA(cudaMemcpyAsync(h, rng, back, cudaMemcpyDeviceToHost, st), "removal count");
+  FS_CUDA(cudaStreamSynchronize(st), "removal count");
+  if (reinterpret_cast<const unsigned long long*>(h + 2)[fs::kLookbackTimeout])
+    return fail(FS_TIMEOUT, "fs_keep_after_removal: a bounded wait gave up");
+  const int64_t kept = h[1];
   *n_keep = kept;
   return FS_OK;
 }

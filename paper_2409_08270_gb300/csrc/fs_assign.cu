@@ -9,6 +9,7 @@
 // the table's precision.
 #include <math.h>
 
+#include "fs_compact.cuh"
 #include "fs_internal.h"
 
 namespace fs {
@@ -157,39 +158,22 @@ __global__ void __launch_bounds__(256) assign_rows_kernel(
   if (margin) margin[i] = d.margin;
 }
 
-// flag[i] = 1 iff Gaussian i belongs to none of the objects in `remove`
-__global__ void __launch_bounds__(256) keep_flag_kernel(int64_t n,
-                                                        const uint64_t* __restrict__ bits,
-                                                        uint64_t remove,
-                                                        uint32_t* __restrict__ flag) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) flag[i] = (bits[i] & remove) ? 0u : 1u;
-}
-
-__global__ void __launch_bounds__(256) keep_scatter_kernel(int64_t n,
-                                                           const uint32_t* __restrict__ flag,
-                                                           const uint32_t* __restrict__ offs,
-                                                           int32_t* __restrict__ keep) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n && flag[i]) keep[offs[i]] = static_cast<int32_t>(i);
-}
+// The Gaussians in none of the objects of `remove`.
+struct KeptGaussians {
+  const uint64_t* bits;
+  uint64_t remove;
+  __device__ __forceinline__ uint32_t value(int64_t p) const { return static_cast<uint32_t>(p); }
+  __device__ __forceinline__ bool keep(uint32_t i) const { return (bits[i] & remove) == 0ull; }
+};
 
 }  // namespace
 
-cudaError_t launch_keep_flags(int64_t n, const uint64_t* member_bits, uint64_t remove,
-                              uint32_t* flag, cudaStream_t stream) {
-  if (n == 0) return cudaSuccess;
-  keep_flag_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(n, member_bits,
-                                                                              remove, flag);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_keep_scatter(int64_t n, const uint32_t* flag, const uint32_t* offs,
-                                int32_t* keep, cudaStream_t stream) {
-  if (n == 0) return cudaSuccess;
-  keep_scatter_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(n, flag, offs,
-                                                                                 keep);
-  return cudaGetLastError();
+cudaError_t launch_keep(int64_t n, const uint64_t* member_bits, uint64_t remove, int32_t* keep,
+                        int64_t* range_out, void* lookback, unsigned long long* counters,
+                        cudaStream_t stream) {
+  return launch_compact(KeptGaussians{member_bits, remove}, 0, n,
+                        reinterpret_cast<uint32_t*>(keep), range_out, lookback, counters, stream,
+                        nullptr);
 }
 
 cudaError_t launch_assign(const void* table, int table_dtype, int64_t n, int E, float gamma,

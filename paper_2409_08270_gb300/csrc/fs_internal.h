@@ -156,12 +156,12 @@ cudaError_t launch_assign(const void* table, int table_dtype, int64_t n, int E, 
                           uint64_t* member_bits, int32_t* label, float* margin,
                           cudaStream_t stream);
 
-// Object removal (Sec. 4.4): flag[i] = no bit of `remove` set in member_bits[i];
-// keep[offs[i]] = i for flagged i (offs: exclusive scan of flag).
-cudaError_t launch_keep_flags(int64_t n, const uint64_t* member_bits, uint64_t remove,
-                              uint32_t* flag, cudaStream_t stream);
-cudaError_t launch_keep_scatter(int64_t n, const uint32_t* flag, const uint32_t* offs,
-                                int32_t* keep, cudaStream_t stream);
+// Object removal (Sec. 4.4): the indices of the Gaussians with no bit of
+// `remove` in member_bits, in order, to keep, and {0, their number} to range_out
+// (device).  lookback: bin_fused_temp_bytes(n) of scratch.
+cudaError_t launch_keep(int64_t n, const uint64_t* member_bits, uint64_t remove, int32_t* keep,
+                        int64_t* range_out, void* lookback, unsigned long long* counters,
+                        cudaStream_t stream);
 
 // dst[i] = (float) src[i], i < count
 cudaError_t launch_round_table(int64_t count, const double* src, float* dst, cudaStream_t stream);
@@ -236,13 +236,13 @@ struct RenderOut {
   float* rho;
   float* depth;
 };
-// flag[k] = 1 iff sorted slot k is visible and member[slot % n] & bit
-cudaError_t launch_member_select(int64_t k_total, int64_t n, const uint32_t* sorted_val,
-                                 const TileBox* box, const uint64_t* member, uint64_t bit,
-                                 uint32_t* flag, cudaStream_t stream);
-// out[offs[k]] = sorted_val[k] for flagged k (order kept)
-cudaError_t launch_member_scatter(int64_t k_total, const uint32_t* flag, const uint32_t* offs,
-                                  const uint32_t* sorted_val, uint32_t* out, cudaStream_t stream);
+// The sorted slots [0, n_pos) whose Gaussian has `bit` in member, in order, to
+// out, and {0, their number} to range_out (device).  lookback:
+// bin_fused_temp_bytes(n_pos) of scratch.
+cudaError_t launch_member_slots(int64_t n_pos, int64_t n, const uint32_t* sorted_val,
+                                const uint64_t* member, uint64_t bit, uint32_t* out,
+                                int64_t* range_out, void* lookback, unsigned long long* counters,
+                                cudaStream_t stream);
 // Object e's tile lists composited per pixel and folded into the masks:
 // rho^e > tau and D^e below best[] (per batch pixel, at state_off) takes label
 // e; first != 0 starts every pixel at label 0 and best = +inf.
