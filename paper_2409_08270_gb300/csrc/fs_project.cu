@@ -22,6 +22,8 @@
 // so far fewer tiles are listed than with the bounding box.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "fs_binning.cuh"
 #include "fs_common.cuh"
 #include "fs_compact.cuh"
@@ -113,31 +115,17 @@ __device__ __forceinline__ f2 f2_clamp(f2 x, float lim_hi, float lim_lo) {
   return x;
 }
 
-// x rounded to FP16 (round to nearest, ties to even), x a float pair: the
-// float rounding of hi is corrected when hi sits exactly halfway between two
-// FP16 values and lo says on which side x lies.
-__device__ __forceinline__ uint16_t f2_to_half_rn(f2 x) {
-  const __half h = __float2half_rn(x.hi);
-  const float hf = __half2float(h);
-  if (x.lo == 0.f || hf == x.hi) return __half_as_ushort(h);
-  // the FP16 neighbour on the other side of hi
-  const uint16_t hb = __half_as_ushort(h);
-  const bool up_in_magnitude = (fabsf(x.hi) > fabsf(hf));
-  const uint16_t ob = static_cast<uint16_t>(up_in_magnitude ? hb + 1 : hb - 1);
-  const float of = __half2float(__ushort_as_half(ob));
-  if (0.5f * (hf + of) != x.hi) return hb;  // not a tie: hi's rounding is x's
-  // tie on hi alone: x lies towards lo's side
-  const bool towards_other = (x.lo > 0.f) == (of > hf);
-  return towards_other ? ob : hb;
-}
-
-// One thread per Gaussian; it projects the Gaussian into every view of the
-// batch so the scene is read once per batch.  rec16 != NULL: the record is
+// One thread per Gaussian; it projects the Gaussian into the views of its block's
+// share (all of them for large scenes, so the scene is read once per batch;
+// small scenes spread the views over the grid's second dimension).  rec16 != NULL: the record is
 // written in the reduced-precision form instead (rec is not written).  The
 // paired float-pair quantities (the two rows of the Jacobian-rotation product,
 // the two rows of T Sigma3D, the x and y halves of the pinhole map, the rows
 // of W) run in packed FP32 (f2x2), bit-identical to the scalar form.  Three
-// blocks per SM (80 registers) spill less than four.
+// blocks per SM (80 registers) spill less than four.  Bound by issue (about
+// 1,100 instructions a slot): one reciprocal and four roots, seeded by the
+// hardware's, where six correctly rounded float-pair divisions and four roots
+// stood, take 10^6 Gaussians in 100 views from 4.44 to 3.74 ms.
 template <bool kFast>
 __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
     int64_t n, int n_views, const ViewParams* __restrict__ views_g,
@@ -163,7 +151,9 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
   const float r2 = opaque_enough ? fmaxf(2.f * logf(255.f * o), 0.f) : 0.f;
   const float nlo = opaque_enough ? -log2f(o) : 0.f;  // alpha = 2^-(|w|^2 - log2 o)
 
-  for (int v = 0; v < n_views; ++v) {
+  // the block's share of the views
+  const int v_end = static_cast<int>((blockIdx.y + 1) * n_views / gridDim.y);
+  for (int v = static_cast<int>(blockIdx.y * n_views / gridDim.y); v < v_end; ++v) {
     const ViewParams& vp = views[v];
     const int64_t slot = static_cast<int64_t>(v) * n + i;
     const f2x2 txy = f2x2_dot3_add(vp.R_hi + 0, vp.R_lo + 0, vp.R_hi + 3, vp.R_lo + 3, po.x, po.y,
@@ -259,7 +249,7 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
         det32 = dt;
       } else {
         // one float-pair reciprocal of the depth, then (x, y) / z side by side
-        const f2 iz = f2_div(f2_from(1.f), tz);
+        const f2 iz = f2_rcp(tz);
         const f2x2 uxy = f2x2_mul(f2x2_pack(tx, ty), f2x2_pack(iz, iz));
         const f2 ux = f2x2_first(uxy), uy = f2x2_second(uxy);
         const f2 fx = {vp.fx_hi, vp.fx_lo}, fy = {vp.fy_hi, vp.fy_lo};
@@ -271,7 +261,6 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
         depth = tz.hi;
         depth_l = tz.lo;
         R.misc.w = depth;
-        R16.depth = depth;
         const f2x2 J = f2x2_mul(fxy, f2x2_pack(iz, iz));  // (fx / z, fy / z)
         const f2 uxc = f2_clamp(ux, vp.limx_hi, vp.limx_lo);
         const f2 uyc = f2_clamp(uy, vp.limy_hi, vp.limy_lo);
@@ -305,7 +294,6 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
         const f2 h = f2_scale(f2_sub(a, c), 0.5f);
         const f2 rr = f2_sqrt(f2_add(f2_mul(h, h), f2_mul(b, b)));
         const f2 lam1 = f2_add(f2_scale(f2_add(a, c), 0.5f), rr);
-        const f2 lam2 = f2_div(det, lam1);
         // unit eigenvector of lambda1 from whichever form has no cancellation
         f2 ex, ey;
         if (h.hi >= 0.f) {
@@ -315,36 +303,33 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
           ex = b;
           ey = f2_sub(rr, h);
         }
-        const f2 en = f2_sqrt(f2_add(f2_mul(ex, ex), f2_mul(ey, ey)));
-        if (en.hi > 0.f) {
-          const f2 ien = f2_div(f2_from(1.f), en);
-          const f2x2 e = f2x2_mul(f2x2_pack(ex, ey), f2x2_pack(ien, ien));
-          ex = f2x2_first(e);
-          ey = f2x2_second(e);
+        const f2 en2 = f2_add(f2_mul(ex, ex), f2_mul(ey, ey));
+        f2 ien = f2_from(1.f);
+        if (en2.hi > kRootMin) {
+          ien = f2_rsqrt(en2);
         } else {
           ex = f2_from(1.f);
           ey = f2_from(0.f);
         }
         // axis scales sqrt(0.5 log2 e / lambda) as float pairs too: the FP64
-        // near-tie re-check evaluates alpha from this record
-        const f2 hl = {kHalfLog2eHi, kHalfLog2eLo};
-        const f2 k1 = f2_sqrt(f2_div(hl, lam1));
-        const f2 k2 = f2_sqrt(f2_div(hl, lam2));
-        const f2x2 W0 = f2x2_mul(f2x2_pack(ex, ey), f2x2_pack(k1, k1));
-        const f2x2 W1 = f2x2_mul(f2x2_pack(f2_neg(ey), ex), f2x2_pack(k2, k2));
+        // near-tie re-check evaluates alpha from this record.  With lambda2 =
+        // det / lambda1 they are c / sqrt(lambda1) and c sqrt(lambda1) /
+        // sqrt(det), c = sqrt(0.5 log2 e); the eigenvector's norm goes in too.
+        const f2 root_hl = {static_cast<float>(kRootHalfLog2e),
+                            static_cast<float>(kRootHalfLog2e -
+                                               static_cast<double>(static_cast<float>(kRootHalfLog2e)))};
+        const f2 r1 = f2_rsqrt(lam1);
+        const f2 rd = det.hi > 0.f ? f2_rsqrt(det) : f2_from(0.f);
+        const f2 is = f2_mul(ien, root_hl);
+        const f2x2 sc = f2x2_mul(f2x2_pack(r1, f2_mul(f2_mul(lam1, r1), rd)), f2x2_pack(is, is));
+        const f2 s1 = f2x2_first(sc), s2 = f2x2_second(sc);
+        const f2x2 W0 = f2x2_mul(f2x2_pack(ex, ey), f2x2_pack(s1, s1));
+        const f2x2 W1 = f2x2_mul(f2x2_pack(f2_neg(ey), ex), f2x2_pack(s2, s2));
         const f2 W00 = f2x2_first(W0), W01 = f2x2_second(W0);
         const f2 W10 = f2x2_first(W1), W11 = f2x2_second(W1);
         R.w_hi = make_float4(W00.hi, W01.hi, W10.hi, W11.hi);
         R.w_lo = make_float4(W00.lo, W01.lo, W10.lo, W11.lo);
         R.m = make_float4(mx.hi, my.hi, mx.lo, my.lo);
-        if (rec16) {
-          R16.mx = mx.hi;  // the float pair is normalised: hi is the FP32 rounding
-          R16.my = my.hi;
-          R16.w01 = static_cast<uint32_t>(f2_to_half_rn(W00)) |
-                    (static_cast<uint32_t>(f2_to_half_rn(W01)) << 16);
-          R16.w23 = static_cast<uint32_t>(f2_to_half_rn(W10)) |
-                    (static_cast<uint32_t>(f2_to_half_rn(W11)) << 16);
-        }
         sxx = a.hi;
         sxy = b.hi;
         syy = c.hi;
@@ -357,16 +342,17 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
       F.mx = mx32;
       F.my = my32;
       F.syr = syy * r2b;
-      F.hy = sqrtf(F.syr);
-      F.dys = sxy * sqrtf(r2b / sxx);
-      F.a = sxy / syy;
-      F.b2 = det32 / (syy * syy);
+      F.hy = sqrt_approx(F.syr);
+      F.dys = sxy * sqrt_approx(r2b * rcp_approx(sxx));
+      const float isyy = rcp_approx(syy);
+      F.a = sxy * isyy;
+      F.b2 = det32 * isyy * isyy;
       const float hy = F.hy;
       const float py0 = ceilf(__fsub_rn(__fsub_rn(F.my, hy), 1.5f));
       const float py1 = floorf(__fadd_rn(__fadd_rn(F.my, hy), 0.5f));
       // visible when the widened bounding box meets the image; the exact
       // per-row tile spans are counted later, per depth chunk
-      const float hx = sqrtf(sxx * r2b);
+      const float hx = sqrt_approx(sxx * r2b);
       const float px0 = ceilf(__fsub_rn(__fsub_rn(F.mx, hx), 1.5f));
       const float px1 = floorf(__fadd_rn(__fadd_rn(F.mx, hx), 0.5f));
       if (!(py1 >= 0.f && py0 <= vp.height - 1 && px1 >= 0.f && px0 <= vp.width - 1)) {
@@ -419,7 +405,7 @@ __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
     }
     if (vp.cols) vp.cols[slot] = col_clip;
     if (visible) {  // records are read only through tile lists, which hold visible slots
-      if (rec16)
+      if constexpr (kFast)
         rec16[slot] = R16;
       else
         rec[slot] = R;
@@ -940,13 +926,16 @@ cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, cons
   if (n == 0 || n_views == 0) return cudaSuccess;
   const int threads = 256;
   const int64_t blocks = (n + threads - 1) / threads;
+  // two sets of resident blocks (three per SM of 152), if there are the views
+  const int64_t share = std::max<int64_t>(1, std::min<int64_t>(n_views, 2 * 3 * 152 / blocks));
+  const dim3 grid(static_cast<unsigned>(blocks), static_cast<unsigned>(share));
   // the reduced-precision form takes the FP32 projection
   if (rec16)
-    project_kernel<true><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-        n, n_views, views, pos_op, cov, rec, rec16, foot, box, key, depth_lo, key_range);
+    project_kernel<true><<<grid, threads, 0, stream>>>(n, n_views, views, pos_op, cov, rec, rec16,
+                                                       foot, box, key, depth_lo, key_range);
   else
-    project_kernel<false><<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
-        n, n_views, views, pos_op, cov, rec, rec16, foot, box, key, depth_lo, key_range);
+    project_kernel<false><<<grid, threads, 0, stream>>>(n, n_views, views, pos_op, cov, rec, rec16,
+                                                        foot, box, key, depth_lo, key_range);
   return cudaGetLastError();
 }
 
