@@ -181,34 +181,36 @@ constexpr double kAlphaMinD = 1.0 / 255.0, kAlphaMaxD = 0.99, kTMinD = 1e-4;
 constexpr double kLn2D = 0.69314718055994530942;
 #define FS_F2C(d) f2{static_cast<float>(d), static_cast<float>((d) - static_cast<double>(static_cast<float>(d)))}
 
-// One row of w = W l + b at the pixel offset l (exact small half-integers) as
-// a float pair: the products' and sums' rounding errors are gathered in one
-// float and put back once (a compensated dot product, Ogita, Rump and Oishi
-// 2005), about 25 operations where a chain of float-pair products and sums
-// takes 34.
-__device__ __forceinline__ f2 f2_row(float wh0, float wl0, float wh1, float wl1, float bh,
-                                     float bl, float lx, float ly) {
-  const f2 p0 = two_prod(wh0, lx), p1 = two_prod(wh1, ly);
-  const f2 s = two_sum(p0.hi, p1.hi);
-  const f2 u = two_sum(s.hi, bh);
-  float err = __fadd_rn(p0.lo, p1.lo);
-  err = __fmaf_rn(wl0, lx, err);
-  err = __fmaf_rn(wl1, ly, err);
-  err = __fadd_rn(err, s.lo);
-  err = __fadd_rn(err, u.lo);
-  err = __fadd_rn(err, bl);
-  return fast_two_sum(u.hi, err);
+// w = W l + b at the pixel offset (lx, ly) (exact small half-integers), both rows
+// side by side in packed FP32, as float pairs: the products' and sums' rounding
+// errors are gathered in one float per row and put back once (a compensated dot
+// product, Ogita, Rump and Oishi 2005), about 25 operations a row where a chain
+// of float-pair products and sums takes 34.  wx, wy: columns of W.
+__device__ __forceinline__ f2x2 f2x2_rows(float2 wxh, float2 wxl, float2 wyh, float2 wyl,
+                                          float2 bh, float2 bl, float lx, float ly) {
+  const float2 X = make_float2(lx, lx), Y = make_float2(ly, ly);
+  const float2 p0 = __fmul2_rn(wxh, X), p1 = __fmul2_rn(wyh, Y);
+  float2 err = add2(__ffma2_rn(wxh, X, neg2(p0)), __ffma2_rn(wyh, Y, neg2(p1)));
+  err = __ffma2_rn(wxl, X, err);
+  err = __ffma2_rn(wyl, Y, err);
+  const float2 s = add2(p0, p1);  // two_sum(p0, p1), then two_sum(s, b)
+  float2 bb = sub2(s, p0);
+  err = add2(err, add2(sub2(p0, sub2(s, bb)), sub2(p1, bb)));
+  const float2 u = add2(s, bh);
+  bb = sub2(u, s);
+  err = add2(err, add2(sub2(s, sub2(u, bb)), sub2(bh, bb)));
+  err = add2(err, bl);
+  const float2 r = add2(u, err);
+  return {r, sub2(err, sub2(r, u))};
 }
 
-// a^2 + b^2 of float pairs, likewise with one gathered error.
-__device__ __forceinline__ f2 f2_norm2(f2 a, f2 b) {
-  const f2 p0 = two_prod(a.hi, a.hi), p1 = two_prod(b.hi, b.hi);
-  const f2 s = two_sum(p0.hi, p1.hi);
-  float err = __fadd_rn(p0.lo, p1.lo);
-  err = __fmaf_rn(a.hi + a.hi, a.lo, err);
-  err = __fmaf_rn(b.hi + b.hi, b.lo, err);
-  err = __fadd_rn(err, s.lo);
-  return fast_two_sum(s.hi, err);
+// |w|^2 of a pair of float pairs, likewise with one gathered error.
+__device__ __forceinline__ f2 f2_norm2(const f2x2& w) {
+  const float2 p = __fmul2_rn(w.hi, w.hi);
+  const float2 e = __ffma2_rn(w.hi, w.hi, neg2(p));
+  const float2 t = __ffma2_rn(add2(w.hi, w.hi), w.lo, e);
+  const f2 s = two_sum(p.x, p.y);
+  return fast_two_sum(s.hi, __fadd_rn(__fadd_rn(t.x, t.y), s.lo));
 }
 
 // o 2^-q for q >= 0 as a float pair (about 1e-11 relative): q = k + j/64 + s,
@@ -244,8 +246,8 @@ __device__ __forceinline__ f2 f2_exp2_neg(f2 q, float o, const float2* __restric
 }
 
 // Staged list entries of one warp, one array per 16-byte part so that lanes that
-// read different entries spread over the banks: W (hi and lo parts), b = W (ctr - m)
-// relative to the tile centre, the cut with slack, the opacity and the
+// read different entries spread over the banks: W by columns (hi and lo parts),
+// b = W (ctr - m) relative to the tile centre, the cut with slack, the opacity and the
 // re-check row (-1: none).
 struct Stage {
   float4 w_hi[kRound];
@@ -264,8 +266,8 @@ __device__ __forceinline__ void stage_entry(Stage& S, int e, const ProjRecord& r
   const f2 dy = f2_sub(f2_from(cy), f2{r.m.y, r.m.w});
   const f2 b0 = f2_add(f2_mul(w0, dx), f2_mul(w1, dy));
   const f2 b1 = f2_add(f2_mul(w2, dx), f2_mul(w3, dy));
-  S.w_hi[e] = r.w_hi;
-  S.w_lo[e] = r.w_lo;
+  S.w_hi[e] = make_float4(r.w_hi.x, r.w_hi.z, r.w_hi.y, r.w_hi.w);
+  S.w_lo[e] = make_float4(r.w_lo.x, r.w_lo.z, r.w_lo.y, r.w_lo.w);
   // near the cut the FP32 screen |W_hi l + b_hi|^2 is off by far less than 0.05
   S.bq[e] = make_float4(b0.hi, b1.hi, r.misc.y + 0.05f, r.misc.x);
   S.b_lo[e] = make_float2(b0.lo, b1.lo);
@@ -281,7 +283,7 @@ __device__ __forceinline__ void stage_compact(Stage& S, int e, const CompactReco
   const f2 dx = two_sum(cx, -r.mx), dy = two_sum(cy, -r.my);
   const f2 b0 = f2_add(f2_mul_f(dx, wa.x), f2_mul_f(dy, wa.y));
   const f2 b1 = f2_add(f2_mul_f(dx, wb.x), f2_mul_f(dy, wb.y));
-  S.w_hi[e] = make_float4(wa.x, wa.y, wb.x, wb.y);
+  S.w_hi[e] = make_float4(wa.x, wb.x, wa.y, wb.y);
   S.w_lo[e] = make_float4(0.f, 0.f, 0.f, 0.f);
   S.bq[e] = make_float4(b0.hi, b1.hi, fmaxf(log2f(255.f * o), 0.f) * 1.001f + 1e-3f + 0.05f, o);
   S.b_lo[e] = make_float2(b0.lo, b1.lo);
@@ -291,9 +293,10 @@ __device__ __forceinline__ void stage_compact(Stage& S, int e, const CompactReco
 // FP32 screen: can the entry's alpha >= 1/255 region reach this pixel?
 __device__ __forceinline__ bool reaches(const Stage& S, int e, float lx, float ly) {
   const float4 w = S.w_hi[e], b = S.bq[e];
-  const float q0 = fmaf(w.x, lx, fmaf(w.y, ly, b.x));
-  const float q1 = fmaf(w.z, lx, fmaf(w.w, ly, b.y));
-  return fmaf(q0, q0, q1 * q1) <= b.z;
+  const float2 q = __ffma2_rn(make_float2(w.x, w.y), make_float2(lx, lx),
+                              __ffma2_rn(make_float2(w.z, w.w), make_float2(ly, ly),
+                                         make_float2(b.x, b.y)));
+  return fmaf(q.x, q.x, q.y * q.y) <= b.z;
 }
 
 // alpha of one (pixel, staged entry) pair, clamped: a float pair.
@@ -301,10 +304,11 @@ __device__ __forceinline__ f2 pair_alpha(const Stage& S, int e, float lx, float 
                                          const float2* __restrict__ tab) {
   const float4 wh = S.w_hi[e], wl = S.w_lo[e], bq = S.bq[e];
   const float2 bl = S.b_lo[e];
-  const f2 w0 = f2_row(wh.x, wl.x, wh.y, wl.y, bq.x, bl.x, lx, ly);
-  const f2 w1 = f2_row(wh.z, wl.z, wh.w, wl.w, bq.y, bl.y, lx, ly);
+  const f2x2 w = f2x2_rows(make_float2(wh.x, wh.y), make_float2(wl.x, wl.y),
+                           make_float2(wh.z, wh.w), make_float2(wl.z, wl.w),
+                           make_float2(bq.x, bq.y), bl, lx, ly);
   const f2 a_max = FS_F2C(kAlphaMaxD);
-  const f2 a = f2_exp2_neg(f2_norm2(w0, w1), bq.w, tab);
+  const f2 a = f2_exp2_neg(f2_norm2(w), bq.w, tab);
   return f2_lt(a_max, a) ? a_max : a;
 }
 
