@@ -110,8 +110,25 @@ __global__ void __launch_bounds__(256) assign_kernel(const T* __restrict__ table
 // The same with the block's rows staged through shared memory: rows of E
 // values at a stride of E are read by consecutive threads at consecutive
 // addresses (the direct form above reads one row per thread, E * 8 bytes
-// apart).  128 rows per block.
+// apart).  128 rows per block.  Bound by HBM for FP32 tables, so the rows go
+// straight to shared memory in 16-byte asynchronous copies, all of a block's
+// in flight at once (3M rows of 33 labels: 92 us with loads and stores, 75 us
+// so, 87 % of the measured copy rate).
 constexpr int kAssignRows = 128;
+
+// bytes (any number) from src to shared memory at dst, by the whole block.
+__device__ __forceinline__ void stage_rows(void* dst, const void* src, int bytes) {
+  const bool aligned = (reinterpret_cast<uintptr_t>(src) & 15u) == 0;
+  const int whole = aligned ? bytes / 16 : 0;
+  const uint32_t to = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  for (int k = threadIdx.x; k < whole; k += kAssignRows)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * k),
+                 "l"(static_cast<const char*>(src) + 16 * k));
+  for (int k = 4 * whole + threadIdx.x; k < bytes / 4; k += kAssignRows)
+    static_cast<uint32_t*>(dst)[k] = static_cast<const uint32_t*>(src)[k];
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+}
 template <typename T>
 __global__ void __launch_bounds__(kAssignRows) assign_staged_kernel(
     const T* __restrict__ table, int64_t n, int E, T gamma, uint64_t* __restrict__ bits,
@@ -120,10 +137,7 @@ __global__ void __launch_bounds__(kAssignRows) assign_staged_kernel(
   T* rows = reinterpret_cast<T*>(smem_raw);
   const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kAssignRows;
   const int n_rows = static_cast<int>(min(static_cast<int64_t>(kAssignRows), n - i0));
-  const int count = n_rows * E;
-  const T* src = table + i0 * E;
-  for (int k = threadIdx.x; k < count; k += kAssignRows) rows[k] = src[k];
-  __syncthreads();
+  stage_rows(rows, table + i0 * E, n_rows * E * static_cast<int>(sizeof(T)));
   if (static_cast<int>(threadIdx.x) >= n_rows) return;
   const int64_t i = i0 + threadIdx.x;
   const Decision d = decide_row(rows + threadIdx.x * E, E, gamma);
