@@ -30,32 +30,41 @@ struct MemberSlots {
   }
 };
 
-constexpr int kRenderThreads = kTilePixels;  // one thread per pixel of a 16x16 tile
+constexpr int kRenderThreads = 128;  // four warps: the 8x8 sub-tiles of a 16x16 tile
+constexpr int kRenderBatch = kRenderThreads;  // records staged at a time, one per thread
+// Records a warp takes between looks at its pixels' stops (1, 2, 4 at ten blocks
+// per SM: 4.18, 4.10, 4.05 ms a call; eight blocks, whose 64 registers hold the
+// loads of a step: 4.02).
+constexpr int kRenderStep = 4;
 
-// One block per (tile, view), one thread per pixel, warps of 8x4 pixels; the
-// tile's list is walked in depth order in batches of 256 records staged in
-// shared memory.  Plain FP32 compositing with the solve's rules: alpha =
-// min(0.99, o 2^-|W (p - m)|^2), skipped below 1/255, and the pixel stops before
-// a Gaussian that takes T below 1e-4.  best[] holds, per pixel of the batch, the
-// smallest depth of a passing object so far (written on the first object).
+// One block per (tile, view), one warp per 8x8 sub-tile, two pixels per lane
+// (rows y and y + 4) in packed FP32; the tile's list is walked in depth order
+// in batches of records staged in shared memory.  Plain FP32 compositing with
+// the solve's rules: alpha = min(0.99, o 2^-|W (p - m)|^2), skipped below
+// 1/255, and the pixel stops before a Gaussian that takes T below 1e-4.
+// best[] holds, per pixel of the batch, the smallest depth of a passing object
+// so far (written on the first object).
 //
-// Bound by issue.  Where a record is staged, it is tested against the eight
-// warps' pixel rectangles (over which w = W (p - m) stays in a box around its
-// centre's); a warp then evaluates only the records that can reach it, about
-// a third of the tile's, and the others are below 1/255 at all of its pixels
-// anyway (500k Gaussians, 8 views 1008x756: 445 -> 384 us for the first of 8
-// objects; eight blocks per SM take the whole call from 4.82 to 4.50 ms).
+// Bound by issue.  Where a record is staged, it is tested against the four
+// sub-tiles (over which w = W (p - m) stays in a box around its centre's); a
+// warp then evaluates only the records that can reach it, and the others are
+// below 1/255 at all of its pixels anyway.  A record's loads, its list entry
+// and the loop are paid once for two pixels, and the pixel step is free of
+// branches: with one pixel per lane, 8x4 pixels per warp and divergent skips
+// and stops, 384 us for the first of 8 objects, 284 us so (500k
+// Gaussians, 8 views 1008x756; the whole call 4.43 -> 4.02 ms).
 template <typename OutT>
 __global__ void __launch_bounds__(kRenderThreads, 8) render_kernel(
     const ViewParams* __restrict__ views, const RenderOut* __restrict__ outs,
     const uint2* __restrict__ ranges, const uint32_t* __restrict__ list_val,
     const ProjRecord* __restrict__ rec, const CompactRecord* __restrict__ rec16, int e,
     int first, float tau, float* __restrict__ best) {
-  __shared__ float4 s_w[kRenderThreads];  // W (row-major 2x2)
-  __shared__ float4 s_m[kRenderThreads];  // mean as float pairs (mx, my, mx_lo, my_lo)
-  __shared__ float4 s_o[kRenderThreads];  // (-log2 o, clamp, depth, -)
-  __shared__ uint8_t s_keep[kRenderThreads];                      // bit w: reaches warp w
-  __shared__ uint8_t s_list[kRenderThreads / 32][kRenderThreads]; // per warp: its records
+  // one record more than the batch: o = 0, which no pixel takes
+  __shared__ float4 s_w[kRenderBatch + 1];  // W (row-major 2x2)
+  __shared__ float4 s_m[kRenderBatch + 1];  // mean as float pairs (mx, my, mx_lo, my_lo)
+  __shared__ float4 s_o[kRenderBatch + 1];  // (-log2 o, clamp, depth, -)
+  __shared__ uint8_t s_keep[kRenderBatch];                             // bit w: reaches warp w
+  __shared__ uint8_t s_list[kRenderThreads / 32][kRenderBatch + kRenderStep];  // per warp: its records
   const int v = blockIdx.y;
   const ViewParams& vp = views[v];
   const int tiles_x = vp.tiles_x;
@@ -64,15 +73,21 @@ __global__ void __launch_bounds__(kRenderThreads, 8) render_kernel(
   const int tx = tile % tiles_x, ty = tile / tiles_x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int px = tx * kTile + 8 * (warp & 1) + (lane & 7);
-  const int py = ty * kTile + 4 * (warp >> 1) + (lane >> 3);
-  const bool inside = px < vp.width && py < vp.height;
+  const int py = ty * kTile + 8 * (warp >> 1) + (lane >> 3);
   const uint2 rg = ranges[vp.tile_base + tile];
-  const float pxc = static_cast<float>(px) + 0.5f, pyc = static_cast<float>(py) + 0.5f;
+  const float pxc = static_cast<float>(px) + 0.5f;
+  const float2 pyc = make_float2(static_cast<float>(py) + 0.5f, static_cast<float>(py + 4) + 0.5f);
   const float tcx = static_cast<float>(tx * kTile), tcy = static_cast<float>(ty * kTile);
-  float T = 1.f, rho = 0.f, zsum = 0.f;
-  bool done = !inside;
-  for (uint32_t base = rg.x; base < rg.y; base += kRenderThreads) {
-    if (__syncthreads_and(done ? 1 : 0)) break;  // every pixel of the tile stopped
+  const float2 one = make_float2(1.f, 1.f);
+  float2 T = one, rho = make_float2(0.f, 0.f), zsum = make_float2(0.f, 0.f);
+  bool done0 = px >= vp.width || py >= vp.height;
+  bool done1 = px >= vp.width || py + 4 >= vp.height;
+  if (threadIdx.x == 0) {
+    s_w[kRenderBatch] = s_m[kRenderBatch] = make_float4(0.f, 0.f, 0.f, 0.f);
+    s_o[kRenderBatch] = make_float4(__int_as_float(0x7f800000), 0.f, 0.f, 0.f);
+  }
+  for (uint32_t base = rg.x; base < rg.y; base += kRenderBatch) {
+    if (__syncthreads_and(done0 && done1 ? 1 : 0)) break;  // every pixel of the tile stopped
     const uint32_t k = base + threadIdx.x;
     uint32_t keep = 0u;
     if (k < rg.y) {
@@ -96,14 +111,14 @@ __global__ void __launch_bounds__(kRenderThreads, 8) render_kernel(
       }
       s_w[threadIdx.x] = w;
       s_m[threadIdx.x] = m;
-      // rectangle of warp q: pixel centres within (3.5, 1.5) of its own centre;
-      // q_cut carries the slack for the rounding of this test
-      const float h0 = fmaf(fabsf(w.x), 3.5f, fabsf(w.y) * 1.5f);
-      const float h1 = fmaf(fabsf(w.z), 3.5f, fabsf(w.w) * 1.5f);
+      // sub-tile q: pixel centres within 3.5 of its own centre; q_cut carries
+      // the slack for the rounding of this test
+      const float h0 = fmaf(fabsf(w.x), 3.5f, fabsf(w.y) * 3.5f);
+      const float h1 = fmaf(fabsf(w.z), 3.5f, fabsf(w.w) * 3.5f);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < 4; ++q) {
         const float dx = ((tcx + 8.f * (q & 1) + 4.f) - m.x) - m.z;
-        const float dy = ((tcy + 4.f * (q >> 1) + 2.f) - m.y) - m.w;
+        const float dy = ((tcy + 8.f * (q >> 1) + 4.f) - m.y) - m.w;
         const float d0 = fmaxf(0.f, fabsf(fmaf(w.x, dx, w.y * dy)) - h0);
         const float d1 = fmaxf(0.f, fabsf(fmaf(w.z, dx, w.w * dy)) - h1);
         if (fmaf(d0, d0, d1 * d1) <= qc) keep |= 1u << q;
@@ -111,54 +126,79 @@ __global__ void __launch_bounds__(kRenderThreads, 8) render_kernel(
     }
     s_keep[threadIdx.x] = static_cast<uint8_t>(keep);
     __syncthreads();
-    // the warp's records, in list order
+    // the warp's records, in list order, filled up to whole steps
     int count = 0;
 #pragma unroll
-    for (int q = 0; q < kRenderThreads; q += 32) {
+    for (int q = 0; q < kRenderBatch; q += 32) {
       const bool on = (s_keep[q + lane] >> warp) & 1u;
       const uint32_t bal = __ballot_sync(0xffffffffu, on);
       if (on)
         s_list[warp][count + __popc(bal & ((1u << lane) - 1u))] = static_cast<uint8_t>(q + lane);
       count += __popc(bal);
     }
+    if (lane < kRenderStep) s_list[warp][count + lane] = static_cast<uint8_t>(kRenderBatch);
     __syncwarp();
-    for (int c = 0; c < count && !done; ++c) {
-      const int j = s_list[warp][c];
-      const float4 w = s_w[j], m = s_m[j], o = s_o[j];
-      const float dx = (pxc - m.x) - m.z, dy = (pyc - m.y) - m.w;
-      const float w0 = fmaf(w.x, dx, w.y * dy), w1 = fmaf(w.z, dx, w.w * dy);
-      float alpha = ex2_approx(-fmaf(w0, w0, fmaf(w1, w1, o.x)));
-      if (o.y != 0.f) alpha = fminf(alpha, kAlphaMax);
-      if (alpha < kAlphaMin) continue;
-      const float t_next = T * (1.f - alpha);
-      if (t_next < kTMin) {
-        done = true;
-        break;
+    for (int c = 0; c < count; c += kRenderStep) {
+      if (__all_sync(0xffffffffu, done0 && done1)) break;
+#pragma unroll
+      for (int u = 0; u < kRenderStep; ++u) {
+        const int j = s_list[warp][c + u];
+        const float4 w = s_w[j], m = s_m[j], o = s_o[j];
+        const float dx = (pxc - m.x) - m.z;
+        const float2 dX = make_float2(dx, dx);
+        const float2 dY = add2(add2(pyc, make_float2(-m.y, -m.y)), make_float2(-m.w, -m.w));
+        const float2 w0 = __ffma2_rn(make_float2(w.x, w.x), dX,
+                                     __fmul2_rn(make_float2(w.y, w.y), dY));
+        const float2 w1 = __ffma2_rn(make_float2(w.z, w.z), dX,
+                                     __fmul2_rn(make_float2(w.w, w.w), dY));
+        const float2 q = __ffma2_rn(w0, w0, __ffma2_rn(w1, w1, make_float2(o.x, o.x)));
+        float a0 = ex2_approx(-q.x), a1 = ex2_approx(-q.y);
+        if (o.y != 0.f) {
+          a0 = fminf(a0, kAlphaMax);
+          a1 = fminf(a1, kAlphaMax);
+        }
+        // a pixel that skips takes alpha = 0, which leaves T as it is
+        if (done0 || a0 < kAlphaMin) a0 = 0.f;
+        if (done1 || a1 < kAlphaMin) a1 = 0.f;
+        const float2 tn = __fmul2_rn(T, __ffma2_rn(make_float2(a0, a1), make_float2(-1.f, -1.f), one));
+        const bool stop0 = tn.x < kTMin, stop1 = tn.y < kTMin;
+        done0 = done0 || stop0;
+        done1 = done1 || stop1;
+        if (stop0) a0 = 0.f;
+        if (stop1) a1 = 0.f;
+        const float2 al = make_float2(a0, a1);
+        const float2 cT = __fmul2_rn(al, T);
+        rho = add2(rho, cT);
+        if (a0 != 0.f) zsum.x = fmaf(cT.x, o.z, zsum.x);  // no 0 times an overflown depth
+        if (a1 != 0.f) zsum.y = fmaf(cT.y, o.z, zsum.y);
+        if (!stop0) T.x = tn.x;
+        if (!stop1) T.y = tn.y;
       }
-      const float cT = alpha * T;
-      rho += cT;
-      zsum = fmaf(cT, o.z, zsum);
-      T = t_next;
     }
     __syncthreads();  // the batch is read by every thread before the next one lands
   }
-  if (!inside) return;
   const int64_t npix = static_cast<int64_t>(vp.width) * vp.height;
-  const int64_t p = static_cast<int64_t>(py) * vp.width + px;
   const RenderOut ro = outs[v];
-  const float depth = rho > 0.f ? zsum / rho : 0.f;
-  if (ro.rho) ro.rho[static_cast<int64_t>(e - 1) * npix + p] = rho;
-  if (ro.depth) ro.depth[static_cast<int64_t>(e - 1) * npix + p] = depth;
-  float* const bp = best + vp.state_off + p;
-  OutT* const mp = static_cast<OutT*>(ro.mask) + p;
-  float b = first ? __int_as_float(0x7f800000) : *bp;
-  OutT lab = first ? static_cast<OutT>(0) : *mp;
-  if (rho > tau && depth < b) {
-    b = depth;
-    lab = static_cast<OutT>(e);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int y = py + 4 * i;
+    if (px >= vp.width || y >= vp.height) continue;
+    const int64_t p = static_cast<int64_t>(y) * vp.width + px;
+    const float r = i ? rho.y : rho.x, zs = i ? zsum.y : zsum.x;
+    const float depth = r > 0.f ? zs / r : 0.f;
+    if (ro.rho) ro.rho[static_cast<int64_t>(e - 1) * npix + p] = r;
+    if (ro.depth) ro.depth[static_cast<int64_t>(e - 1) * npix + p] = depth;
+    float* const bp = best + vp.state_off + p;
+    OutT* const mp = static_cast<OutT*>(ro.mask) + p;
+    float b = first ? __int_as_float(0x7f800000) : *bp;
+    OutT lab = first ? static_cast<OutT>(0) : *mp;
+    if (r > tau && depth < b) {
+      b = depth;
+      lab = static_cast<OutT>(e);
+    }
+    *bp = b;
+    *mp = lab;
   }
-  *bp = b;
-  *mp = lab;
 }
 
 }  // namespace
