@@ -468,13 +468,16 @@ __device__ __forceinline__ void fix_tie_run(int64_t k, int64_t n_total, const Sl
 // from one 16-byte load each (when both arrays are 16-byte aligned) and the
 // words around them.  Nearly every same-view run is a pair: the pairs' low
 // words are gathered together, where walking each run as it is met costs a
-// chain of gathers per run.  Longer runs are walked.  Bound by the gathers:
-// every sixth slot of a 10^6-Gaussian view shares its key (4.8 10^7 slots of
-// 48 views: 328 us, 375 us with every run walked).
-__global__ void depth_tie_fix_kernel(int64_t n_total, int64_t n, const uint32_t* __restrict__ key,
-                                     uint32_t* __restrict__ val,
-                                     const uint32_t* __restrict__ depth_lo,
-                                     const uint32_t* __restrict__ n_dev) {
+// chain of gathers per run.  Longer runs are walked.  Bound by the latency of
+// its loads and gathers: every sixth slot of a 10^6-Gaussian view shares its
+// key.  4.8 10^7 slots of 48 views: 375 us with every run walked, 329 us with
+// the pairs gathered, 313 us with the slots loaded beside the keys instead of
+// after them, 249 us with blocks of 128, twelve to an SM (42 registers; 256
+// threads, six: 268; 128, fourteen or sixteen: 281).
+constexpr int kTieThreads = 128;
+__global__ void __launch_bounds__(kTieThreads, 12) depth_tie_fix_kernel(
+    int64_t n_total, int64_t n, const uint32_t* __restrict__ key, uint32_t* __restrict__ val,
+    const uint32_t* __restrict__ depth_lo, const uint32_t* __restrict__ n_dev) {
   if (n_dev) n_total = min(n_total, static_cast<int64_t>(*n_dev));
   const int64_t k0 = 4 * (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
   if (k0 + 1 >= n_total) return;
@@ -499,11 +502,11 @@ __global__ void depth_tie_fix_kernel(int64_t n_total, int64_t n, const uint32_t*
     dst[6] = k0 + 5 < n_total ? src[k0 + 5] : none;
   };
   load(key, 0xFFFFFFFFu, t);
+  load(val, 0u, w);
   bool any = false;  // an equal neighbour somewhere among the four
 #pragma unroll
   for (int i = 1; i <= 4; ++i) any = any || (t[i] != 0xFFFFFFFFu && t[i + 1] == t[i]);
   if (!any) return;
-  load(val, 0u, w);
   const SlotView view_of(n);
   bool tie[6];  // positions k0 + i - 1 and k0 + i: equal keys, one view
 #pragma unroll
@@ -947,9 +950,8 @@ cudaError_t launch_depth_tie_fix(int64_t n_total, int64_t n, const uint32_t* key
                                  const uint32_t* depth_lo, cudaStream_t stream,
                                  const uint32_t* n_dev) {
   if (n_total < 2) return cudaSuccess;
-  const int threads = 256;
-  const int64_t blocks = ((n_total + 3) / 4 + threads - 1) / threads;
-  depth_tie_fix_kernel<<<static_cast<unsigned>(blocks), threads, 0, stream>>>(n_total, n, key, val,
+  const int64_t blocks = ((n_total + 3) / 4 + kTieThreads - 1) / kTieThreads;
+  depth_tie_fix_kernel<<<static_cast<unsigned>(blocks), kTieThreads, 0, stream>>>(n_total, n, key, val,
                                                                               depth_lo, n_dev);
   return cudaGetLastError();
 }
