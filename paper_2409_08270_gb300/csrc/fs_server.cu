@@ -249,6 +249,28 @@ fs_status solve_with_graph(fs_server* s, int slot, SceneEntry& se, Request* r,
   return status;
 }
 
+// Frees the captured solve used longest ago that is not replaying (another
+// scene's than `self`).  False when there is none.
+bool drop_oldest_graph(fs_server* s, SceneEntry* self) {
+  std::lock_guard<std::mutex> lk(s->graphs_mu);
+  SceneEntry* lru = nullptr;
+  std::lock_guard<std::mutex> g(s->scenes_mu);
+  for (auto& e : s->scenes) {
+    if (e.get() == self || !e->graph_mu.try_lock()) continue;
+    const bool older = e->graph && (!lru || e->last_use < lru->last_use);
+    if (older && lru) lru->graph_mu.unlock();
+    if (older)
+      lru = e.get();  // stays locked
+    else
+      e->graph_mu.unlock();
+  }
+  if (!lru) return false;
+  drop_graph(*lru);
+  lru->graph_mu.unlock();
+  --s->live_graphs;
+  return true;
+}
+
 // The first request of a scene (autotune on): time a few batching settings
 // on a sample of its views and keep the fastest for the scene.
 void tune_scene(fs_server* s, int slot, SceneEntry& se, Request* r) {
@@ -296,16 +318,26 @@ void worker(fs_server* s, int slot) {
       if (!se->tuned) {
         tune_scene(s, slot, *se, r);
         se->tuned = true;
+        // captured solves have workspaces of their own
+        if (s->max_graphs > 0) fs::ctx_release_workspace(s->ctx[slot]);
       }
     }
     fs::ctx_set_batching(s->ctx[slot], se->views_per_batch, se->depth_chunks);
     r->info.views_per_batch = se->views_per_batch;
     r->info.depth_chunks = fs::ctx_depth_chunks(s->ctx[slot], se->n);
-    const fs_status st =
-        s->max_graphs > 0
-            ? solve_with_graph(s, slot, *se, r, &r->info.stats)
-            : solve_request(s, slot, *se, r, static_cast<int32_t>(r->cams.size()),
-                            &r->info.stats);
+    auto solve = [&] {
+      return s->max_graphs > 0
+                 ? solve_with_graph(s, slot, *se, r, &r->info.stats)
+                 : solve_request(s, slot, *se, r, static_cast<int32_t>(r->cams.size()),
+                                 &r->info.stats);
+    };
+    fs_status st = solve();
+    // out of device memory: other scenes' captured solves give way, oldest first
+    while (st == FS_OUT_OF_MEMORY && s->max_graphs > 0) {
+      cudaStreamSynchronize(s->streams[slot]);
+      if (!drop_oldest_graph(s, se)) break;
+      st = solve();
+    }
     if (st != FS_OK) r->error = fs_last_error();
     // keep the slot's retained workspace within its share of the budget
     if (static_cast<int64_t>(fs::ctx_workspace_bytes(s->ctx[slot])) > s->budget / s->n_slots) {
