@@ -273,22 +273,46 @@ void fs::ctx_set_batching(fs_ctx* c, int views_per_batch, int depth_chunks) {
   if (depth_chunks >= 0) c->depth_chunks = std::min(depth_chunks, 16);
 }
 
-// Front-to-back depth chunks of a solve of n Gaussians (sizes 1/32, 1/32, 1/16,
-// ..., 1/2 of a batch's visible slots with six): the context's setting, or by n.
-// A chunk costs its launches, a readback and the blend's start on every tile,
-// and spares later chunks the entries of the tiles it saturates, of which there
-// are more the deeper a view's lists are.  Solve times in ms with
-// 1 | 2 | 3 | 4 | 5 | 6 | 7 | 8 chunks:
-//   50k Gaussians, 60 views 300x200      2.0   2.3   2.6   2.8   3.0   3.2   3.4   3.5
-//   300k, 24 views 512x512               3.0   3.1   3.3   3.4   3.6   3.7   3.8   3.9
-//   333k, 37 views 799x601               6.6   6.3   6.3   6.5   6.7   6.9   7.0   7.2
-//   500k, 50 views 1008x756             15.7  13.9  13.6  13.6  13.7  13.9  14.2  14.5
-//   1M, 100 views 1008x756              51.3  37.6  30.2  27.5  26.6  26.7  27.1  27.6
-//   3M, 100 views 1256x828               158   118    97  86.1  79.8  77.2  76.5  76.6
-int fs::ctx_depth_chunks(const fs_ctx* c, int64_t n) {
+// Front-to-back depth chunks of a solve (sizes 1/32, 1/32, 1/16, ..., 1/2 of a
+// batch's visible slots with six): the context's setting, or by the solve's
+// size.  A chunk costs its launches, a readback and the blend's start on every
+// tile, and spares later chunks the entries of the tiles it saturates.  The
+// share of those grows with a view's depth, that is with n; views of few tiles
+// leave a chunk's kernels short, so its fixed costs weigh more; and a batch
+// must hold enough entries (about 3 + tiles / 350 a slot) to pay for them at
+// all: 5.6 10^7 per chunk after the first at 300,000 Gaussians, fewer the
+// larger the share that a chunk spares (300,000 in 24 views of 512x512: 3.0 |
+// 3.1 | 3.3; in one of 1600x1200: 0.51 with 1).  Solve times in ms with 1 | 2 |
+// 3 | 4 | 5 | 6 | 8 chunks, 40 views (30 of 1600x1200), a forward-facing arc:
+//   180k Gaussians, 400x300    2.45   2.47   2.52   2.64   2.78   2.90   3.11
+//   180k, 1600x1200            7.64   7.06   7.03   7.31   7.77   8.26   9.18
+//   300k, 160x120              3.17   3.53   3.80   4.08   4.26   4.43   4.61
+//   300k, 400x300              3.38   3.18   3.16   3.24   3.38   3.50   3.72
+//   300k, 900x640              6.48   5.60   5.27   5.28   5.43   5.67   6.11
+//   300k, 1600x1200           10.73   8.84   8.29   8.31   8.66   9.08  10.04
+//   600k, 400x300              5.65   4.93   4.68   4.64   4.73   4.86   5.07
+//   600k, 1600x1200           18.02  13.53  11.18  10.51  10.55  10.85  11.70
+//   1M, 160x120                8.08   7.56   7.71   7.75   8.01   8.13   8.45
+//   1M, 900x640               17.17  12.35  10.15   9.28   9.01   9.00   9.38
+//   1.5M, 1600x1200           39.01  26.43  19.72  16.40  15.10  14.88  15.43
+// and for 3M Gaussians in 100 views of 1256x828, the re-check included, 158
+// 118  97  86.1  79.8  77.2 (7: 76.5) 76.6.
+int fs::ctx_depth_chunks(const fs_ctx* c, int64_t n, const fs_camera* cams, int32_t V) {
   if (c->depth_chunks > 0) return std::min(c->depth_chunks, fs::kMaxChunks);
-  const double by_size = 1.0 + 2.0 * log2(static_cast<double>(std::max<int64_t>(n, 1)) / 262144.0);
-  return std::max(1, std::min(8, static_cast<int>(lround(by_size))));
+  if (n <= 0 || V <= 0) return 1;
+  double tiles = 0;  // mean over the views
+  for (int32_t v = 0; v < V; ++v)
+    tiles += static_cast<double>((cams[v].width + fs::kTile - 1) / fs::kTile) *
+             ((cams[v].height + fs::kTile - 1) / fs::kTile);
+  tiles /= V;
+  const double views = std::min<double>(c->views_per_batch, V);
+  const double entries = views * static_cast<double>(n) * (3.0 + tiles / 350.0);
+  const double by_depth = 3.0 + 1.3 * log2(static_cast<double>(n) / 3e5) -
+                          0.9 * std::max(0.0, log2(3000.0 / tiles));
+  const double per_chunk = 5.6e7 * pow(3e5 / static_cast<double>(n), 0.6);
+  const double chunks =
+      std::min({std::floor(by_depth + 0.5), std::floor(1.0 + entries / per_chunk), 8.0});
+  return std::max(1, static_cast<int>(chunks));
 }
 
 extern "C" {
@@ -855,7 +879,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   if (vb < 1) return fail(FS_UNSUPPORTED, "fs_accumulate: scene too large");
   const int64_t kcap = static_cast<int64_t>(vb) * n;
-  const int chunks = fs::ctx_depth_chunks(c, n);
+  const int chunks = fs::ctx_depth_chunks(c, n, cams, V);
   FS_TRY(ensure_window(c, n, vb, V, keep));
   FS_TRY(stage_masks(c, cams, V, masks, mask_dtype, mask_memory, stream));
   if (keep) FS_TRY(kept_layout(c, cams, V, vb, chunks));

@@ -255,8 +255,8 @@ cudaError_t launch_render(const ViewParams* views, const RenderOut* outs, int n_
 size_t ctx_workspace_bytes(const fs_ctx* c);
 void ctx_release_workspace(fs_ctx* c);
 void ctx_set_batching(fs_ctx* c, int views_per_batch, int depth_chunks);
-// Depth chunks a solve of n Gaussians takes in this context.
-int ctx_depth_chunks(const fs_ctx* c, int64_t n);
+// Depth chunks a solve of n Gaussians in V views takes in this context.
+int ctx_depth_chunks(const fs_ctx* c, int64_t n, const fs_camera* cams, int32_t V);
 
 // View parameters of a camera (fs_api.cu): float pairs of R, t and the
 // intrinsics, near plane 0.2, Jacobian clamp 1.3 tan(half field of view),

@@ -324,7 +324,8 @@ void worker(fs_server* s, int slot) {
     }
     fs::ctx_set_batching(s->ctx[slot], se->views_per_batch, se->depth_chunks);
     r->info.views_per_batch = se->views_per_batch;
-    r->info.depth_chunks = fs::ctx_depth_chunks(s->ctx[slot], se->n);
+    r->info.depth_chunks = fs::ctx_depth_chunks(s->ctx[slot], se->n, r->cams.data(),
+                                                static_cast<int32_t>(r->cams.size()));
     auto solve = [&] {
       return s->max_graphs > 0
                  ? solve_with_graph(s, slot, *se, r, &r->info.stats)
