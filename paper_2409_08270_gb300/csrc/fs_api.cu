@@ -211,10 +211,10 @@ struct fs_ctx {
   DevBuf lb_tmp;     // look-back words of the fused binning
   // the main pass's tile lists, kept for the re-check (see kept_layout)
   bool kl_valid = false;
-  int kl_chunks = 1;
-  std::vector<DevBuf> kl_val;
+  std::vector<int> kl_parts;            // lists of each batch
+  std::vector<DevBuf> kl_val, kl_rng;   // [batch * kMaxChunks + part]: values, tile ranges
   std::vector<int64_t> kl_tile_off;
-  DevBuf kl_ranges, kl_satc, kl_bound;
+  DevBuf kl_satc, kl_bound;
   std::vector<const void*> mask_dev;  // device pointer of every view's mask (last solve)
   HostBuf views_host, total_host, counters_host;
   fs_stats stats{};
@@ -236,7 +236,7 @@ DevBuf* const* workspace_bufs(fs_ctx* c, size_t* count) {
                     &c->lv_a, &c->lk_b, &c->lv_b, &c->ranges, &c->sort_tmp, &c->scan_tmp,
                     &c->mask_stage, &c->table_tmp, &c->table32_tmp, &c->bits_tmp,
                     &c->label_tmp, &c->margin_tmp, &c->rk_flag, &c->rk_offs,
-                    &c->rk_F, &c->rk_map, &c->rk_R, &c->rk_Rb, &c->rk_tiles, &c->kl_ranges, &c->kl_satc,
+                    &c->rk_F, &c->rk_map, &c->rk_R, &c->rk_Rb, &c->rk_tiles, &c->kl_satc,
                     &c->kl_bound, &c->key_range, &c->lb_tmp, &c->key_a2, &c->val_a2,
                     &c->key_b2, &c->val_b2, &c->cols, &c->rd_val,
                     &c->render_out, &c->chunk_bnd, &c->free_tab, &c->live, &c->live_val,
@@ -253,6 +253,7 @@ size_t fs::ctx_workspace_bytes(const fs_ctx* c) {
   DevBuf* const* b = workspace_bufs(const_cast<fs_ctx*>(c), &count);
   for (size_t k = 0; k < count; ++k) total += b[k]->bytes;
   for (const DevBuf& v : c->kl_val) total += v.bytes;
+  for (const DevBuf& v : c->kl_rng) total += v.bytes;
   return total;
 }
 
@@ -264,6 +265,7 @@ void fs::ctx_release_workspace(fs_ctx* c) {
   DevBuf* const* b = workspace_bufs(c, &count);
   for (size_t k = 0; k < count; ++k) b[k]->release();
   for (DevBuf& v : c->kl_val) v.release();
+  for (DevBuf& v : c->kl_rng) v.release();
   c->kl_valid = false;
 }
 
@@ -386,12 +388,13 @@ fs_status fs_destroy(fs_ctx* c) {
                     &c->sort_tmp, &c->scan_tmp, &c->total, &c->counters, &c->mask_stage,
                     &c->table_tmp, &c->table32_tmp, &c->bits_tmp, &c->label_tmp, &c->margin_tmp,
                     &c->rk_flag, &c->rk_offs, &c->rk_F, &c->rk_map, &c->rk_R,
-                    &c->rk_Rb, &c->rk_tiles, &c->kl_ranges, &c->kl_satc, &c->kl_bound, &c->key_range,
+                    &c->rk_Rb, &c->rk_tiles, &c->kl_satc, &c->kl_bound, &c->key_range,
                     &c->lb_tmp,
                     &c->key_a2, &c->val_a2, &c->key_b2, &c->val_b2, &c->cols,
                     &c->rd_val, &c->render_out, &c->chunk_bnd,
                     &c->free_tab, &c->live, &c->live_val, &c->live_range};
   for (DevBuf& b : c->kl_val) b.release();
+  for (DevBuf& b : c->kl_rng) b.release();
   for (DevBuf* b : bufs) b->release();
   c->views_host.release();
   c->render_out_host.release();
@@ -682,7 +685,8 @@ fs_status read_total(fs_ctx* c, cudaStream_t stream, int64_t* out) {
 // range (may be NULL): the positions' bounds in device memory (at most n_pos).
 // live: the positions are first reduced to the slots with an unsaturated tile
 // in their box (for large chunks behind saturated tiles).  limit > 0: more
-// entries than that are left unsorted and unlisted, and *I_out is -1.
+// entries than that, or than there is memory for, are left unsorted and
+// unlisted, and *I_out is minus their number.
 //
 // Captured form (range_dev != NULL): the chunk's positions are read on the
 // device from range_dev[0 .. 1] (at most n_pos of them: the grid), nothing is
@@ -760,22 +764,32 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
     FS_TRY(stage_end(c, tb, stream));
     FS_TRY(read_total(c, stream, &I));
     if (limit > 0 && I > limit) {
-      *I_out = -1;
+      *I_out = -I;
       return FS_OK;
     }
     if (I >= (static_cast<int64_t>(1) << 31))
       return fail(FS_UNSUPPORTED, "%lld list entries in one chunk; use fewer views per batch",
                   (long long)I);
+    // room for the list and its sort
+    const size_t bytes = static_cast<size_t>(I) * 4;
+    fs_status st = c->lk_a.ensure(bytes, "list keys");
+    if (st == FS_OK) st = val_dst->ensure(bytes, "list values");
+    if (st == FS_OK) st = c->lk_b.ensure(bytes, "list keys");
+    if (st == FS_OK) st = c->lv_b.ensure(bytes, "list values");
+    if (st == FS_OK)
+      st = c->sort_tmp.ensure(fs::radix_temp_bytes(std::max<int64_t>(I, kcap)), "sort temp");
+    if (st == FS_OUT_OF_MEMORY && limit > 0) {
+      for (DevBuf* b : {&c->lk_a, val_dst, &c->lk_b, &c->lv_b}) b->release();
+      FS_TRY(c->sort_tmp.ensure(fs::radix_temp_bytes(kcap), "sort temp"));
+      *I_out = -std::max<int64_t>(I, 1);
+      return FS_OK;
+    }
+    FS_TRY(st);
     if (I <= static_cast<int64_t>(capacity)) break;
-    FS_TRY(c->lk_a.ensure(static_cast<size_t>(I) * 4, "list keys"));
-    FS_TRY(val_dst->ensure(static_cast<size_t>(I) * 4, "list values"));
   }
   if (count_entries) c->stats.list_entries += I;
   *I_out = I;
   if (I == 0) return FS_OK;
-  FS_TRY(c->lk_b.ensure(static_cast<size_t>(I) * 4, "list keys"));
-  FS_TRY(c->lv_b.ensure(static_cast<size_t>(I) * 4, "list values"));
-  FS_TRY(c->sort_tmp.ensure(fs::radix_temp_bytes(std::max<int64_t>(I, kcap)), "sort temp"));
   c->stats.kernel_launches += 1 + radix_launches(I, tile_bits);
   bool alt2 = false;
   int tt = -1;
@@ -800,9 +814,15 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
 // chunk's slots lie behind saturated tiles: its last two chunks 600 and 1041
 // us without, 545 and 645 us with the bits; earlier and smaller chunks lose.
 constexpr int64_t kLiveMin = 1 << 22;
-// A chunk with more list entries than this (8 GB of lists) is halved when the
-// context chose the number of chunks.
+// A list of more entries than this (8 GB with its sort's buffers) is cut into
+// parts: a depth chunk by its positions, when the context chose the number of
+// chunks, the re-check's list by its views.
 constexpr int64_t kSplitEntries = static_cast<int64_t>(1) << 29;
+// The next size of a part that had `entries` list entries, which were too many.
+int64_t smaller_part(int64_t part, int64_t entries) {
+  const double fits = 0.85 * static_cast<double>(kSplitEntries) / static_cast<double>(entries);
+  return std::max<int64_t>(1, std::min(part / 2, static_cast<int64_t>(part * fits)));
+}
 
 // Front-to-back depth chunk boundaries of a batch of k_total sorted slots:
 // chunk ci covers positions [chunk_begin(ci), chunk_begin(ci + 1)).
@@ -811,10 +831,10 @@ int64_t chunk_end(int64_t k_total, int chunks, int ci) {
 }
 
 // Layout of the main pass's tile lists kept for the near-tie re-check: per
-// view batch and depth chunk, the list values and the ranges over the
-// batch's tiles; per batch tile, the chunk in which it saturated; per batch
-// and chunk, the last slot of the chunk.
-fs_status kept_layout(fs_ctx* c, const fs_camera* cams, int32_t V, int vb, int chunks) {
+// view batch and depth chunk (or part of one), the list values and the ranges
+// over the batch's tiles; per batch tile, the list in which it saturated; per
+// batch and list, the last slot of its positions.
+fs_status kept_layout(fs_ctx* c, const fs_camera* cams, int32_t V, int vb) {
   c->kl_tile_off.clear();
   int64_t tiles = 0;
   for (int32_t v0 = 0; v0 < V; v0 += vb) {
@@ -828,11 +848,13 @@ fs_status kept_layout(fs_ctx* c, const fs_camera* cams, int32_t V, int vb, int c
   }
   c->kl_tile_off.push_back(tiles);
   const size_t batches = c->kl_tile_off.size() - 1;
-  c->kl_chunks = chunks;
-  if (c->kl_val.size() < batches * chunks) c->kl_val.resize(batches * chunks);
-  FS_TRY(c->kl_ranges.ensure(static_cast<size_t>(tiles) * chunks * 8 + 8, "kept ranges"));
+  c->kl_parts.assign(batches, 0);
+  if (c->kl_val.size() < batches * fs::kMaxChunks) {
+    c->kl_val.resize(batches * fs::kMaxChunks);
+    c->kl_rng.resize(batches * fs::kMaxChunks);
+  }
   FS_TRY(c->kl_satc.ensure(static_cast<size_t>(tiles) + 8, "kept saturation chunks"));
-  FS_TRY(c->kl_bound.ensure(batches * chunks * 4 + 4, "kept chunk bounds"));
+  FS_TRY(c->kl_bound.ensure(batches * fs::kMaxChunks * 4, "kept chunk bounds"));
   return FS_OK;
 }
 
@@ -882,7 +904,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
   const int chunks = fs::ctx_depth_chunks(c, n, cams, V);
   FS_TRY(ensure_window(c, n, vb, V, keep));
   FS_TRY(stage_masks(c, cams, V, masks, mask_dtype, mask_memory, stream));
-  if (keep) FS_TRY(kept_layout(c, cams, V, vb, chunks));
+  if (keep) FS_TRY(kept_layout(c, cams, V, vb));
 
   unsigned long long* ctr = c->counters.as<unsigned long long>();
   const int batches = static_cast<int>((V + vb - 1) / vb);
@@ -970,7 +992,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
     return FS_OK;
   };
   FS_TRY(ensure_prologue_events(c));
-  bool split = false;
+  bool all_kept = true;
   if (overlap) FS_TRY(launch_prologue(0, stream));
   for (int32_t v0 = 0, b = 0; v0 < V; v0 += vb, ++b) {
     const int nb = std::min(vb, V - v0);
@@ -1049,50 +1071,50 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
     FS_TRY(stage_end(c, ts, stream));
     c->stats.views += nb;
     c->stats.pixels += L.pixels;
-    if (keep) {  // the last slot of every chunk but the last (0xFFFFFFFF: empty chunk)
-      uint32_t* bound = c->kl_bound.as<uint32_t>() + static_cast<int64_t>(b) * chunks;
-      FS_CUDA(cudaMemsetAsync(bound, 0xFF, static_cast<size_t>(chunks) * 4, stream), "bounds");
+    uint32_t* bound = nullptr;
+    if (keep) {  // the last slot of every list (0xFFFFFFFF: empty)
+      bound = c->kl_bound.as<uint32_t>() + static_cast<int64_t>(b) * fs::kMaxChunks;
+      FS_CUDA(cudaMemsetAsync(bound, 0xFF, fs::kMaxChunks * 4, stream), "bounds");
       if (plan)
         FS_CUDA(fs::launch_chunk_last(c->chunk_bnd.as<int64_t>(), chunks, sorted_val, bound,
                                       stream),
                 "bounds");
-      for (int ci = 0; ci + 1 < chunks && !plan; ++ci) {
-        const int64_t pb = ci == 0 ? 0 : chunk_end(k_vis, chunks, ci - 1);
-        const int64_t p1 = chunk_end(k_vis, chunks, ci);
-        if (p1 > pb)
-          FS_CUDA(cudaMemcpyAsync(bound + ci, sorted_val + (p1 - 1), 4, cudaMemcpyDeviceToDevice,
-                                  stream),
-                  "bounds");
-      }
     }
 
     // front-to-back depth chunks over the visible slots: a chunk lists only
-    // tiles not yet saturated
+    // tiles not yet saturated.  Chunks of the context's own choosing are taken
+    // in parts where they hold too many entries; every part is a list of its
+    // own to the re-check, as long as there are kMaxChunks of them at most.
     int64_t p0 = 0;
+    int part = 0;
     for (int ci = 0; ci < chunks; ++ci) {
       const size_t pi = static_cast<size_t>(b) * chunks + ci;
       const int64_t p1 = plan ? 0 : chunk_end(k_vis, chunks, ci);
       const int64_t n_pos = plan ? plan->npos[pi] : p1 - p0;
       if (record) record->npos[pi] = n_pos;
-      DevBuf* val_dst = keep ? &c->kl_val[static_cast<size_t>(b) * chunks + ci] : &c->lv_a;
-      uint2* ranges_dst =
-          keep ? c->kl_ranges.as<uint2>() + (c->kl_tile_off[b] * chunks +
-                                             static_cast<int64_t>(ci) * total_tiles)
-               : c->ranges.as<uint2>();
-      if (n_pos <= 0) {
+      int64_t want = std::max<int64_t>(n_pos, 1);  // positions of the next part
+      for (int64_t a0 = p0; a0 < p0 + n_pos || (n_pos <= 0 && a0 == p0);) {
+        if (part + (chunks - ci) > fs::kMaxChunks) {  // more lists than can be kept
+          part = fs::kMaxChunks - (chunks - ci);
+          all_kept = false;
+        }
+        const size_t slot = static_cast<size_t>(b) * fs::kMaxChunks + part;
+        DevBuf* val_dst = keep ? &c->kl_val[slot] : &c->lv_a;
         if (keep)
-          FS_CUDA(cudaMemsetAsync(ranges_dst, 0, static_cast<size_t>(total_tiles) * 8, stream),
-                  "ranges clear");
-        if (plan)  // the plan's chunk is empty: so must the replay's be
-          FS_CUDA(fs::launch_graph_check(nullptr, 0u, nullptr, 0, c->chunk_bnd.as<int64_t>() + ci,
-                                         0, ctr, stream),
-                  "plan check");
-        continue;
-      }
-      // a chunk of the context's own choosing is halved while it has too many
-      // entries (its parts are not kept for the re-check, which then bins anew)
-      for (int64_t a0 = p0, a1 = p0 + n_pos; a0 < p0 + n_pos;) {
-        const int64_t n_part = a1 - a0;
+          FS_TRY(c->kl_rng[slot].ensure(static_cast<size_t>(total_tiles) * 8, "kept ranges"));
+        uint2* ranges_dst = (keep ? c->kl_rng[slot] : c->ranges).as<uint2>();
+        if (n_pos <= 0) {
+          if (keep)
+            FS_CUDA(cudaMemsetAsync(ranges_dst, 0, static_cast<size_t>(total_tiles) * 8, stream),
+                    "ranges clear");
+          if (plan)  // the plan's chunk is empty: so must the replay's be
+            FS_CUDA(fs::launch_graph_check(nullptr, 0u, nullptr, 0,
+                                           c->chunk_bnd.as<int64_t>() + ci, 0, ctr, stream),
+                    "plan check");
+          ++part;
+          break;
+        }
+        const int64_t n_part = std::min(want, p0 + n_pos - a0);
         const int64_t limit =
             c->depth_chunks == 0 && !plan && !record && n_part > 1 ? kSplitEntries : 0;
         const bool live = ci > 0 && n_part >= kLiveMin && 5 * n_part >= k_total;
@@ -1102,31 +1124,37 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
                              plan ? c->chunk_bnd.as<int64_t>() + ci : nullptr,
                              plan ? plan->entries[pi] : 0));
         if (I < 0) {
-          a1 = a0 + n_part / 2;
-          split = true;
+          want = smaller_part(n_part, -I);
           continue;
         }
         if (record) record->entries[pi] = I;
-        a0 = a1;
-        a1 = p0 + n_pos;
+        a0 += n_part;
+        if (keep && !plan)
+          FS_CUDA(cudaMemcpyAsync(bound + part, sorted_val + (a0 - 1), 4,
+                                  cudaMemcpyDeviceToDevice, stream),
+                  "bounds");
+        const int list = part++;
         if (I == 0) continue;
         int tb = -1;
         FS_TRY(stage_begin(c, FS_STAGE_BLEND, stream, plan != nullptr, &tb));
         FS_CUDA(fs::launch_blend(vd, nb, max_tiles, ranges_dst, val_dst->as<uint32_t>(), P.rec,
                                  P.rec16, n, E, mask_dtype, table, table_dtype, state, sat, subsat,
-                                 satc, ci, ctr, c->census, stream),
+                                 satc, list, ctr, c->census, stream),
                 "blend");
         FS_TRY(stage_end(c, tb, stream));
       }
       p0 = p1;
     }
+    if (keep) c->kl_parts[b] = part;
   }
-  c->kl_valid = keep && !split;
+  c->kl_valid = keep && all_kept;
   return FS_OK;
 }
 
 // Dedicated binning of the tiles whose `skip` bit is clear (all depths, one
-// list per tile) and the re-check compositing of them into R.
+// list per tile) and the re-check compositing of them into R.  A list of more
+// than kSplitEntries entries, or one there is no memory for, is made for some
+// of the views at a time; `skip` then ends with the last views' tiles only.
 fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, int64_t kcap,
                               const BatchLayout& L, const fs::ViewParams* vd, const ProjPtrs& P,
                               uint64_t* skip, int32_t mask_dtype,
@@ -1139,44 +1167,67 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
   FS_TRY(c->ccnt.ensure(static_cast<size_t>(kcap) * 4, "candidate flags"));
   FS_TRY(c->offs.ensure(static_cast<size_t>(kcap) * 4, "candidate offsets"));
   FS_TRY(c->scan_tmp.ensure(fs::scan_temp_bytes(kcap), "scan temp"));
-  c->stats.kernel_launches += 1 + scan_launches(k_total);
-  FS_CUDA(fs::launch_candidates(k_total, n, vd, P.box, P.foot, skip, c->ccnt.as<uint32_t>(),
-                                stream),
-          "candidates");
-  FS_CUDA(fs::exclusive_scan(c->ccnt.as<uint32_t>(), nullptr, c->offs.as<uint32_t>(), k_total,
-                             c->total.as<uint32_t>(), c->scan_tmp.p, stream),
-          "candidate scan");
-  int64_t C = 0;
-  FS_TRY(read_total(c, stream, &C));
-  if (C == 0) return FS_OK;
-  c->stats.kernel_launches += 2 + radix_launches(C, 32);
-  FS_CUDA(fs::launch_compact(k_total, c->ccnt.as<uint32_t>(), c->offs.as<uint32_t>(), P.rec, P.rec16,
-                             c->key_b.as<uint32_t>(), c->val_b.as<uint32_t>(), stream),
-          "compact");
-  bool alt = false;
-  FS_CUDA(fs::radix_sort_pairs(c->key_b.as<uint32_t>(), c->val_b.as<uint32_t>(),
-                               c->key_a.as<uint32_t>(), c->val_a.as<uint32_t>(), C, 32,
-                               c->sort_tmp.p, &alt, stream, ctr),
-          "candidate sort");
-  uint32_t* sorted_key = alt ? c->key_a.as<uint32_t>() : c->key_b.as<uint32_t>();
-  uint32_t* sorted_val = alt ? c->val_a.as<uint32_t>() : c->val_b.as<uint32_t>();
-  FS_CUDA(fs::launch_depth_tie_fix(C, n, sorted_key, sorted_val, P.dlo, stream), "depth ties");
-  int64_t I = 0;
-  FS_TRY(bin_positions(c, 0, C, n, vd, nb, sorted_val, P, skip, total_tiles, tile_bits, kcap, false,
-                       &c->lv_a, c->ranges.as<uint2>(), stream, &I));
-  if (I == 0) return FS_OK;
-  fs::RecheckLists Ls{};
-  Ls.val[0] = c->lv_a.as<uint32_t>();
-  Ls.ranges[0] = c->ranges.as<uint2>();
-  Ls.chunks = 1;
-  Ls.flagged = F;
-  Ls.n_flagged = static_cast<int>(std::min<int64_t>(nF, 0x7FFFFFFF));
-  Ls.box = P.box;
-  Ls.foot = P.foot;
-  c->stats.kernel_launches += 2;
-  FS_CUDA(fs::launch_recheck_blend(vd, nb, L.max_tiles, Ls, skip, c->rk_tiles.p, c->n_sm, P.rec, P.rec16,
-                                   s->pos_op.as<float4>(), n, E, mask_dtype, map, R, ctr, stream),
-          "re-check blend");
+  int want = nb;  // views at a time
+  for (int g0 = 0; g0 < nb;) {
+    const int ng = std::min(want, nb - g0);
+    if (ng < nb) {  // only the tiles of views [g0, g0 + ng)
+      FS_CUDA(cudaMemsetAsync(skip, 0xFF, static_cast<size_t>((total_tiles + 63) / 64) * 8, stream),
+              "skip bits");
+      c->stats.kernel_launches += 1;
+      FS_CUDA(fs::launch_mark_tiles(nF, g0, ng, n, F, vd, P.box, P.foot, skip,
+                                    c->total.as<uint32_t>(), nullptr, 0, P.rec, P.rec16, P.dlo,
+                                    nullptr, nullptr, stream),
+              "mark tiles");
+    }
+    c->stats.kernel_launches += 1 + scan_launches(k_total);
+    FS_CUDA(fs::launch_candidates(k_total, n, vd, P.box, P.foot, skip, c->ccnt.as<uint32_t>(),
+                                  stream),
+            "candidates");
+    FS_CUDA(fs::exclusive_scan(c->ccnt.as<uint32_t>(), nullptr, c->offs.as<uint32_t>(), k_total,
+                               c->total.as<uint32_t>(), c->scan_tmp.p, stream),
+            "candidate scan");
+    int64_t C = 0;
+    FS_TRY(read_total(c, stream, &C));
+    if (C == 0) {
+      g0 += ng;
+      continue;
+    }
+    c->stats.kernel_launches += 2 + radix_launches(C, 32);
+    FS_CUDA(fs::launch_compact(k_total, c->ccnt.as<uint32_t>(), c->offs.as<uint32_t>(), P.rec,
+                               P.rec16, c->key_b.as<uint32_t>(), c->val_b.as<uint32_t>(), stream),
+            "compact");
+    bool alt = false;
+    FS_CUDA(fs::radix_sort_pairs(c->key_b.as<uint32_t>(), c->val_b.as<uint32_t>(),
+                                 c->key_a.as<uint32_t>(), c->val_a.as<uint32_t>(), C, 32,
+                                 c->sort_tmp.p, &alt, stream, ctr),
+            "candidate sort");
+    uint32_t* sorted_key = alt ? c->key_a.as<uint32_t>() : c->key_b.as<uint32_t>();
+    uint32_t* sorted_val = alt ? c->val_a.as<uint32_t>() : c->val_b.as<uint32_t>();
+    FS_CUDA(fs::launch_depth_tie_fix(C, n, sorted_key, sorted_val, P.dlo, stream), "depth ties");
+    int64_t I = 0;
+    FS_TRY(bin_positions(c, 0, C, n, vd, nb, sorted_val, P, skip, total_tiles, tile_bits, kcap,
+                         false, &c->lv_a, c->ranges.as<uint2>(), stream, &I, nullptr, false,
+                         ng > 1 ? kSplitEntries : 0));
+    if (I < 0) {
+      want = static_cast<int>(smaller_part(ng, -I));
+      continue;
+    }
+    g0 += ng;
+    if (I == 0) continue;
+    fs::RecheckLists Ls{};
+    Ls.val[0] = c->lv_a.as<uint32_t>();
+    Ls.ranges[0] = c->ranges.as<uint2>();
+    Ls.chunks = 1;
+    Ls.flagged = F;
+    Ls.n_flagged = static_cast<int>(std::min<int64_t>(nF, 0x7FFFFFFF));
+    Ls.box = P.box;
+    Ls.foot = P.foot;
+    c->stats.kernel_launches += 2;
+    FS_CUDA(fs::launch_recheck_blend(vd, nb, L.max_tiles, Ls, skip, c->rk_tiles.p, c->n_sm, P.rec,
+                                     P.rec16, s->pos_op.as<float4>(), n, E, mask_dtype, map, R,
+                                     ctr, stream),
+            "re-check blend");
+  }
   return FS_OK;
 }
 
@@ -1231,7 +1282,6 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
   const int vb = batch_views(c, n);
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   const int64_t kcap = static_cast<int64_t>(vb) * n;
-  const int chunks = K->kl_chunks;
   fs::ViewParams* vh = c->views_host.as<fs::ViewParams>();
   unsigned long long* ctr = c->counters.as<unsigned long long>();
   unsigned long long* ctr_h = c->counters_host.as<unsigned long long>();
@@ -1262,10 +1312,11 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
     FS_CUDA(cudaMemsetAsync(deep, 0, sat_bytes, stream), "deep bits");
     FS_CUDA(cudaMemsetAsync(c->total.p, 0, sizeof(uint32_t), stream), "visible clear");
     const uint8_t* satc = kept ? K->kl_satc.as<uint8_t>() + K->kl_tile_off[b] : nullptr;
-    const uint32_t* bound = kept ? K->kl_bound.as<uint32_t>() + static_cast<int64_t>(b) * chunks
-                                 : nullptr;
+    const int chunks = kept ? K->kl_parts[b] : 0;
+    const uint32_t* bound =
+        kept ? K->kl_bound.as<uint32_t>() + static_cast<int64_t>(b) * fs::kMaxChunks : nullptr;
     c->stats.kernel_launches += 1;
-    FS_CUDA(fs::launch_mark_tiles(nF, nb, n, F, vd, P.box, P.foot, skip, c->total.as<uint32_t>(),
+    FS_CUDA(fs::launch_mark_tiles(nF, 0, nb, n, F, vd, P.box, P.foot, skip, c->total.as<uint32_t>(),
                                   bound, chunks, P.rec, P.rec16, P.dlo, satc, deep, stream),
             "mark tiles");
     int64_t visible = 0;
@@ -1275,9 +1326,9 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
       // walk the main pass's kept chunk lists
       fs::RecheckLists Ls{};
       for (int ci = 0; ci < chunks; ++ci) {
-        Ls.val[ci] = K->kl_val[static_cast<size_t>(b) * chunks + ci].as<uint32_t>();
-        Ls.ranges[ci] = K->kl_ranges.as<uint2>() +
-                        (K->kl_tile_off[b] * chunks + static_cast<int64_t>(ci) * total_tiles);
+        const size_t slot = static_cast<size_t>(b) * fs::kMaxChunks + ci;
+        Ls.val[ci] = K->kl_val[slot].as<uint32_t>();
+        Ls.ranges[ci] = K->kl_rng[slot].as<uint2>();
       }
       Ls.chunks = chunks;
       Ls.sat_chunk = satc;

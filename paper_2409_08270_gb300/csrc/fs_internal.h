@@ -178,13 +178,13 @@ cudaError_t launch_flag_margin(int64_t n, const float* margin, float tau, uint32
 // F[offs[i]] = i and map[i] = offs[i] for flagged i; map[i] = -1 otherwise
 cudaError_t launch_scatter_flagged(int64_t n, const uint32_t* flag, const uint32_t* offs,
                                    uint32_t* F, int32_t* map, cudaStream_t stream);
-// clears the skip bits of every tile a flagged Gaussian reaches in the batch;
-// *visible += the number of visible (view, flagged Gaussian) pairs.  With
+// clears the skip bits of every tile a flagged Gaussian reaches in the batch's
+// views [v_begin, v_begin + n_views); *visible += the number of visible (view, flagged Gaussian) pairs.  With
 // kept chunk lists (bound: the last slot of each depth chunk; rec / rec16 and
 // dlo: the batch's records and low depth words, which order its slots; sat_chunk: the chunk in which each tile
 // saturated, 0xFF = never), sets the `deep` bit of every tile that saturated
 // before the flagged Gaussian's own chunk.  bound == NULL: no kept lists.
-cudaError_t launch_mark_tiles(int64_t n_flagged, int n_views, int64_t n, const uint32_t* F,
+cudaError_t launch_mark_tiles(int64_t n_flagged, int v_begin, int n_views, int64_t n, const uint32_t* F,
                               const ViewParams* views, const TileBox* box, const Footprint* foot,
                               uint64_t* skip, uint32_t* visible, const uint32_t* bound,
                               int chunks, const ProjRecord* rec, const CompactRecord* rec16,

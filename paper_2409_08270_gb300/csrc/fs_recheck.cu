@@ -84,7 +84,7 @@ __device__ __forceinline__ bool order_le(uint32_t a, uint32_t b, int64_t n,
 // counts the visible (view, re-checked Gaussian) pairs in *visible.  With
 // kept chunk lists (bound != NULL), a tile that saturated in an earlier chunk
 // than the re-checked Gaussian's own gets its `deep` bit set.
-__global__ void mark_tiles_kernel(int64_t n_flagged, int n_views, int64_t n,
+__global__ void mark_tiles_kernel(int64_t n_flagged, int v_begin, int n_views, int64_t n,
                                   const uint32_t* __restrict__ F,
                                   const ViewParams* __restrict__ views,
                                   const TileBox* __restrict__ box,
@@ -99,7 +99,7 @@ __global__ void mark_tiles_kernel(int64_t n_flagged, int n_views, int64_t n,
                                   unsigned long long* __restrict__ deep) {
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= n_flagged * n_views) return;
-  const int v = static_cast<int>(idx / n_flagged);
+  const int v = v_begin + static_cast<int>(idx / n_flagged);
   const int64_t slot = static_cast<int64_t>(v) * n + F[idx % n_flagged];
   if (!box_visible(box[slot])) return;
   atomicAdd(visible, 1u);
@@ -572,7 +572,7 @@ cudaError_t launch_scatter_flagged(int64_t n, const uint32_t* flag, const uint32
   return cudaGetLastError();
 }
 
-cudaError_t launch_mark_tiles(int64_t n_flagged, int n_views, int64_t n, const uint32_t* F,
+cudaError_t launch_mark_tiles(int64_t n_flagged, int v_begin, int n_views, int64_t n, const uint32_t* F,
                               const ViewParams* views, const TileBox* box, const Footprint* foot,
                               uint64_t* skip, uint32_t* visible, const uint32_t* bound,
                               int chunks, const ProjRecord* rec, const CompactRecord* rec16,
@@ -581,7 +581,8 @@ cudaError_t launch_mark_tiles(int64_t n_flagged, int n_views, int64_t n, const u
   const int64_t total = n_flagged * n_views;
   if (total == 0) return cudaSuccess;
   mark_tiles_kernel<<<blocks_for(total, 256), 256, 0, stream>>>(
-      n_flagged, n_views, n, F, views, box, foot, reinterpret_cast<unsigned long long*>(skip),
+      n_flagged, v_begin, n_views, n, F, views, box, foot,
+      reinterpret_cast<unsigned long long*>(skip),
       visible, bound, chunks, rec, rec16, dlo, sat_chunk, reinterpret_cast<unsigned long long*>(deep));
   return cudaGetLastError();
 }
