@@ -1116,13 +1116,16 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
         }
         const int64_t n_part = std::min(want, p0 + n_pos - a0);
         const int64_t limit =
-            c->depth_chunks == 0 && !plan && !record && n_part > 1 ? kSplitEntries : 0;
+            c->depth_chunks == 0 && !plan && n_part > 1 ? kSplitEntries : 0;
         const bool live = ci > 0 && n_part >= kLiveMin && 5 * n_part >= k_total;
         int64_t I = 0;
         FS_TRY(bin_positions(c, a0, n_part, n, vd, nb, sorted_val, P, sat, total_tiles, tile_bits,
                              kcap, !plan, val_dst, ranges_dst, stream, &I, nullptr, live, limit,
                              plan ? c->chunk_bnd.as<int64_t>() + ci : nullptr,
                              plan ? plan->entries[pi] : 0));
+        if (I < 0 && record)  // a plan's chunks are cut by the replay's counts alone
+          return fail(FS_UNSUPPORTED, "%lld list entries in one chunk of a captured solve",
+                      (long long)-I);
         if (I < 0) {
           want = smaller_part(n_part, -I);
           continue;
@@ -1823,8 +1826,11 @@ fs_status fs_graph_create(fs_ctx* tmpl, const fs_scene* s, const fs_camera* cams
                            g->keep, g->stream, &g->plan, nullptr);
   };
   st = record();
-  if (st == FS_UNSUPPORTED && c->depth_chunks == 0) {
-    // too many entries for the chunks its size suggests: the most there are
+  if ((st == FS_UNSUPPORTED || st == FS_OUT_OF_MEMORY) && c->depth_chunks == 0) {
+    // more entries than a list of the chunks its size suggests may have, or
+    // than there is memory for: as many chunks as there can be
+    for (DevBuf* b : {&c->lk_a, &c->lv_a, &c->lk_b, &c->lv_b}) b->release();
+    for (DevBuf& b : c->kl_val) b.release();
     c->depth_chunks = fs::kMaxChunks;
     st = record();
   }

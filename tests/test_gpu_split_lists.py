@@ -54,6 +54,40 @@ def test_more_entries_than_one_list_holds():
     _same(_solve(*work, recheck_reproject=True, **kw), six)  # the re-check bins by views
 
 
+def test_captured_solve_fits_where_six_chunks_do():
+    """A capture's plan cannot cut its chunks: it takes more of them instead."""
+    import torch
+    from paper_2409_08270_gb300 import flashsplat
+    g, cams, masks = _workload(125_000, 256, 0.38)
+    six = _solve(g, cams, masks, depth_chunks=6, recheck_margin=1e-4)
+
+    def captured(chunks, held_to=None):
+        s = flashsplat.Solver(g, depth_chunks=chunks, recheck_margin=1e-4)
+        held = graph = None
+        try:
+            dm = s.upload_masks(masks)
+            torch.cuda.synchronize()
+            free = torch.cuda.mem_get_info()[0]
+            if held_to:
+                held = torch.empty(free - held_to, dtype=torch.uint8, device="cuda")
+            graph = s.capture(cams, dm, 2, 0.0, table_dtype="float64")
+            used = free - torch.cuda.mem_get_info()[0]
+            graph.launch()
+            graph.synchronize()
+            out = graph.outputs
+            return used, (out["table"].cpu().numpy(), out["bits"].cpu().numpy())
+        finally:
+            if graph is not None:
+                graph.close()
+            s.close()
+            del held
+            torch.cuda.empty_cache()
+
+    used, first = captured(6)
+    _same(first, six)
+    _same(captured(0, used + used // 5)[1], six)
+
+
 def test_lists_that_do_not_fit_in_memory():
     """With no more memory than six chunks take and a fifth."""
     import torch
