@@ -201,6 +201,7 @@ fs_status solve_with_graph(fs_server* s, int slot, SceneEntry& se, Request* r,
     }
     fs_status status = FS_OK;
     if (e != cudaSuccess) {
+      cudaGetLastError();  // not the next launch's error: the request may be tried again
       status = fail(FS_OUT_OF_MEMORY, std::string("captured solve buffers: ") +
                                           cudaGetErrorString(e));
     } else {
