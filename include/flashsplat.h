@@ -345,7 +345,12 @@ fs_status fs_check_wait_timeout(int32_t device, int32_t spins);
  * fs_test_tile_ranges: for n keys in non-decreasing order (device uint32,
  *   each < n_tiles, checked on the host), ranges (device, n_tiles pairs of
  *   uint32) receives per tile t the run [first, last + 1) of key t, and
- *   [0, 0) for a tile without an entry. */
+ *   [0, 0) for a tile without an entry.
+ * fs_test_wait_timeout: while `on`, every call on the context counts one
+ *   bounded wait of its kernels as run out, so fs_keep_after_removal,
+ *   fs_render_masks, and fs_synchronize after fs_accumulate or fs_solve
+ *   return FS_TIMEOUT. */
+fs_status fs_test_wait_timeout(fs_ctx* ctx, int32_t on);
 fs_status fs_test_sort_pairs(int32_t device, uint32_t* keys, uint32_t* vals, int64_t n,
                              int32_t bits);
 fs_status fs_test_exclusive_scan(int32_t device, const uint32_t* in, uint32_t* out, int64_t n,

@@ -196,9 +196,10 @@ struct fs_ctx {
   bool recheck_reproject = false;
   bool compact = false;  // reduced-precision records (FP16 whitening matrix, FP32 mean)
   bool census = false;   // blend counts its pairs (slower variant)
+  bool test_timeout = false;  // calls count one bounded wait as run out (test hook)
   bool sigma3 = false;   // 3-sigma tile coverage (per-slot tile columns in `cols`)
   DevBuf rk_flag, rk_offs, rk_F, rk_map, rk_R, rk_Rb, rk_tiles, cols;
-  DevBuf rd_val, render_out;  // novel-view mask rendering
+  DevBuf rd_val, render_out, rd_counters;  // novel-view mask rendering
   DevBuf chunk_bnd;                             // captured solves: chunk boundaries
   HostBuf render_out_host;
   DevBuf key_range;  // min / max visible depth key of the batch (two slots, by batch parity)
@@ -391,7 +392,7 @@ fs_status fs_destroy(fs_ctx* c) {
                     &c->rk_Rb, &c->rk_tiles, &c->kl_satc, &c->kl_bound, &c->key_range,
                     &c->lb_tmp,
                     &c->key_a2, &c->val_a2, &c->key_b2, &c->val_b2, &c->cols,
-                    &c->rd_val, &c->render_out, &c->chunk_bnd,
+                    &c->rd_val, &c->render_out, &c->rd_counters, &c->chunk_bnd,
                     &c->free_tab, &c->live, &c->live_val, &c->live_range};
   for (DevBuf& b : c->kl_val) b.release();
   for (DevBuf& b : c->kl_rng) b.release();
@@ -674,6 +675,17 @@ fs_status read_total(fs_ctx* c, cudaStream_t stream, int64_t* out) {
           "count readback");
   FS_CUDA(cudaStreamSynchronize(stream), "count readback");
   *out = *total_h;
+  return FS_OK;
+}
+
+// Clears a call's device counters (kNumCounters of them).
+fs_status clear_counters(fs_ctx* c, void* counters, cudaStream_t stream) {
+  const size_t word = sizeof(unsigned long long);
+  FS_CUDA(cudaMemsetAsync(counters, 0, word * fs::kNumCounters, stream), "counters clear");
+  if (c->test_timeout)
+    FS_CUDA(cudaMemsetAsync(static_cast<unsigned long long*>(counters) + fs::kLookbackTimeout, 1,
+                            word, stream),
+            "counters clear");
   return FS_OK;
 }
 
@@ -1410,6 +1422,18 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
     }
     return FS_OK;
   }
+  // the sorts, compactions and binnings count in words of the call's own, read
+  // back with each batch: a solve before it may not have been synchronised yet
+  const size_t ctr_bytes = sizeof(unsigned long long) * fs::kNumCounters;
+  FS_TRY(c->rd_counters.ensure(ctr_bytes, "render counters"));
+  FS_TRY(clear_counters(c, c->rd_counters.p, stream));
+  struct OwnCounters {
+    fs_ctx* c;
+    explicit OwnCounters(fs_ctx* ctx) : c(ctx) { std::swap(c->counters, c->rd_counters); }
+    ~OwnCounters() { std::swap(c->counters, c->rd_counters); }
+  } own_counters(c);
+  unsigned long long* const ctr_h =
+      reinterpret_cast<unsigned long long*>(c->total_host.as<char>() + 64);
   const int vb = batch_views(c, n);
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   if (vb < 1) return fail(FS_UNSUPPORTED, "fs_render_masks: scene too large");
@@ -1494,7 +1518,13 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
     }
     // the host staging of this batch is read by the copies above before the
     // next batch rewrites it
+    FS_CUDA(cudaMemcpyAsync(ctr_h, c->counters.p, ctr_bytes, cudaMemcpyDeviceToHost, stream),
+            "counters readback");
     FS_CUDA(cudaStreamSynchronize(stream), "render");
+    if (ctr_h[fs::kLookbackTimeout])
+      return fail(FS_TIMEOUT, "fs_render_masks: a bounded wait of a sort or the binning gave up");
+    if (ctr_h[fs::kBinningMismatch])
+      return fail(FS_CUDA_ERROR, "fs_render_masks: internal binning mismatch");
   }
   return FS_OK;
 }
@@ -1514,7 +1544,7 @@ fs_status fs_accumulate(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   c->stats = fs_stats{};
   c->events_used = 0;
-  FS_CUDA(cudaMemsetAsync(c->counters.p, 0, c->counters.bytes, st), "counters clear");
+  FS_TRY(clear_counters(c, c->counters.p, st));
   return accumulate_impl(c, s, cams, V, masks, mask_dtype, mask_memory, E, table, table_dtype,
                          false, st);
 }
@@ -1584,7 +1614,7 @@ fs_status fs_solve(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32_t 
   }
   c->stats = fs_stats{};
   c->events_used = 0;
-  FS_CUDA(cudaMemsetAsync(c->counters.p, 0, c->counters.bytes, st), "counters clear");
+  FS_TRY(clear_counters(c, c->counters.p, st));
   if (tbytes) FS_CUDA(cudaMemsetAsync(table, 0, tbytes, st), "table clear");
   const bool recheck = c->recheck_margin > 0.f && n > 0 && V > 0;
   // keep every view's projection resident for the re-check when it fits in
@@ -1674,7 +1704,7 @@ fs_status fs_keep_after_removal(fs_ctx* c, const uint64_t* member_bits, int64_t 
   int64_t* const rng = c->live_range.as<int64_t>();
   unsigned long long* const ctr = reinterpret_cast<unsigned long long*>(rng + 2);
   const size_t back = 16 + sizeof(unsigned long long) * fs::kNumCounters;
-  FS_CUDA(cudaMemsetAsync(ctr, 0, back - 16, st), "counters clear");
+  FS_TRY(clear_counters(c, ctr, st));
   FS_CUDA(fs::launch_keep(n, member_bits, remove, keep_index, rng, c->lb_tmp.p, ctr, st),
           "removal");
   c->stats.kernel_launches += 1;
@@ -1731,7 +1761,7 @@ void graph_free(fs_graph* g) {
 fs_status graph_body(fs_graph* g, cudaStream_t st) {
   fs_ctx* c = g->c;
   const int64_t n = g->s->n;
-  FS_CUDA(cudaMemsetAsync(c->counters.p, 0, c->counters.bytes, st), "counters clear");
+  FS_TRY(clear_counters(c, c->counters.p, st));
   FS_CUDA(cudaMemsetAsync(g->table, 0, static_cast<size_t>(n) * g->E * 8, st), "table clear");
   FS_TRY(accumulate_impl(c, g->s, g->cams.data(), static_cast<int32_t>(g->cams.size()),
                          g->masks.data(), g->mask_dtype, FS_MEM_DEVICE, g->E, g->table, FS_F64,
@@ -1868,7 +1898,7 @@ fs_status fs_graph_launch(fs_graph* g, void* stream) {
     fs_ctx* rc = g->rc;
     rc->stats = fs_stats{};
     rc->events_used = 0;
-    FS_CUDA(cudaMemsetAsync(rc->counters.p, 0, rc->counters.bytes, st), "counters clear");
+    FS_TRY(clear_counters(rc, rc->counters.p, st));
     FS_TRY(recheck_impl(rc, g->s, g->cams.data(), V, g->mask_dtype, g->E, g->gamma, g->table,
                         FS_F64, g->bits, g->label, g->margin, g->keep, st,
                         g->keep ? g->c : nullptr));
@@ -1961,6 +1991,12 @@ fs_status test_device(int32_t device, const char* what) {
 }
 
 }  // namespace
+
+fs_status fs_test_wait_timeout(fs_ctx* c, int32_t on) {
+  if (!c) return fail(FS_INVALID_ARGUMENT, "fs_test_wait_timeout: NULL context");
+  c->test_timeout = on != 0;
+  return FS_OK;
+}
 
 fs_status fs_test_sort_pairs(int32_t device, uint32_t* keys, uint32_t* vals, int64_t n,
                              int32_t bits) {

@@ -32,8 +32,8 @@ STATUS_NAMES = {0: "FS_OK", 1: "FS_INVALID_ARGUMENT", 2: "FS_OUT_OF_MEMORY", 3: 
 EXPORTS = ["fs_version", "fs_last_error", "fs_create", "fs_destroy", "fs_scene_create",
            "fs_scene_destroy", "fs_scene_size", "fs_accumulate", "fs_assign", "fs_solve",
            "fs_synchronize", "fs_keep_after_removal", "fs_check_wait_timeout", "fs_render_masks",
-           "fs_test_sort_pairs", "fs_test_exclusive_scan", "fs_test_tile_ranges",
-           "fs_graph_create", "fs_graph_launch", "fs_graph_synchronize", "fs_graph_destroy",
+           "fs_test_wait_timeout", "fs_test_sort_pairs", "fs_test_exclusive_scan",
+           "fs_test_tile_ranges", "fs_graph_create", "fs_graph_launch", "fs_graph_synchronize", "fs_graph_destroy",
            "fs_solve_noalloc", "fs_server_create", "fs_server_add_scene",
            "fs_server_submit", "fs_server_fetch", "fs_server_fetch_for", "fs_server_cancel",
            "fs_server_destroy"]
@@ -137,6 +137,7 @@ def load(path: str | None = None):
                            i32, f32, ctypes.POINTER(fs_result), vp]),
         "fs_synchronize": (i32, [vp, vp, ctypes.POINTER(fs_stats)]),
         "fs_check_wait_timeout": (i32, [i32, i32]),
+        "fs_test_wait_timeout": (i32, [vp, i32]),
         "fs_test_sort_pairs": (i32, [i32, vp, vp, i64, i32]),
         "fs_test_exclusive_scan": (i32, [i32, vp, vp, i64, ctypes.POINTER(ctypes.c_uint32)]),
         "fs_test_tile_ranges": (i32, [i32, vp, i64, i32, vp]),
@@ -245,6 +246,11 @@ def fs_synchronize(ctx, stream=0) -> fs_stats:
 def fs_check_wait_timeout(device: int, spins: int) -> int:
     """Status of the bounded-wait diagnostic (FS_TIMEOUT expected)."""
     return load().fs_check_wait_timeout(device, spins)
+
+
+def fs_test_wait_timeout(ctx: int, on: bool) -> None:
+    """While on, calls on the context count one bounded wait as run out."""
+    check(load().fs_test_wait_timeout(ctx, 1 if on else 0))
 
 
 def fs_test_sort_pairs(device: int, keys, vals, bits: int) -> None:
