@@ -57,3 +57,19 @@ def test_a_render_keeps_an_unfinished_solves_counters():
         assert st.bad_labels == 14
     finally:
         s.close()
+
+
+def test_the_wait_limit_is_seconds():
+    """The limit on the polls of a look-back wait amounts to some two seconds,
+    by the time a sixteenth of them takes (at most a quarter of a second)."""
+    import os
+    import re
+    import time
+    from paper_2409_08270_gb300 import build, flashsplat as fsb
+    build.build()
+    text = open(os.path.join(build.CSRC, "fs_internal.h")).read()
+    polls = 1 << int(re.search(r"kLookbackSpinLimit = 1 << (\d+)", text).group(1))
+    assert fsb.fs_check_wait_timeout(0, 1) == fsb.FS_TIMEOUT
+    t = time.perf_counter()
+    assert fsb.fs_check_wait_timeout(0, polls // 16) == fsb.FS_TIMEOUT
+    assert time.perf_counter() - t < 0.25
