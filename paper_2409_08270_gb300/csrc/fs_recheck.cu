@@ -405,8 +405,10 @@ __global__ void __launch_bounds__(32 * kRWarps, 8) recheck_blend_kernel(
     const float ry = 4.f * static_cast<float>(sub >> 1) - 6.f;
     const uint32_t slot0 = static_cast<uint32_t>(static_cast<int64_t>(view) * n);
 
-    // can the slot reach one of the piece's pixel centres? (FP32, with the
-    // slack of the per-pixel screen)
+    // can the slot reach one of the piece's pixel centres?  (FP32: the rows'
+    // products are off by less than 2^-21 of their terms' sizes, which is taken
+    // off them, so that means any distance away lose no pixel; the rest is
+    // within the slack of the per-pixel screen)
     auto meets = [&](uint32_t slot) -> bool {
       float4 w;
       float bx, by, qc;
@@ -426,10 +428,12 @@ __global__ void __launch_bounds__(32 * kRWarps, 8) recheck_blend_kernel(
         by = ((cy + ry) - m.y) - m.w;
         qc = r.misc.y;
       }
+      const float rel = 0x1p-21f;
+      const float sx = fmaf(rel, fabsf(bx), 3.5f), sy = fmaf(rel, fabsf(by), 1.5f);
       const float d0 = fmaxf(0.f, fabsf(fmaf(w.x, bx, w.y * by)) -
-                                      fmaf(fabsf(w.x), 3.5f, fabsf(w.y) * 1.5f));
+                                      fmaf(fabsf(w.x), sx, fabsf(w.y) * sy));
       const float d1 = fmaxf(0.f, fabsf(fmaf(w.z, bx, w.w * by)) -
-                                      fmaf(fabsf(w.z), 3.5f, fabsf(w.w) * 1.5f));
+                                      fmaf(fabsf(w.z), sx, fabsf(w.w) * sy));
       return fmaf(d0, d0, d1 * d1) <= qc + 0.05f;
     };
     // ring entries first .. first + count - 1 into the stage, one per lane
