@@ -111,10 +111,14 @@ __global__ void __launch_bounds__(kRenderThreads, 8) render_kernel(
       }
       s_w[threadIdx.x] = w;
       s_m[threadIdx.x] = m;
-      // sub-tile q: pixel centres within 3.5 of its own centre; q_cut carries
-      // the slack for the rounding of this test
-      const float h0 = fmaf(fabsf(w.x), 3.5f, fabsf(w.y) * 3.5f);
-      const float h1 = fmaf(fabsf(w.z), 3.5f, fabsf(w.w) * 3.5f);
+      // sub-tile q: pixel centres within 3.5 of its own centre.  This test's rows
+      // and a pixel's are each off by less than 2^-21 of their terms' sizes
+      // (|p - m| <= the tile centre's + 8), taken off here: means any distance
+      // away lose no pixel that its own evaluation would take
+      const float ex = fmaf(0x1p-20f, fabsf((tcx + 8.f) - m.x) + 8.f, 3.5f);
+      const float ey = fmaf(0x1p-20f, fabsf((tcy + 8.f) - m.y) + 8.f, 3.5f);
+      const float h0 = fmaf(fabsf(w.x), ex, fabsf(w.y) * ey);
+      const float h1 = fmaf(fabsf(w.z), ex, fabsf(w.w) * ey);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const float dx = ((tcx + 8.f * (q & 1) + 4.f) - m.x) - m.z;
