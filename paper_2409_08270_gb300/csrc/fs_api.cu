@@ -276,6 +276,19 @@ void fs::ctx_set_batching(fs_ctx* c, int views_per_batch, int depth_chunks) {
   if (depth_chunks >= 0) c->depth_chunks = std::min(depth_chunks, 16);
 }
 
+// Tiles of a view, on average.
+static double mean_tiles(const fs_camera* cams, int32_t V) {
+  double tiles = 0;
+  for (int32_t v = 0; v < V; ++v)
+    tiles += static_cast<double>((cams[v].width + fs::kTile - 1) / fs::kTile) *
+             ((cams[v].height + fs::kTile - 1) / fs::kTile);
+  return tiles / std::max(V, 1);
+}
+
+double fs::entries_per_slot(const fs_camera* cams, int32_t V) {
+  return 3.0 + mean_tiles(cams, V) / 350.0;
+}
+
 // Front-to-back depth chunks of a solve (sizes 1/32, 1/32, 1/16, ..., 1/2 of a
 // batch's visible slots with six): the context's setting, or by the solve's
 // size.  A chunk costs its launches, a readback and the blend's start on every
@@ -300,22 +313,22 @@ void fs::ctx_set_batching(fs_ctx* c, int views_per_batch, int depth_chunks) {
 //   1.5M, 1600x1200           39.01  26.43  19.72  16.40  15.10  14.88  15.43
 // and for 3M Gaussians in 100 views of 1256x828, the re-check included, 158
 // 118  97  86.1  79.8  77.2 (7: 76.5) 76.6.
-int fs::ctx_depth_chunks(const fs_ctx* c, int64_t n, const fs_camera* cams, int32_t V) {
-  if (c->depth_chunks > 0) return std::min(c->depth_chunks, fs::kMaxChunks);
+int fs::chunks_by_size(int views_per_batch, int64_t n, const fs_camera* cams, int32_t V) {
   if (n <= 0 || V <= 0) return 1;
-  double tiles = 0;  // mean over the views
-  for (int32_t v = 0; v < V; ++v)
-    tiles += static_cast<double>((cams[v].width + fs::kTile - 1) / fs::kTile) *
-             ((cams[v].height + fs::kTile - 1) / fs::kTile);
-  tiles /= V;
-  const double views = std::min<double>(c->views_per_batch, V);
-  const double entries = views * static_cast<double>(n) * (3.0 + tiles / 350.0);
+  const double tiles = mean_tiles(cams, V);
+  const double views = std::min(views_per_batch, V);
+  const double entries = views * static_cast<double>(n) * fs::entries_per_slot(cams, V);
   const double by_depth = 3.0 + 1.3 * log2(static_cast<double>(n) / 3e5) -
                           0.9 * std::max(0.0, log2(3000.0 / tiles));
   const double per_chunk = 5.6e7 * pow(3e5 / static_cast<double>(n), 0.6);
   const double chunks =
       std::min({std::floor(by_depth + 0.5), std::floor(1.0 + entries / per_chunk), 8.0});
   return std::max(1, static_cast<int>(chunks));
+}
+
+int fs::ctx_depth_chunks(const fs_ctx* c, int64_t n, const fs_camera* cams, int32_t V) {
+  if (c->depth_chunks > 0) return std::min(c->depth_chunks, fs::kMaxChunks);
+  return chunks_by_size(c->views_per_batch, n, cams, V);
 }
 
 extern "C" {
@@ -624,10 +637,10 @@ BatchLayout layout_batch(fs_ctx* c, fs::ViewParams* vh, const fs_camera* cams, i
   return L;
 }
 
-// Views per batch: (view, Gaussian) slots of one batch must fit in 31 bits.
-int batch_views(const fs_ctx* c, int64_t n) {
+// Views per batch of V: (view, Gaussian) slots of one batch must fit in 31 bits.
+int batch_views(const fs_ctx* c, int64_t n, int32_t V) {
   const int64_t max_vb = ((static_cast<int64_t>(1) << 31) - 1) / n;
-  return static_cast<int>(std::min<int64_t>(c->views_per_batch, max_vb));
+  return static_cast<int>(std::min<int64_t>(std::min(c->views_per_batch, V), max_vb));
 }
 
 // Projection storage of a batch: either the batch window (slot = view in
@@ -909,7 +922,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
   const int64_t n = s->n;
   c->kl_valid = false;
   if (n == 0 || V == 0) return FS_OK;
-  const int vb = batch_views(c, n);
+  const int vb = batch_views(c, n, V);
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   if (vb < 1) return fail(FS_UNSUPPORTED, "fs_accumulate: scene too large");
   const int64_t kcap = static_cast<int64_t>(vb) * n;
@@ -1294,7 +1307,7 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
     Rb = c->rk_Rb.as<double>();
   }
 
-  const int vb = batch_views(c, n);
+  const int vb = batch_views(c, n, V);
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   const int64_t kcap = static_cast<int64_t>(vb) * n;
   fs::ViewParams* vh = c->views_host.as<fs::ViewParams>();
@@ -1434,7 +1447,7 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
   } own_counters(c);
   unsigned long long* const ctr_h =
       reinterpret_cast<unsigned long long*>(c->total_host.as<char>() + 64);
-  const int vb = batch_views(c, n);
+  const int vb = batch_views(c, n, V);
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   if (vb < 1) return fail(FS_UNSUPPORTED, "fs_render_masks: scene too large");
   const int64_t kcap = static_cast<int64_t>(vb) * n;
@@ -1839,7 +1852,7 @@ fs_status fs_graph_create(fs_ctx* tmpl, const fs_scene* s, const fs_camera* cams
   g->keep = g->recheck && keep_fits(c, n, V);
   if (g->recheck) {
     if ((st = fs_create(&g->rc, tmpl->device, &o)) != FS_OK) return bail(st);
-    const int vbr = batch_views(g->rc, n);
+    const int vbr = batch_views(g->rc, n, V);
     if ((st = ensure_window(g->rc, n, vbr, V, false)) != FS_OK) return bail(st);
     if ((st = stage_masks(g->rc, cams, V, masks, mask_dtype, FS_MEM_DEVICE, nullptr)) != FS_OK)
       return bail(st);
@@ -1867,7 +1880,7 @@ fs_status fs_graph_create(fs_ctx* tmpl, const fs_scene* s, const fs_camera* cams
   if (st != FS_OK) return bail(st);
   if ((ce = cudaStreamSynchronize(g->stream)) != cudaSuccess)
     return bail(cuda_fail(ce, "fs_graph_create"));
-  const int vb = batch_views(c, n);
+  const int vb = batch_views(c, n, V);
   const size_t batches = static_cast<size_t>((V + vb - 1) / vb);
   if ((st = g->plan.views.ensure(batches * fs::kMaxViewsPerBatch * sizeof(fs::ViewParams))) !=
       FS_OK)

@@ -258,6 +258,10 @@ void ctx_release_workspace(fs_ctx* c);
 void ctx_set_batching(fs_ctx* c, int views_per_batch, int depth_chunks);
 // Depth chunks a solve of n Gaussians in V views takes in this context.
 int ctx_depth_chunks(const fs_ctx* c, int64_t n, const fs_camera* cams, int32_t V);
+// The same by the solve's size alone, and the list entries of a (view, Gaussian)
+// slot it reckons with, were no tile saturated.
+int chunks_by_size(int views_per_batch, int64_t n, const fs_camera* cams, int32_t V);
+double entries_per_slot(const fs_camera* cams, int32_t V);
 
 // View parameters of a camera (fs_api.cu): float pairs of R, t and the
 // intrinsics, near plane 0.2, Jacobian clamp 1.3 tan(half field of view),

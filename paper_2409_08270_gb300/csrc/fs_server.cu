@@ -65,12 +65,19 @@ struct SceneEntry {
 };
 
 // Device bytes a request needs while it runs: the context's per-batch
-// window (records, footprints, keys, list entries), the FP64 table and its
-// rounding, the staged masks and the per-pixel state of one batch.
-int64_t footprint(int64_t n, int vb, const std::vector<fs_camera>& cams, int32_t mask_dtype,
-                  int32_t E) {
-  const int64_t nb = std::min<int64_t>(vb, static_cast<int64_t>(cams.size()));
-  const int64_t window = nb * n * (64 + 32 + 4 * 9) + nb * n * 2 * 16;
+// window (records, footprints, boxes, keys, re-check flags), a depth chunk's
+// list and its sort's buffers (16 B an entry; one chunk lists a whole batch,
+// several list ever fewer of its entries; scenes seen from near have about
+// twice the entries of the chunk rule's), the FP64 table and its rounding, the
+// staged masks and the per-pixel state of one batch.
+int64_t footprint(int64_t n, int vb, int chunks, const std::vector<fs_camera>& cams,
+                  int32_t mask_dtype, int32_t E) {
+  const int32_t V = static_cast<int32_t>(cams.size());
+  const int64_t nb = std::min<int64_t>(vb, V);
+  if (chunks == 0) chunks = fs::chunks_by_size(vb, n, cams.data(), V);
+  const double entries = std::max(2.0, 2.0 * fs::entries_per_slot(cams.data(), V) / chunks);
+  const int64_t window = nb * n * (64 + 32 + 4 * 9) +
+                         static_cast<int64_t>(static_cast<double>(nb * n) * entries * 16);
   int64_t pixels = 0, batch_pixels = 0;
   for (size_t v = 0; v < cams.size(); ++v) {
     const int64_t p = static_cast<int64_t>(cams[v].width) * cams[v].height;
@@ -430,7 +437,7 @@ fs_status fs_server_submit(fs_server* s, int32_t scene_id, const fs_camera* cams
   if (!(gamma >= -1.f && gamma <= 1.f))
     return fail(FS_INVALID_ARGUMENT, "fs_server_submit: gamma outside [-1, 1]");
   int64_t n = 0;
-  int vb = 16;
+  int vb = 16, chunks = 0;
   {
     std::lock_guard<std::mutex> lk(s->scenes_mu);
     if (scene_id < 0 || scene_id >= static_cast<int32_t>(s->scenes.size()))
@@ -439,6 +446,7 @@ fs_status fs_server_submit(fs_server* s, int32_t scene_id, const fs_camera* cams
     n = e.n;
     // before its scene is tuned a request may run with the largest batch
     vb = (s->autotune && !e.tuned) ? 64 : e.views_per_batch;
+    chunks = e.depth_chunks;
   }
   std::unique_ptr<Request> r(new Request());
   r->scene = scene_id;
@@ -458,7 +466,7 @@ fs_status fs_server_submit(fs_server* s, int32_t scene_id, const fs_camera* cams
   r->bits.resize(static_cast<size_t>(n > 0 ? n : 1));
   r->label.resize(static_cast<size_t>(n > 0 ? n : 1));
   r->margin.resize(static_cast<size_t>(n > 0 ? n : 1));
-  r->est = footprint(n, vb, r->cams, mask_dtype, E);
+  r->est = footprint(n, vb, chunks, r->cams, mask_dtype, E);
   {
     std::lock_guard<std::mutex> lk(s->mu);
     if (s->stopping) return fail(FS_CANCELLED, "fs_server_submit: server is stopping");
