@@ -1157,7 +1157,8 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
         }
         if (record) record->entries[pi] = I;
         a0 += n_part;
-        if (keep && !plan)
+        // the last list's bound is never looked at
+        if (keep && !plan && (a0 < p0 + n_pos || ci + 1 < chunks))
           FS_CUDA(cudaMemcpyAsync(bound + part, sorted_val + (a0 - 1), 4,
                                   cudaMemcpyDeviceToDevice, stream),
                   "bounds");
