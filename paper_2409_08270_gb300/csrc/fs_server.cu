@@ -17,6 +17,7 @@
 #include <string>
 #include <thread>
 #include <unordered_map>
+#include <utility>
 #include <vector>
 
 #include "../../include/flashsplat.h"
@@ -280,21 +281,33 @@ bool drop_oldest_graph(fs_server* s, SceneEntry* self) {
 }
 
 // The first request of a scene (autotune on): time a few batching settings
-// on a sample of its views and keep the fastest for the scene.
+// (views per batch, depth chunks) on a sample of its views and keep the fastest
+// for the scene.  The untuned setting, chunks by the size, comes first, after a
+// solve that takes the allocations, so that tuning does not end below it (one
+// request of 300,000 Gaussians, 24 views of 512x512: 4.95 ms untuned, 5.32 ms
+// with the best of four to six chunks).  A scene under kTuneBySize Gaussians
+// takes some milliseconds whichever it is and has fixed settings.
+constexpr int64_t kTuneBySize = 1 << 16;
 void tune_scene(fs_server* s, int slot, SceneEntry& se, Request* r) {
-  static const int cand[][2] = {{50, 6}, {32, 5}, {64, 6}, {16, 4}, {50, 4}};
   const int32_t V = static_cast<int32_t>(std::min<size_t>(r->cams.size(), 32));
-  double best = 1e300;
+  const int by_size = fs::chunks_by_size(se.views_per_batch, se.n, r->cams.data(), V);
+  std::vector<std::pair<int, int>> cand = {{50, 6}, {32, 5}, {64, 6}, {16, 4}, {50, 4}};
   fs_stats st{};
+  if (se.n >= kTuneBySize) {
+    cand = {{50, 0}, {32, 0}, {64, 0}, {50, by_size + 1}, {50, by_size + 2}};
+    fs::ctx_set_batching(s->ctx[slot], 50, 0);
+    solve_request(s, slot, se, r, V, &st);
+  }
+  double best = 1e300;
   for (const auto& c : cand) {
-    fs::ctx_set_batching(s->ctx[slot], c[0], c[1]);
+    fs::ctx_set_batching(s->ctx[slot], c.first, c.second);
     const double t0 = now_s();
     if (solve_request(s, slot, se, r, V, &st) != FS_OK) continue;
     const double dt = now_s() - t0;
     if (dt < best) {
       best = dt;
-      se.views_per_batch = c[0];
-      se.depth_chunks = c[1];
+      se.views_per_batch = c.first;
+      se.depth_chunks = c.second;
     }
   }
 }
