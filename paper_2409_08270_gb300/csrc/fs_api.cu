@@ -723,8 +723,8 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
                         const uint64_t* sat, int total_tiles, int tile_bits, int64_t kcap,
                         bool count_entries, DevBuf* val_dst, uint2* ranges_dst,
                         cudaStream_t stream, int64_t* I_out,
-                        const int64_t* range = nullptr, bool live = false, int64_t limit = 0, const int64_t* range_dev = nullptr,
-                        int64_t plan_cap = 0) {
+                        const int64_t* range = nullptr, bool live = false, int64_t limit = 0,
+                        const int64_t* range_dev = nullptr, int64_t plan_cap = 0) {
   unsigned long long* ctr = c->counters.as<unsigned long long>();
   *I_out = 0;
   FS_CUDA(cudaMemsetAsync(ranges_dst, 0, static_cast<size_t>(total_tiles) * 8, stream),
@@ -751,9 +751,9 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
   if (range_dev) {
     uint32_t* total = c->total.as<uint32_t>();
     const uint32_t capacity = static_cast<uint32_t>(plan_cap);
-    FS_CUDA(fs::launch_bin_fused(0, n_pos, n, vd, nb, sorted_val, P.foot, sat, c->lk_a.as<uint32_t>(),
-                                 val_dst->as<uint32_t>(), capacity, c->lb_tmp.p, total, ctr,
-                                 stream, range),
+    FS_CUDA(fs::launch_bin_fused(0, n_pos, n, vd, nb, sorted_val, P.foot, sat,
+                                 c->lk_a.as<uint32_t>(), val_dst->as<uint32_t>(), capacity,
+                                 c->lb_tmp.p, total, ctr, stream, range),
             "binning");
     FS_CUDA(fs::launch_graph_check(total, capacity, nullptr, 0, range_dev, n_pos, ctr, stream),
             "plan check");
@@ -762,8 +762,8 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
     bool alt2 = false;
     FS_CUDA(fs::radix_sort_pairs(c->lk_a.as<uint32_t>(), val_dst->as<uint32_t>(),
                                  c->lk_b.as<uint32_t>(), c->lv_b.as<uint32_t>(), plan_cap,
-                                 tile_bits, c->sort_tmp.p, &alt2, stream, ctr, false, 0u, 0xFFFFFFFFu,
-                                 total),
+                                 tile_bits, c->sort_tmp.p, &alt2, stream, ctr, false, 0u,
+                                 0xFFFFFFFFu, total),
             "tile sort");
     const uint32_t* lkey = alt2 ? c->lk_b.as<uint32_t>() : c->lk_a.as<uint32_t>();
     if (alt2)
@@ -1212,7 +1212,7 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
     FS_CUDA(fs::launch_candidates(k_total, n, vd, P.box, P.foot, skip, c->ccnt.as<uint32_t>(),
                                   stream),
             "candidates");
-    FS_CUDA(fs::exclusive_scan(c->ccnt.as<uint32_t>(), nullptr, c->offs.as<uint32_t>(), k_total,
+    FS_CUDA(fs::exclusive_scan(c->ccnt.as<uint32_t>(), c->offs.as<uint32_t>(), k_total,
                                c->total.as<uint32_t>(), c->scan_tmp.p, stream),
             "candidate scan");
     int64_t C = 0;
@@ -1287,7 +1287,7 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
   c->stats.kernel_launches += 2 + scan_launches(n);
   FS_CUDA(fs::launch_flag_margin(n, margin, c->recheck_margin, c->rk_flag.as<uint32_t>(), stream),
           "re-check flags");
-  FS_CUDA(fs::exclusive_scan(c->rk_flag.as<uint32_t>(), nullptr, c->rk_offs.as<uint32_t>(), n,
+  FS_CUDA(fs::exclusive_scan(c->rk_flag.as<uint32_t>(), c->rk_offs.as<uint32_t>(), n,
                              c->total.as<uint32_t>(), c->scan_tmp.p, stream),
           "re-check scan");
   FS_CUDA(fs::launch_scatter_flagged(n, c->rk_flag.as<uint32_t>(), c->rk_offs.as<uint32_t>(), F,
@@ -1370,8 +1370,8 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
       FS_CUDA(cudaMemsetAsync(ctr + fs::kRecheckIncomplete, 0, 8, stream), "incomplete clear");
       c->stats.kernel_launches += 2;
       FS_CUDA(fs::launch_recheck_blend(vd, nb, L.max_tiles, Ls, skip, c->rk_tiles.p, c->n_sm,
-                                       P.rec, P.rec16, s->pos_op.as<float4>(), n, E, mask_dtype, map, Rb, ctr,
-                                       stream),
+                                       P.rec, P.rec16, s->pos_op.as<float4>(), n, E, mask_dtype,
+                                       map, Rb, ctr, stream),
               "re-check blend");
       FS_CUDA(cudaMemcpyAsync(ctr_h + fs::kRecheckIncomplete, ctr + fs::kRecheckIncomplete, 8,
                               cudaMemcpyDeviceToHost, stream),
@@ -1502,8 +1502,8 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
     bool alt = false;
     FS_CUDA(fs::radix_sort_pairs(c->key_a.as<uint32_t>(), c->val_a.as<uint32_t>(),
                                  c->key_b.as<uint32_t>(), c->val_b.as<uint32_t>(), k_total,
-                                 key_bits, c->sort_tmp.p, &alt, stream, c->counters.as<unsigned long long>(),
-                                 true, kmin, span),
+                                 key_bits, c->sort_tmp.p, &alt, stream,
+                                 c->counters.as<unsigned long long>(), true, kmin, span),
             "depth sort");
     uint32_t* sorted_key = alt ? c->key_b.as<uint32_t>() : c->key_a.as<uint32_t>();
     uint32_t* sorted_val = alt ? c->val_b.as<uint32_t>() : c->val_a.as<uint32_t>();
@@ -2056,7 +2056,7 @@ fs_status fs_test_exclusive_scan(int32_t device, const uint32_t* in, uint32_t* o
   DevBuf tmp, tot;
   FS_TRY(tmp.ensure(fs::scan_temp_bytes(n), "scan temp"));
   FS_TRY(tot.ensure(4, "scan total"));
-  cudaError_t e = fs::exclusive_scan(in, nullptr, out, n, tot.as<uint32_t>(), tmp.p, nullptr);
+  cudaError_t e = fs::exclusive_scan(in, out, n, tot.as<uint32_t>(), tmp.p, nullptr);
   if (e == cudaSuccess) e = cudaMemcpy(total, tot.p, 4, cudaMemcpyDeviceToHost);
   tmp.release();
   tot.release();

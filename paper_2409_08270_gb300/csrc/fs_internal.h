@@ -26,9 +26,9 @@ constexpr int kLookbackSpinLimit = 1 << 23;
 // scan / sort (fs_sort.cu) --------------------------------------------------
 // Temporary storage needed by exclusive_scan for n elements (bytes).
 size_t scan_temp_bytes(int64_t n);
-// out[k] = sum_{j<k} in[gather ? gather[j] : j]; *total = the full sum (device).
-cudaError_t exclusive_scan(const uint32_t* in, const uint32_t* gather, uint32_t* out, int64_t n,
-                           uint32_t* total, void* temp, cudaStream_t stream);
+// out[k] = sum_{j<k} in[j]; *total = the full sum (device).
+cudaError_t exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total,
+                           void* temp, cudaStream_t stream);
 // Passes radix_sort_pairs makes for a `bits`-bit key (8- or 9-bit digits).
 int radix_passes(int bits);
 // Temporary storage of radix_sort_pairs for n elements (bytes).
@@ -180,16 +180,17 @@ cudaError_t launch_flag_margin(int64_t n, const float* margin, float tau, uint32
 cudaError_t launch_scatter_flagged(int64_t n, const uint32_t* flag, const uint32_t* offs,
                                    uint32_t* F, int32_t* map, cudaStream_t stream);
 // clears the skip bits of every tile a flagged Gaussian reaches in the batch's
-// views [v_begin, v_begin + n_views); *visible += the number of visible (view, flagged Gaussian) pairs.  With
-// kept chunk lists (bound: the last slot of each depth chunk; rec / rec16 and
-// dlo: the batch's records and low depth words, which order its slots; sat_chunk: the chunk in which each tile
-// saturated, 0xFF = never), sets the `deep` bit of every tile that saturated
-// before the flagged Gaussian's own chunk.  bound == NULL: no kept lists.
-cudaError_t launch_mark_tiles(int64_t n_flagged, int v_begin, int n_views, int64_t n, const uint32_t* F,
-                              const ViewParams* views, const TileBox* box, const Footprint* foot,
-                              uint64_t* skip, uint32_t* visible, const uint32_t* bound,
-                              int chunks, const ProjRecord* rec, const CompactRecord* rec16,
-                              const uint32_t* dlo,
+// views [v_begin, v_begin + n_views); *visible += the number of visible (view,
+// flagged Gaussian) pairs.  With kept lists (bound: the last slot of each list;
+// rec / rec16 and dlo: the batch's records and low depth words, which order
+// its slots; sat_chunk: the list in which each tile saturated, 0xFF = never),
+// sets the `deep` bit of every tile that saturated before the flagged
+// Gaussian's own list.  bound == NULL: no kept lists.
+cudaError_t launch_mark_tiles(int64_t n_flagged, int v_begin, int n_views, int64_t n,
+                              const uint32_t* F, const ViewParams* views, const TileBox* box,
+                              const Footprint* foot, uint64_t* skip, uint32_t* visible,
+                              const uint32_t* bound, int chunks, const ProjRecord* rec,
+                              const CompactRecord* rec16, const uint32_t* dlo,
                               const uint8_t* sat_chunk, uint64_t* deep, cudaStream_t stream);
 // dst[i] += src[i], i < count
 cudaError_t launch_add_rows(int64_t count, const double* src, double* dst, cudaStream_t stream);

@@ -115,17 +115,18 @@ __device__ __forceinline__ f2 f2_clamp(f2 x, float lim_hi, float lim_lo) {
   return x;
 }
 
-// One thread per Gaussian; it projects the Gaussian into the views of its block's
-// share (all of them for large scenes, so the scene is read once per batch;
-// small scenes spread the views over the grid's second dimension).  rec16 != NULL: the record is
-// written in the reduced-precision form instead (rec is not written).  The
-// paired float-pair quantities (the two rows of the Jacobian-rotation product,
-// the two rows of T Sigma3D, the x and y halves of the pinhole map, the rows
-// of W) run in packed FP32 (f2x2), bit-identical to the scalar form.  Three
-// blocks per SM (80 registers) spill less than four.  Bound by issue (about
-// 1,100 instructions a slot): one reciprocal and four roots, seeded by the
-// hardware's, where six correctly rounded float-pair divisions and four roots
-// stood, take 10^6 Gaussians in 100 views from 4.44 to 3.74 ms.
+// One thread per Gaussian; it projects the Gaussian into the views of its
+// block's share (all of them for large scenes, so the scene is read once per
+// batch; small scenes spread the views over the grid's second dimension).
+// rec16 != NULL: the record is written in the reduced-precision form instead
+// (rec is not written).  The paired float-pair quantities (the two rows of the
+// Jacobian-rotation product, the two rows of T Sigma3D, the x and y halves of
+// the pinhole map, the rows of W) run in packed FP32 (f2x2), bit-identical to
+// the scalar form.  Three blocks per SM (80 registers) spill less than four.
+// Bound by issue (about 1,100 instructions a slot): one reciprocal and four
+// roots, seeded by the hardware's, where six correctly rounded float-pair
+// divisions and four roots stood, take 10^6 Gaussians in 100 views from 4.44 to
+// 3.74 ms.
 template <bool kFast>
 __global__ void __launch_bounds__(256, kFast ? 4 : 3) project_kernel(
     int64_t n, int n_views, const ViewParams* __restrict__ views_g,
@@ -951,8 +952,8 @@ cudaError_t launch_depth_tie_fix(int64_t n_total, int64_t n, const uint32_t* key
                                  const uint32_t* n_dev) {
   if (n_total < 2) return cudaSuccess;
   const int64_t blocks = ((n_total + 3) / 4 + kTieThreads - 1) / kTieThreads;
-  depth_tie_fix_kernel<<<static_cast<unsigned>(blocks), kTieThreads, 0, stream>>>(n_total, n, key, val,
-                                                                              depth_lo, n_dev);
+  depth_tie_fix_kernel<<<static_cast<unsigned>(blocks), kTieThreads, 0, stream>>>(
+      n_total, n, key, val, depth_lo, n_dev);
   return cudaGetLastError();
 }
 

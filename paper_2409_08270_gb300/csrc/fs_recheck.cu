@@ -162,7 +162,8 @@ __global__ void candidates_kernel(int64_t k_total, int64_t n, const ViewParams* 
 __global__ void compact_kernel(int64_t k_total, const uint32_t* __restrict__ flag,
                                const uint32_t* __restrict__ offs,
                                const ProjRecord* __restrict__ rec,
-                               const CompactRecord* __restrict__ rec16, uint32_t* __restrict__ out_key, uint32_t* __restrict__ out_val) {
+                               const CompactRecord* __restrict__ rec16,
+                               uint32_t* __restrict__ out_key, uint32_t* __restrict__ out_val) {
   const int64_t slot = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (slot >= k_total || !flag[slot]) return;
   const uint32_t o = offs[slot];
@@ -607,18 +608,19 @@ cudaError_t launch_scatter_flagged(int64_t n, const uint32_t* flag, const uint32
   return cudaGetLastError();
 }
 
-cudaError_t launch_mark_tiles(int64_t n_flagged, int v_begin, int n_views, int64_t n, const uint32_t* F,
-                              const ViewParams* views, const TileBox* box, const Footprint* foot,
-                              uint64_t* skip, uint32_t* visible, const uint32_t* bound,
-                              int chunks, const ProjRecord* rec, const CompactRecord* rec16,
-                              const uint32_t* dlo,
+cudaError_t launch_mark_tiles(int64_t n_flagged, int v_begin, int n_views, int64_t n,
+                              const uint32_t* F, const ViewParams* views, const TileBox* box,
+                              const Footprint* foot, uint64_t* skip, uint32_t* visible,
+                              const uint32_t* bound, int chunks, const ProjRecord* rec,
+                              const CompactRecord* rec16, const uint32_t* dlo,
                               const uint8_t* sat_chunk, uint64_t* deep, cudaStream_t stream) {
   const int64_t total = n_flagged * n_views;
   if (total == 0) return cudaSuccess;
   mark_tiles_kernel<<<blocks_for(total, 256), 256, 0, stream>>>(
       n_flagged, v_begin, n_views, n, F, views, box, foot,
       reinterpret_cast<unsigned long long*>(skip),
-      visible, bound, chunks, rec, rec16, dlo, sat_chunk, reinterpret_cast<unsigned long long*>(deep));
+      visible, bound, chunks, rec, rec16, dlo, sat_chunk,
+      reinterpret_cast<unsigned long long*>(deep));
   return cudaGetLastError();
 }
 

@@ -55,12 +55,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* s
   return warp_pre + inc - x;
 }
 
-__device__ __forceinline__ uint32_t load_in(const uint32_t* in, const uint32_t* gather, int64_t j) {
-  return gather ? in[gather[j]] : in[j];
-}
-
 __global__ void __launch_bounds__(kThreads) scan_reduce_kernel(const uint32_t* __restrict__ in,
-                                                               const uint32_t* __restrict__ gather,
                                                                int64_t n,
                                                                uint32_t* __restrict__ block_sums) {
   __shared__ uint32_t s_warp[kWarps];
@@ -69,7 +64,7 @@ __global__ void __launch_bounds__(kThreads) scan_reduce_kernel(const uint32_t* _
 #pragma unroll
   for (int r = 0; r < kRounds; ++r) {
     const int64_t j = base + r * kThreads + threadIdx.x;
-    x[r] = j < n ? load_in(in, gather, j) : 0u;
+    x[r] = j < n ? in[j] : 0u;
   }
   uint32_t acc = 0;
 #pragma unroll
@@ -103,7 +98,6 @@ __global__ void __launch_bounds__(kThreads) scan_blocks_kernel(uint32_t* __restr
 }
 
 __global__ void __launch_bounds__(kThreads) scan_down_kernel(const uint32_t* __restrict__ in,
-                                                             const uint32_t* __restrict__ gather,
                                                              int64_t n,
                                                              const uint32_t* __restrict__ block_pre,
                                                              uint32_t* __restrict__ out) {
@@ -114,7 +108,7 @@ __global__ void __launch_bounds__(kThreads) scan_down_kernel(const uint32_t* __r
 #pragma unroll
   for (int r = 0; r < kRounds; ++r) {
     const int64_t j = base + r * kThreads + threadIdx.x;
-    x[r] = j < n ? load_in(in, gather, j) : 0u;
+    x[r] = j < n ? in[j] : 0u;
   }
   uint32_t carry = block_pre[blockIdx.x];
 #pragma unroll
@@ -475,17 +469,17 @@ size_t scan_temp_bytes(int64_t n) {
   return static_cast<size_t>(tiles_of(n) + 1) * sizeof(uint32_t);
 }
 
-cudaError_t exclusive_scan(const uint32_t* in, const uint32_t* gather, uint32_t* out, int64_t n,
-                           uint32_t* total, void* temp, cudaStream_t stream) {
+cudaError_t exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total,
+                           void* temp, cudaStream_t stream) {
   if (n <= 0) {
     if (total) return cudaMemsetAsync(total, 0, sizeof(uint32_t), stream);
     return cudaSuccess;
   }
   const int64_t nb = tiles_of(n);
   uint32_t* sums = static_cast<uint32_t*>(temp);
-  scan_reduce_kernel<<<static_cast<unsigned>(nb), kThreads, 0, stream>>>(in, gather, n, sums);
+  scan_reduce_kernel<<<static_cast<unsigned>(nb), kThreads, 0, stream>>>(in, n, sums);
   scan_blocks_kernel<<<1, kThreads, 0, stream>>>(sums, nb, total);
-  scan_down_kernel<<<static_cast<unsigned>(nb), kThreads, 0, stream>>>(in, gather, n, sums, out);
+  scan_down_kernel<<<static_cast<unsigned>(nb), kThreads, 0, stream>>>(in, n, sums, out);
   return cudaGetLastError();
 }
 
