@@ -508,6 +508,20 @@ size_t status_bytes(int64_t n) {
   return static_cast<size_t>(tiles) * kMaxRadix * (n < kWideSort ? 4 : 8);
 }
 
+// Dynamic shared memory above 48 KB needs the opt-in, once per kernel (`set`: its
+// devices so far) and device.
+cudaError_t allow_smem(const void* kernel, size_t bytes, std::atomic<uint64_t>* set) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (set->load() & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(bytes));
+  if (e == cudaSuccess) set->fetch_or(bit);
+  return e;
+}
+
 template <int DB, int K, typename Word>
 cudaError_t radix_pass(const uint32_t* src_k, const uint32_t* src_v, uint32_t* dst_k,
                        uint32_t* dst_v, int64_t n, int pass, int shift, uint32_t kmin,
@@ -516,19 +530,10 @@ cudaError_t radix_pass(const uint32_t* src_k, const uint32_t* src_v, uint32_t* d
                        const uint32_t* range_dev, unsigned long long* counters) {
   constexpr int T = kPassThreads, kBlocks = K > 8 ? 2 : 3;
   const size_t smem = sizeof(PassSmem<DB, T, K>);
-  // dynamic shared memory above 48 KB needs the opt-in, once per device
   static std::atomic<uint64_t> attr_set{0};
-  int dev = 0;
-  cudaError_t e0 = cudaGetDevice(&dev);
+  const cudaError_t e0 = allow_smem(
+      reinterpret_cast<const void*>(radix_pass_kernel<DB, T, K, kBlocks, Word>), smem, &attr_set);
   if (e0 != cudaSuccess) return e0;
-  const uint64_t bit = 1ull << (dev & 63);
-  if (!(attr_set.load() & bit)) {
-    cudaError_t e = cudaFuncSetAttribute(radix_pass_kernel<DB, T, K, kBlocks, Word>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    attr_set.fetch_or(bit);
-  }
   const int64_t tiles = (n + T * K - 1) / (T * K);
   radix_pass_kernel<DB, T, K, kBlocks, Word><<<static_cast<unsigned>(tiles), T, smem, stream>>>(
       src_k, src_v, n, pass, shift, kmin, span, head, static_cast<Word*>(status),
@@ -576,8 +581,9 @@ cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
   if (e != cudaSuccess) return e;
   const int64_t hist_blocks = std::min<int64_t>((n + 8 * kHistThreads - 1) / (8 * kHistThreads), 304);
   const size_t hist_bytes = hist_smem(shape);
-  e = cudaFuncSetAttribute(radix_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(kMaxPasses * kMaxRadix * kHistCopies * 4));
+  static std::atomic<uint64_t> attr_set{0};
+  e = allow_smem(reinterpret_cast<const void*>(radix_hist_kernel),
+                 kMaxPasses * kMaxRadix * kHistCopies * 4, &attr_set);
   if (e != cudaSuccess) return e;
   radix_hist_kernel<<<static_cast<unsigned>(hist_blocks), kHistThreads, hist_bytes, stream>>>(
       keys, n, shape, kmin, span, head, n_dev, range_dev);
