@@ -691,6 +691,17 @@ fs_status read_total(fs_ctx* c, cudaStream_t stream, int64_t* out) {
   return FS_OK;
 }
 
+// FS_TIMEOUT if a bounded wait of the call's kernels has given up.
+fs_status check_waits(fs_ctx* c, cudaStream_t stream) {
+  unsigned long long* h = c->counters_host.as<unsigned long long>() + fs::kLookbackTimeout;
+  FS_CUDA(cudaMemcpyAsync(h, c->counters.as<unsigned long long>() + fs::kLookbackTimeout,
+                          sizeof(*h), cudaMemcpyDeviceToHost, stream),
+          "counter readback");
+  FS_CUDA(cudaStreamSynchronize(stream), "counter readback");
+  if (*h == 0) return FS_OK;
+  return fail(FS_TIMEOUT, "a bounded wait of a sort, a compaction or the binning gave up");
+}
+
 // Clears a call's device counters (kNumCounters of them).
 fs_status clear_counters(fs_ctx* c, void* counters, cudaStream_t stream) {
   const size_t word = sizeof(unsigned long long);
@@ -770,7 +781,7 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
       FS_CUDA(fs::launch_copy_count(c->lv_b.as<uint32_t>(), val_dst->as<uint32_t>(), total,
                                     plan_cap, stream),
               "list copy");
-    FS_CUDA(fs::launch_ranges(plan_cap, lkey, ranges_dst, stream, total), "ranges");
+    FS_CUDA(fs::launch_ranges(plan_cap, lkey, ranges_dst, ctr, stream, total), "ranges");
     return FS_OK;
   }
   // count, offsets and emission in one launch into the buffers' current
@@ -788,6 +799,7 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
             "binning");
     FS_TRY(stage_end(c, tb, stream));
     FS_TRY(read_total(c, stream, &I));
+    if (I == fs::kGaveUpTotal) FS_TRY(check_waits(c, stream));
     if (limit > 0 && I > limit) {
       *I_out = -I;
       return FS_OK;
@@ -828,7 +840,7 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
     FS_CUDA(cudaMemcpyAsync(val_dst->p, c->lv_b.p, static_cast<size_t>(I) * 4,
                             cudaMemcpyDeviceToDevice, stream),
             "list copy");
-  FS_CUDA(fs::launch_ranges(I, lkey, ranges_dst, stream), "ranges");
+  FS_CUDA(fs::launch_ranges(I, lkey, ranges_dst, ctr, stream), "ranges");
   FS_TRY(stage_end(c, tt, stream));
   return FS_OK;
 }
@@ -1075,7 +1087,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
             "depth sort");
     uint32_t* sorted_key = alt ? pr.key_alt : pr.key;
     uint32_t* sorted_val = alt ? pr.val_alt : pr.val;
-    FS_CUDA(fs::launch_depth_tie_fix(k_total, n, sorted_key, sorted_val, P.dlo, stream),
+    FS_CUDA(fs::launch_depth_tie_fix(k_total, n, sorted_key, sorted_val, P.dlo, ctr, stream),
             "depth ties");
     FS_TRY(stage_end(c, td, stream));
     if (overlap && b + 1 < batches) {
@@ -1101,7 +1113,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
       bound = c->kl_bound.as<uint32_t>() + static_cast<int64_t>(b) * fs::kMaxChunks;
       FS_CUDA(cudaMemsetAsync(bound, 0xFF, fs::kMaxChunks * 4, stream), "bounds");
       if (plan)
-        FS_CUDA(fs::launch_chunk_last(c->chunk_bnd.as<int64_t>(), chunks, sorted_val, bound,
+        FS_CUDA(fs::launch_chunk_last(c->chunk_bnd.as<int64_t>(), chunks, sorted_val, bound, ctr,
                                       stream),
                 "bounds");
     }
@@ -1232,7 +1244,7 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
             "candidate sort");
     uint32_t* sorted_key = alt ? c->key_a.as<uint32_t>() : c->key_b.as<uint32_t>();
     uint32_t* sorted_val = alt ? c->val_a.as<uint32_t>() : c->val_b.as<uint32_t>();
-    FS_CUDA(fs::launch_depth_tie_fix(C, n, sorted_key, sorted_val, P.dlo, stream), "depth ties");
+    FS_CUDA(fs::launch_depth_tie_fix(C, n, sorted_key, sorted_val, P.dlo, ctr, stream), "depth ties");
     int64_t I = 0;
     FS_TRY(bin_positions(c, 0, C, n, vd, nb, sorted_val, P, skip, total_tiles, tile_bits, kcap,
                          false, &c->lv_a, c->ranges.as<uint2>(), stream, &I, nullptr, false,
@@ -1507,7 +1519,8 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
             "depth sort");
     uint32_t* sorted_key = alt ? c->key_b.as<uint32_t>() : c->key_a.as<uint32_t>();
     uint32_t* sorted_val = alt ? c->val_b.as<uint32_t>() : c->val_a.as<uint32_t>();
-    FS_CUDA(fs::launch_depth_tie_fix(k_total, n, sorted_key, sorted_val, P.dlo, stream),
+    FS_CUDA(fs::launch_depth_tie_fix(k_total, n, sorted_key, sorted_val, P.dlo,
+                                     c->counters.as<unsigned long long>(), stream),
             "depth ties");
     // no tile saturates: every list is complete
     const size_t sat_bytes = static_cast<size_t>((total_tiles + 63) / 64) * 8;
@@ -2083,7 +2096,7 @@ fs_status fs_test_tile_ranges(int32_t device, const uint32_t* keys, int64_t n, i
                   (long long)k);
   e = cudaMemset(ranges, 0, static_cast<size_t>(n_tiles) * 8);
   if (e == cudaSuccess && n > 0)
-    e = fs::launch_ranges(n, keys, reinterpret_cast<uint2*>(ranges), nullptr);
+    e = fs::launch_ranges(n, keys, reinterpret_cast<uint2*>(ranges), nullptr, nullptr);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(e, "fs_test_tile_ranges");
   return FS_OK;

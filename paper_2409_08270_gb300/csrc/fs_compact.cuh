@@ -71,9 +71,13 @@ __global__ void __launch_bounds__(32 * kCompactWarps) compact_kernel(
     n_pos = min(n_pos, range_in[1] - range_in[0]);
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_vb = atomicAdd(ticket, 1u);
+  if (threadIdx.x == 0) {
+    const uint32_t t = atomicAdd(ticket, 1u);
+    s_vb = gave_up(counters) ? kGaveUpTotal : t;  // the values may be incomplete
+  }
   __syncthreads();
   const uint32_t vb = s_vb;
+  if (vb == kGaveUpTotal) return;
   const int64_t j0 = static_cast<int64_t>(vb) * kCompactTile + warp * 32 * kCompactItems + lane;
   uint32_t g[kCompactItems], bal[kCompactItems], cnt = 0;
 #pragma unroll

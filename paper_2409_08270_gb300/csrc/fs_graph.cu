@@ -23,11 +23,12 @@ __global__ void chunk_bounds_kernel(const uint32_t* __restrict__ key_range, int 
 
 __global__ void chunk_last_kernel(const int64_t* __restrict__ bnd, int chunks,
                                   const uint32_t* __restrict__ sorted_val,
-                                  uint32_t* __restrict__ bound) {
+                                  uint32_t* __restrict__ bound,
+                                  const unsigned long long* __restrict__ counters) {
   const int ci = threadIdx.x;
   if (ci + 1 >= chunks) return;
   const int64_t p0 = bnd[ci], p1 = bnd[ci + 1];
-  bound[ci] = p1 > p0 ? sorted_val[p1 - 1] : 0xFFFFFFFFu;
+  bound[ci] = p1 > p0 && !gave_up(counters) ? sorted_val[p1 - 1] : 0xFFFFFFFFu;
 }
 
 __global__ void __launch_bounds__(256) copy_count_kernel(const uint32_t* __restrict__ src,
@@ -63,9 +64,10 @@ cudaError_t launch_chunk_bounds(const uint32_t* key_range, int chunks, int64_t* 
 }
 
 cudaError_t launch_chunk_last(const int64_t* bnd, int chunks, const uint32_t* sorted_val,
-                              uint32_t* bound, cudaStream_t stream) {
+                              uint32_t* bound, const unsigned long long* counters,
+                              cudaStream_t stream) {
   if (chunks < 2) return cudaSuccess;
-  chunk_last_kernel<<<1, 32, 0, stream>>>(bnd, chunks, sorted_val, bound);
+  chunk_last_kernel<<<1, 32, 0, stream>>>(bnd, chunks, sorted_val, bound, counters);
   return cudaGetLastError();
 }
 

@@ -22,6 +22,11 @@ typedef uint2 TileBox;
 // Polls of a predecessor's look-back word before the wait gives up: one takes
 // 0.24 us (a 32 ns sleep and a load past L1), so a wait lasts two seconds.
 constexpr int kLookbackSpinLimit = 1 << 23;
+// A wait that gave up leaves words of its launch's outputs unwritten.  Launches
+// that would index memory by them find the count of such waits in the solve's
+// counters (kLookbackTimeout) and do nothing; a binning then reports this number
+// of entries, on which the host looks at the counter and returns FS_TIMEOUT.
+constexpr uint32_t kGaveUpTotal = 0xFFFFFFFFu;
 
 // scan / sort (fs_sort.cu) --------------------------------------------------
 // Temporary storage needed by exclusive_scan for n elements (bytes).
@@ -67,8 +72,8 @@ cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, cons
 // re-orders runs of equal 32-bit depth keys by the depth's low word, then slot
 // (n_total elements; slot / n is the view of a slot)
 cudaError_t launch_depth_tie_fix(int64_t n_total, int64_t n, const uint32_t* key, uint32_t* val,
-                                 const uint32_t* depth_lo, cudaStream_t stream,
-                                 const uint32_t* n_dev = nullptr);
+                                 const uint32_t* depth_lo, const unsigned long long* counters,
+                                 cudaStream_t stream);
 // Binning of sorted positions [p0, p0 + n_pos): one list entry (key = tile id,
 // value = slot) per (tile, Gaussian) whose footprint reaches the tile, unless
 // the tile's `sat` bit is set, in one launch (count, decoupled look-back,
@@ -107,7 +112,8 @@ cudaError_t launch_lookback_probe(void* lookback, uint32_t* total, unsigned long
 cudaError_t launch_free_tables(const ViewParams* views, int n_views, const uint64_t* sat,
                                cudaStream_t stream);
 cudaError_t launch_ranges(int64_t n_entries, const uint32_t* key, uint2* ranges,
-                          cudaStream_t stream, const uint32_t* n_dev = nullptr);
+                          const unsigned long long* counters, cudaStream_t stream,
+                          const uint32_t* n_dev = nullptr);
 
 // Captured solves (fs_graph.cu) ----------------------------------------------
 // Device-side sizes for a solve captured into a CUDA graph: no host readback.
@@ -117,7 +123,8 @@ cudaError_t launch_chunk_bounds(const uint32_t* key_range, int chunks, int64_t* 
                                 cudaStream_t stream);
 // bound[ci] = the last sorted slot of chunk ci < chunks - 1 (0xFFFFFFFF: empty)
 cudaError_t launch_chunk_last(const int64_t* bnd, int chunks, const uint32_t* sorted_val,
-                              uint32_t* bound, cudaStream_t stream);
+                              uint32_t* bound, const unsigned long long* counters,
+                              cudaStream_t stream);
 // dst[k] = src[k] for k < min(*n_dev, cap)
 cudaError_t launch_copy_count(const uint32_t* src, uint32_t* dst, const uint32_t* n_dev,
                               int64_t cap, cudaStream_t stream);
@@ -290,5 +297,11 @@ enum Counter {
   kGraphKeyRange = 13,   // a captured solve's depth keys outgrew the plan's sort bits
   kNumCounters = 14
 };
+
+// Whether a bounded wait had given up when the launch began (counters may be
+// NULL); later ones may or may not be seen, so the load may come from L1.
+__device__ __forceinline__ bool gave_up(const unsigned long long* counters) {
+  return counters && counters[kLookbackTimeout] != 0ull;
+}
 
 }  // namespace fs

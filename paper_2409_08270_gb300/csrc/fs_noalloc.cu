@@ -233,7 +233,7 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
             "sort");
     uint32_t* skey = alt ? key_b : key_a;
     uint32_t* sval = alt ? val_b : val_a;
-    NA_CUDA(launch_depth_tie_fix(n, n, skey, sval, dlo, strm), "ties");
+    NA_CUDA(launch_depth_tie_fix(n, n, skey, sval, dlo, ctr, strm), "ties");
     NA_CUDA(cudaMemsetAsync(sat, 0, static_cast<size_t>((tiles + 63) / 64) * 8, strm), "clear");
     NA_CUDA(cudaMemsetAsync(subsat, 0, static_cast<size_t>((4 * tiles + 63) / 64) * 8, strm),
             "clear");
@@ -255,6 +255,8 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
         NA_CUDA(cudaMemcpyAsync(&I, total_d, 4, cudaMemcpyDeviceToHost, strm), "readback");
         NA_CUDA(cudaStreamSynchronize(strm), "readback");
         if (I <= static_cast<uint32_t>(kNA_Entries)) break;
+        if (I == kGaveUpTotal)  // more than 2^32 - 2 entries are not possible here
+          return na_fail(FS_TIMEOUT, "fs_solve_noalloc: a bounded wait of a sort gave up");
         int ci = 0;  // the chunk p0 lies in ends at n >> (chunks - 1 - ci)
         while (ci < chunks - 1 && (n >> (chunks - 1 - ci)) <= p0) ++ci;
         const int64_t end = ci == chunks - 1 ? n : n >> (chunks - 1 - ci);
@@ -272,7 +274,7 @@ extern "C" fs_status fs_solve_noalloc(int32_t device, const fs_gaussians* g, con
         const uint32_t* lkey = alt2 ? lk_b : lk_a;
         const uint32_t* lval = alt2 ? lv_b : lv_a;
         NA_CUDA(cudaMemsetAsync(ranges, 0, static_cast<size_t>(tiles) * 8, strm), "clear");
-        NA_CUDA(launch_ranges(I, lkey, ranges, strm), "ranges");
+        NA_CUDA(launch_ranges(I, lkey, ranges, ctr, strm), "ranges");
         NA_CUDA(launch_blend(vd, 1, tiles, ranges, lval, rec, nullptr, n, E, mask_dtype, table,
                              FS_F32, state, sat, subsat, nullptr, 0, ctr, false, strm),
                 "blend");

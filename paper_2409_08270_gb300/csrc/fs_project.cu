@@ -478,8 +478,7 @@ __device__ __forceinline__ void fix_tie_run(int64_t k, int64_t n_total, const Sl
 constexpr int kTieThreads = 128;
 __global__ void __launch_bounds__(kTieThreads, 12) depth_tie_fix_kernel(
     int64_t n_total, int64_t n, const uint32_t* __restrict__ key, uint32_t* __restrict__ val,
-    const uint32_t* __restrict__ depth_lo, const uint32_t* __restrict__ n_dev) {
-  if (n_dev) n_total = min(n_total, static_cast<int64_t>(*n_dev));
+    const uint32_t* __restrict__ depth_lo, const unsigned long long* __restrict__ counters) {
   const int64_t k0 = 4 * (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
   if (k0 + 1 >= n_total) return;
   // t[1 + i], w[1 + i]: key and slot of position k0 + i (key 0xFFFFFFFF where
@@ -504,6 +503,7 @@ __global__ void __launch_bounds__(kTieThreads, 12) depth_tie_fix_kernel(
   };
   load(key, 0xFFFFFFFFu, t);
   load(val, 0u, w);
+  if (gave_up(counters)) return;
   bool any = false;  // an equal neighbour somewhere among the four
 #pragma unroll
   for (int i = 1; i <= 4; ++i) any = any || (t[i] != 0xFFFFFFFFu && t[i + 1] == t[i]);
@@ -681,7 +681,12 @@ __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
     n_pos = min(n_pos, range_dev[1] - range_dev[0]);  // the launch's scratch is sized for n_pos
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_vb = atomicAdd(ticket, 1u);
+  if (threadIdx.x == 0) {
+    const uint32_t t = atomicAdd(ticket, 1u);
+    const bool off = gave_up(counters);  // the sorted slots may be incomplete
+    s_vb = off ? kGaveUpTotal : t;
+    if (off) *total = kGaveUpTotal;
+  }
   const uint32_t* const cols = views[0].cols;
   const uint32_t* const free_tab = views[0].free_tab;
   for (int v = threadIdx.x; v < n_views; v += kBinThreads) {
@@ -691,6 +696,7 @@ __global__ void __launch_bounds__(kBinThreads, 12) bin_fused_kernel(
   }
   __syncthreads();
   const uint32_t vb = s_vb;
+  if (vb == kGaveUpTotal) return;
   const int64_t j = static_cast<int64_t>(vb) * kBinThreads + threadIdx.x;
   if (j - threadIdx.x >= n_pos) return;  // whole block: the grid was sized for more
   uint32_t g = 0u, nrows = 0u;
@@ -885,7 +891,9 @@ __global__ void __launch_bounds__(256) free_table_kernel(const ViewParams* __res
 // takes four consecutive entries (one 16-byte load when the list is 16-byte
 // aligned, as the library's buffers are) and the entries on either side.
 __global__ void ranges_kernel(int64_t n_entries, const uint32_t* __restrict__ key,
-                              uint2* __restrict__ ranges, const uint32_t* __restrict__ n_dev) {
+                              uint2* __restrict__ ranges,
+                              const unsigned long long* __restrict__ counters,
+                              const uint32_t* __restrict__ n_dev) {
   if (n_dev) n_entries = min(n_entries, static_cast<int64_t>(*n_dev));
   const int64_t k0 = 4 * (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
   if (k0 >= n_entries) return;
@@ -902,6 +910,7 @@ __global__ void ranges_kernel(int64_t n_entries, const uint32_t* __restrict__ ke
     for (int i = 0; i < 4; ++i) t[1 + i] = k0 + i < n_entries ? key[k0 + i] : 0xFFFFFFFFu;
   }
   t[5] = k0 + 4 < n_entries ? key[k0 + 4] : 0xFFFFFFFFu;
+  if (gave_up(counters)) return;  // keys of the list may be missing
 #pragma unroll
   for (int i = 1; i <= 4; ++i) {
     const int64_t k = k0 + i - 1;
@@ -948,12 +957,12 @@ cudaError_t launch_project(int64_t n, int n_views, const ViewParams* views, cons
 }
 
 cudaError_t launch_depth_tie_fix(int64_t n_total, int64_t n, const uint32_t* key, uint32_t* val,
-                                 const uint32_t* depth_lo, cudaStream_t stream,
-                                 const uint32_t* n_dev) {
+                                 const uint32_t* depth_lo, const unsigned long long* counters,
+                                 cudaStream_t stream) {
   if (n_total < 2) return cudaSuccess;
   const int64_t blocks = ((n_total + 3) / 4 + kTieThreads - 1) / kTieThreads;
   depth_tie_fix_kernel<<<static_cast<unsigned>(blocks), kTieThreads, 0, stream>>>(
-      n_total, n, key, val, depth_lo, n_dev);
+      n_total, n, key, val, depth_lo, counters);
   return cudaGetLastError();
 }
 
@@ -1047,12 +1056,13 @@ cudaError_t launch_free_tables(const ViewParams* views, int n_views, const uint6
 }
 
 cudaError_t launch_ranges(int64_t n_entries, const uint32_t* key, uint2* ranges,
-                          cudaStream_t stream, const uint32_t* n_dev) {
+                          const unsigned long long* counters, cudaStream_t stream,
+                          const uint32_t* n_dev) {
   if (n_entries == 0) return cudaSuccess;
   const int threads = 256;
   const int64_t blocks = ((n_entries + 3) / 4 + threads - 1) / threads;
   ranges_kernel<<<static_cast<unsigned>(blocks), threads, 0, stream>>>(n_entries, key, ranges,
-                                                                       n_dev);
+                                                                       counters, n_dev);
   return cudaGetLastError();
 }
 

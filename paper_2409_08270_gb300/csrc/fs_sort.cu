@@ -300,7 +300,11 @@ __global__ void __launch_bounds__(T, kBlocks) radix_pass_kernel(
   PassSmem<DB, T, K>& S = *reinterpret_cast<PassSmem<DB, T, K>*>(smem_raw);
   device_sizes(n_dev, range_dev, &n, &kmin, &span);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) S.tile = atomicAdd(&head->ticket[pass], 1u);
+  if (threadIdx.x == 0) {
+    const uint32_t t = atomicAdd(&head->ticket[pass], 1u);
+    // after a wait that gave up the pairs are not those the digits were counted of
+    S.tile = gave_up(counters) ? 0xFFFFFFFFu : t;
+  }
   uint32_t* const cnt2 = reinterpret_cast<uint32_t*>(S.wcnt[warp]);
 #pragma unroll
   for (int k = 0; k < kRad / 64; ++k) cnt2[lane + 32 * k] = 0;
