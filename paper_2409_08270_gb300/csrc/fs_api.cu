@@ -293,37 +293,39 @@ double fs::entries_per_slot(const fs_camera* cams, int32_t V) {
 // batch's visible slots with six): the context's setting, or by the solve's
 // size.  A chunk costs its launches, a readback and the blend's start on every
 // tile, and spares later chunks the entries of the tiles it saturates.  The
-// share of those grows with a view's depth, that is with n; views of few tiles
-// leave a chunk's kernels short, so its fixed costs weigh more; and a batch
-// must hold enough entries (about 3 + tiles / 350 a slot) to pay for them at
-// all: 5.6 10^7 per chunk after the first at 300,000 Gaussians, fewer the
-// larger the share that a chunk spares (300,000 in 24 views of 512x512: 3.0 |
-// 3.1 | 3.3; in one of 1600x1200: 0.51 with 1).  Solve times in ms with 1 | 2 |
-// 3 | 4 | 5 | 6 | 8 chunks, 40 views (30 of 1600x1200), a forward-facing arc:
+// share of those grows with a view's depth, that is with n: the count by n alone
+// (1 up to 310,000 Gaussians, 5 at 10^6, 8 at 3 10^6) serves views up to about
+// 1000x750.  In larger ones a slot has more entries (about 3 + tiles / 350) and
+// scenes of some 10^5 Gaussians take more chunks, as far as the batch's entries
+// pay for them: 5.6 10^7 for each after the first at 300,000 Gaussians, fewer
+// the larger the share that a chunk spares (300,000 in 24 views of 512x512: 3.0
+// | 3.1 | 3.3 ms; in one of 1600x1200: 0.51 with 1).  Fewer chunks than by n are
+// better in views that show little of each Gaussian and worse in others of as
+// many tiles (460,000 in 126x995: 3.8 ms with 1, 6.0 with 3; in 726x163: 3.4 and
+// 2.8), which is not known beforehand.  Solve times in ms with 1 | 2 | 3 | 4 | 5
+// | 6 | 8 chunks, 40 views (30 of 1600x1200), a forward-facing arc:
 //   180k Gaussians, 400x300    2.45   2.47   2.52   2.64   2.78   2.90   3.11
 //   180k, 1600x1200            7.64   7.06   7.03   7.31   7.77   8.26   9.18
-//   300k, 160x120              3.17   3.53   3.80   4.08   4.26   4.43   4.61
 //   300k, 400x300              3.38   3.18   3.16   3.24   3.38   3.50   3.72
 //   300k, 900x640              6.48   5.60   5.27   5.28   5.43   5.67   6.11
 //   300k, 1600x1200           10.73   8.84   8.29   8.31   8.66   9.08  10.04
 //   600k, 400x300              5.65   4.93   4.68   4.64   4.73   4.86   5.07
 //   600k, 1600x1200           18.02  13.53  11.18  10.51  10.55  10.85  11.70
-//   1M, 160x120                8.08   7.56   7.71   7.75   8.01   8.13   8.45
 //   1M, 900x640               17.17  12.35  10.15   9.28   9.01   9.00   9.38
 //   1.5M, 1600x1200           39.01  26.43  19.72  16.40  15.10  14.88  15.43
 // and for 3M Gaussians in 100 views of 1256x828, the re-check included, 158
 // 118  97  86.1  79.8  77.2 (7: 76.5) 76.6.
 int fs::chunks_by_size(int views_per_batch, int64_t n, const fs_camera* cams, int32_t V) {
   if (n <= 0 || V <= 0) return 1;
-  const double tiles = mean_tiles(cams, V);
-  const double views = std::min(views_per_batch, V);
-  const double entries = views * static_cast<double>(n) * fs::entries_per_slot(cams, V);
-  const double by_depth = 3.0 + 1.3 * log2(static_cast<double>(n) / 3e5) -
-                          0.9 * std::max(0.0, log2(3000.0 / tiles));
-  const double per_chunk = 5.6e7 * pow(3e5 / static_cast<double>(n), 0.6);
-  const double chunks =
-      std::min({std::floor(by_depth + 0.5), std::floor(1.0 + entries / per_chunk), 8.0});
-  return std::max(1, static_cast<int>(chunks));
+  const double count = static_cast<double>(n), tiles = mean_tiles(cams, V);
+  const double by_n = std::floor(1.5 + 2.0 * log2(count / 262144.0));
+  const double by_tiles =
+      std::floor(3.5 + 1.3 * log2(count / 3e5) - 0.9 * std::max(0.0, log2(3000.0 / tiles)));
+  const double entries =
+      std::min(views_per_batch, V) * count * fs::entries_per_slot(cams, V);
+  const double paid = std::floor(1.0 + entries / (5.6e7 * pow(3e5 / count, 0.6)));
+  const double chunks = std::max(by_n, std::min(by_tiles, paid));
+  return std::max(1, static_cast<int>(std::min(chunks, 8.0)));
 }
 
 int fs::ctx_depth_chunks(const fs_ctx* c, int64_t n, const fs_camera* cams, int32_t V) {
