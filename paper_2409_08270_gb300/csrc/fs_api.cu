@@ -856,10 +856,12 @@ fs_status bin_positions(fs_ctx* c, int64_t p0, int64_t n_pos, int64_t n,
 // is not known before the pass: Gaussians of opacity 0.01 to 0.05, of which 81 %
 // and 57 % are live there, pay 0.3 ms of a solve's 31.
 constexpr int64_t kLiveMin = 1 << 22;
-// A list of more entries than this (8 GB with its sort's buffers) is cut into
-// parts: a depth chunk by its positions, when the context chose the number of
-// chunks, the re-check's list by its views.
+// A depth chunk's list of more entries than this (8 GB with its sort's buffers)
+// is cut into parts by its positions, when the context chose the number of
+// chunks.  The re-check's list is cut by its views only from kListEntries on,
+// the most one list can hold: every cut reads all of the batch's slots again.
 constexpr int64_t kSplitEntries = static_cast<int64_t>(1) << 29;
+constexpr int64_t kListEntries = (static_cast<int64_t>(1) << 31) - 1;
 // The next size of a part that had `entries` list entries, which were too many.
 int64_t smaller_part(int64_t part, int64_t entries) {
   const double fits = 0.85 * static_cast<double>(kSplitEntries) / static_cast<double>(entries);
@@ -1199,7 +1201,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
 
 // Dedicated binning of the tiles whose `skip` bit is clear (all depths, one
 // list per tile) and the re-check compositing of them into R.  A list of more
-// than kSplitEntries entries, or one there is no memory for, is made for some
+// than kListEntries entries, or one there is no memory for, is made for some
 // of the views at a time; `skip` then ends with the last views' tiles only.
 fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, int64_t kcap,
                               const BatchLayout& L, const fs::ViewParams* vd, const ProjPtrs& P,
@@ -1253,7 +1255,7 @@ fs_status recheck_batch_rebin(fs_ctx* c, const fs_scene* s, int64_t n, int nb, i
     int64_t I = 0;
     FS_TRY(bin_positions(c, 0, C, n, vd, nb, sorted_val, P, skip, total_tiles, tile_bits, kcap,
                          false, &c->lv_a, c->ranges.as<uint2>(), stream, &I, nullptr, false,
-                         ng > 1 ? kSplitEntries : 0));
+                         ng > 1 ? kListEntries : 0));
     if (I < 0) {
       want = static_cast<int>(smaller_part(ng, -I));
       continue;
