@@ -639,10 +639,12 @@ BatchLayout layout_batch(fs_ctx* c, fs::ViewParams* vh, const fs_camera* cams, i
   return L;
 }
 
-// Views per batch of V: (view, Gaussian) slots of one batch must fit in 31 bits.
-int batch_views(const fs_ctx* c, int64_t n, int32_t V) {
+// Views per batch: (view, Gaussian) slots of one batch must fit in 31 bits.  The
+// batch's buffers are sized for them whatever the call's own number of views: a
+// context that serves calls of differing numbers does not grow them again.
+int batch_views(const fs_ctx* c, int64_t n) {
   const int64_t max_vb = ((static_cast<int64_t>(1) << 31) - 1) / n;
-  return static_cast<int>(std::min<int64_t>(std::min(c->views_per_batch, V), max_vb));
+  return static_cast<int>(std::min<int64_t>(c->views_per_batch, max_vb));
 }
 
 // Projection storage of a batch: either the batch window (slot = view in
@@ -941,7 +943,7 @@ fs_status accumulate_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, i
   const int64_t n = s->n;
   c->kl_valid = false;
   if (n == 0 || V == 0) return FS_OK;
-  const int vb = batch_views(c, n, V);
+  const int vb = batch_views(c, n);
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   if (vb < 1) return fail(FS_UNSUPPORTED, "fs_accumulate: scene too large");
   const int64_t kcap = static_cast<int64_t>(vb) * n;
@@ -1327,7 +1329,7 @@ fs_status recheck_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int3
     Rb = c->rk_Rb.as<double>();
   }
 
-  const int vb = batch_views(c, n, V);
+  const int vb = batch_views(c, n);
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   const int64_t kcap = static_cast<int64_t>(vb) * n;
   fs::ViewParams* vh = c->views_host.as<fs::ViewParams>();
@@ -1467,7 +1469,7 @@ fs_status render_impl(fs_ctx* c, const fs_scene* s, const fs_camera* cams, int32
   } own_counters(c);
   unsigned long long* const ctr_h =
       reinterpret_cast<unsigned long long*>(c->total_host.as<char>() + 64);
-  const int vb = batch_views(c, n, V);
+  const int vb = batch_views(c, n);
   FS_TRY(ensure_free_tabs(c, cams, V, vb));
   if (vb < 1) return fail(FS_UNSUPPORTED, "fs_render_masks: scene too large");
   const int64_t kcap = static_cast<int64_t>(vb) * n;
@@ -1873,7 +1875,7 @@ fs_status fs_graph_create(fs_ctx* tmpl, const fs_scene* s, const fs_camera* cams
   g->keep = g->recheck && keep_fits(c, n, V);
   if (g->recheck) {
     if ((st = fs_create(&g->rc, tmpl->device, &o)) != FS_OK) return bail(st);
-    const int vbr = batch_views(g->rc, n, V);
+    const int vbr = batch_views(g->rc, n);
     if ((st = ensure_window(g->rc, n, vbr, V, false)) != FS_OK) return bail(st);
     if ((st = stage_masks(g->rc, cams, V, masks, mask_dtype, FS_MEM_DEVICE, nullptr)) != FS_OK)
       return bail(st);
@@ -1901,7 +1903,7 @@ fs_status fs_graph_create(fs_ctx* tmpl, const fs_scene* s, const fs_camera* cams
   if (st != FS_OK) return bail(st);
   if ((ce = cudaStreamSynchronize(g->stream)) != cudaSuccess)
     return bail(cuda_fail(ce, "fs_graph_create"));
-  const int vb = batch_views(c, n, V);
+  const int vb = batch_views(c, n);
   const size_t batches = static_cast<size_t>((V + vb - 1) / vb);
   if ((st = g->plan.views.ensure(batches * fs::kMaxViewsPerBatch * sizeof(fs::ViewParams))) !=
       FS_OK)

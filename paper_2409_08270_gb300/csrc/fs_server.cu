@@ -65,8 +65,9 @@ struct SceneEntry {
   double last_use = 0.0;
 };
 
-// Device bytes a request needs while it runs: the context's per-batch
-// window (records, footprints, boxes, keys, re-check flags), a depth chunk's
+// Device bytes a request needs while it runs: the context's window of one full
+// batch (records, footprints, boxes, keys, re-check flags; packed live slots and
+// their bits), a depth chunk's
 // list and its sort's buffers (16 B an entry; one chunk lists a whole batch,
 // several list ever fewer of its entries; scenes seen from near have about
 // twice the entries of the chunk rule's), the FP64 table and its rounding, the
@@ -77,7 +78,7 @@ int64_t footprint(int64_t n, int vb, int chunks, const std::vector<fs_camera>& c
   const int64_t nb = std::min<int64_t>(vb, V);
   if (chunks == 0) chunks = fs::chunks_by_size(vb, n, cams.data(), V);
   const double entries = std::max(2.0, 2.0 * fs::entries_per_slot(cams.data(), V) / chunks);
-  const int64_t window = nb * n * (64 + 32 + 4 * 9) +
+  const int64_t window = vb * n * (64 + 32 + 4 * 9) + vb * n * 9 / 4 +
                          static_cast<int64_t>(static_cast<double>(nb * n) * entries * 16);
   int64_t pixels = 0, batch_pixels = 0;
   for (size_t v = 0; v < cams.size(); ++v) {
@@ -282,19 +283,20 @@ bool drop_oldest_graph(fs_server* s, SceneEntry* self) {
 
 // The first request of a scene (autotune on): time a few batching settings
 // (views per batch, depth chunks) on a sample of its views and keep the fastest
-// for the scene.  The untuned setting, chunks by the size, comes first, after a
-// solve that takes the allocations, so that tuning does not end below it (one
-// request of 300,000 Gaussians, 24 views of 512x512: 4.95 ms untuned, 5.32 ms
-// with the best of four to six chunks).  A scene under kTuneBySize Gaussians
-// takes some milliseconds whichever it is and has fixed settings.
+// for the scene.  Where the size asks for fewer chunks than the fixed settings
+// have, the untuned setting is among them, after a solve that takes the
+// allocations, so that tuning does not end below it (one request of 300,000
+// Gaussians, 24 views of 512x512: 4.95 ms untuned, 5.32 ms with the best of four
+// to six chunks); five solves either way.  A scene under kTuneBySize Gaussians
+// takes some milliseconds whichever it is and has the fixed settings too.
 constexpr int64_t kTuneBySize = 1 << 16;
 void tune_scene(fs_server* s, int slot, SceneEntry& se, Request* r) {
   const int32_t V = static_cast<int32_t>(std::min<size_t>(r->cams.size(), 32));
   const int by_size = fs::chunks_by_size(se.views_per_batch, se.n, r->cams.data(), V);
   std::vector<std::pair<int, int>> cand = {{50, 6}, {32, 5}, {64, 6}, {16, 4}, {50, 4}};
   fs_stats st{};
-  if (se.n >= kTuneBySize) {
-    cand = {{50, 0}, {32, 0}, {64, 0}, {50, by_size + 1}, {50, by_size + 2}};
+  if (se.n >= kTuneBySize && by_size < 4) {
+    cand = {{50, 0}, {32, 0}, {64, 0}, {50, by_size + 1}};
     fs::ctx_set_batching(s->ctx[slot], 50, 0);
     solve_request(s, slot, se, r, V, &st);
   }

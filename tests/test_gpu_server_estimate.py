@@ -1,7 +1,7 @@
 """A request is admitted by an estimate of the device memory it needs, which
-must not lie below what a scene of few entries a slot then takes: its batch's
-views (not the largest batch's), and, with the one depth chunk that small scenes
-take, the lists of the whole batch."""
+must not lie below what a scene of few entries a slot then takes: the window of
+a full batch, and, with the one depth chunk that small scenes take, the lists
+of all its views."""
 import numpy as np
 import pytest
 
