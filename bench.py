@@ -493,7 +493,8 @@ def run_flashsplat(args, rank, world, local_rank):
                 "frac": (achieved / peak_tflops) if achieved else None,
                 "traffic": (BLEND_DRAM_BYTES_PER_PAIR * pairs / max(1, blend_launches)
                             if BLEND_DRAM_BYTES_PER_PAIR and blend_launches else None),
-                "traffic_unit": "DRAM bytes per launch (ncu capture scaled by work units)",
+                "traffic_unit": "DRAM bytes per launch (ncu capture, six depth chunks, scaled by work "
+                                "units)",
                 "peak_source": f"{n_sm} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {sm_clk:.0f} MHz",
                 "unit_of_work": "pair with alpha >= 1/255 reached before the pixel's stop "
                                 "(stop included), counted by a census solve",

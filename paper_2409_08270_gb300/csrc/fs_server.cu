@@ -67,11 +67,10 @@ struct SceneEntry {
 
 // Device bytes a request needs while it runs: the context's window of one full
 // batch (records, footprints, boxes, keys, re-check flags; packed live slots and
-// their bits), a depth chunk's
-// list and its sort's buffers (16 B an entry; one chunk lists a whole batch,
-// several list ever fewer of its entries; scenes seen from near have about
-// twice the entries of the chunk rule's), the FP64 table and its rounding, the
-// staged masks and the per-pixel state of one batch.
+// their bits), a depth chunk's list and its sort's buffers (16 B an entry; one
+// chunk lists a whole batch, several list ever fewer of its entries; scenes
+// seen from near have about twice the entries of the chunk rule's), the FP64
+// table and its rounding, the staged masks and the per-pixel state of one batch.
 int64_t footprint(int64_t n, int vb, int chunks, const std::vector<fs_camera>& cams,
                   int32_t mask_dtype, int32_t E) {
   const int32_t V = static_cast<int32_t>(cams.size());
